@@ -69,6 +69,62 @@ size_t factored_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
     return kStatusBytes + (most > skinny ? most : skinny);
 }
 
+// ---- operands that TMA cannot address ----
+// A bf16 operand whose rows do not all start on 16-byte boundaries is copied to the end of the workspace with a padded
+// pitch (pack_rows.cu) and the tensor-core kernels run on the copy.  velora_workspace_bytes reports the room for the
+// operands whose width is no multiple of 8; a workspace without that room is as good as it ever was (the call then
+// runs on the CUDA cores), and other misaligned operands (an offset view) are copied where the room happens to be
+// there.  Measured on a 4096 x 2048 -> 5461 layer with dense rows: 3360 us a product on the CUDA cores.
+bool packable(int64_t rows, int64_t cols) { return rows >= 1 && rows < (1 << 30) && cols >= 1 && cols < (1 << 30); }
+
+size_t pack_bytes_if_ragged(int64_t rows, int64_t cols)
+{
+    return cols % 8 && packable(rows, cols) ? pack_rows_bytes(rows, cols) : 0;
+}
+
+struct Operand {
+    const void* p;
+    int64_t ld;
+    int64_t rows, cols;
+};
+
+// Replaces those of the operands (at most two) that need it by copies at ws + used; all of them or none.
+int pack_operands(Operand** ops, int count, void* ws, size_t ws_bytes, size_t used, cudaStream_t stream)
+{
+    PackJob jobs[2];
+    Operand* packed[2];
+    int n = 0;
+    char* at = static_cast<char*>(ws) + used;
+    size_t need = used;
+    for (int i = 0; i < count; ++i) {
+        Operand& o = *ops[i];
+        if (tc_operand_ok(o.p, o.ld)) continue;
+        if (!packable(o.rows, o.cols)) return VELORA_OK;
+        const size_t bytes = pack_rows_bytes(o.rows, o.cols);
+        need += bytes;
+        if (need > ws_bytes) return VELORA_OK;
+        jobs[n] = PackJob{o.p, o.ld, o.rows, o.cols, at};
+        packed[n++] = &o;
+        at += bytes;
+    }
+    if (n == 0) return VELORA_OK;
+    const int rc = launch_pack_rows(jobs, n, stream);
+    if (rc == VELORA_ERR_UNSUPPORTED) return VELORA_OK;
+    if (rc != VELORA_OK) return rc;
+    for (int i = 0; i < n; ++i) {
+        packed[i]->p = jobs[i].dst;
+        packed[i]->ld = pack_rows_pitch(packed[i]->cols);
+    }
+    return VELORA_OK;
+}
+
+// The weight gradient's kernels that read dY through TMA: the dense product, and the factored form but for adapter
+// shapes (plain loads) and rows of more than 256 sub-tokens (CUDA cores).
+bool weight_grad_wants_tma(int64_t D, int64_t O, int Dsub, int mode)
+{
+    return mode == VELORA_WG_EXPLICIT || (O > 64 && num_subtokens(D, Dsub) <= 256);
+}
+
 // ---- weight gradient routing ----
 int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
                      const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
@@ -198,11 +254,12 @@ size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub)
     if (N < 0 || D < 1 || Dsub < 1 || Dsub > D || Dsub > VELORA_MAX_DSUB) return 0;
     switch (op) {
         case VELORA_OP_INIT_V: return init_v_workspace_bytes(Dsub);
-        case VELORA_OP_WEIGHT_GRAD_FACTORED:
-        case VELORA_OP_LINEAR_BACKWARD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub);
-        case VELORA_OP_WEIGHT_GRAD_EXPLICIT:
-        case VELORA_OP_LINEAR_BACKWARD_EXPLICIT: return xhat_bytes(N, D);
-        case VELORA_OP_LINEAR_FORWARD: return kStatusBytes;
+        case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O);
+        case VELORA_OP_LINEAR_BACKWARD_FACTORED:
+            return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O) + pack_bytes_if_ragged(O, D);
+        case VELORA_OP_WEIGHT_GRAD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O);
+        case VELORA_OP_LINEAR_BACKWARD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O) + pack_bytes_if_ragged(O, D);
+        case VELORA_OP_LINEAR_FORWARD: return kStatusBytes + pack_bytes_if_ragged(N, D) + pack_bytes_if_ragged(O, D);
         case VELORA_OP_UPDATE_V: return update_v_workspace_bytes(Dsub);
         case VELORA_OP_Z8_CALIBRATE: return z8_calibrate_workspace_bytes(N, D, Dsub);
         default: return 0;
@@ -261,11 +318,15 @@ int velora_weight_grad(const void* dY, int dy_dtype, int64_t N, int64_t O, int64
     int rc = check_weight_grad_args(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub,
                                     dW, dw_dtype, lddw, beta, mode, ws);
     if (rc != VELORA_OK) return rc;
-    const size_t need = velora_workspace_bytes(mode == VELORA_WG_FACTORED ? VELORA_OP_WEIGHT_GRAD_FACTORED
-                                                                          : VELORA_OP_WEIGHT_GRAD_EXPLICIT,
-                                               N, D, O, Dsub);
+    const size_t need = mode == VELORA_WG_FACTORED ? factored_bytes(N, D, O, Dsub) : xhat_bytes(N, D);
     if (ws_bytes < need) return VELORA_ERR_WORKSPACE;
-    return weight_grad_impl(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
+    Operand y{dY, lddy, N, O};
+    if (N > 0 && dy_dtype == VELORA_BF16 && weight_grad_wants_tma(D, O, Dsub, mode)) {
+        Operand* ops[1] = {&y};
+        rc = pack_operands(ops, 1, ws, ws_bytes, need, static_cast<cudaStream_t>(stream));
+        if (rc != VELORA_OK) return rc;
+    }
+    return weight_grad_impl(y.p, dy_dtype, N, O, y.ld, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
                             beta, mode, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }
 
@@ -287,7 +348,13 @@ int velora_linear_forward(const void* X, int64_t ldx, const void* W, int64_t ldw
     if (!ws || ws_bytes < kStatusBytes) return VELORA_ERR_WORKSPACE;
     if (!aligned16(ws)) return VELORA_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    rc = launch_linear_forward_tc(X, ldx, W, ldw, v, Y, ldy, Z, z_dtype, ldz, dtype, N, D, O, Dsub,
+    Operand x{X, ldx, N, D}, w{W, ldw, O, D};
+    if (dtype == VELORA_BF16) {
+        Operand* ops[2] = {&x, &w};
+        rc = pack_operands(ops, 2, ws, ws_bytes, kStatusBytes, s);
+        if (rc != VELORA_OK) return rc;
+    }
+    rc = launch_linear_forward_tc(x.p, x.ld, w.p, w.ld, v, Y, ldy, Z, z_dtype, ldz, dtype, N, D, O, Dsub,
                                   static_cast<int*>(ws), s);
     if (rc != VELORA_ERR_UNSUPPORTED) return rc;
     rc = launch_gemm_simt(X, dtype, ldx, 1, W, dtype, ldw, 1, Y, dtype, ldy, 0, N, O, D, s);
@@ -315,20 +382,27 @@ int velora_linear_backward(const void* dY, int64_t lddy, const void* W, int64_t 
         if (ldw < D || lddx < D) return VELORA_ERR_INVALID_ARG;
         if (!elem_aligned(W, dtype) || !elem_aligned(dX, dtype)) return VELORA_ERR_ALIGNMENT;
     }
+    size_t used = kStatusBytes;                               /* of the workspace, before the copies of ragged operands */
     if (dW) {
         rc = check_weight_grad_args(dY, dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub,
                                     dW, dw_dtype, lddw, beta, mode, ws);
         if (rc != VELORA_OK) return rc;
-        const size_t need = velora_workspace_bytes(mode == VELORA_WG_FACTORED ? VELORA_OP_LINEAR_BACKWARD_FACTORED
-                                                                              : VELORA_OP_LINEAR_BACKWARD_EXPLICIT,
-                                                   N, D, O, Dsub);
-        if (ws_bytes < need) return VELORA_ERR_WORKSPACE;
+        used = mode == VELORA_WG_FACTORED ? factored_bytes(N, D, O, Dsub) : xhat_bytes(N, D);
+        if (ws_bytes < used) return VELORA_ERR_WORKSPACE;
     }
     if (!ws || ws_bytes < kStatusBytes) return VELORA_ERR_WORKSPACE;
     if (!aligned16(ws)) return VELORA_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    Operand y{dY, lddy, N, O}, w{W, ldw, O, D};
+    if (N > 0 && dtype == VELORA_BF16 && (dX || (dW && weight_grad_wants_tma(D, O, Dsub, mode)))) {
+        Operand* ops[2] = {&y, &w};
+        rc = pack_operands(ops, dX ? 2 : 1, ws, ws_bytes, used, s);
+        if (rc != VELORA_OK) return rc;
+    }
+    dY = y.p;
+    lddy = y.ld;
     if (dX && N > 0) {
-        rc = launch_gemm_tc(GEMM_NN_K_MN, dY, lddy, W, ldw, dX, dtype, lddx, 0, N, D, O, dtype,
+        rc = launch_gemm_tc(GEMM_NN_K_MN, dY, lddy, w.p, w.ld, dX, dtype, lddx, 0, N, D, O, dtype,
                             static_cast<int*>(ws), s);
         if (rc == VELORA_ERR_UNSUPPORTED)
             rc = launch_gemm_simt(dY, dtype, lddy, 1, W, dtype, 1, ldw, dX, dtype, lddx, 0, N, D, O, s);
@@ -503,6 +577,14 @@ int velora_weight_grad_p(const void* dY, int dy_dtype, int64_t N, int64_t O, int
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* status = static_cast<int*>(ws);
     char* body = static_cast<char*>(ws) + kStatusBytes;
+    Operand y{dY, lddy, N, O};
+    if (N > 0 && dy_dtype == VELORA_BF16 && weight_grad_wants_tma(D, O, Dsub, VELORA_WG_FACTORED)) {
+        Operand* ops[1] = {&y};
+        rc = pack_operands(ops, 1, ws, ws_bytes, factored_bytes(N, D, O, Dsub), st);
+        if (rc != VELORA_OK) return rc;
+        dY = y.p;
+        lddy = y.ld;
+    }
     if (N > 0) {
         rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D,
                                        beta, body, ws_bytes - kStatusBytes, st, P, ldp);

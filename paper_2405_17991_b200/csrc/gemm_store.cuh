@@ -16,6 +16,9 @@ __device__ __forceinline__ void st_global_32B(void* p, const uint4& a, const uin
                  ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
 }
 
+// Whether every row of an output starts on a 16-byte boundary (vector stores) or not (staged rows).
+inline int c_rows_vec(const void* C, int64_t ldc, size_t elem) { return aligned16(C) && (ldc * static_cast<int64_t>(elem)) % 16 == 0; }
+
 template <typename CT> struct Store32;
 template <> struct Store32<__nv_bfloat16> {
     // 32 consecutive outputs of one row.
@@ -93,5 +96,32 @@ template <> struct Store32<float> {
         }
     }
 };
+
+// Output rows that start on any element (odd pitch, no padding): a lane that stores its own row would touch 32
+// sectors per instruction, two bytes in each.  The warp turns its 32 x 32 block over through shared memory (32 rows of
+// kStagePitch floats; the odd pitch keeps both directions free of bank conflicts) and writes one row at a time,
+// consecutive lanes to consecutive columns.  All lanes call; `valid` columns are the same for all of them.
+constexpr int kStagePitch = 33;
+constexpr int kStageFloats = 32 * kStagePitch;
+
+template <typename CT>
+__device__ __forceinline__ void store_rows_staged(CT* block, int64_t ldc, int rows, int valid, const uint32_t (&r)[32], int beta,
+                                                  float* stage, int lane)
+{
+#pragma unroll
+    for (int e = 0; e < 32; ++e) stage[lane * kStagePitch + e] = __uint_as_float(r[e]);
+    __syncwarp();
+    if (lane < valid) {
+        CT* p = block + lane;
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i, p += ldc) {
+            if (i >= rows) break;
+            float f = stage[i * kStagePitch + lane];
+            if (beta) f += Elem<CT>::load(p);
+            Elem<CT>::store(p, f);
+        }
+    }
+    __syncwarp();
+}
 
 }  // namespace velora

@@ -27,7 +27,8 @@ constexpr int SLAB_BYTES = 64 * BK * 2;           // one 64-wide MN-major slab: 
 constexpr int GEMM_THREADS = 192;
 constexpr int TMEM_COLS = 512;
 constexpr int FUSE_THREADS = GEMM_THREADS + 192;    // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
-constexpr size_t GEMM_SMEM = 1024 + static_cast<size_t>(STAGES) * (A_BYTES + B_BYTES) + 256;
+constexpr int STAGE_OFF = 256;                    // behind the ring: barriers, then the staging of unaligned output rows
+constexpr size_t GEMM_SMEM = 1024 + static_cast<size_t>(STAGES) * (A_BYTES + B_BYTES) + STAGE_OFF + 4 * kStageFloats * sizeof(float);
 constexpr size_t FUSE_SMEM = GEMM_SMEM;
 
 struct TileCoord {
@@ -59,7 +60,7 @@ template <bool A_MN, bool B_MN, typename CT, int FUSE>
 __global__ void __launch_bounds__(FUSE ? FUSE_THREADS : GEMM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
-               int tiles_m, int tiles_n, int* __restrict__ status, const FuseArgs fz)
+               int tiles_m, int tiles_n, int c_vec, int* __restrict__ status, const FuseArgs fz)
 {
     static_assert(FUSE == 0 || (!A_MN && !B_MN), "compress rides on the K-major forward GEMM only");
     extern __shared__ uint8_t smem_raw[];
@@ -224,7 +225,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (lane == 0) mbar_arrive(tempty + 8 * acc);
                 }
                 const int valid = Ndim - (tc0.n0 + c * 32);
-                if (row < Mdim && valid > 0) Store32<CT>::run(crow + c * 32, r, valid, beta);
+                if (valid <= 0) continue;
+                if (!c_vec) {
+                    const int row0 = tc0.m0 + quarter * 32;
+                    if (row0 < Mdim)
+                        store_rows_staged<CT>(C + static_cast<int64_t>(row0) * ldc + tc0.n0 + c * 32, ldc, Mdim - row0, valid, r, beta,
+                                              reinterpret_cast<float*>(tail + STAGE_OFF) + quarter * kStageFloats, lane);
+                } else if (row < Mdim) {
+                    Store32<CT>::run(crow + c * 32, r, valid, beta);
+                }
             }
         }
         if (failed) *abort_flag = 1;
@@ -281,7 +290,7 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     const int64_t tiles = static_cast<int64_t>(tiles_m) * tiles_n;
     const int grid = static_cast<int>(tiles < di.sm_count ? tiles : di.sm_count);
     kern<<<grid, FUSE ? FUSE_THREADS : GEMM_THREADS, FUSE ? FUSE_SMEM : GEMM_SMEM, stream>>>(
-        ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, status, fz);
+        ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, c_rows_vec(C, ldc, sizeof(CT)), status, fz);
     return after_launch();
 }
 
@@ -340,7 +349,6 @@ int launch_gemm_tc(int kind, const void* A, int64_t lda, const void* B, int64_t 
     if (Mdim < 1 || Ndim < 1 || Kdim < 1) return VELORA_ERR_UNSUPPORTED;
     if (Mdim > (1 << 30) || Ndim > (1 << 30) || Kdim > (1 << 30)) return VELORA_ERR_UNSUPPORTED;
     if (!tc_operand_ok(A, lda) || !tc_operand_ok(B, ldb)) return VELORA_ERR_UNSUPPORTED;
-    if (!aligned16(C) || (ldc * static_cast<int64_t>(dtype_size(c_dtype))) % 16) return VELORA_ERR_UNSUPPORTED;
     if ((static_cast<int64_t>((Mdim + BM - 1) / BM) * ((Ndim + BN - 1) / BN)) > (1 << 30)) return VELORA_ERR_UNSUPPORTED;
 
     if (gemm_pair_preferred(Mdim, Ndim)) {
@@ -380,7 +388,7 @@ int launch_linear_forward_tc(const void* X, int64_t ldx, const void* W, int64_t 
     }
     const bool pow2 = Dsub >= 8 && Dsub <= VELORA_MAX_DSUB && (Dsub & (Dsub - 1)) == 0;
     const bool gemm_ok = dtype == VELORA_BF16 && N >= 1 && N < (1 << 30) && D < (1 << 30) && O < (1 << 30) &&
-                         tc_operand_ok(X, ldx) && tc_operand_ok(W, ldw) && aligned16(Y) && ldy % 8 == 0;
+                         tc_operand_ok(X, ldx) && tc_operand_ok(W, ldw);
     // One CTA compresses one k-block in tiles_n; with fewer than four n-tiles the compress warps would
     // hold the producer back, so narrow outputs take the two-kernel route as well.
     const bool wide = (O + BN - 1) / BN >= 4;

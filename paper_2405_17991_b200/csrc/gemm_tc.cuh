@@ -42,6 +42,19 @@ bool gemm_pair_preferred(int64_t Mdim, int64_t Ndim);
 int make_tmap_bf16_2d(CUtensorMap* map, const void* base, int64_t inner, int64_t outer, int64_t ld_elems,
                       int box_inner, int box_outer, bool swizzle128 = true);
 bool tc_operand_ok(const void* p, int64_t ld_elems);
+
+// Copies of bf16 matrices with a row pitch of pack_rows_pitch(cols) elements, for operands whose rows a tensor map
+// cannot describe.  `dst` is 16-byte aligned and holds pack_rows_bytes(rows, cols); up to two matrices a launch.
+// Columns cols .. pitch - 1 of the copy hold anything.  (pack_rows.cu)
+struct PackJob {
+    const void* src;
+    int64_t ld, rows, cols;
+    void* dst;
+};
+int64_t pack_rows_pitch(int64_t cols);
+size_t pack_rows_bytes(int64_t rows, int64_t cols);
+int launch_pack_rows(const PackJob* jobs, int count, cudaStream_t stream);
+
 // The same matrix seen as [64 elements][outer rows][inner / 64 column chunks] (inner a multiple of 64): a box of
 // box_rows rows x box_chunks chunks lands in shared memory as box_chunks tiles of box_rows x 128 bytes, each
 // swizzled like a two-dimensional 64-column box, from box_chunks * 128 contiguous bytes of every row.

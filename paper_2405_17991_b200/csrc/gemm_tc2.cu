@@ -47,7 +47,8 @@ constexpr int P_SLAB = 64 * P_BK * 2;               // 8 KB, one 64-wide MN-majo
 constexpr int P_THREADS = 192;
 constexpr int P_TMEM_COLS = 512;
 constexpr int P_FUSE_THREADS = P_THREADS + 192;      // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
-constexpr size_t P_SMEM = 1024 + static_cast<size_t>(P_STAGES) * P_STAGE_BYTES + 256;
+constexpr int P_STAGE_OFF = 256;                     // behind the ring: barriers, then the staging of unaligned output rows
+constexpr size_t P_SMEM = 1024 + static_cast<size_t>(P_STAGES) * P_STAGE_BYTES + P_STAGE_OFF + 4 * kStageFloats * sizeof(float);
 constexpr size_t P_FUSE_SMEM = P_SMEM;
 
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank)
@@ -118,7 +119,7 @@ template <bool A_MN, bool B_MN, typename CT, int FUSE>
 __global__ void __launch_bounds__(FUSE ? P_FUSE_THREADS : P_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
-                 int tiles_m, int tiles_n, int* __restrict__ status, const FuseArgs fz)
+                 int tiles_m, int tiles_n, int c_vec, int* __restrict__ status, const FuseArgs fz)
 {
     static_assert(FUSE == 0 || (!A_MN && !B_MN), "compress rides on the K-major forward GEMM only");
     namespace cg = cooperative_groups;
@@ -301,7 +302,15 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8 * acc);
                 }
                 const int valid = Ndim - (t0.n0 + c * 32);
-                if (row < Mdim && valid > 0) Store32<CT>::run(crow + c * 32, r, valid, beta);
+                if (valid <= 0) continue;
+                if (!c_vec) {
+                    const int row0 = row - lane;
+                    if (row0 < Mdim)
+                        store_rows_staged<CT>(C + static_cast<int64_t>(row0) * ldc + t0.n0 + c * 32, ldc, Mdim - row0, valid, r, beta,
+                                              reinterpret_cast<float*>(tail + P_STAGE_OFF) + quarter * kStageFloats, lane);
+                } else if (row < Mdim) {
+                    Store32<CT>::run(crow + c * 32, r, valid, beta);
+                }
             }
         }
         if (failed) *abort_flag = 1;
@@ -349,7 +358,8 @@ int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t l
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, status, fz) !=
+    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n,
+                           c_rows_vec(C, ldc, sizeof(CT)), status, fz) !=
         cudaSuccess) {
         cudaGetLastError();
         return VELORA_ERR_CUDA;
@@ -367,7 +377,6 @@ int launch_gemm_tc_pair(int kind, const void* A, int64_t lda, const void* B, int
     if (Mdim < 1 || Ndim < 1 || Kdim < 1) return VELORA_ERR_UNSUPPORTED;
     if (Mdim > (1 << 30) || Ndim > (1 << 30) || Kdim > (1 << 30)) return VELORA_ERR_UNSUPPORTED;
     if (!tc_operand_ok(A, lda) || !tc_operand_ok(B, ldb)) return VELORA_ERR_UNSUPPORTED;
-    if (!aligned16(C) || (ldc * static_cast<int64_t>(dtype_size(c_dtype))) % 16) return VELORA_ERR_UNSUPPORTED;
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc != VELORA_OK) return rc;

@@ -1,0 +1,125 @@
+// Rows that TMA cannot address, copied to rows that it can.
+//
+// A tensor map wants a 16-byte aligned base and a row pitch that is a multiple of 16 bytes; a bf16 matrix as a
+// framework allocates it (5461 columns, no padding) has neither.  Such an operand is copied once into the
+// workspace and the tensor-core kernels run on the copy.  The copy is one read and one write of the operand; without
+// it the product runs on the CUDA cores.  The copy's pitch is a multiple of 128 bytes, not of the 16 that TMA asks for:
+// a 4096 x 5461 -> 2048 product took 84 us with both operands at a pitch of 10928 bytes (every other row starts in
+// the middle of a 32-byte sector) and 70 us at 11008.
+//
+// A warp takes 256 consecutive 16-byte chunks of a row, eight per lane, all loads issued before the first is used.
+// The source of a chunk sits at any even byte offset, so a lane loads the two aligned 16-byte chunks that cover it
+// (the second is its neighbour's first: an L1 hit) and shifts; the offset is the same for a whole row.
+#include "gemm_tc.cuh"
+
+namespace velora {
+namespace {
+
+constexpr int PK_THREADS = 256;
+constexpr int PK_U = 8;                                    // chunks per lane
+constexpr int PK_SEG = 32 * PK_U;                          // chunks per warp and step
+
+struct PackArgs {
+    const char* src[2];
+    const char* src_end[2];                                // one past the last element
+    int64_t src_pitch[2];                                  // bytes
+    uint4* dst[2];
+    int64_t dst_pitch[2];                                  // chunks
+    int chunks[2], segs[2];
+    int64_t items[2];                                      // rows x segments
+};
+
+__device__ __forceinline__ uint4 load_unaligned(const char* p, const char* lo_limit, const char* hi_limit)
+{
+    const uint32_t s = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p) & 15u);
+    const char* a = p - s;
+    uint32_t w[8];
+    if (a >= lo_limit && a + (s ? 32 : 16) <= hi_limit) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(a));
+        uint4 y = make_uint4(0u, 0u, 0u, 0u);
+        if (s) y = __ldg(reinterpret_cast<const uint4*>(a) + 1);
+        w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
+        w[4] = y.x; w[5] = y.y; w[6] = y.z; w[7] = y.w;
+    } else {
+        // The first and the last chunks of the matrix: no byte outside it is touched.
+        uint32_t o[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (p + 2 * e < hi_limit)
+                o[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(p + 2 * e)) << (16 * (e & 1));
+        return make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    if (s & 8u) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+    }
+    if (s & 4u) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+    }
+    const uint32_t bits = (s & 2u) * 8u;
+    return make_uint4(__funnelshift_r(w[0], w[1], bits), __funnelshift_r(w[1], w[2], bits),
+                      __funnelshift_r(w[2], w[3], bits), __funnelshift_r(w[3], w[4], bits));
+}
+
+__global__ void __launch_bounds__(PK_THREADS)
+pack_rows_kernel(const PackArgs a)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (PK_THREADS / 32);
+    const int64_t total = a.items[0] + a.items[1];
+    for (int64_t it = static_cast<int64_t>(blockIdx.x) * (PK_THREADS / 32) + (threadIdx.x >> 5); it < total; it += warps) {
+        const int k = it < a.items[0] ? 0 : 1;
+        const unsigned item = static_cast<unsigned>(it - (k ? a.items[0] : 0));
+        const unsigned row = item / static_cast<unsigned>(a.segs[k]);
+        const int c0 = static_cast<int>(item - row * a.segs[k]) * PK_SEG + lane;
+        const char* rp = a.src[k] + static_cast<int64_t>(row) * a.src_pitch[k];
+        uint4 d[PK_U];
+#pragma unroll
+        for (int u = 0; u < PK_U; ++u)
+            if (c0 + 32 * u < a.chunks[k]) d[u] = load_unaligned(rp + 16 * static_cast<int64_t>(c0 + 32 * u), a.src[k], a.src_end[k]);
+        uint4* op = a.dst[k] + static_cast<int64_t>(row) * a.dst_pitch[k];
+#pragma unroll
+        for (int u = 0; u < PK_U; ++u)
+            if (c0 + 32 * u < a.chunks[k]) op[c0 + 32 * u] = d[u];
+    }
+}
+
+}  // namespace
+
+int64_t pack_rows_pitch(int64_t cols) { return (cols + 63) / 64 * 64; }
+
+size_t pack_rows_bytes(int64_t rows, int64_t cols)
+{
+    return (static_cast<size_t>(rows) * static_cast<size_t>(pack_rows_pitch(cols)) * 2 + 255) / 256 * 256;
+}
+
+int launch_pack_rows(const PackJob* jobs, int count, cudaStream_t stream)
+{
+    PackArgs a{};
+    for (int k = 0; k < count && k < 2; ++k) {
+        const PackJob& j = jobs[k];
+        if (j.rows < 1 || j.rows >= (1 << 30) || j.cols < 1 || j.cols >= (1 << 30)) return VELORA_ERR_UNSUPPORTED;
+        a.src[k] = static_cast<const char*>(j.src);
+        a.src_pitch[k] = j.ld * 2;
+        a.src_end[k] = a.src[k] + ((j.rows - 1) * j.ld + j.cols) * 2;
+        a.dst[k] = static_cast<uint4*>(j.dst);
+        a.chunks[k] = static_cast<int>((j.cols + 7) / 8);
+        a.dst_pitch[k] = pack_rows_pitch(j.cols) / 8;
+        a.segs[k] = (a.chunks[k] + PK_SEG - 1) / PK_SEG;
+        a.items[k] = j.rows * a.segs[k];
+        if (a.items[k] >= (static_cast<int64_t>(1) << 31)) return VELORA_ERR_UNSUPPORTED;
+    }
+    const int64_t items = a.items[0] + a.items[1];
+    if (items == 0) return VELORA_OK;
+    DeviceInfo di;
+    const int rc = device_info(&di);
+    if (rc != VELORA_OK) return rc;
+    int64_t grid = ceil_div64(items, PK_THREADS / 32);
+    const int64_t cap = static_cast<int64_t>(di.sm_count) * kStreamCtasPerSm;
+    if (grid > cap) grid = cap;
+    pack_rows_kernel<<<static_cast<int>(grid), PK_THREADS, 0, stream>>>(a);
+    return after_launch();
+}
+
+}  // namespace velora

@@ -1,0 +1,92 @@
+"""Rows on odd boundaries (no padding, odd pitch, offset views): the tensor-core path through packed copies, the staged
+output stores, and the same calls with a workspace that has no room for the copies.
+
+Outputs are guard-banded with the pitch under test, so a store next to a row is seen; bounds are those of ``_util``.
+"""
+import pytest
+import torch
+
+import oracle
+import velora_inputs as vi
+from _util import C_ROUNDED, TOL_GEMM, TOL_Z, Guard, assert_matches, to_f64
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def vl():
+    import paper_2405_17991_b200 as pkg
+    pkg.lib()
+    return pkg
+
+
+@pytest.fixture
+def guard():
+    g = Guard(DEV)
+    yield g
+    g.check()
+
+
+def _view(t, ld, offset):
+    """The same values with row pitch ``ld``, starting ``offset`` elements into a buffer that ends with the last one."""
+    n, d = t.shape
+    buf = torch.full((offset + (n - 1) * ld + d,), float("nan"), dtype=t.dtype, device=t.device)
+    out = buf.as_strided((n, d), (ld, 1), offset)
+    out.copy_(t)
+    return out
+
+
+# N, D, O, Dsub: one tile and less, tile edges, several tiles of the CTA-pair kernel, adapter width, whole rows of
+# 8-element chunks beside ragged ones, sub-tokens that are no power of two.
+CASES = [(37, 257, 131, 16), (300, 321, 520, 64), (129, 200, 77, 24), (1100, 2049, 1801, 128), (2500, 640, 2731, 64), (513, 1023, 16, 32),
+         (200, 130, 1031, 130)]
+
+
+@pytest.mark.parametrize("N,D,O,Dsub", CASES)
+@pytest.mark.parametrize("pad,offset", [(0, 0), (3, 1), (8, 4)])
+@pytest.mark.parametrize("room", [True, False])
+def test_layer_on_rows_that_start_anywhere(vl, guard, N, D, O, Dsub, pad, offset, room):
+    if not room and N * D * O > 1 << 27:
+        pytest.skip("the CUDA-core route at this size adds nothing")
+    case = vi.small_case(11 * N + D, N, D, O, dtype="bf16", mean_offset=0.1)
+    X, W, dY = (_view(case[k].torch(DEV), case[k].torch(DEV).shape[1] + pad, offset) for k in ("X", "W", "dY"))
+    X64, W64, dY64 = (case[k].f64() for k in ("X", "W", "dY"))
+    v = vl.velora_init_v(X, Dsub)
+    v64 = to_f64(v)
+    assert_matches(v, oracle.init_v(X64, Dsub), TOL_Z, "v")
+    M = vl.num_subtokens(D, Dsub)
+
+    def ws(op):
+        nbytes = vl.velora_workspace_bytes(op, N, D, O, Dsub)
+        if not room:                                     # what the same widths need with padded rows
+            nbytes = 256 if op == vl.OP_LINEAR_FORWARD else vl.velora_workspace_bytes(op, N, D, -(-O // 8) * 8, Dsub)
+        return guard.workspace(vl, nbytes)
+
+    Y, Z = vl.velora_linear_forward(X, W, v, Y=guard.mat(N, O, ld=O + pad), Z=guard.mat(N, M, torch.float32), ws=ws(vl.OP_LINEAR_FORWARD))
+    assert_matches(Z, oracle.compress(X64, v64), TOL_Z, "Z")
+    assert_matches(Y, oracle.linear_forward(X64, W64), TOL_GEMM, "Y")
+    dX, dW = vl.velora_linear_backward(dY, W, Z, v, dX=guard.mat(N, D, ld=D + pad), dW=guard.mat(O, D, ld=D + pad),
+                                       ws=ws(vl.OP_LINEAR_BACKWARD_FACTORED))
+    dW_ref = oracle.weight_grad(dY64, to_f64(Z), v64, D)
+    assert_matches(dX, oracle.input_grad(dY64, W64), TOL_GEMM, "dX")
+    assert_matches(dW, dW_ref, TOL_GEMM, "dW", c=C_ROUNDED)
+    for mode, op in ((vl.WG_FACTORED, vl.OP_WEIGHT_GRAD_FACTORED), (vl.WG_EXPLICIT, vl.OP_WEIGHT_GRAD_EXPLICIT)):
+        got = vl.velora_weight_grad(dY, Z, v, D, dW=guard.mat(O, D, torch.float32, ld=D + pad), mode=mode, ws=ws(op))
+        assert_matches(got, dW_ref, TOL_GEMM, "dW mode %d" % mode, c=C_ROUNDED)
+    P = vl.velora_weight_grad_p(dY, Z, D, Dsub, P=guard.mat(O, M, torch.float32), ws=ws(vl.OP_WEIGHT_GRAD_FACTORED))
+    assert_matches(P, oracle.linear_forward(dY64.T, to_f64(Z).T), TOL_GEMM, "P", c=C_ROUNDED)
+
+
+@pytest.mark.parametrize("c_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("Mdim,Ndim,Kdim", [(130, 259, 64), (40, 31, 264), (2600, 2051, 128)])
+def test_products_add_to_an_output_with_odd_rows(vl, guard, c_dtype, Mdim, Ndim, Kdim):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(Mdim)
+    A = torch.randn((Mdim, Kdim), generator=g, device=DEV).to(torch.bfloat16)
+    B = torch.randn((Ndim, Kdim), generator=g, device=DEV).to(torch.bfloat16)
+    C0 = torch.randn((Mdim, Ndim), generator=g, device=DEV).to(c_dtype)
+    C = guard.mat(Mdim, Ndim, c_dtype, ld=Ndim, init=C0)
+    vl.velora_dense_product(vl.PRODUCT_A_BT, A, B, C=C, beta=1)
+    assert_matches(C, to_f64(A) @ to_f64(B).T + to_f64(C0), TOL_GEMM, "C")
