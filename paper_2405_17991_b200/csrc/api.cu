@@ -142,7 +142,7 @@ int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t
     }
     if (mode == VELORA_WG_FACTORED) {
         if (ws_bytes < factored_bytes(N, D, O, Dsub)) return VELORA_ERR_WORKSPACE;
-        // Adapter-shaped layers (O <= 64) first: too few output tiles for the tensor-core kernel to spread.
+        // Adapter-shaped layers (O <= 64; too few output tiles for the tensor-core kernel to spread) and fp32 first.
         int rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
                                            beta, body, ws_bytes - kStatusBytes, stream, nullptr, 0);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;

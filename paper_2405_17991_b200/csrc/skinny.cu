@@ -8,6 +8,8 @@
 // most 8 CTAs pull on dY and Z); here the tokens are cut into up to 512 slices, each CTA forms the partial P of
 // its slice on the CUDA cores, a second kernel adds the partials in a fixed order, and the common expansion
 // kernel writes dW.  All sums are fp32, products are formed from the stored values (Z is not rounded to bf16).
+// The same kernel, with the output columns in blocks of 64, serves fp32 layers of any width (12608 tokens, 768 columns, 24
+// sub-tokens: 904 us as a general fp32 product whose 12 output tiles left most SMs idle, 39 us here).
 //
 //  2. the forward, Y = X W^T and Z = compress(X, v) in one pass over X (further down).
 #include "common.cuh"
@@ -25,16 +27,19 @@ constexpr int SK_THREADS = 256;
 constexpr int SK_CHUNK = 32;          // tokens staged in shared memory at a time
 constexpr int SK_MAX_O = 64;
 constexpr int SK_MAX_M = 256;
+constexpr int SK_DIRECT_PARTS = 8;    // slices that the expansion kernel adds up itself
 
-// Thread (warp w, lane l) owns outputs o = w + 8 i (i < OI), m = l + 32 j (j < MJ).
+// Thread (warp w, lane l) owns outputs o = OI w + i (i < OI; one or two broadcast loads bring them), m = l + 32 j (j < MJ)
+// of the 8 OI columns of block blockIdx.y.
 template <typename YT, typename ZT, int OI, int MJ>
 __global__ void __launch_bounds__(SK_THREADS)
 wg_skinny_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __restrict__ Z, int64_t ldz,
                          int N, int O, int M, int tokens_per_cta, float* __restrict__ partials)
 {
-    __shared__ float sdy[SK_CHUNK][8 * OI];
+    __shared__ __align__(16) float sdy[SK_CHUNK][8 * OI];
     __shared__ float sz[SK_CHUNK][32 * MJ];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int o0 = blockIdx.y * 8 * OI;
     const int n_begin = blockIdx.x * tokens_per_cta;
     const int n_end = (n_begin + tokens_per_cta < N) ? n_begin + tokens_per_cta : N;
     float acc[OI][MJ];
@@ -43,23 +48,43 @@ wg_skinny_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __re
 #pragma unroll
         for (int j = 0; j < MJ; ++j) acc[i][j] = 0.f;
 
+    constexpr int NY = SK_CHUNK * 8 * OI / SK_THREADS, NZ = SK_CHUNK * 32 * MJ / SK_THREADS;
+    float ly[NY], lz[NZ];
+    auto fetch = [&](int n0) {
+#pragma unroll
+        for (int u = 0; u < NY; ++u) {
+            const int idx = threadIdx.x + u * SK_THREADS;
+            const int n = n0 + idx / (8 * OI), o = o0 + idx % (8 * OI);
+            ly[u] = (n < n_end && o < O) ? Elem<YT>::load(dY + static_cast<int64_t>(n) * lddy + o) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < NZ; ++u) {
+            const int idx = threadIdx.x + u * SK_THREADS;
+            const int n = n0 + idx / (32 * MJ), m = idx % (32 * MJ);
+            lz[u] = (n < n_end && m < M) ? Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m) : 0.f;
+        }
+    };
+    fetch(n_begin);
     for (int n0 = n_begin; n0 < n_end; n0 += SK_CHUNK) {
-        for (int idx = threadIdx.x; idx < SK_CHUNK * 8 * OI; idx += SK_THREADS) {
-            const int r = idx / (8 * OI), o = idx - r * (8 * OI);
-            const int n = n0 + r;
-            sdy[r][o] = (n < n_end && o < O) ? Elem<YT>::load(dY + static_cast<int64_t>(n) * lddy + o) : 0.f;
-        }
-        for (int idx = threadIdx.x; idx < SK_CHUNK * 32 * MJ; idx += SK_THREADS) {
-            const int r = idx / (32 * MJ), m = idx - r * (32 * MJ);
-            const int n = n0 + r;
-            sz[r][m] = (n < n_end && m < M) ? Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m) : 0.f;
-        }
+#pragma unroll
+        for (int u = 0; u < NY; ++u) (&sdy[0][0])[threadIdx.x + u * SK_THREADS] = ly[u];
+#pragma unroll
+        for (int u = 0; u < NZ; ++u) (&sz[0][0])[threadIdx.x + u * SK_THREADS] = lz[u];
         __syncthreads();
+        if (n0 + SK_CHUNK < n_end) fetch(n0 + SK_CHUNK);      // on its way while this chunk is multiplied
 #pragma unroll 4
         for (int r = 0; r < SK_CHUNK; ++r) {
             float y[OI], z[MJ];
+            if (OI == 2) {
+                const float2 q = *reinterpret_cast<const float2*>(&sdy[r][warp * OI]);
+                y[0] = q.x; y[1] = q.y;
+            } else {
 #pragma unroll
-            for (int i = 0; i < OI; ++i) y[i] = sdy[r][warp + 8 * i];
+                for (int i = 0; i < OI / 4; ++i) {
+                    const float4 q = *reinterpret_cast<const float4*>(&sdy[r][warp * OI + 4 * i]);
+                    y[(4 * i) % OI] = q.x; y[(4 * i + 1) % OI] = q.y; y[(4 * i + 2) % OI] = q.z; y[(4 * i + 3) % OI] = q.w;
+                }
+            }
 #pragma unroll
             for (int j = 0; j < MJ; ++j) z[j] = sz[r][lane + 32 * j];
 #pragma unroll
@@ -74,7 +99,7 @@ wg_skinny_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __re
     for (int i = 0; i < OI; ++i)
 #pragma unroll
         for (int j = 0; j < MJ; ++j) {
-            const int o = warp + 8 * i, m = lane + 32 * j;
+            const int o = o0 + warp * OI + i, m = lane + 32 * j;
             if (o < O && m < M) out[o * M + m] = acc[i][j];
         }
 }
@@ -383,7 +408,7 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 
 struct SkinnyPlan {
     bool ok;
-    int M, oi, mj, tokens_per_cta, parts;
+    int M, oi, mj, o_blocks, tokens_per_cta, parts;
     size_t partial_bytes, p_bytes;
 };
 
@@ -391,16 +416,26 @@ SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
 {
     SkinnyPlan p{};
     const int64_t M = ceil_div64(D, Dsub);
-    if (O < 1 || O > SK_MAX_O || M > SK_MAX_M || N < 1 || N > (1 << 30)) return p;
+    if (O < 1 || M > SK_MAX_M || N < 1 || N > (1 << 30) || O * M >= (1 << 30)) return p;
     p.M = static_cast<int>(M);
-    p.oi = static_cast<int>((O + 7) / 8);
+    p.oi = O > SK_MAX_O ? 8 : static_cast<int>((O + 7) / 8);
     p.oi = p.oi <= 2 ? 2 : (p.oi <= 4 ? 4 : 8);
     p.mj = static_cast<int>((M + 31) / 32);
-    p.mj = p.mj <= 2 ? 2 : (p.mj <= 4 ? 4 : 8);
+    p.mj = p.mj <= 1 ? 1 : (p.mj <= 2 ? 2 : (p.mj <= 4 ? 4 : 8));
+    p.o_blocks = static_cast<int>(ceil_div64(O, 8 * p.oi));
     // One 32-token chunk per CTA where that gives at most 512 partials: the partial kernel is a single round
     // trip to memory plus a little arithmetic, so more, shorter CTAs finish sooner.
-    (void)sm_count;
-    int64_t tpc = ceil_div64(N, 512);
+    int64_t max_parts = 512;
+    if (O > SK_MAX_O) {
+        // Wide fp32 layers: four CTAs per SM over all column blocks, as many slices as the tensor-core form's
+        // workspace holds (that size is what velora_workspace_bytes has always reported for them).
+        const int64_t bytes = static_cast<int64_t>(weight_grad_tc_workspace_bytes(N, D, O, Dsub)) - 512;   // two roundings to 256
+        const int64_t room = bytes / static_cast<int64_t>(sizeof(float) * O * M) - 1;                       // and P itself
+        max_parts = ceil_div64(4 * static_cast<int64_t>(sm_count), p.o_blocks);
+        if (max_parts > room) max_parts = room;
+        if (max_parts < 1 || p.o_blocks > 65535) return p;
+    }
+    int64_t tpc = ceil_div64(N, max_parts);
     tpc = ceil_div64(tpc, SK_CHUNK) * SK_CHUNK;
     p.tokens_per_cta = static_cast<int>(tpc);
     p.parts = static_cast<int>(ceil_div64(N, tpc));
@@ -416,13 +451,13 @@ int launch_partial(const SkinnyPlan& p, const void* dY, int64_t lddy, const void
 {
 #define VELORA_SK_CASE(OIV, MJV)                                                                                  \
     if (p.oi == OIV && p.mj == MJV) {                                                                             \
-        wg_skinny_partial_kernel<YT, ZT, OIV, MJV><<<p.parts, SK_THREADS, 0, stream>>>(                           \
+        wg_skinny_partial_kernel<YT, ZT, OIV, MJV><<<dim3(p.parts, p.o_blocks), SK_THREADS, 0, stream>>>(         \
             static_cast<const YT*>(dY), lddy, static_cast<const ZT*>(Z), ldz, N, O, p.M, p.tokens_per_cta, partials); \
         return after_launch();                                                                                    \
     }
-    VELORA_SK_CASE(2, 2) VELORA_SK_CASE(2, 4) VELORA_SK_CASE(2, 8)
-    VELORA_SK_CASE(4, 2) VELORA_SK_CASE(4, 4) VELORA_SK_CASE(4, 8)
-    VELORA_SK_CASE(8, 2) VELORA_SK_CASE(8, 4) VELORA_SK_CASE(8, 8)
+    VELORA_SK_CASE(2, 1) VELORA_SK_CASE(2, 2) VELORA_SK_CASE(2, 4) VELORA_SK_CASE(2, 8)
+    VELORA_SK_CASE(4, 1) VELORA_SK_CASE(4, 2) VELORA_SK_CASE(4, 4) VELORA_SK_CASE(4, 8)
+    VELORA_SK_CASE(8, 1) VELORA_SK_CASE(8, 2) VELORA_SK_CASE(8, 4) VELORA_SK_CASE(8, 8)
 #undef VELORA_SK_CASE
     return VELORA_ERR_UNSUPPORTED;
 }
@@ -431,18 +466,21 @@ int launch_partial(const SkinnyPlan& p, const void* dY, int64_t lddy, const void
 
 size_t weight_grad_skinny_workspace_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
 {
+    if (O > SK_MAX_O) return 0;                          // planned into the tensor-core form's room
     const SkinnyPlan p = skinny_plan(N > 0 ? N : 1, D, O, Dsub, 148);
     // The token range is always cut into at most 512 slices, whatever the device, so the size is fixed.
     return p.ok ? p.partial_bytes + p.p_bytes : 0;
 }
 
-// Returns VELORA_ERR_UNSUPPORTED (nothing launched) when the shape is not adapter-like (O > 64 or M > 256).
+// Returns VELORA_ERR_UNSUPPORTED (nothing launched) for more than 256 sub-tokens, and for bf16 gradients of more than 64
+// columns (those have the tensor cores).
 // P_out != NULL: only the factor, P_out = beta * P_out + dY^T Z (dW, v unused).
 int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
                               const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
                               void* dW, int dw_dtype, int64_t lddw, int beta,
                               void* ws, size_t ws_bytes, cudaStream_t stream, float* P_out, int64_t ldp_out)
 {
+    if (O > SK_MAX_O && dy_dtype != VELORA_F32) return VELORA_ERR_UNSUPPORTED;
     const SkinnyPlan p = skinny_plan(N, D, O, Dsub, 148);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
     if (ws_bytes < p.partial_bytes + p.p_bytes) return VELORA_ERR_WORKSPACE;
@@ -466,6 +504,9 @@ int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O
         wg_skinny_reduce_kernel<<<grid, SK_THREADS, 0, stream>>>(partials, p.parts, o, p.M, P_out, ldp_out, beta);
         return after_launch();
     }
+    // A handful of slices is added up by the expansion itself: one launch less.
+    if (p.parts <= SK_DIRECT_PARTS)
+        return launch_expand_p(partials, p.parts, static_cast<int64_t>(o) * p.M, p.M, v, O, D, Dsub, dW, dw_dtype, lddw, beta, stream);
     wg_skinny_reduce_kernel<<<grid, SK_THREADS, 0, stream>>>(partials, p.parts, o, p.M, P, p.M, 0);
     rc = after_launch();
     if (rc != VELORA_OK) return rc;
