@@ -67,11 +67,11 @@ int launch_linear_forward_tc(const void* X, int64_t ldx, const void* W, int64_t 
                              void* Y, int64_t ldy, void* Z, int z_dtype, int64_t ldz,
                              int dtype, int64_t N, int64_t D, int64_t O, int Dsub, int* status, cudaStream_t stream);
 
-// Row-streaming kernels (stream_rows.cu): bf16 X with 16-byte aligned rows, Dsub = 8 * 2^k up to 1024.
+// Row-streaming kernels (stream_rows.cu): Dsub = 8 * 2^k up to 1024.
 // Return VELORA_ERR_UNSUPPORTED (nothing launched) when the shape does not fit them.
-int launch_compress_rows(const void* X, int64_t N, int64_t D, int64_t ldx, int Dsub, const float* v,
+int launch_compress_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx, int Dsub, const float* v,
                          void* Z, int z_dtype, int64_t ldz, cudaStream_t stream);
-int launch_init_v_partials_rows(const void* X, int64_t N, int64_t D, int64_t ldx, int Dsub,
+int launch_init_v_partials_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx, int Dsub,
                                 float* partials, int max_partials, int* num_partials, cudaStream_t stream);
 
 // One tiny CTA whose bounded waits run out (limit_ns for the first, the abort flag for the second); raises

@@ -1,12 +1,12 @@
 // HBM-bound streaming kernels of the VeLoRA path: init_v, compress, reconstruct and the expansion
 // of the factored weight gradient (arxiv 2405.17991, Section 3.1 Eq. 1 / Eq. 2, Section 3.2).
 //
-// The common case (bf16 rows that are 16-byte aligned, Dsub = 8 * 2^k) is served by stream_rows.cu
-// (compress, init_v) and expand_kernels.cu (reconstruct, expansion of the factored weight gradient).  This
-// file holds the kernels for everything else and the routing between all of them.
+// Dsub = 8 * 2^k is served by stream_rows.cu (compress, init_v) and expand_kernels.cu (reconstruct, expansion of the
+// factored weight gradient), whatever the type and the alignment of the rows.  This file holds the kernels for
+// everything else and the routing between all of them.
 //
-// Element kernels cover everything else (fp32 data, Dsub not a multiple of 8, unaligned rows) with
-// the same arithmetic, one element per lane.
+// Element kernels cover what no vector kernel takes (Dsub not a multiple of 8 on unaligned rows, mixed storage
+// types) with the same arithmetic, one element per lane.
 #include "common.cuh"
 #include "gemm_tc.cuh"
 
@@ -553,9 +553,7 @@ int launch_init_v(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx,
     const int M = static_cast<int>(ceil_div64(D, Dsub));
     int num_partials = 0;
 
-    int rows_rc = VELORA_ERR_UNSUPPORTED;
-    if (x_dtype == VELORA_BF16)
-        rows_rc = launch_init_v_partials_rows(X, N, D, ldx, Dsub, partials, kInitVMaxCtas, &num_partials, stream);
+    const int rows_rc = launch_init_v_partials_rows(X, x_dtype, N, D, ldx, Dsub, partials, kInitVMaxCtas, &num_partials, stream);
     if (rows_rc != VELORA_ERR_UNSUPPORTED) {
         if (rows_rc != VELORA_OK) return rows_rc;
     } else {
@@ -586,10 +584,8 @@ int launch_compress(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ld
                     const float* v, void* Z, int z_dtype, int64_t ldz, cudaStream_t stream)
 {
     const int M = static_cast<int>(ceil_div64(D, Dsub));
-    if (x_dtype == VELORA_BF16) {                        // aligned rows, Dsub = 8 * 2^k: the row-streaming kernel
-        const int rc = launch_compress_rows(X, N, D, ldx, Dsub, v, Z, z_dtype, ldz, stream);
-        if (rc != VELORA_ERR_UNSUPPORTED) return rc;
-    }
+    const int rows_rc = launch_compress_rows(X, x_dtype, N, D, ldx, Dsub, v, Z, z_dtype, ldz, stream);   // Dsub = 8 * 2^k
+    if (rows_rc != VELORA_ERR_UNSUPPORTED) return rows_rc;
     const bool z8 = z_dtype == VELORA_FP8_E4M3;          // 8-bit Z: the TMA kernel above or the element kernel below
     if (!z8 && x_dtype == VELORA_BF16 && (Dsub == 1 || Dsub == 2 || Dsub == 4) && rows_vectorisable(X, ldx) && D < (1 << 30)) {
         int grid = 0;
@@ -665,10 +661,9 @@ static int launch_expand_any(const void* S, int s_dtype, int splits, int64_t spl
 int launch_reconstruct(const void* Z, int z_dtype, int64_t ldz, int64_t N, int64_t D, int Dsub,
                        const float* v, void* Xhat, int x_dtype, int64_t ldxhat, cudaStream_t stream)
 {
-    if (x_dtype == VELORA_BF16) {                        // Xhat = Z (x) v is the one-split, beta = 0 expansion
-        const int rc = launch_expand_rows_vec(Z, z_dtype, 1, 0, ldz, v, N, D, Dsub, Xhat, x_dtype, ldxhat, 0, stream);
-        if (rc != VELORA_ERR_UNSUPPORTED) return rc;
-    }
+    // Xhat = Z (x) v is the one-split, beta = 0 expansion
+    const int vrc = launch_expand_rows_vec(Z, z_dtype, 1, 0, ldz, v, N, D, Dsub, Xhat, x_dtype, ldxhat, 0, stream);
+    if (vrc != VELORA_ERR_UNSUPPORTED) return vrc;
     const bool z8 = z_dtype == VELORA_FP8_E4M3;          // 8-bit Z: the vector expansion above or the element kernel below
     if (!z8 && x_dtype == VELORA_BF16 && (Dsub == 1 || Dsub == 2 || Dsub == 4) && D % 8 == 0 && rows_vectorisable(Xhat, ldxhat) &&
         D < (1 << 30)) {

@@ -90,3 +90,24 @@ def test_products_add_to_an_output_with_odd_rows(vl, guard, c_dtype, Mdim, Ndim,
     C = guard.mat(Mdim, Ndim, c_dtype, ld=Ndim, init=C0)
     vl.velora_dense_product(vl.PRODUCT_A_BT, A, B, C=C, beta=1)
     assert_matches(C, to_f64(A) @ to_f64(B).T + to_f64(C0), TOL_GEMM, "C")
+
+
+# Sub-tokens of every length class of the one-element walk (8 .. 1024), fp32 and bf16, last sub-token ragged or whole.
+@pytest.mark.parametrize("N,D,Dsub", [(1, 9, 8), (37, 257, 8), (300, 1041, 16), (129, 1375, 32), (70, 2049, 64), (33, 2051, 256), (20, 3071, 1024)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("pad", [0, 3])
+def test_streams_on_odd_rows(vl, guard, N, D, Dsub, dtype, pad):
+    case = vi.small_case(3 * N + D, N, D, 8, dtype=dtype, mean_offset=0.1)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    X = _view(case["X"].torch(DEV), D + pad, 1)
+    v = vl.velora_init_v(X, Dsub)
+    assert_matches(v, oracle.init_v(case["X"].f64(), Dsub), TOL_Z, "v")
+    M, v64 = vl.num_subtokens(D, Dsub), to_f64(v)
+    Z = vl.velora_compress(X, v, Z=guard.mat(N, M, torch.float32))
+    assert_matches(Z, oracle.compress(case["X"].f64(), v64), TOL_Z, "Z")
+    Xhat = vl.velora_reconstruct(Z, v, D, Xhat=guard.mat(N, D, dt, ld=D + pad))
+    assert_matches(Xhat, oracle.reconstruct(to_f64(Z), v64, D), TOL_Z, "Xhat")
+    W0 = torch.randn((N, D), device=DEV).to(dt)
+    W = guard.mat(N, D, dt, ld=D + pad, init=W0)
+    vl.velora_expand_p(Z, v, D, dW=W, beta=1)
+    assert_matches(W, oracle.reconstruct(to_f64(Z), v64, D) + to_f64(W0), TOL_Z, "W + P v", c=2e-3)
