@@ -37,12 +37,14 @@ struct DeviceOnce {
 };
 
 inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
-// Programmatic dependent launch.  A kernel launched with pdl_attribute() may become resident while the
-// kernel before it in the stream is still running; it must call pdl_wait() before it touches anything
-// that kernel writes (the wait returns once that kernel has completed and its writes are visible).
-// pdl_trigger() in a kernel lets the NEXT kernel in the stream, if launched this way, start early.
-// Used between the Z conversion and the weight-gradient kernel; tried on the dense products as well,
-// where hiding the launch latency of a 200-500 us kernel made no measurable difference.
+// Programmatic dependent launch.  A kernel launched with pdl_attribute() may become resident while the kernel before it
+// in the stream is still running: its launch, its barriers and its TMEM are then ready when that kernel ends.  Every
+// thread of such a kernel calls pdl_wait() before it touches global memory (the wait returns once the kernel before
+// has completed and its writes are visible), and only then pdl_trigger(), which lets the NEXT kernel start early: so
+// when kernel k + 1 becomes resident, everything up to k - 1 has completed.  A small layer is a chain of kernels of
+// 5-10 us with about 2 us of launch and set-up between them.
+// Not launched this way: the CTA-pair product (long queues of layers with it stopped making progress on the one
+// occasion it was, for a reason that has not been found; it runs long enough for 2 us not to matter).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -54,6 +56,27 @@ inline cudaLaunchAttribute pdl_attribute()
     a.val.programmaticStreamSerializationAllowed = 1;
     return a;
 }
+
+#ifdef __CUDACC__
+// Launches a kernel that keeps to the rules above; counts it and reports a launch error as a status.
+template <typename... KArgs, typename... Args>
+inline int launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = pdl_attribute();
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...) != cudaSuccess) {
+        cudaGetLastError();
+        return VELORA_ERR_CUDA;
+    }
+    return after_launch();
+}
+#endif
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t dtype_size(int dt) { return dt == VELORA_BF16 ? 2 : (dt == VELORA_FP8_E4M3 ? 1 : 4); }

@@ -80,8 +80,8 @@ expand_rows_vec_kernel(const ST* __restrict__ S, int splits, int64_t split_strid
     const int q = lane & (LPS - 1);
     const int sub = lane / LPS;
     // Programmatic stream serialisation (see common.cuh): resident early, nothing read or written before the wait.
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     float vr[CH][VEC];
 #pragma unroll
     for (int i = 0; i < CH; ++i)

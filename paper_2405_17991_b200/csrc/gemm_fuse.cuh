@@ -58,6 +58,7 @@ __device__ __forceinline__ uint4 ld_x_chunk(const uint4* p)
 // The slice of v a lane of a compress warp works with: lane l always meets chunk (32 * part + l) % L of a
 // sub-token of L = Dsub / 8 chunks, part = 0 .. CH - 1 (CH = L / 32 for L > 32, else 1).
 template <int CH> struct VSlice {
+    static constexpr int kParts = CH;
     float v[CH][8];
     __device__ __forceinline__ void load(const float* vg, int Dsub, int lane)
     {
@@ -71,29 +72,37 @@ template <int CH> struct VSlice {
     }
 };
 
-// The compress of one "group" of a row block by ONE warp, read straight from global memory (the lines are
-// in L2 around the time the GEMM's own loads of the same row block run, so X still crosses HBM once):
-// rows [r0, r0 + 32) of X, columns [8 * cpr * g, 8 * cpr * (g + 1)), cpr = max(Dsub / 8, 8) 16-byte chunks
-// per row, i.e. one whole sub-token per row (Dsub >= 64) or the 64 / Dsub sub-tokens of a 64-column block.
-// A load instruction covers 32 consecutive chunks of the warp's 32 x cpr chunk rectangle in row-major
-// order; eight instructions are issued before the first is used.  L = Dsub / 8 chunks form a sub-token:
-// lps = min(L, 32) adjacent lanes hold (a part of) it, for L > 32 the CH = L / 32 consecutive instructions
-// complete it.  fp32 products and sums, xor-shuffle reduction, one lane stores Z[row, m].  Columns at or
-// beyond D count as zeros (ragged last sub-token), rows at or beyond N are skipped.  No shared memory and
-// no barrier (v sits in registers): the warps that do this never touch the GEMM's pipeline, and in
-// particular not the shared-memory bandwidth the tensor cores live on.
-template <int ZK, int CH>
-__device__ __forceinline__ void compress_group_direct(const FuseArgs& fz, const VSlice<CH>& vs, int r0, int N, int D, int g, int lane)
-{
-    const int L = fz.Dsub >> 3;                         // a power of two, 1 .. 128 (host)
-    const int lps = L < 32 ? L : 32;
-    const int cpr = L < 8 ? 8 : L;
-    const int cshift = 31 - __clz(cpr), lshift = 31 - __clz(L);
-    const int d8 = D >> 3, tail = D & 7;
-    const int c_base = g * cpr;                         // first chunk of the group in a row
-    const int subs_per_row = cpr >> lshift;             // sub-tokens of one row inside the group (1 if Dsub >= 64)
-    for (int i0 = 0; i0 < cpr; i0 += 8) {               // cpr instructions cover the warp's 32 rows
-        uint4 d[8];
+// The compress of a row block's column groups g0, g0 + step, ... by ONE warp, read straight from global memory (the lines
+// are in L2 around the time the GEMM's own loads of the same row block run, so X still crosses HBM once): rows
+// [r0, r0 + 32) of X, columns [8 * cpr * g, 8 * cpr * (g + 1)) of group g, cpr = max(Dsub / 8, 8) 16-byte chunks per
+// row, i.e. one whole sub-token per row (Dsub >= 64) or the 64 / Dsub sub-tokens of a 64-column block.
+// A load instruction covers 32 consecutive chunks of the warp's 32 x cpr chunk rectangle in row-major order; eight make
+// a batch, and the next batch is on its way while this one is multiplied (beside the tensor cores' operand stream a
+// load takes microseconds: one batch at a time kept 16 KB per SM in flight and moved 3.4 GB/s per SM).
+// L = Dsub / 8 chunks form a sub-token: lps = min(L, 32) adjacent lanes hold (a part of) it, for L > 32 the CH = L / 32
+// consecutive instructions complete it.  fp32 products and sums, xor-shuffle reduction, one lane stores Z[row, m].
+// Columns at or beyond D count as zeros (ragged last sub-token), rows at or beyond N are skipped.  No shared memory and
+// no barrier (v sits in registers): the warps that do this never touch the GEMM's pipeline, and in particular not
+// the shared-memory bandwidth the tensor cores live on.
+template <int ZK, int CH> struct CompressWalk {
+    const FuseArgs& fz;
+    const VSlice<CH>& vs;
+    int r0, N, lane, lps, cpr, cshift, lshift, d8, tail;
+
+    __device__ __forceinline__ CompressWalk(const FuseArgs& fz_, const VSlice<CH>& vs_, int r0_, int N_, int D, int lane_)
+        : fz(fz_), vs(vs_), r0(r0_), N(N_), lane(lane_)
+    {
+        const int L = fz.Dsub >> 3;                     // a power of two, 1 .. 128 (host)
+        lps = L < 32 ? L : 32;
+        cpr = L < 8 ? 8 : L;
+        cshift = 31 - __clz(cpr);
+        lshift = 31 - __clz(L);
+        d8 = D >> 3;
+        tail = D & 7;
+    }
+    __device__ __forceinline__ void load(uint4 (&d)[8], int g, int i0) const
+    {
+        const int c_base = g << cshift;                 // first chunk of the group in a row
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int flat = 32 * (i0 + u) + lane;
@@ -113,7 +122,16 @@ __device__ __forceinline__ void compress_group_direct(const FuseArgs& fz, const 
             }
             d[u] = x;
         }
-        float part = 0.f;
+    }
+    // The sums over the lanes of a sub-token, all of a batch's at once: at each step a lane hands on half of the values it
+    // holds and takes its partner's share of the other half, so a batch costs 7 or 8 shuffles where one reduction
+    // after the other costs 24 to 40 (the additions and their order are the same).  Shuffles pass through the
+    // shared-memory pipe that feeds the tensor cores: a 4096 x 5461 -> 2048 forward took 127 us with them and 100 without.
+    __device__ __forceinline__ void reduce(const uint4 (&d)[8], int g, int i0) const
+    {
+        constexpr int NV = 8 / CH;                      // values of a batch
+        const int subs_per_row = cpr >> lshift;         // sub-tokens of one row inside the group (1 if Dsub >= 64)
+        float k[NV];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int pi = u & (CH - 1);                // which 32-chunk part of the sub-token (i0 is a multiple of 8)
@@ -122,17 +140,57 @@ __device__ __forceinline__ void compress_group_direct(const FuseArgs& fz, const 
             a0 = fmaf(bf16_lo(d[u].y), v[2], a0); a1 = fmaf(bf16_hi(d[u].y), v[3], a1);
             a0 = fmaf(bf16_lo(d[u].z), v[4], a0); a1 = fmaf(bf16_hi(d[u].z), v[5], a1);
             a0 = fmaf(bf16_lo(d[u].w), v[6], a0); a1 = fmaf(bf16_hi(d[u].w), v[7], a1);
-            part = (pi == 0) ? a0 + a1 : part + (a0 + a1);
-            if (pi == CH - 1) {
-                float k = part;
-                for (int off = lps >> 1; off >= 1; off >>= 1) k += __shfl_xor_sync(0xffffffffu, k, off);
-                const int flat = 32 * (i0 + u) + lane;
-                const int row = r0 + (flat >> cshift);
-                const int m = g * subs_per_row + ((flat & (cpr - 1)) >> lshift);
-                if ((lane & (lps - 1)) == 0 && row < N && m < fz.M) store_z<ZK>(fz, row, m, k);
+            k[u / CH] = (pi == 0) ? a0 + a1 : k[u / CH] + (a0 + a1);
+        }
+        int off = lps >> 1, first = 0, held = NV;       // this lane holds the values first .. first + held - 1
+#pragma unroll
+        for (int half = NV / 2; half >= 1; half >>= 1) {
+            if (off == 0) break;
+            const bool upper = (lane & off) != 0;
+#pragma unroll
+            for (int j = 0; j < half; ++j) {
+                const float give = upper ? k[j] : k[j + half], keep = upper ? k[j + half] : k[j];
+                k[j] = keep + __shfl_xor_sync(0xffffffffu, give, off);
             }
+            first += upper ? half : 0;
+            held = half;
+            off >>= 1;
+        }
+        const int writer_mask = off ? 2 * off - 1 : 0;  // of the lanes that come to hold the same value the first writes
+        for (; off >= 1; off >>= 1) k[0] += __shfl_xor_sync(0xffffffffu, k[0], off);
+        if (lane & writer_mask) return;
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            if (j >= held) break;
+            const int flat = 32 * (i0 + (first + j) * CH + CH - 1) + lane;
+            const int row = r0 + (flat >> cshift);
+            const int m = g * subs_per_row + ((flat & (cpr - 1)) >> lshift);
+            if (row < N && m < fz.M) store_z<ZK>(fz, row, m, k[j]);
         }
     }
-}
+    __device__ __forceinline__ void run(int g, int step, int n_groups) const
+    {
+        if (r0 >= N || g >= n_groups) return;
+        uint4 a[8], b[8];
+        int i = 0;                                      // cpr instructions (a multiple of 8) cover the warp's 32 rows
+        auto next = [&](int& gg, int& ii) {
+            ii += 8;
+            if (ii >= cpr) { ii = 0; gg += step; }
+        };
+        load(a, g, i);
+        for (;;) {
+            int g1 = g, i1 = i;
+            next(g1, i1);
+            if (g1 < n_groups) load(b, g1, i1);
+            reduce(a, g, i);
+            if (g1 >= n_groups) return;
+            g = g1; i = i1;
+            next(g, i);
+            if (g < n_groups) load(a, g, i);
+            reduce(b, g1, i1);
+            if (g >= n_groups) return;
+        }
+    }
+};
 
 }  // namespace velora

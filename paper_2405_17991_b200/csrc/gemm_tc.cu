@@ -105,6 +105,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();                                              // nothing in global memory has been touched so far
+    pdl_trigger();
 
     bool failed = false;
     if (warp == 0) {
@@ -194,9 +196,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (!wait_for_tile(tiles_started, ti, abort_flag)) { failed = true; break; }
                 const TileCoord tc0 = tile_coord(tile, tiles_m, tiles_n);
                 const int r0 = tc0.m0 + cwi * 32;
-                if (r0 >= Mdim) continue;
-                for (int g = tc0.n0 / BN; g < n_groups; g += tiles_n)
-                    compress_group_direct<FUSE>(fz, vs, r0, Mdim, Kdim, g, lane);
+                CompressWalk<FUSE, vs.kParts>(fz, vs, r0, Mdim, Kdim, lane).run(tc0.n0 / BN, tiles_n, n_groups);
             }
         };
         if (fz.Dsub <= 256) walk(VSlice<1>{});
@@ -215,24 +215,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t taddr = tmem_base + acc * BN + (static_cast<uint32_t>(quarter * 32) << 16);
             CT* crow = C + static_cast<int64_t>(row) * ldc + tc0.n0;
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                uint32_t r[32];
-                tmem_ld_32x32(taddr + c * 32, r);
+            for (int c = 0; c < BN / 32; c += 2) {            // 64 columns a step: two TMEM loads in flight
+                uint32_t r[2][32];
+                tmem_ld_32x32(taddr + c * 32, r[0]);
+                tmem_ld_32x32(taddr + c * 32 + 32, r[1]);
                 tmem_ld_wait();
-                if (c == BN / 32 - 1) {                   // accumulator fully read: hand it back
+                if (c == BN / 32 - 2) {                       // accumulator fully read: hand it back
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty + 8 * acc);
                 }
                 const int valid = Ndim - (tc0.n0 + c * 32);
-                if (valid <= 0) continue;
-                if (!c_vec) {
-                    const int row0 = tc0.m0 + quarter * 32;
-                    if (row0 < Mdim)
-                        store_rows_staged<CT>(C + static_cast<int64_t>(row0) * ldc + tc0.n0 + c * 32, ldc, Mdim - row0, valid, r, beta,
-                                              reinterpret_cast<float*>(tail + STAGE_OFF) + quarter * kStageFloats, lane);
-                } else if (row < Mdim) {
-                    Store32<CT>::run(crow + c * 32, r, valid, beta);
+                if (c_vec) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);
+                } else if (row - lane < Mdim) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (valid > 32 * h)
+                            store_rows_staged<CT>(crow - static_cast<int64_t>(lane) * ldc + (c + h) * 32, ldc, Mdim - (row - lane), valid - 32 * h,
+                                                  r[h], beta, reinterpret_cast<float*>(tail + STAGE_OFF) + quarter * kStageFloats, lane);
                 }
             }
         }
@@ -289,9 +292,8 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     const int tiles_m = (Mdim + BM - 1) / BM, tiles_n = (Ndim + BN - 1) / BN;
     const int64_t tiles = static_cast<int64_t>(tiles_m) * tiles_n;
     const int grid = static_cast<int>(tiles < di.sm_count ? tiles : di.sm_count);
-    kern<<<grid, FUSE ? FUSE_THREADS : GEMM_THREADS, FUSE ? FUSE_SMEM : GEMM_SMEM, stream>>>(
-        ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, c_rows_vec(C, ldc, sizeof(CT)), status, fz);
-    return after_launch();
+    return launch_chained(kern, dim3(static_cast<unsigned>(grid)), FUSE ? FUSE_THREADS : GEMM_THREADS, FUSE ? FUSE_SMEM : GEMM_SMEM, stream,
+                          ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, c_rows_vec(C, ldc, sizeof(CT)), status, fz);
 }
 
 }  // namespace
@@ -389,9 +391,11 @@ int launch_linear_forward_tc(const void* X, int64_t ldx, const void* W, int64_t 
     const bool pow2 = Dsub >= 8 && Dsub <= VELORA_MAX_DSUB && (Dsub & (Dsub - 1)) == 0;
     const bool gemm_ok = dtype == VELORA_BF16 && N >= 1 && N < (1 << 30) && D < (1 << 30) && O < (1 << 30) &&
                          tc_operand_ok(X, ldx) && tc_operand_ok(W, ldw);
-    // One CTA compresses one k-block in tiles_n; with fewer than four n-tiles the compress warps would
-    // hold the producer back, so narrow outputs take the two-kernel route as well.
-    const bool wide = (O + BN - 1) / BN >= 4;
+    // A CTA compresses one tiles_n-th of its row block's columns while it multiplies all of them; the loads and
+    // shuffles of that compete with the tensor cores' operand stream, so with few n-tiles the two kernels in turn are
+    // faster.  Fused / in turn, us: 47 / 34 at 8192 x 1376 -> 1024 (4 n-tiles), 59 / 62 at 4096 x 4096 -> 2048 (8), 98 / 93
+    // there with D = 5461 and a pitch of 10928 bytes (each load touches a line more), 51 / 58 at 12608 x 768 -> 3072 (12).
+    const bool wide = (O + BN - 1) / BN >= (ldx % 64 == 0 ? 8 : 12);
     if (pow2 && gemm_ok && wide) {
         if (gemm_pair_preferred(N, O)) {
             const int prc = launch_linear_forward_tc_pair(X, ldx, W, ldw, v, Y, ldy, Z, z_dtype, ldz, N, D, O, Dsub, status, stream);

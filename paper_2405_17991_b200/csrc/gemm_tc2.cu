@@ -270,9 +270,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (!wait_for_tile(tiles_started, ti, abort_flag)) { failed = true; break; }
                 const PairTile t0 = pair_tile(tile, tiles_m, tiles_n);
                 const int r0 = t0.m0 + static_cast<int>(rank) * P_BM + cwi * 32;
-                if (r0 >= Mdim) continue;
-                for (int g = t0.n0 / P_BN; g < n_groups; g += tiles_n)
-                    compress_group_direct<FUSE>(fz, vs, r0, Mdim, Kdim, g, lane);
+                CompressWalk<FUSE, vs.kParts>(fz, vs, r0, Mdim, Kdim, lane).run(t0.n0 / P_BN, tiles_n, n_groups);
             }
         };
         if (fz.Dsub <= 256) walk(VSlice<1>{});
@@ -292,24 +290,27 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const uint32_t taddr = tmem_base + acc * P_BN + (static_cast<uint32_t>(quarter * 32) << 16);
             CT* crow = C + static_cast<int64_t>(row) * ldc + t0.n0;
 #pragma unroll 1
-            for (int c = 0; c < P_BN / 32; ++c) {
-                uint32_t r[32];
-                tmem_ld_32x32(taddr + c * 32, r);
+            for (int c = 0; c < P_BN / 32; c += 2) {            // 64 columns a step: two TMEM loads in flight
+                uint32_t r[2][32];
+                tmem_ld_32x32(taddr + c * 32, r[0]);
+                tmem_ld_32x32(taddr + c * 32 + 32, r[1]);
                 tmem_ld_wait();
-                if (c == P_BN / 32 - 1) {                     // accumulator fully read: tell the leader
+                if (c == P_BN / 32 - 2) {                       // accumulator fully read: hand it back
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8 * acc);
                 }
                 const int valid = Ndim - (t0.n0 + c * 32);
-                if (valid <= 0) continue;
-                if (!c_vec) {
-                    const int row0 = row - lane;
-                    if (row0 < Mdim)
-                        store_rows_staged<CT>(C + static_cast<int64_t>(row0) * ldc + t0.n0 + c * 32, ldc, Mdim - row0, valid, r, beta,
-                                              reinterpret_cast<float*>(tail + P_STAGE_OFF) + quarter * kStageFloats, lane);
-                } else if (row < Mdim) {
-                    Store32<CT>::run(crow + c * 32, r, valid, beta);
+                if (c_vec) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);
+                } else if (row - lane < Mdim) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (valid > 32 * h)
+                            store_rows_staged<CT>(crow - static_cast<int64_t>(lane) * ldc + (c + h) * 32, ldc, Mdim - (row - lane), valid - 32 * h,
+                                                  r[h], beta, reinterpret_cast<float*>(tail + P_STAGE_OFF) + quarter * kStageFloats, lane);
                 }
             }
         }

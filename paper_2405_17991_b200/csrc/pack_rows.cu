@@ -65,6 +65,8 @@ __device__ __forceinline__ uint4 load_unaligned(const char* p, const char* lo_li
 __global__ void __launch_bounds__(PK_THREADS)
 pack_rows_kernel(const PackArgs a)
 {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (PK_THREADS / 32);
     const int64_t total = a.items[0] + a.items[1];
@@ -118,8 +120,7 @@ int launch_pack_rows(const PackJob* jobs, int count, cudaStream_t stream)
     int64_t grid = ceil_div64(items, PK_THREADS / 32);
     const int64_t cap = static_cast<int64_t>(di.sm_count) * kStreamCtasPerSm;
     if (grid > cap) grid = cap;
-    pack_rows_kernel<<<static_cast<int>(grid), PK_THREADS, 0, stream>>>(a);
-    return after_launch();
+    return launch_chained(pack_rows_kernel, dim3(static_cast<unsigned>(grid)), PK_THREADS, 0, stream, a);
 }
 
 }  // namespace velora

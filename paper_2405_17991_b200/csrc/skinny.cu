@@ -64,6 +64,8 @@ wg_skinny_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __re
             lz[u] = (n < n_end && m < M) ? Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m) : 0.f;
         }
     };
+    pdl_wait();
+    pdl_trigger();
     fetch(n_begin);
     for (int n0 = n_begin; n0 < n_end; n0 += SK_CHUNK) {
 #pragma unroll
@@ -112,6 +114,8 @@ wg_skinny_reduce_kernel(const float* __restrict__ partials, int parts, int O, in
                         int64_t ldp, int beta)
 {
     __shared__ float sred[8][32];
+    pdl_wait();
+    pdl_trigger();
     const int total = O * M;
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int idx = blockIdx.x * 32 + lane;
@@ -224,6 +228,8 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         tmem_alloc(smem_u32(tmem_slot), 64);
         tmem_relinquish();
     }
+    pdl_wait();
+    pdl_trigger();
     for (int j = threadIdx.x; j < fz.Dsub; j += SF_THREADS) sv[j] = fz.v[j];
     tc_fence_before_sync();
     __syncthreads();
@@ -451,9 +457,8 @@ int launch_partial(const SkinnyPlan& p, const void* dY, int64_t lddy, const void
 {
 #define VELORA_SK_CASE(OIV, MJV)                                                                                  \
     if (p.oi == OIV && p.mj == MJV) {                                                                             \
-        wg_skinny_partial_kernel<YT, ZT, OIV, MJV><<<dim3(p.parts, p.o_blocks), SK_THREADS, 0, stream>>>(         \
+        return launch_chained(wg_skinny_partial_kernel<YT, ZT, OIV, MJV>, dim3(p.parts, p.o_blocks), SK_THREADS, 0, stream, \
             static_cast<const YT*>(dY), lddy, static_cast<const ZT*>(Z), ldz, N, O, p.M, p.tokens_per_cta, partials); \
-        return after_launch();                                                                                    \
     }
     VELORA_SK_CASE(2, 1) VELORA_SK_CASE(2, 2) VELORA_SK_CASE(2, 4) VELORA_SK_CASE(2, 8)
     VELORA_SK_CASE(4, 1) VELORA_SK_CASE(4, 2) VELORA_SK_CASE(4, 4) VELORA_SK_CASE(4, 8)
@@ -501,14 +506,12 @@ int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O
     const int total = o * p.M;
     const int grid = (total + 31) / 32;
     if (P_out) {
-        wg_skinny_reduce_kernel<<<grid, SK_THREADS, 0, stream>>>(partials, p.parts, o, p.M, P_out, ldp_out, beta);
-        return after_launch();
+        return launch_chained(wg_skinny_reduce_kernel, dim3(grid), SK_THREADS, 0, stream, partials, p.parts, o, p.M, P_out, ldp_out, beta);
     }
     // A handful of slices is added up by the expansion itself: one launch less.
     if (p.parts <= SK_DIRECT_PARTS)
         return launch_expand_p(partials, p.parts, static_cast<int64_t>(o) * p.M, p.M, v, O, D, Dsub, dW, dw_dtype, lddw, beta, stream);
-    wg_skinny_reduce_kernel<<<grid, SK_THREADS, 0, stream>>>(partials, p.parts, o, p.M, P, p.M, 0);
-    rc = after_launch();
+    rc = launch_chained(wg_skinny_reduce_kernel, dim3(grid), SK_THREADS, 0, stream, partials, p.parts, o, p.M, P, p.M, 0);
     if (rc != VELORA_OK) return rc;
     return launch_expand_p(P, 1, 0, p.M, v, O, D, Dsub, dW, dw_dtype, lddw, beta, stream);
 }
@@ -551,14 +554,12 @@ int launch_linear_forward_skinny(const void* X, int64_t ldx, const void* W, int6
     FuseArgs fz{v, Z, ldz, Dsub, static_cast<int>(ceil_div64(D, Dsub))};
     const int grid = static_cast<int>(ceil_div64(N, SF_TOKENS));
     if (z_dtype == VELORA_BF16)
-        skinny_forward_kernel<true><<<grid, SF_THREADS, SF_SMEM, stream>>>(
+        return launch_chained(skinny_forward_kernel<true>, dim3(grid), SF_THREADS, SF_SMEM, stream,
             tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D),
             w_rows, stages, status, fz);
-    else
-        skinny_forward_kernel<false><<<grid, SF_THREADS, SF_SMEM, stream>>>(
+    return launch_chained(skinny_forward_kernel<false>, dim3(grid), SF_THREADS, SF_SMEM, stream,
             tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D),
             w_rows, stages, status, fz);
-    return after_launch();
 }
 
 }  // namespace velora

@@ -81,6 +81,8 @@ init_v_finalize_kernel(const float* __restrict__ partials, int num_partials, int
     __shared__ double s_sum[VELORA_MAX_DSUB];
     __shared__ double s_red[kFinThreads * VEC];
     __shared__ double s_warp[kFinThreads / 32];
+    pdl_wait();
+    pdl_trigger();
     const int groups = Dsub / VEC;                             // VEC divides Dsub (host)
     for (int g0 = 0; g0 < groups; g0 += kFinThreads) {
         const int width = (groups - g0 < kFinThreads) ? groups - g0 : kFinThreads;
@@ -146,13 +148,12 @@ init_v_finalize_kernel(const float* __restrict__ partials, int num_partials, int
 }
 
 // Partial rows start 16-byte aligned and are Dsub floats apart: four positions per load when Dsub allows it.
-inline void launch_init_v_finalize(const float* partials, int num_partials, int Dsub, float* v, int* status,
-                                   int normalize, cudaStream_t stream)
+inline int launch_init_v_finalize(const float* partials, int num_partials, int Dsub, float* v, int* status,
+                                  int normalize, cudaStream_t stream)
 {
-    if (Dsub % 4 == 0 && aligned16(partials))
-        init_v_finalize_kernel<4><<<1, kFinThreads, 0, stream>>>(partials, num_partials, Dsub, v, status, normalize);
-    else
-        init_v_finalize_kernel<1><<<1, kFinThreads, 0, stream>>>(partials, num_partials, Dsub, v, status, normalize);
+    const bool vec = Dsub % 4 == 0 && aligned16(partials);
+    return launch_chained(vec ? init_v_finalize_kernel<4> : init_v_finalize_kernel<1>, dim3(1), kFinThreads, 0, stream,
+                          partials, num_partials, Dsub, v, status, normalize);
 }
 
 // Running-average variant of the initialisation (Section 5, ablation on the initialisation strategy):
@@ -522,8 +523,7 @@ int launch_normalize_v(const float* s, int Dsub, float* v, void* ws, size_t ws_b
 {
     if (ws_bytes < kStatusBytes) return VELORA_ERR_WORKSPACE;
     int* status = static_cast<int*>(ws) + 1;
-    launch_init_v_finalize(s, 1, Dsub, v, status, 1, stream);
-    if (check_launch() != VELORA_OK) return VELORA_ERR_CUDA;
+    if (launch_init_v_finalize(s, 1, Dsub, v, status, 1, stream) != VELORA_OK) return VELORA_ERR_CUDA;
     return read_degenerate_flag(status, stream);
 }
 
@@ -574,8 +574,7 @@ int launch_init_v(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx,
                 static_cast<const float*>(X), N, static_cast<int>(D), ldx, Dsub, M, rows_per_cta, partials);
     }
     if (check_launch() != VELORA_OK) return VELORA_ERR_CUDA;
-    launch_init_v_finalize(partials, num_partials, Dsub, v, status, sum_only ? 0 : 1, stream);
-    if (check_launch() != VELORA_OK) return VELORA_ERR_CUDA;
+    if (launch_init_v_finalize(partials, num_partials, Dsub, v, status, sum_only ? 0 : 1, stream) != VELORA_OK) return VELORA_ERR_CUDA;
     if (sum_only) return VELORA_OK;                            // v holds s; nothing to report, no synchronisation
     return read_degenerate_flag(status, stream);
 }

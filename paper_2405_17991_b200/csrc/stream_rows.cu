@@ -101,8 +101,8 @@ stream_rows_kernel(const XT* __restrict__ X, int N, int D, int64_t ldx, int M,
     static_assert(U % CH == 0, "a round must hold whole sub-tokens");
     typedef Chunk<XT, VEC> C;
     // Programmatic stream serialisation (common.cuh): resident early, nothing read or written before the wait.
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int q = lane & (LPS - 1);               // position of this lane's chunk inside a 32-chunk part
     const int full = D / VEC, tail = D % VEC;

@@ -360,13 +360,15 @@ __global__ void __launch_bounds__(256)
 reduce_partials_kernel(const float* __restrict__ partials, int splits, int64_t split_stride, int ldpart,
                        int O, int M, float* __restrict__ P, int64_t ldp, int beta)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t total = static_cast<int64_t>(O) * M;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total; idx += stride) {
         const int o = static_cast<int>(idx / M);
         const int m = static_cast<int>(idx - static_cast<int64_t>(o) * M);
         float p = beta ? P[o * ldp + m] : 0.f;
-        for (int s = 0; s < splits; ++s) p += __ldg(partials + s * split_stride + static_cast<int64_t>(o) * ldpart + m);
+        for (int s = 0; s < splits; ++s) p += partials[s * split_stride + static_cast<int64_t>(o) * ldpart + m];
         P[o * ldp + m] = p;
     }
 }
@@ -554,9 +556,8 @@ int launch_weight_grad_tc(const void* dY, int dy_dtype, int64_t N, int64_t O, in
         int64_t grid = ceil_div64(total, 256);
         const int64_t cap = static_cast<int64_t>(di.sm_count) * 8;
         if (grid > cap) grid = cap;
-        reduce_partials_kernel<<<static_cast<int>(grid), 256, 0, stream>>>(
-            partials, p.splits, a.split_stride, p.npad, static_cast<int>(O), p.M, P_out, ldp_out, beta);
-        return after_launch();
+        return launch_chained(reduce_partials_kernel, dim3(static_cast<unsigned>(grid)), 256, 0, stream,
+                              partials, p.splits, a.split_stride, p.npad, static_cast<int>(O), p.M, P_out, ldp_out, beta);
     }
     // 2a. one launch: cluster of the tile's splits, reduction through distributed shared memory
     const int L = (Dsub % 8 == 0) ? Dsub / 8 : 0;
