@@ -43,8 +43,8 @@ inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // has completed and its writes are visible), and only then pdl_trigger(), which lets the NEXT kernel start early: so
 // when kernel k + 1 becomes resident, everything up to k - 1 has completed.  A small layer is a chain of kernels of
 // 5-10 us with about 2 us of launch and set-up between them.
-// Not launched this way: the CTA-pair product (long queues of layers with it stopped making progress on the one
-// occasion it was, for a reason that has not been found; it runs long enough for 2 us not to matter).
+// Not launched this way: cluster launches, but for the weight gradient behind its own conversion (a long queue of layers
+// with the CTA-pair product among the chained kernels stopped making progress once, for a reason not found).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -158,7 +158,7 @@ gemm_simt_kernel(const AT* __restrict__ A, int64_t a_sm, int64_t a_sk, int a_mod
         for (int j = 0; j < 2 * G; ++j) acc[i][j] = 0ull;       // two zeros
 
     pdl_wait();
-    pdl_trigger();
+    if (gridDim.z == 1) pdl_trigger();
     float ra[8], rb[8];
     Tile<AT, T, TK>::load(A, a_sm, a_sk, m0, Mdim, k_begin, k_end, a_mode, ra);
     Tile<BT, T, TK>::load(B, b_sn, b_sk, n0, Ndim, k_begin, k_end, b_mode, rb);
@@ -251,14 +251,16 @@ int launch_tiles(const void* A, int64_t a_sm, int64_t a_sk, int a_mode, const vo
     cfg.gridDim = dim3(static_cast<unsigned>(ceil_div64(Ndim, T)), static_cast<unsigned>(ceil_div64(Mdim, T)), static_cast<unsigned>(splits));
     cfg.blockDim = dim3(SG_THREADS, 1, 1);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0] = pdl_attribute();
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = static_cast<unsigned>(splits);
+    cudaLaunchAttribute attr[1];
+    attr[0] = pdl_attribute();                                  // not for clusters (common.cuh)
+    if (splits > 1) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = static_cast<unsigned>(splits);
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = splits > 1 ? 2 : 1;
+    cfg.numAttrs = 1;
     const int64_t k_per_split = ceil_div64(ceil_div64(Kdim, TK), splits) * TK;
     if (cudaLaunchKernelEx(&cfg, gemm_simt_kernel<G, AT, BT, CT>, static_cast<const AT*>(A), a_sm, a_sk, a_mode,
                            static_cast<const BT*>(B), b_sn, b_sk, b_mode, static_cast<CT*>(C), ldc, beta, c_vec, Mdim, Ndim, Kdim,

@@ -97,6 +97,31 @@ template <> struct Store32<float> {
     }
 };
 
+// Four consecutive outputs of a row at a multiple of four columns, rows on 16-byte boundaries.
+template <typename CT> struct Store4;
+template <> struct Store4<__nv_bfloat16> {
+    static __device__ __forceinline__ void run(__nv_bfloat16* p, float (&y)[4], int beta)
+    {
+        uint2* q = reinterpret_cast<uint2*>(p);
+        if (beta) {
+            const uint2 old = *q;
+            y[0] += bf16_lo(old.x); y[1] += bf16_hi(old.x); y[2] += bf16_lo(old.y); y[3] += bf16_hi(old.y);
+        }
+        *q = make_uint2(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]));
+    }
+};
+template <> struct Store4<float> {
+    static __device__ __forceinline__ void run(float* p, float (&y)[4], int beta)
+    {
+        float4* q = reinterpret_cast<float4*>(p);
+        if (beta) {
+            const float4 old = *q;
+            y[0] += old.x; y[1] += old.y; y[2] += old.z; y[3] += old.w;
+        }
+        *q = make_float4(y[0], y[1], y[2], y[3]);
+    }
+};
+
 // Output rows that start on any element (odd pitch, no padding): a lane that stores its own row would touch 32
 // sectors per instruction, two bytes in each.  The warp turns its 32 x 32 block over through shared memory (32 rows of
 // kStagePitch floats; the odd pitch keeps both directions free of bank conflicts) and writes one row at a time,

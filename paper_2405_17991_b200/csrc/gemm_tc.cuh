@@ -62,6 +62,16 @@ int launch_pack_rows(const PackJob* jobs, int count, cudaStream_t stream);
 int make_tmap_bf16_chunks3d(CUtensorMap* map, const void* base, int64_t inner, int64_t outer, int64_t ld_elems,
                             int box_rows, int box_chunks);
 
+// A shape of the tensor-core product: the CTA-pair kernel, or the single-CTA kernel with tiles of 128 x bn and `splits` CTAs
+// (a cluster) sharing a tile's contraction.
+struct GemmShape {
+    bool pair;
+    int bn, splits;
+};
+int launch_linear_forward_tc_single(const GemmShape& shape, const void* X, int64_t ldx, const void* W, int64_t ldw, const float* v,
+                                    void* Y, int64_t ldy, void* Z, int z_dtype, int64_t ldz,
+                                    int64_t N, int64_t D, int64_t O, int Dsub, int* status, cudaStream_t stream);
+
 // Y = X W^T with compress(X, v) computed from the same staged X tiles.
 int launch_linear_forward_tc(const void* X, int64_t ldx, const void* W, int64_t ldw, const float* v,
                              void* Y, int64_t ldy, void* Z, int z_dtype, int64_t ldz,
