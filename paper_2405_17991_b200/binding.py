@@ -87,40 +87,47 @@ def lib() -> ctypes.CDLL:
 Z8_TORCH = getattr(torch, "float8_e4m3fn", None)      # torch's name for the E4M3 byte; torch.uint8 is accepted as well
 
 
+# uint8 / float8_e4m3fn: only Z may have this type; the library checks.
+_DTYPES = {torch.float32: F32, torch.bfloat16: BF16, torch.uint8: FP8_E4M3}
+if Z8_TORCH is not None:
+    _DTYPES[Z8_TORCH] = FP8_E4M3
+
+
 def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.uint8 or (Z8_TORCH is not None and t.dtype == Z8_TORCH):
-        return FP8_E4M3                                 # only Z may have this type; the library checks
-    raise TypeError("unsupported dtype %s (float32, bfloat16, or uint8 / float8_e4m3fn for Z)" % t.dtype)
+    dt = _DTYPES.get(t.dtype)
+    if dt is None:
+        raise TypeError("unsupported dtype %s (float32, bfloat16, or uint8 / float8_e4m3fn for Z)" % t.dtype)
+    return dt
 
 
 def _mat(t: torch.Tensor, name: str):
     if t.ndim != 2 or not t.is_cuda:
         raise ValueError("%s must be a 2-d CUDA tensor" % name)
-    if t.shape[1] > 1 and t.stride(1) != 1:
+    rows, cols = t.shape
+    ld, step = t.stride()
+    if step != 1 and cols > 1:
         raise ValueError("%s must have contiguous rows" % name)
-    ld = t.stride(0) if t.shape[0] > 1 else max(t.stride(0), t.shape[1])
-    return ctypes.c_void_p(t.data_ptr()), int(ld)
+    return t.data_ptr(), ld if rows > 1 else max(ld, cols)
 
 
-def _vec(v: torch.Tensor):
+def _vec(v: torch.Tensor) -> int:
     if v.ndim != 1 or v.dtype != torch.float32 or not v.is_cuda or not v.is_contiguous():
         raise ValueError("v must be a contiguous 1-d float32 CUDA tensor")
-    return ctypes.c_void_p(v.data_ptr())
+    return v.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+# The current stream of the current device as an integer, without building a Stream object (2 us of a call that
+# otherwise takes 6).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
-def _ws(ws: Optional[torch.Tensor], need: int, device) -> torch.Tensor:
-    if ws is None:
-        ws = velora_workspace_alloc(need, device)
-    return ws
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def velora_workspace_alloc(nbytes: int, device) -> torch.Tensor:
@@ -131,14 +138,14 @@ def velora_workspace_alloc(nbytes: int, device) -> torch.Tensor:
 
 
 def velora_workspace_init(ws: torch.Tensor, stream=None) -> None:
-    _check(lib().velora_workspace_init(ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream)),
+    _check(lib().velora_workspace_init(ws.data_ptr(), ws.numel(), _stream(stream)),
            "velora_workspace_init")
 
 
 def velora_workspace_status(ws: torch.Tensor, stream=None) -> int:
     """Synchronises the stream; 0, ERR_TIMEOUT if a kernel's bounded wait expired, or ERR_DEGENERATE_V
     left by velora_update_v."""
-    return int(lib().velora_workspace_status(ctypes.c_void_p(ws.data_ptr()), _stream(stream)))
+    return int(lib().velora_workspace_status(ws.data_ptr(), _stream(stream)))
 
 
 def velora_device_error(stream=None) -> int:
@@ -150,8 +157,8 @@ def velora_selftest_wait_timeout(ws: torch.Tensor, limit_ns: int, observed: torc
     """Runs the one-CTA kernel whose bounded waits expire; ``observed`` is a 4-element int32 CUDA tensor."""
     if observed.dtype != torch.int32 or observed.numel() < 4 or not observed.is_cuda or not observed.is_contiguous():
         raise ValueError("observed must be a contiguous int32 CUDA tensor with 4 elements")
-    _check(lib().velora_selftest_wait_timeout(ctypes.c_void_p(ws.data_ptr()), ws.numel(), int(limit_ns),
-                                              ctypes.c_void_p(observed.data_ptr()), _stream(stream)),
+    _check(lib().velora_selftest_wait_timeout(ws.data_ptr(), ws.numel(), int(limit_ns),
+                                              observed.data_ptr(), _stream(stream)),
            "velora_selftest_wait_timeout")
 
 
@@ -182,8 +189,9 @@ def velora_init_v(X: torch.Tensor, Dsub: int, v: Optional[torch.Tensor] = None,
     N, D = X.shape
     if v is None:
         v = torch.empty(Dsub, dtype=torch.float32, device=X.device)
-    ws = _ws(ws, velora_workspace_bytes(OP_INIT_V, N, D, 1, Dsub), X.device)
-    rc = lib().velora_init_v(xp, _dt(X), N, D, ldx, Dsub, _vec(v), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_INIT_V, N, D, 1, Dsub), X.device)
+    rc = lib().velora_init_v(xp, _dt(X), N, D, ldx, Dsub, _vec(v), ws.data_ptr(), ws.numel(),
                              _stream(stream))
     _check(rc, "velora_init_v")
     return v
@@ -239,9 +247,10 @@ def velora_weight_grad(dY: torch.Tensor, Z: torch.Tensor, v: torch.Tensor, D: in
         dW = torch.empty((O, D), dtype=dw_dtype or dY.dtype, device=dY.device)
     wp, lddw = _mat(dW, "dW")
     op = OP_WEIGHT_GRAD_FACTORED if mode == WG_FACTORED else OP_WEIGHT_GRAD_EXPLICIT
-    ws = _ws(ws, velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
     rc = lib().velora_weight_grad(yp, _dt(dY), N, O, lddy, zp, _dt(Z), ldz, _vec(v), D, Dsub,
-                                  wp, _dt(dW), lddw, beta, mode, ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+                                  wp, _dt(dW), lddw, beta, mode, ws.data_ptr(), ws.numel(),
                                   _stream(stream))
     _check(rc, "velora_weight_grad")
     return dW
@@ -263,9 +272,10 @@ def velora_linear_forward(X: torch.Tensor, W: torch.Tensor, v: torch.Tensor,
         Z = torch.empty((N, num_subtokens(D, Dsub)), dtype=z_dtype, device=X.device)
     yp, ldy = _mat(Y, "Y")
     zp, ldz = _mat(Z, "Z")
-    ws = _ws(ws, velora_workspace_bytes(OP_LINEAR_FORWARD, N, D, O, Dsub), X.device)
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_LINEAR_FORWARD, N, D, O, Dsub), X.device)
     rc = lib().velora_linear_forward(xp, ldx, wp, ldw, _vec(v), yp, ldy, zp, _dt(Z), ldz,
-                                     _dt(X), N, D, O, Dsub, ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+                                     _dt(X), N, D, O, Dsub, ws.data_ptr(), ws.numel(),
                                      _stream(stream))
     _check(rc, "velora_linear_forward")
     return Y, Z
@@ -285,13 +295,14 @@ def velora_linear_backward(dY: torch.Tensor, W: torch.Tensor, Z: torch.Tensor, v
         dX = torch.empty((N, D), dtype=dY.dtype, device=dY.device)
     if need_dW and dW is None:
         dW = torch.empty((O, D), dtype=dw_dtype or dY.dtype, device=dY.device)
-    xp, lddx = _mat(dX, "dX") if need_dX else (ctypes.c_void_p(0), D)
-    gp, lddw = _mat(dW, "dW") if need_dW else (ctypes.c_void_p(0), D)
+    xp, lddx = _mat(dX, "dX") if need_dX else (None, D)
+    gp, lddw = _mat(dW, "dW") if need_dW else (None, D)
     op = OP_LINEAR_BACKWARD_FACTORED if mode == WG_FACTORED else OP_LINEAR_BACKWARD_EXPLICIT
-    ws = _ws(ws, velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
     rc = lib().velora_linear_backward(yp, lddy, wp, ldw, zp, _dt(Z), ldz, _vec(v), xp, lddx,
                                       gp, _dt(dW) if need_dW else _dt(dY), lddw, beta, mode,
-                                      _dt(dY), N, D, O, Dsub, ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+                                      _dt(dY), N, D, O, Dsub, ws.data_ptr(), ws.numel(),
                                       _stream(stream))
     _check(rc, "velora_linear_backward")
     return dX, dW
@@ -309,9 +320,10 @@ def velora_dense_product(kind: int, A: torch.Tensor, B: torch.Tensor, C: Optiona
     if C is None:
         C = torch.empty((Mdim, Ndim), dtype=c_dtype or A.dtype, device=A.device)
     cp, ldc = _mat(C, "C")
-    ws = _ws(ws, 256, A.device)
+    if ws is None:
+        ws = velora_workspace_alloc(256, A.device)
     rc = lib().velora_dense_product(kind, ap, lda, bp, ldb, cp, _dt(C), ldc, beta, Mdim, Ndim, Kdim, _dt(A),
-                                    ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+                                    ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_dense_product")
     return C
 
@@ -324,9 +336,10 @@ def velora_z8_calibrate(X: torch.Tensor, v: torch.Tensor, headroom: float = 2.0,
     Dsub = v.shape[0]
     zscale = torch.empty(1, dtype=torch.float32, device=X.device)
     v_store, v_load = torch.empty_like(v), torch.empty_like(v)
-    ws = _ws(ws, velora_workspace_bytes(OP_Z8_CALIBRATE, N, D, 0, Dsub), X.device)
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_Z8_CALIBRATE, N, D, 0, Dsub), X.device)
     rc = lib().velora_z8_calibrate(xp, _dt(X), N, D, ldx, Dsub, _vec(v), float(headroom), _vec(zscale), _vec(v_store),
-                                   _vec(v_load), ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+                                   _vec(v_load), ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_z8_calibrate")
     return zscale, v_store, v_load
 
@@ -339,12 +352,12 @@ def velora_host_step_staging_bytes(N: int, D: int, O: int, Dsub: int) -> int:
     return int(lib().velora_host_step_staging_bytes(N, D, O, Dsub))
 
 
-def _host_ptr(t: Optional[torch.Tensor], shape, name: str) -> ctypes.c_void_p:
+def _host_ptr(t: Optional[torch.Tensor], shape, name: str) -> Optional[int]:
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     if t.is_cuda or t.dtype != torch.bfloat16 or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
         raise ValueError("%s must be a contiguous CPU bfloat16 tensor of shape %r" % (name, tuple(shape)))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def velora_linear_step_host(hX: torch.Tensor, hdY: torch.Tensor, W: torch.Tensor, v: torch.Tensor,
@@ -361,8 +374,8 @@ def velora_linear_step_host(hX: torch.Tensor, hdY: torch.Tensor, W: torch.Tensor
     rc = lib().velora_linear_step_host(
         _host_ptr(hX, (N, D), "hX"), _host_ptr(hdY, (N, O), "hdY"), _host_ptr(hY, (N, O), "hY"),
         _host_ptr(hdX, (N, D), "hdX"), _host_ptr(hdW, (O, D), "hdW"), wp, _vec(v),
-        ctypes.c_void_p(staging.data_ptr()), staging.numel(), N, D, O, Dsub,
-        ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+        staging.data_ptr(), staging.numel(), N, D, O, Dsub,
+        ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_linear_step_host")
 
 
@@ -370,11 +383,12 @@ def velora_subtoken_sum(X: torch.Tensor, Dsub: int, s: Optional[torch.Tensor] = 
                         ws: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Un-normalised sub-token sum of this rank's shard (add the ranks' sums, then velora_normalize_v)."""
     N, D = X.shape
-    xp, ldx = (_mat(X, "X") if N > 0 else (ctypes.c_void_p(0), D))
+    xp, ldx = (_mat(X, "X") if N > 0 else (None, D))
     if s is None:
         s = torch.empty(Dsub, dtype=torch.float32, device=X.device)
-    ws = _ws(ws, velora_workspace_bytes(OP_INIT_V, max(N, 1), D, 1, Dsub), X.device)
-    rc = lib().velora_subtoken_sum(xp, _dt(X), N, D, ldx, Dsub, _vec(s), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_INIT_V, max(N, 1), D, 1, Dsub), X.device)
+    rc = lib().velora_subtoken_sum(xp, _dt(X), N, D, ldx, Dsub, _vec(s), ws.data_ptr(), ws.numel(),
                                    _stream(stream))
     _check(rc, "velora_subtoken_sum")
     return s
@@ -388,7 +402,7 @@ def velora_update_v(X: torch.Tensor, Dsub: int, rho: float, a: torch.Tensor, v: 
     if ws is None:
         ws = velora_workspace_alloc(velora_workspace_bytes(OP_UPDATE_V, N, D, 1, Dsub), X.device)
     rc = lib().velora_update_v(xp, _dt(X), N, D, ldx, Dsub, float(rho), _vec(a), _vec(v),
-                               ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+                               ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_update_v")
 
 
@@ -397,8 +411,9 @@ def velora_normalize_v(s: torch.Tensor, v: Optional[torch.Tensor] = None, ws: Op
     Dsub = s.shape[0]
     if v is None:
         v = torch.empty_like(s)
-    ws = _ws(ws, 256, s.device)
-    rc = lib().velora_normalize_v(_vec(s), Dsub, _vec(v), ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+    if ws is None:
+        ws = velora_workspace_alloc(256, s.device)
+    rc = lib().velora_normalize_v(_vec(s), Dsub, _vec(v), ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_normalize_v")
     return v
 
@@ -408,14 +423,15 @@ def velora_weight_grad_p(dY: torch.Tensor, Z: torch.Tensor, D: int, Dsub: int, P
     """P[O, M] = beta * P + dY^T Z in fp32: the weight gradient before its expansion by v."""
     N, O = dY.shape
     M = num_subtokens(D, Dsub)
-    yp, lddy = (_mat(dY, "dY") if N > 0 else (ctypes.c_void_p(0), O))
-    zp, ldz = (_mat(Z, "Z") if N > 0 else (ctypes.c_void_p(0), M))
+    yp, lddy = (_mat(dY, "dY") if N > 0 else (None, O))
+    zp, ldz = (_mat(Z, "Z") if N > 0 else (None, M))
     if P is None:
         P = torch.zeros((O, M), dtype=torch.float32, device=dY.device)
     pp, ldp = _mat(P, "P")
-    ws = _ws(ws, velora_workspace_bytes(OP_WEIGHT_GRAD_FACTORED, N, D, O, Dsub), dY.device)
+    if ws is None:
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_WEIGHT_GRAD_FACTORED, N, D, O, Dsub), dY.device)
     rc = lib().velora_weight_grad_p(yp, _dt(dY), N, O, lddy, zp, _dt(Z), ldz, D, Dsub, pp, ldp, beta,
-                                    ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream))
+                                    ws.data_ptr(), ws.numel(), _stream(stream))
     _check(rc, "velora_weight_grad_p")
     return P
 
