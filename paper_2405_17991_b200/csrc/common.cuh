@@ -138,6 +138,21 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
+#ifdef __CUDACC__
+// Eight consecutive floats at a 16-byte boundary.  In one 32-byte store where that is a whole sector: as two 16-byte
+// stores every sector is written twice, half of it each time (fp32 gradient of a 4096 x 5461 -> 2048 layer: 33 -> 27 us).
+__device__ __forceinline__ void store_f32x8(float* p, const float (&y)[8])
+{
+    if ((reinterpret_cast<uintptr_t>(p) & 31u) == 0) {
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"l"(p), "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7]) : "memory");
+    } else {
+        __stcs(reinterpret_cast<float4*>(p), make_float4(y[0], y[1], y[2], y[3]));
+        __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(y[4], y[5], y[6], y[7]));
+    }
+}
+#endif
+
 // One byte of the 8-bit floating-point format E4M3 (4 exponent bits, bias 7; 3 mantissa bits; no infinities,
 // largest finite value 448): a storage type for Z only.  Conversions are the hardware's: round to nearest
 // even, saturating at +-448.

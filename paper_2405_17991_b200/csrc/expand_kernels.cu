@@ -59,8 +59,7 @@ template <> struct Out8<float> {
             y[0] += a.x; y[1] += a.y; y[2] += a.z; y[3] += a.w;
             y[4] += b.x; y[5] += b.y; y[6] += b.z; y[7] += b.w;
         }
-        __stcs(q, make_float4(y[0], y[1], y[2], y[3]));
-        __stcs(q + 1, make_float4(y[4], y[5], y[6], y[7]));
+        store_f32x8(p, y);
     }
 };
 

@@ -20,8 +20,11 @@
 //                      Two launch shapes: two CTAs of six warps per SM (ring of 2..4 stages), or, where the
 //                      partial products are large and the row blocks few, one CTA of twelve warps per SM with
 //                      half as many splits (half the reduction traffic, four stages, as many warps writing).
-//     CLUSTER = false  the partials go to the workspace and launch_expand_p sums and expands them
-//                      (shapes the cluster form does not take: Dsub not 8 * 2^k, unaligned dW rows).
+//     CLUSTER = false  the partials go to the workspace (L2), and launch_expand_p sums and expands them with every SM full
+//                      of warps: shapes the cluster form does not take (Dsub not 8 * 2^k, unaligned dW rows), and
+//                      outputs of so few row blocks that its grid would fill less than half of the chip.
+//                      Clustered / through the workspace, us: 14.4 / 13.3 at 8192 x 512 -> 512 (32 CTAs), 27 / 23 at
+//                      4096 x 5461 -> 2048 in fp32 (128), 28.8 / 29.0 at 8192 x 4096 -> 4096 (256).
 // Summing the partials in a fixed order keeps the result run-to-run identical.
 #include <cooperative_groups.h>
 
@@ -112,8 +115,7 @@ template <> struct WgOut8<float> {
             y[0] += a.x; y[1] += a.y; y[2] += a.z; y[3] += a.w;
             y[4] += b.x; y[5] += b.y; y[6] += b.z; y[7] += b.w;
         }
-        __stcs(q, make_float4(y[0], y[1], y[2], y[3]));
-        __stcs(q + 1, make_float4(y[4], y[5], y[6], y[7]));
+        store_f32x8(p, y);
     }
 };
 
@@ -561,7 +563,8 @@ int launch_weight_grad_tc(const void* dY, int dy_dtype, int64_t N, int64_t O, in
     }
     // 2a. one launch: cluster of the tile's splits, reduction through distributed shared memory
     const int L = (Dsub % 8 == 0) ? Dsub / 8 : 0;
-    const bool vec = L >= 1 && L <= 128 && (L & (L - 1)) == 0 && aligned16(dW) &&
+    const bool filled = p.fat || static_cast<int64_t>(p.tiles_o) * p.splits > di.sm_count;
+    const bool vec = filled && L >= 1 && L <= 128 && (L & (L - 1)) == 0 && aligned16(dW) &&
                      (lddw * static_cast<int64_t>(dtype_size(dw_dtype))) % 16 == 0 &&
                      static_cast<size_t>(WG_BM) * (p.npad + 4) * 4 <= static_cast<size_t>(p.tail_off);
     if (vec) {
