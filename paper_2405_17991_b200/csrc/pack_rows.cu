@@ -7,16 +7,17 @@
 // a 4096 x 5461 -> 2048 product took 84 us with both operands at a pitch of 10928 bytes (every other row starts in
 // the middle of a 32-byte sector) and 70 us at 11008.
 //
-// A warp takes 256 consecutive 16-byte chunks of a row, eight per lane, all loads issued before the first is used.
-// The source of a chunk sits at any even byte offset, so a lane loads the two aligned 16-byte chunks that cover it
-// (the second is its neighbour's first: an L1 hit) and shifts; the offset is the same for a whole row.
+// A warp takes 128 consecutive 16-byte chunks of a row, four per lane, all loads issued before the first is used.
+// The source of a chunk sits at any even byte offset, the same for a whole row.  A lane loads the aligned 16 bytes in which
+// its chunk begins, takes the rest from its neighbour (whose chunk begins there) and shifts; only the last lane of the
+// last step loads a second time.
 #include "gemm_tc.cuh"
 
 namespace velora {
 namespace {
 
 constexpr int PK_THREADS = 256;
-constexpr int PK_U = 8;                                    // chunks per lane
+constexpr int PK_U = 4;                                    // chunks per lane
 constexpr int PK_SEG = 32 * PK_U;                          // chunks per warp and step
 
 struct PackArgs {
@@ -29,26 +30,22 @@ struct PackArgs {
     int64_t items[2];                                      // rows x segments
 };
 
-__device__ __forceinline__ uint4 load_unaligned(const char* p, const char* lo_limit, const char* hi_limit)
+// The aligned 16 bytes at `a`; bytes outside the matrix are not touched and read as zero.
+__device__ __forceinline__ uint4 load_aligned(const char* a, const char* lo_limit, const char* hi_limit)
 {
-    const uint32_t s = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p) & 15u);
-    const char* a = p - s;
-    uint32_t w[8];
-    if (a >= lo_limit && a + (s ? 32 : 16) <= hi_limit) {
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(a));
-        uint4 y = make_uint4(0u, 0u, 0u, 0u);
-        if (s) y = __ldg(reinterpret_cast<const uint4*>(a) + 1);
-        w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
-        w[4] = y.x; w[5] = y.y; w[6] = y.z; w[7] = y.w;
-    } else {
-        // The first and the last chunks of the matrix: no byte outside it is touched.
-        uint32_t o[4] = {0u, 0u, 0u, 0u};
+    if (a >= lo_limit && a + 16 <= hi_limit) return __ldcs(reinterpret_cast<const uint4*>(a));
+    uint32_t o[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            if (p + 2 * e < hi_limit)
-                o[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(p + 2 * e)) << (16 * (e & 1));
-        return make_uint4(o[0], o[1], o[2], o[3]);
-    }
+    for (int e = 0; e < 8; ++e)
+        if (a + 2 * e >= lo_limit && a + 2 * e < hi_limit)
+            o[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(a + 2 * e)) << (16 * (e & 1));
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Sixteen bytes from byte s (even) of the 32 in x, y.
+__device__ __forceinline__ uint4 shift_pair(const uint4& x, const uint4& y, uint32_t s)
+{
+    uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
     if (s & 8u) {
 #pragma unroll
         for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
@@ -76,14 +73,28 @@ pack_rows_kernel(const PackArgs a)
         const unsigned row = item / static_cast<unsigned>(a.segs[k]);
         const int c0 = static_cast<int>(item - row * a.segs[k]) * PK_SEG + lane;
         const char* rp = a.src[k] + static_cast<int64_t>(row) * a.src_pitch[k];
-        uint4 d[PK_U];
+        const uint32_t shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(rp) & 15u);
+        const char* ap = rp - shift;
+        uint4 d[PK_U], over = make_uint4(0u, 0u, 0u, 0u);     // chunks at or beyond the row's end are loaded, not used
 #pragma unroll
         for (int u = 0; u < PK_U; ++u)
-            if (c0 + 32 * u < a.chunks[k]) d[u] = load_unaligned(rp + 16 * static_cast<int64_t>(c0 + 32 * u), a.src[k], a.src_end[k]);
+            d[u] = c0 - lane + 32 * u <= a.chunks[k] ? load_aligned(ap + 16 * static_cast<int64_t>(c0 + 32 * u), a.src[k], a.src_end[k])
+                                                     : make_uint4(0u, 0u, 0u, 0u);
+        if (lane == 31) over = load_aligned(ap + 16 * static_cast<int64_t>(c0 + 32 * PK_U - 31), a.src[k], a.src_end[k]);
+        over.x = __shfl_sync(0xffffffffu, over.x, 31); over.y = __shfl_sync(0xffffffffu, over.y, 31);
+        over.z = __shfl_sync(0xffffffffu, over.z, 31); over.w = __shfl_sync(0xffffffffu, over.w, 31);
         uint4* op = a.dst[k] + static_cast<int64_t>(row) * a.dst_pitch[k];
 #pragma unroll
-        for (int u = 0; u < PK_U; ++u)
-            if (c0 + 32 * u < a.chunks[k]) op[c0 + 32 * u] = d[u];
+        for (int u = 0; u < PK_U; ++u) {
+            // The next chunk's beginning: lane + 1 of this step, for lane 31 lane 0 of the next.
+            const uint4 nx = u + 1 < PK_U ? d[(u + 1) % PK_U] : over;
+            const uint4 give = lane == 0 ? nx : d[u];
+            const int from = (lane + 1) & 31;
+            uint4 y;
+            y.x = __shfl_sync(0xffffffffu, give.x, from); y.y = __shfl_sync(0xffffffffu, give.y, from);
+            y.z = __shfl_sync(0xffffffffu, give.z, from); y.w = __shfl_sync(0xffffffffu, give.w, from);
+            if (c0 + 32 * u < a.chunks[k]) op[c0 + 32 * u] = shift_pair(d[u], y, shift);
+        }
     }
 }
 
