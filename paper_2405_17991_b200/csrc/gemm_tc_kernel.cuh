@@ -30,8 +30,10 @@ constexpr int BM = 128, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;              // 16 KB
 constexpr int SLAB_BYTES = 64 * BK * 2;           // one 64-wide MN-major slab: 64 k-rows x 128 bytes
 constexpr int MAX_SPLITS = 8;                     // the portable cluster size
-constexpr int GEMM_THREADS = 192;
-constexpr int FUSE_THREADS = GEMM_THREADS + 192;    // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
+constexpr int GEMM_THREADS = 192;                   // producer, issuer, four epilogue warps
+constexpr int GEMM_THREADS_SHORT = 320;             // eight epilogue warps, for contractions of up to SHORT_KBLOCKS k-blocks
+constexpr int SHORT_KBLOCKS = 8;
+constexpr int FUSE_THREADS = 384;    // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
 constexpr int STAGE_OFF = 256;                    // behind the ring: barriers, then the staging of unaligned output rows
 
 // What depends on the tile's width: as many stages as fit 200 KB, at most eight.
@@ -72,7 +74,7 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, int tiles_m, int tiles
 // and they sit on warps 6, 7, 10, 11 so that none of them shares a warp scheduler (warp % 4) with the TMA
 // producer (warp 0) or the MMA issuer (warp 1).
 template <bool A_MN, bool B_MN, typename CT, int FUSE, int BN>
-__global__ void __launch_bounds__(FUSE ? FUSE_THREADS : GEMM_THREADS, 1)
+__global__ void __launch_bounds__(FUSE ? FUSE_THREADS : GEMM_THREADS_SHORT, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
                int tiles_m, int tiles_n, int kb_per_split, int c_vec, int* __restrict__ status, const FuseArgs fz)
@@ -109,7 +111,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull + 8 * a, 1);
-            mbar_init(tempty + 8 * a, 4);
+            mbar_init(tempty + 8 * a, FUSE ? 4 : (blockDim.x - 64) / 32);        // the epilogue's warps
         }
         *abort_flag = 0;
         *tiles_started = 0;
@@ -223,8 +225,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         else if (fz.Dsub == 512) walk(VSlice<2>{});
         else walk(VSlice<4>{});
     } else {
-        // ------------------------------------------------ epilogue (4 warps, one TMEM lane quarter each)
+        // ------------------------------------------------ epilogue (one TMEM lane quarter per warp; short contractions have
+        // two sets of four warps, which take the 64-column steps in turn: 22 -> 20 us for 8192 x 4096 with K = 16, no gain at
+        // K = 3072)
         const int quarter = warp & 3;
+        const int set = FUSE ? 0 : (warp - 2) >> 2;
+        const int sets = FUSE || blockDim.x == GEMM_THREADS || (!c_vec && splits == 1) ? 1 : 2;     // staging room for four warps
         uint32_t t = 0;
         for (int tile = blockIdx.x; tile < num_tiles && !failed; tile += gridDim.x, ++t) {
             const TileCoord tc0 = tile_coord<BN>(tile, tiles_m, tiles_n);
@@ -236,7 +242,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (splits > 1) {                                 // one tile per CTA: park the partial product
                 float* prow = reinterpret_cast<float*>(smem) + (quarter * 32 + lane) * S::kPartialPitch;
 #pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
+                for (int c = set; c < BN / 32; c += sets) {
                     uint32_t r[32];
                     tmem_ld_32x32(taddr + c * 32, r);
                     tmem_ld_wait();
@@ -247,13 +253,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 continue;
             }
             CT* crow = C + static_cast<int64_t>(row) * ldc + tc0.n0;
+            const int last = set >= sets ? -1 : ((BN / 64 - 1 - set) / sets * sets + set) * 2;    // this warp's last step
+            if (last < 0 || set >= BN / 64) {                 // nothing for this set in a tile of this width
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty + 8 * acc);
+                continue;
+            }
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; c += 2) {            // 64 columns a step: two TMEM loads in flight
+            for (int c = 2 * set; c < BN / 32; c += 2 * sets) {       // 64 columns a step: two TMEM loads in flight
                 uint32_t r[2][32];
                 tmem_ld_32x32(taddr + c * 32, r[0]);
                 tmem_ld_32x32(taddr + c * 32 + 32, r[1]);
                 tmem_ld_wait();
-                if (c == BN / 32 - 2) {                       // accumulator fully read: hand it back
+                if (c == last) {                              // this warp has read its share: hand it back
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty + 8 * acc);
@@ -343,7 +355,7 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     const int tiles_m = (Mdim + BM - 1) / BM, tiles_n = (Ndim + BN - 1) / BN;
     const int64_t tiles = static_cast<int64_t>(tiles_m) * tiles_n;
     const int kblocks = (Kdim + BK - 1) / BK;
-    const int threads = FUSE ? FUSE_THREADS : GEMM_THREADS;
+    const int threads = FUSE ? FUSE_THREADS : (kblocks <= SHORT_KBLOCKS * splits ? GEMM_THREADS_SHORT : GEMM_THREADS);
     const int c_vec = c_rows_vec(C, ldc, sizeof(CT));
     if (splits <= 1) {
         const int grid = static_cast<int>(tiles < di.sm_count ? tiles : di.sm_count);
