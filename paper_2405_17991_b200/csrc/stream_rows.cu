@@ -37,14 +37,16 @@ template <> __device__ __forceinline__ void put_z<float>(float* p, float z) { *p
 template <> __device__ __forceinline__ void put_z<__nv_bfloat16>(__nv_bfloat16* p, float z) { *p = __float2bfloat16_rn(z); }
 template <> __device__ __forceinline__ void put_z<e4m3_t>(e4m3_t* p, float z) { *p = float_to_e4m3(z); }
 
-// Chunk c of a row as loaded, and its VEC values; zeros beyond column D.  full = D / VEC whole chunks, tail = D % VEC.
+// Chunk c of a row as loaded (KEEP: a compress of the same rows is likely to follow, so they
+// are left in L2), and its VEC values; zeros beyond column D.  full = D / VEC whole chunks, tail = D % VEC.
 template <typename XT, int VEC> struct Chunk;
 template <> struct Chunk<__nv_bfloat16, 8> {
     typedef uint4 Raw;
+    template <bool KEEP>
     static __device__ __forceinline__ Raw load(const __nv_bfloat16* __restrict__ row, int c, int full, int tail)
     {
         const uint4* q = reinterpret_cast<const uint4*>(row) + c;
-        if (c < full) return __ldcs(q);
+        if (c < full) return KEEP ? __ldg(q) : __ldcs(q);
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
         if (c == full && tail) {
             x = __ldcs(q);                       // inside the row's pitch (a multiple of 8 elements)
@@ -68,10 +70,11 @@ template <> struct Chunk<__nv_bfloat16, 8> {
 };
 template <> struct Chunk<float, 4> {
     typedef float4 Raw;
+    template <bool KEEP>
     static __device__ __forceinline__ Raw load(const float* __restrict__ row, int c, int full, int tail)
     {
         const float4* q = reinterpret_cast<const float4*>(row) + c;
-        if (c < full) return __ldcs(q);
+        if (c < full) return KEEP ? __ldg(q) : __ldcs(q);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c == full && tail) {                 // the row may end inside the chunk and so may the buffer
             x.x = row[4 * c];
@@ -84,6 +87,7 @@ template <> struct Chunk<float, 4> {
 };
 template <typename XT> struct Chunk<XT, 1> {
     typedef XT Raw;
+    template <bool KEEP>
     static __device__ __forceinline__ Raw load(const XT* __restrict__ row, int c, int full, int)
     {
         return c < full ? __ldg(row + c) : static_cast<XT>(0.f);
@@ -114,14 +118,17 @@ stream_rows_kernel(const XT* __restrict__ X, int N, int D, int64_t ldx, int M,
 #pragma unroll
         for (int e = 0; e < VEC; ++e) vr[i][e] = INIT ? 0.f : __ldg(v + VEC * (q + LPS * i) + e);
 
+    // compress goes through the rows from the last to the first: whatever read or wrote X before it went the other way, so the
+    // last rows are the ones still in L2 (a 180 MB X right behind its sub-token sum: 32 -> 23 us).
     const int warps = gridDim.x * RW_WARPS;
-    for (int row = blockIdx.x * RW_WARPS + (threadIdx.x >> 5); row < N; row += warps) {
+    for (int at = blockIdx.x * RW_WARPS + (threadIdx.x >> 5); at < N; at += warps) {
+        const int row = INIT ? at : N - 1 - at;
         const XT* rp = X + static_cast<int64_t>(row) * ldx;
         ZT* zrow = INIT ? nullptr : Z + static_cast<int64_t>(row) * ldz;
         for (int c0 = 0; c0 < cpr; c0 += 32 * U) {
             typename C::Raw d[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) d[u] = C::load(rp, c0 + 32 * u + lane, full, tail);
+            for (int u = 0; u < U; ++u) d[u] = C::template load<INIT>(rp, c0 + 32 * u + lane, full, tail);
             float part = 0.f;                     // CH > 1: sum over the parts of one sub-token so far
 #pragma unroll
             for (int u = 0; u < U; ++u) {
