@@ -44,10 +44,11 @@
  *     empty sum, dW = beta * dW: beta = 0 fills dW with zeros, beta = 1 leaves it.
  *   - Vector (128-bit) kernels are used when base pointers are 16-byte aligned,
  *     leading dimensions are multiples of 16 bytes and Dsub is a multiple of 8
- *     (fastest for 8 * 2^k) or one of 1, 2, 4; otherwise the element-wise kernels
+ *     (fastest for 8 * 2^k) or one of 1, 2, 4; otherwise kernels that take one element at a time
  *     run (same results, lower speed).  The
- *     tensor-core GEMMs need 16-byte aligned bf16 rows; other cases run on the
- *     CUDA-core GEMM.
+ *     tensor-core GEMMs read 16-byte aligned bf16 rows; operands whose rows are not are copied
+ *     into the workspace first, where it has the room that velora_workspace_bytes reports
+ *     for widths that are no multiple of 8.  Without it, and for fp32, the CUDA-core GEMM runs.
  */
 #ifndef VELORA_H
 #define VELORA_H
@@ -103,7 +104,9 @@ const char* velora_status_string(int status);
 
 /*
  * Bytes of device workspace the given entry point needs for these sizes
- * (0 if it needs none).  Independent of pointer values; deterministic.
+ * (0 if it needs none).  Independent of pointer values; deterministic.  Where D or O is no multiple of 8 the
+ * figure includes room for aligned copies of the bf16 operands of that width; a workspace
+ * smaller by that much is accepted and costs speed on rows that are not 16-byte aligned.
  */
 size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub);
 
@@ -281,7 +284,7 @@ int velora_z8_calibrate(const void* X, int x_dtype, int64_t N, int64_t D, int64_
  *   VELORA_PRODUCT_A_BT:  A[Mdim, Kdim], B[Ndim, Kdim]    (C = A B^T)
  *   VELORA_PRODUCT_A_B:   A[Mdim, Kdim], B[Kdim, Ndim]    (C = A B)
  *   VELORA_PRODUCT_AT_B:  A[Kdim, Mdim], B[Kdim, Ndim]    (C = A^T B)
- * `dtype`: storage type of A and B (bf16: tensor cores when rows are 16-byte aligned; otherwise and for
+ * `dtype`: storage type of A and B (bf16: tensor cores when their rows are 16-byte aligned; otherwise and for
  * f32 the CUDA-core product).  C: c_dtype, bf16 or f32.  ws: at least 256 bytes, initialised (status header).
  */
 typedef enum { VELORA_PRODUCT_A_BT = 0, VELORA_PRODUCT_A_B = 1, VELORA_PRODUCT_AT_B = 2 } velora_product;
