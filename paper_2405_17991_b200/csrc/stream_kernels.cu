@@ -69,8 +69,8 @@ init_v_partial_elem_kernel(const XT* __restrict__ X, int64_t N, int D, int64_t l
 // The partial rows come from up to ~1200 CTAs and sit in L2; adding them is a chain of load latencies, so
 // the CTA is as wide as it can be (1024 threads) and a thread owns VEC consecutive positions (one 16-byte
 // load for VEC = 4): for a block of up to 1024 position groups the threads split the partial rows into
-// `slots` interleaved sets (eight independent loads in flight each), then one thread per group adds the
-// sets in order.  The order depends only on the sizes, so the result is run-to-run identical.
+// `slots` interleaved sets (eight independent loads in flight each), then a tree adds the
+// sets.  The order depends only on the sizes, so the result is run-to-run identical.
 constexpr int kFinThreads = 1024;
 
 template <int VEC>
@@ -117,13 +117,18 @@ init_v_finalize_kernel(const float* __restrict__ partials, int num_partials, int
 #pragma unroll
         for (int e = 0; e < VEC; ++e) s_red[threadIdx.x * VEC + e] = s[e];
         __syncthreads();
+        for (int n = slots; n > 1;) {                              // a tree over the sets: 64 of them one after the other took 2 us
+            const int half = (n + 1) / 2;
+            if (slot < n - half) {
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) s_red[threadIdx.x * VEC + e] += s_red[(threadIdx.x + half * width) * VEC + e];
+            }
+            __syncthreads();
+            n = half;
+        }
         if (threadIdx.x < width) {
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) {
-                double t = 0.0;
-                for (int k = 0; k < slots; ++k) t += s_red[(k * width + threadIdx.x) * VEC + e];
-                s_sum[g * VEC + e] = t;
-            }
+            for (int e = 0; e < VEC; ++e) s_sum[g * VEC + e] = s_red[threadIdx.x * VEC + e];
         }
         __syncthreads();
     }
