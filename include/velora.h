@@ -49,6 +49,8 @@
  *     tensor-core GEMMs read 16-byte aligned bf16 rows; operands whose rows are not are copied
  *     into the workspace first, where it has the room that velora_workspace_bytes reports
  *     for widths that are no multiple of 8.  Without it, and for fp32, the CUDA-core GEMM runs.
+ *     The factored weight gradient of such bf16 rows runs on the CUDA cores in either case, with Z
+ *     as stored; on aligned rows of more than 64 columns it rounds an fp32 Z to bf16 for the tensor cores.
  */
 #ifndef VELORA_H
 #define VELORA_H

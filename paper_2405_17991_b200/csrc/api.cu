@@ -118,12 +118,10 @@ int pack_operands(Operand** ops, int count, void* ws, size_t ws_bytes, size_t us
     return VELORA_OK;
 }
 
-// The weight gradient's kernels that read dY through TMA: the dense product, and the factored form but for adapter
-// shapes (plain loads) and rows of more than 256 sub-tokens (CUDA cores).
-bool weight_grad_wants_tma(int64_t D, int64_t O, int Dsub, int mode)
-{
-    return mode == VELORA_WG_EXPLICIT || (O > 64 && num_subtokens(D, Dsub) <= 256);
-}
+// Whether the weight gradient runs on a packed copy of dY: the dense product with a bf16 result only.  The factored form
+// keeps such rows on the CUDA cores: its tensor-core kernel rounds an fp32 Z to bf16 (error of P at 4096 tokens: 2e-3
+// instead of 2e-7) and adds up with truncation, as the tensor cores do (P from a bf16 Z of 12608 tokens: 3.4e-6 instead of 2e-7).
+bool weight_grad_packs(int mode, int dw_dtype) { return mode == VELORA_WG_EXPLICIT && dw_dtype == VELORA_BF16; }
 
 // ---- weight gradient routing ----
 int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
@@ -142,7 +140,8 @@ int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t
     }
     if (mode == VELORA_WG_FACTORED) {
         if (ws_bytes < factored_bytes(N, D, O, Dsub)) return VELORA_ERR_WORKSPACE;
-        // Adapter-shaped layers (O <= 64; too few output tiles for the tensor-core kernel to spread) and fp32 first.
+        // Adapter-shaped layers (O <= 64; too few output tiles for the tensor-core kernel to spread), fp32 and bf16 rows
+        // on odd boundaries first.
         int rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
                                            beta, body, ws_bytes - kStatusBytes, stream, nullptr, 0);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;
@@ -254,7 +253,7 @@ size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub)
     if (N < 0 || D < 1 || Dsub < 1 || Dsub > D || Dsub > VELORA_MAX_DSUB) return 0;
     switch (op) {
         case VELORA_OP_INIT_V: return init_v_workspace_bytes(Dsub);
-        case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O);
+        case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub);
         case VELORA_OP_LINEAR_BACKWARD_FACTORED:
             return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O) + pack_bytes_if_ragged(O, D);
         case VELORA_OP_WEIGHT_GRAD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O);
@@ -321,7 +320,7 @@ int velora_weight_grad(const void* dY, int dy_dtype, int64_t N, int64_t O, int64
     const size_t need = mode == VELORA_WG_FACTORED ? factored_bytes(N, D, O, Dsub) : xhat_bytes(N, D);
     if (ws_bytes < need) return VELORA_ERR_WORKSPACE;
     Operand y{dY, lddy, N, O};
-    if (N > 0 && dy_dtype == VELORA_BF16 && weight_grad_wants_tma(D, O, Dsub, mode)) {
+    if (N > 0 && dy_dtype == VELORA_BF16 && weight_grad_packs(mode, dw_dtype)) {
         Operand* ops[1] = {&y};
         rc = pack_operands(ops, 1, ws, ws_bytes, need, static_cast<cudaStream_t>(stream));
         if (rc != VELORA_OK) return rc;
@@ -394,23 +393,22 @@ int velora_linear_backward(const void* dY, int64_t lddy, const void* W, int64_t 
     if (!aligned16(ws)) return VELORA_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Operand y{dY, lddy, N, O}, w{W, ldw, O, D};
-    if (N > 0 && dtype == VELORA_BF16 && (dX || (dW && weight_grad_wants_tma(D, O, Dsub, mode)))) {
+    const bool pack_for_dw = dW && weight_grad_packs(mode, dw_dtype);
+    if (N > 0 && dtype == VELORA_BF16 && (dX || pack_for_dw)) {
         Operand* ops[2] = {&y, &w};
         rc = pack_operands(ops, dX ? 2 : 1, ws, ws_bytes, used, s);
         if (rc != VELORA_OK) return rc;
     }
-    dY = y.p;
-    lddy = y.ld;
     if (dX && N > 0) {
-        rc = launch_gemm_tc(GEMM_NN_K_MN, dY, lddy, w.p, w.ld, dX, dtype, lddx, 0, N, D, O, dtype,
+        rc = launch_gemm_tc(GEMM_NN_K_MN, y.p, y.ld, w.p, w.ld, dX, dtype, lddx, 0, N, D, O, dtype,
                             static_cast<int*>(ws), s);
         if (rc == VELORA_ERR_UNSUPPORTED)
             rc = launch_gemm_simt(dY, dtype, lddy, 1, W, dtype, 1, ldw, dX, dtype, lddx, 0, N, D, O, s);
         if (rc != VELORA_OK) return rc;
     }
     if (dW)
-        return weight_grad_impl(dY, dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
-                                beta, mode, ws, ws_bytes, s);
+        return weight_grad_impl(pack_for_dw ? y.p : dY, dtype, N, O, pack_for_dw ? y.ld : lddy, Z, z_dtype, ldz, v, D, Dsub,
+                                dW, dw_dtype, lddw, beta, mode, ws, ws_bytes, s);
     return VELORA_OK;
 }
 
@@ -577,14 +575,6 @@ int velora_weight_grad_p(const void* dY, int dy_dtype, int64_t N, int64_t O, int
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* status = static_cast<int*>(ws);
     char* body = static_cast<char*>(ws) + kStatusBytes;
-    Operand y{dY, lddy, N, O};
-    if (N > 0 && dy_dtype == VELORA_BF16 && weight_grad_wants_tma(D, O, Dsub, VELORA_WG_FACTORED)) {
-        Operand* ops[1] = {&y};
-        rc = pack_operands(ops, 1, ws, ws_bytes, factored_bytes(N, D, O, Dsub), st);
-        if (rc != VELORA_OK) return rc;
-        dY = y.p;
-        lddy = y.ld;
-    }
     if (N > 0) {
         rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D,
                                        beta, body, ws_bytes - kStatusBytes, st, P, ldp);

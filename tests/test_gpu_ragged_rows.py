@@ -79,6 +79,35 @@ def test_layer_on_rows_that_start_anywhere(vl, guard, N, D, O, Dsub, pad, offset
     assert_matches(P, oracle.linear_forward(dY64.T, to_f64(Z).T), TOL_GEMM, "P", c=C_ROUNDED)
 
 
+# The factored gradient of rows on odd boundaries is an fp32 sum of products with Z as stored, whatever the workspace holds:
+# a Z rounded to bf16 on the way would show as 2e-3.  One slice, several, blocks of 1 .. 8 times 32 sub-tokens, more than 256
+# sub-tokens (the general fp32 product), adapter width.  Bound as in the fp32 tests: 3.84 * N * 2^-24 of the column's rms.
+@pytest.mark.parametrize("N,D,O,Dsub", [(37, 257, 131, 16), (1100, 2049, 1801, 128), (2500, 640, 2731, 64), (777, 1025, 97, 8), (700, 1031, 203, 4),
+                                        (513, 1023, 13, 32)])
+@pytest.mark.parametrize("z_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("room", [True, False])
+def test_factored_gradient_keeps_every_bit_of_z(vl, guard, N, D, O, Dsub, z_dtype, room):
+    case = vi.small_case(13 * N + D, N, D, O, dtype="bf16", mean_offset=0.1)
+    X, W, dY = (_view(case[k].torch(DEV), case[k].torch(DEV).shape[1], 1) for k in ("X", "W", "dY"))
+    v = vl.velora_init_v(X, Dsub)
+    M = vl.num_subtokens(D, Dsub)
+    Z = vl.velora_compress(X, v, z_dtype=z_dtype)
+    c = 3.84 * 2500 * 2.0 ** -24
+
+    def ws(op):
+        return guard.workspace(vl, vl.velora_workspace_bytes(op, N, D, O if room else -(-O // 8) * 8, Dsub))
+
+    P = vl.velora_weight_grad_p(dY, Z, D, Dsub, P=guard.mat(O, M, torch.float32), ws=ws(vl.OP_WEIGHT_GRAD_FACTORED))
+    assert_matches(P, case["dY"].f64().T @ to_f64(Z), 1e-5, "P", c=c)
+    ref = oracle.weight_grad(case["dY"].f64(), to_f64(Z), to_f64(v), D)
+    dW = vl.velora_weight_grad(dY, Z, v, D, dW=guard.mat(O, D, torch.float32, ld=D), ws=ws(vl.OP_WEIGHT_GRAD_FACTORED))
+    assert_matches(dW, ref, 1e-5, "dW", c=c)
+    for need_dX in (True, False):
+        _, dW = vl.velora_linear_backward(dY, W, Z, v, dX=guard.mat(N, D, ld=D), dW=guard.mat(O, D, torch.float32, ld=D), need_dX=need_dX,
+                                          ws=ws(vl.OP_LINEAR_BACKWARD_FACTORED))
+        assert_matches(dW, ref, 1e-5, "dW of the backward", c=c)
+
+
 @pytest.mark.parametrize("c_dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("Mdim,Ndim,Kdim", [(130, 259, 64), (40, 31, 264), (2600, 2051, 128)])
 def test_products_add_to_an_output_with_odd_rows(vl, guard, c_dtype, Mdim, Ndim, Kdim):
