@@ -122,7 +122,7 @@ template <> struct Store4<float> {
     }
 };
 
-// Output rows that start on any element (odd pitch, no padding): a lane that stores its own row would touch 32
+// Output rows of bf16 that start on any element (odd pitch, no padding): a lane that stores its own row would touch 32
 // sectors per instruction, two bytes in each.  The warp turns its 32 x 32 block over through shared memory (32 rows of
 // kStagePitch floats; the odd pitch keeps both directions free of bank conflicts) and writes one row at a time,
 // consecutive lanes to consecutive columns.  All lanes call; `valid` columns are the same for all of them.

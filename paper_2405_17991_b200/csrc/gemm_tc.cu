@@ -105,6 +105,9 @@ int launch_gemm_tc(int kind, const void* A, int64_t lda, const void* B, int64_t 
     if (Mdim < 1 || Ndim < 1 || Kdim < 1) return VELORA_ERR_UNSUPPORTED;
     if (Mdim > (1 << 30) || Ndim > (1 << 30) || Kdim > (1 << 30)) return VELORA_ERR_UNSUPPORTED;
     if (!tc_operand_ok(A, lda) || !tc_operand_ok(B, ldb)) return VELORA_ERR_UNSUPPORTED;
+    // An fp32 result on rows that vector stores cannot write stays with the CUDA-core product, whose sums are rounded and
+    // not truncated (relative error of 8192 positive terms: 1.6e-7, 3.5e-5 here); a bf16 result hides the difference.
+    if (c_dtype == VELORA_F32 && !c_rows_vec(C, ldc, sizeof(float))) return VELORA_ERR_UNSUPPORTED;
     if ((static_cast<int64_t>((Mdim + BM - 1) / BM) * ((Ndim + 255) / 256)) > (1 << 30)) return VELORA_ERR_UNSUPPORTED;
 
     DeviceInfo di;

@@ -301,7 +301,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8 * acc);
                 }
                 const int valid = Ndim - (t0.n0 + c * 32);
-                if (c_vec) {
+                if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
                         if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);

@@ -230,7 +230,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // K = 3072)
         const int quarter = warp & 3;
         const int set = FUSE ? 0 : (warp - 2) >> 2;
-        const int sets = FUSE || blockDim.x == GEMM_THREADS || (!c_vec && splits == 1) ? 1 : 2;     // staging room for four warps
+        const int sets = FUSE || blockDim.x == GEMM_THREADS || (sizeof(CT) == 2 && !c_vec && splits == 1) ? 1 : 2;     // staging room for four warps
         uint32_t t = 0;
         for (int tile = blockIdx.x; tile < num_tiles && !failed; tile += gridDim.x, ++t) {
             const TileCoord tc0 = tile_coord<BN>(tile, tiles_m, tiles_n);
@@ -271,7 +271,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (lane == 0) mbar_arrive(tempty + 8 * acc);
                 }
                 const int valid = Ndim - (tc0.n0 + c * 32);
-                if (c_vec) {
+                if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
                         if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);

@@ -140,3 +140,35 @@ def test_streams_on_odd_rows(vl, guard, N, D, Dsub, dtype, pad):
     W = guard.mat(N, D, dt, ld=D + pad, init=W0)
     vl.velora_expand_p(Z, v, D, dW=W, beta=1)
     assert_matches(W, oracle.reconstruct(to_f64(Z), v64, D) + to_f64(W0), TOL_Z, "W + P v", c=2e-3)
+
+
+# fp32 results on odd rows are sums rounded at every step.  Positive terms: a chain of K additions, each off by 2^-24 / sqrt(3) of
+# the running sum at most (rms), ends up off by 2^-24 / sqrt(3) * sqrt(K / 3) = 1.8e-6 of the result at K = 8192 and less in
+# shares; twice that is allowed.  Sums that are truncated, as the tensor cores', are 3.5e-5 off.
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("Mdim,Ndim", [(130, 259), (2600, 2051)])
+def test_fp32_results_on_odd_rows_are_rounded_sums(vl, guard, kind, Mdim, Ndim):
+    K = 8192
+    g = torch.Generator(device=DEV)
+    g.manual_seed(Mdim + kind)
+    mat = lambda r, c: torch.rand((r, -(-c // 8) * 8), generator=g, device=DEV).to(torch.bfloat16)[:, :c]
+    A = mat(K, Mdim) if kind == vl.PRODUCT_AT_B else mat(Mdim, K)
+    B = mat(Ndim, K) if kind == vl.PRODUCT_A_BT else mat(K, Ndim)
+    C = vl.velora_dense_product(kind, A, B, C=guard.mat(Mdim, Ndim, torch.float32, ld=Ndim))
+    a = (A.T if kind == vl.PRODUCT_AT_B else A).double()
+    b = (B.T if kind == vl.PRODUCT_A_BT else B).double()
+    ref = a @ b
+    assert float((C.double() - ref).norm() / ref.norm()) < 3.6e-6
+
+
+@pytest.mark.parametrize("dy_pad,dw_pad", [(0, 1), (1, 0), (1, 1)])
+def test_explicit_fp32_gradient_on_odd_rows_is_a_rounded_sum(vl, guard, dy_pad, dw_pad):
+    N, D, O, Dsub = 8192, 520, 264, 8
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+    dY = _view(torch.rand((N, O), generator=g, device=DEV).to(torch.bfloat16), O + dy_pad, 0)
+    Z = torch.rand((N, vl.num_subtokens(D, Dsub)), generator=g, device=DEV)
+    v = torch.rand(Dsub, generator=g, device=DEV)
+    dW = vl.velora_weight_grad(dY, Z, v, D, dW=guard.mat(O, D, torch.float32, ld=D + dw_pad), mode=vl.WG_EXPLICIT)
+    ref = dY.double().T @ vl.velora_reconstruct(Z, v, D, x_dtype=torch.bfloat16).double()
+    assert float((dW.double() - ref).norm() / ref.norm()) < 3.6e-6
