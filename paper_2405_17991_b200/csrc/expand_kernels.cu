@@ -23,7 +23,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 template <typename T> __device__ __forceinline__ float load_scalar(const T* p);
-template <> __device__ __forceinline__ float load_scalar<float>(const float* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float load_scalar<float>(const float* p) { return ld_chained(p); }
 template <> __device__ __forceinline__ float load_scalar<__nv_bfloat16>(const __nv_bfloat16* p)
 {
     return __bfloat162float(*p);
@@ -68,8 +68,8 @@ template <> struct Out8<float> {
 // MODE 2: ragged last sub-token as well (column checks, element-wise tail).
 template <int VEC, int LPS, int CH, int MODE, typename ST, typename WT>
 __global__ void __launch_bounds__(kStreamThreads)
-expand_rows_vec_kernel(const ST* __restrict__ S, int splits, int64_t split_stride, int lds,
-                       const float* __restrict__ v, int R, int D, int M, int mblocks,
+expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
+                       const float* v, int R, int D, int M, int mblocks,
                        WT* __restrict__ out, int64_t ldo, int beta)
 {
     static_assert(VEC == 8 || MODE == 2, "single elements are checked one by one");
@@ -85,7 +85,7 @@ expand_rows_vec_kernel(const ST* __restrict__ S, int splits, int64_t split_strid
 #pragma unroll
     for (int i = 0; i < CH; ++i)
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) vr[i][e] = __ldg(v + VEC * (q + LPS * i) + e);
+        for (int e = 0; e < VEC; ++e) vr[i][e] = ld_chained(v + VEC * (q + LPS * i) + e);
 
     // One warp per output row at a time.  The row's scalars are fetched for up to PB blocks of 32 sub-tokens
     // before the first store, so a row costs one load latency per PB blocks instead of one per block (a row of

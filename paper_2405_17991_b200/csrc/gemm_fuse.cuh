@@ -45,12 +45,12 @@ template <int ZK> __device__ __forceinline__ void store_z(const FuseArgs& fz, in
     else static_cast<float*>(fz.Z)[static_cast<int64_t>(row) * fz.ldz + m] = z;
 }
 
-// 16 bytes of X for the compress warps: read-only path, not kept in L1 (each line is used once here, and
+// 16 bytes of X for the compress warps: a plain load (common.cuh), not kept in L1 (each line is used once here, and
 // L1 shares its storage and bandwidth with the shared memory the tensor cores are reading).
 __device__ __forceinline__ uint4 ld_x_chunk(const uint4* p)
 {
     uint4 x;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
     return x;
 }
@@ -67,7 +67,7 @@ template <int CH> struct VSlice {
         for (int i = 0; i < CH; ++i) {
             const int pos = (32 * i + lane) & (L - 1);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[i][e] = __ldg(vg + 8 * pos + e);
+            for (int e = 0; e < 8; ++e) v[i][e] = ld_chained(vg + 8 * pos + e);
         }
     }
 };

@@ -32,7 +32,7 @@ template <typename T, int ROWS, int TK>
 struct Tile {
     static constexpr int E = ROWS * TK / SG_THREADS;
     static_assert(ROWS * TK == E * SG_THREADS && E % 4 == 0, "whole vectors per thread");
-    static __device__ __forceinline__ void load(const T* __restrict__ p, int64_t s_row, int64_t s_k, int64_t row0, int64_t rows,
+    static __device__ __forceinline__ void load(const T* p, int64_t s_row, int64_t s_k, int64_t row0, int64_t rows,
                                                 int64_t k0, int64_t k_end, int mode, float (&r)[E])
     {
         const int t = threadIdx.x;
@@ -47,7 +47,7 @@ struct Tile {
                 const int64_t fast_left = row_fast ? rows - (row0 + row) : k_end - (k0 + kk);
                 const bool slow_in = row_fast ? k0 + kk < k_end : row0 + row < rows;
                 if (sizeof(T) == 4 && slow_in && fast_left >= 4) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(q));
+                    const float4 x = ld_chained(reinterpret_cast<const float4*>(q));
                     r[4 * i] = x.x; r[4 * i + 1] = x.y; r[4 * i + 2] = x.z; r[4 * i + 3] = x.w;
                 } else {
 #pragma unroll
@@ -141,8 +141,8 @@ __host__ __device__ constexpr int slice_depth(int gm, int gn) { return gm * gn =
 // share a tile's contraction (a cluster; 64 x 64 tiles only).
 template <int GM, int GN, typename AT, typename BT, typename CT>
 __global__ void __launch_bounds__(SG_THREADS, 2)
-gemm_simt_kernel(const AT* __restrict__ A, int64_t a_sm, int64_t a_sk, int a_mode,
-                 const BT* __restrict__ B, int64_t b_sn, int64_t b_sk, int b_mode,
+gemm_simt_kernel(const AT* A, int64_t a_sm, int64_t a_sk, int a_mode,
+                 const BT* B, int64_t b_sn, int64_t b_sk, int b_mode,
                  CT* __restrict__ C, int64_t ldc, int beta, int c_vec,
                  int64_t Mdim, int64_t Ndim, int64_t Kdim, int64_t k_per_split)
 {

@@ -34,7 +34,7 @@ constexpr int SK_DIRECT_PARTS = 8;    // slices that the expansion kernel adds u
 // of the 8 OI columns of block blockIdx.y.
 template <typename YT, typename ZT, int OI, int MJ>
 __global__ void __launch_bounds__(SK_THREADS)
-wg_skinny_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __restrict__ Z, int64_t ldz,
+wg_skinny_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
                          int N, int O, int M, int tokens_per_cta, float* __restrict__ partials)
 {
     __shared__ __align__(16) float sdy[SK_CHUNK][8 * OI];
@@ -117,7 +117,7 @@ constexpr int SK_TILE_O = 64, SK_TILE_M = 32;
 
 template <typename YT, typename ZT, int MT>
 __global__ void __launch_bounds__(SK_THREADS, MT == 4 ? 3 : 2)
-wg_tile_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __restrict__ Z, int64_t ldz,
+wg_tile_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
                        int N, int O, int M, int tokens_per_cta, float* __restrict__ partials)
 {
     constexpr int TM = 4 * MT;
@@ -205,7 +205,7 @@ wg_tile_partial_kernel(const YT* __restrict__ dY, int64_t lddy, const ZT* __rest
 // each add every eighth partial (four loads in flight), then the eight sums are added in a fixed order: a
 // thread per element walking all the partials one after the other took 12 us for 148 of them.
 __global__ void __launch_bounds__(SK_THREADS)
-wg_skinny_reduce_kernel(const float* __restrict__ partials, int parts, int O, int M, float* __restrict__ P,
+wg_skinny_reduce_kernel(const float* partials, int parts, int O, int M, float* __restrict__ P,
                         int64_t ldp, int beta)
 {
     __shared__ float sred[8][32];

@@ -75,7 +75,7 @@ constexpr int kFinThreads = 1024;
 
 template <int VEC>
 __global__ void __launch_bounds__(kFinThreads)
-init_v_finalize_kernel(const float* __restrict__ partials, int num_partials, int Dsub,
+init_v_finalize_kernel(const float* partials, int num_partials, int Dsub,
                        float* __restrict__ v, int* __restrict__ status, int normalize)
 {
     __shared__ double s_sum[VELORA_MAX_DSUB];

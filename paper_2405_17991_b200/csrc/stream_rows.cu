@@ -43,13 +43,13 @@ template <typename XT, int VEC> struct Chunk;
 template <> struct Chunk<__nv_bfloat16, 8> {
     typedef uint4 Raw;
     template <bool KEEP>
-    static __device__ __forceinline__ Raw load(const __nv_bfloat16* __restrict__ row, int c, int full, int tail)
+    static __device__ __forceinline__ Raw load(const __nv_bfloat16* row, int c, int full, int tail)
     {
         const uint4* q = reinterpret_cast<const uint4*>(row) + c;
-        if (c < full) return KEEP ? __ldg(q) : __ldcs(q);
+        if (c < full) return ld_chained<!KEEP>(q);
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
         if (c == full && tail) {
-            x = __ldcs(q);                       // inside the row's pitch (a multiple of 8 elements)
+            x = ld_chained<true>(q);                       // inside the row's pitch (a multiple of 8 elements)
             uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -71,10 +71,10 @@ template <> struct Chunk<__nv_bfloat16, 8> {
 template <> struct Chunk<float, 4> {
     typedef float4 Raw;
     template <bool KEEP>
-    static __device__ __forceinline__ Raw load(const float* __restrict__ row, int c, int full, int tail)
+    static __device__ __forceinline__ Raw load(const float* row, int c, int full, int tail)
     {
         const float4* q = reinterpret_cast<const float4*>(row) + c;
-        if (c < full) return KEEP ? __ldg(q) : __ldcs(q);
+        if (c < full) return ld_chained<!KEEP>(q);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c == full && tail) {                 // the row may end inside the chunk and so may the buffer
             x.x = row[4 * c];
@@ -88,17 +88,17 @@ template <> struct Chunk<float, 4> {
 template <typename XT> struct Chunk<XT, 1> {
     typedef XT Raw;
     template <bool KEEP>
-    static __device__ __forceinline__ Raw load(const XT* __restrict__ row, int c, int full, int)
+    static __device__ __forceinline__ Raw load(const XT* row, int c, int full, int)
     {
-        return c < full ? __ldg(row + c) : static_cast<XT>(0.f);
+        return c < full ? ld_chained(row + c) : static_cast<XT>(0.f);
     }
     static __device__ __forceinline__ void unpack(const Raw& d, float (&x)[1]) { x[0] = static_cast<float>(d); }
 };
 
 template <typename XT, int VEC, int LPS, int CH, bool INIT, typename ZT>
 __global__ void __launch_bounds__(RW_THREADS)
-stream_rows_kernel(const XT* __restrict__ X, int N, int D, int64_t ldx, int M,
-                   const float* __restrict__ v, ZT* __restrict__ Z, int64_t ldz, float* __restrict__ partials)
+stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M,
+                   const float* v, ZT* __restrict__ Z, int64_t ldz, float* __restrict__ partials)
 {
     constexpr int U = CH > RW_U ? CH : RW_U;
     static_assert(CH == 1 || LPS == 32, "several chunks per lane only for sub-tokens wider than a warp's span");
@@ -116,7 +116,7 @@ stream_rows_kernel(const XT* __restrict__ X, int N, int D, int64_t ldx, int M,
 #pragma unroll
     for (int i = 0; i < CH; ++i)
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) vr[i][e] = INIT ? 0.f : __ldg(v + VEC * (q + LPS * i) + e);
+        for (int e = 0; e < VEC; ++e) vr[i][e] = INIT ? 0.f : ld_chained(v + VEC * (q + LPS * i) + e);
 
     // compress goes through the rows from the last to the first: whatever read or wrote X before it went the other way, so the
     // last rows are the ones still in L2 (a 180 MB X right behind its sub-token sum: 32 -> 23 us).

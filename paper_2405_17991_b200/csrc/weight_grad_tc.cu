@@ -359,7 +359,7 @@ wg_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUten
 
 // P[o, m] = beta * P[o, m] + sum_s partials[s][o][m], splits added in a fixed order.
 __global__ void __launch_bounds__(256)
-reduce_partials_kernel(const float* __restrict__ partials, int splits, int64_t split_stride, int ldpart,
+reduce_partials_kernel(const float* partials, int splits, int64_t split_stride, int ldpart,
                        int O, int M, float* __restrict__ P, int64_t ldp, int beta)
 {
     pdl_wait();

@@ -139,3 +139,23 @@ def test_memory_model_matches_table_5b_structure():
     full = saved_activation_bytes(1 << 20, D, None)
     for zb, ratio in ((4, 32), (2, 64), (1, 128)):
         assert abs(full / saved_activation_bytes(1 << 20, D, 64, z_bytes=zb) / ratio - 1) < 1e-3
+
+
+# A kernel that waits for the one before it while that one runs may not read through the read-only path: ld.global.nc is for data
+# that nothing writes while the reader lives, and the compiler makes it of const __restrict__ inputs too.  Exempt: the conversion of
+# Z, which is launched when everything before it has completed, and the kernel behind it, which reads nothing else early.
+def test_kernels_that_start_early_do_not_read_through_the_read_only_path():
+    csrc = os.path.join(ROOT, "paper_2405_17991_b200", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        with open(os.path.join(csrc, name)) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        parts = text.split("__global__")
+        kernels = [p.split("\n}\n", 1)[0] for p in parts[1:]]
+        early = [k for k in kernels if "pdl_wait()" in k and not re.search(r"z_to_bf16_kernel|\bwg_kernel", k)]
+        seen += len(early)
+        helpers = [parts[0]] if early and name != "stream_kernels.cu" or name == "gemm_fuse.cuh" else []
+        for body in early + helpers:
+            bad = re.findall(r"__ldg\b|\bld\.global\.nc|const\s+\w+\s*\*\s*__restrict__", body)
+            assert not bad, (name, bad, body[:200])
+    assert seen >= 8
