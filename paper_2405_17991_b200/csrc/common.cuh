@@ -40,11 +40,22 @@ inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // Programmatic dependent launch.  A kernel launched with pdl_attribute() may become resident while the kernel before it
 // in the stream is still running: its launch, its barriers and its TMEM are then ready when that kernel ends.  Every
 // thread of such a kernel calls pdl_wait() before it touches global memory (the wait returns once the kernel before
-// has completed and its writes are visible), and only then pdl_trigger(), which lets the NEXT kernel start early: so
-// when kernel k + 1 becomes resident, everything up to k - 1 has completed.  A small layer is a chain of kernels of
-// 5-10 us with about 2 us of launch and set-up between them.
-// Not launched this way: cluster launches, but for the weight gradient behind its own conversion (a long queue of layers
-// with the CTA-pair product among the chained kernels stopped making progress once, for a reason not found).
+// has completed and its writes are visible), and then, when its CTA holds all that it will allocate, pdl_trigger(), which
+// lets the NEXT kernel start early: so when kernel k + 1 becomes resident, everything up to k - 1 has completed.  A small layer
+// is a chain of kernels of 5-10 us with about 2 us of launch and set-up between them.
+// Two kernels keep to another order and depend on how they are launched.  z_to_bf16_kernel triggers first: it is launched
+// the ordinary way, so all before it has completed.  wg_kernel behind it therefore reads dY before its wait, which one thread makes,
+// ahead of the conversion's result; behind anything else it is launched the ordinary way.
+// Not launched this way: the other cluster kernels (a long queue of layers with the CTA-pair product and the split products
+// in the chain stopped making progress once; the form is gone and its cause was not found).
+//
+// Why no kernel of a chain can wait for ever.  Waits on barriers of a CTA are bounded (tc_common.cuh).  Three are not:
+//   griddepcontrol.wait  waits for the kernel before, all of whose CTAs are resident or done when this one starts (each has
+//                        triggered): nothing that this kernel occupies can keep it from ending.
+//   tcgen05.alloc        never finds TMEM short.  Every kernel that allocates TMEM takes more than half of an SM's 228 KB of shared
+//                        memory and so has an SM to itself among them (products 209 KB or more, adapter forward 222 KB),
+//                        but for wg_kernel, of which two CTAs fit (96 KB or more each) with at most 256 of the 512 columns each.
+//   cluster barriers     all CTAs of a cluster are placed together, and each reaches both barriers whatever happened before.
 // What such a kernel reads is still being written while it is resident, so none of it may go through the read-only path:
 // neither __ldg nor ld.global.nc, and no `const __restrict__` on its inputs, of which the compiler makes the same loads (a line
 // that the kernel before had read on this SM, next to what another SM has written since, would be served as it was).  ld_chained

@@ -324,11 +324,11 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         tmem_relinquish();
     }
     pdl_wait();
-    pdl_trigger();
     for (int j = threadIdx.x; j < fz.Dsub; j += SF_THREADS) sv[j] = fz.v[j];
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    pdl_trigger();                                           // this CTA holds its TMEM now
     const uint32_t tmem_base = *tmem_slot;
 
     bool failed = false;

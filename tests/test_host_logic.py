@@ -159,3 +159,20 @@ def test_kernels_that_start_early_do_not_read_through_the_read_only_path():
             bad = re.findall(r"__ldg\b|\bld\.global\.nc|const\s+\w+\s*\*\s*__restrict__", body)
             assert not bad, (name, bad, body[:200])
     assert seen >= 8
+
+
+# Each CTA of a kernel that lets the next one in holds its TMEM by then: otherwise the next kernel could take the columns and wait
+# for a kernel that waits for them.
+def test_kernels_trigger_the_next_one_after_they_have_allocated():
+    csrc = os.path.join(ROOT, "paper_2405_17991_b200", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        with open(os.path.join(csrc, name)) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        for kernel in text.split("__global__")[1:]:
+            body = kernel.split("\n}\n", 1)[0]
+            if "tmem_alloc(" in body and "pdl_trigger()" in body:
+                seen += 1
+                allocated = body.index("__syncthreads()", body.index("tmem_alloc("))
+                assert body.index("pdl_wait()") < body.index("pdl_trigger()") and allocated < body.index("pdl_trigger()"), name
+    assert seen >= 2
