@@ -58,38 +58,20 @@ inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 //   cluster barriers     all CTAs of a cluster are placed together, and each reaches both barriers whatever happened before.
 // What such a kernel reads is still being written while it is resident, so none of it may go through the read-only path:
 // neither __ldg nor ld.global.nc, and no `const __restrict__` on its inputs, of which the compiler makes the same loads (a line
-// that the kernel before had read on this SM, next to what another SM has written since, would be served as it was).  ld_chained
-// is a plain load that stays behind pdl_wait(); STREAM: the line is not needed again.
+// that the kernel before had read on this SM, next to what another SM has written since, would be served as it was): plain loads,
+// which stay behind pdl_wait(), or ld_stream_if where the line is not needed again.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-template <bool STREAM = false>
-__device__ __forceinline__ uint4 ld_chained(const uint4* p)
+// Four words, or zeros where `take` is false.
+__device__ __forceinline__ uint4 ld_stream_if(const void* p, bool take)
 {
     uint4 x;
-    if (STREAM) asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
-    else asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
+    asm volatile("{\n\t.reg .pred t;\n\tsetp.ne.s32 t, %5, 0;\n\t"
+                 "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+                 "@t ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "=&r"(x.x), "=&r"(x.y), "=&r"(x.z), "=&r"(x.w) : "l"(p), "r"(static_cast<int>(take)));
     return x;
-}
-template <bool STREAM = false>
-__device__ __forceinline__ float4 ld_chained(const float4* p)
-{
-    float4 x;
-    if (STREAM) asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p));
-    else asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p));
-    return x;
-}
-__device__ __forceinline__ float ld_chained(const float* p)
-{
-    float x;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
-    return x;
-}
-__device__ __forceinline__ __nv_bfloat16 ld_chained(const __nv_bfloat16* p)
-{
-    unsigned short x;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(x) : "l"(p));
-    return __ushort_as_bfloat16(x);
 }
 #endif
 inline cudaLaunchAttribute pdl_attribute()

@@ -12,6 +12,9 @@
 // pointer advances by a constant, so one store instruction costs one shuffle, eight multiplies, four
 // packs and the store; every store instruction writes one contiguous 512-byte span.
 //
+// Fewer rows than warps: a row is cut into spans of sub-tokens, one warp each.  16 rows of 11005 unpadded bf16 elements, Dsub 64,
+// added to what is there: 3 us, 111 with a warp per row.
+//
 // Output rows that are not 16-byte aligned take the same walk with single elements in the place of the groups of eight
 // (VEC = 1): a store instruction then writes 32 consecutive elements.  8192 x 11005 unpadded bf16: 62 us, 322 with an
 // integer division per element.
@@ -23,7 +26,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 template <typename T> __device__ __forceinline__ float load_scalar(const T* p);
-template <> __device__ __forceinline__ float load_scalar<float>(const float* p) { return ld_chained(p); }
+template <> __device__ __forceinline__ float load_scalar<float>(const float* p) { return *p; }
 template <> __device__ __forceinline__ float load_scalar<__nv_bfloat16>(const __nv_bfloat16* p)
 {
     return __bfloat162float(*p);
@@ -69,7 +72,7 @@ template <> struct Out8<float> {
 template <int VEC, int LPS, int CH, int MODE, typename ST, typename WT>
 __global__ void __launch_bounds__(kStreamThreads)
 expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
-                       const float* v, int R, int D, int M, int mblocks,
+                       const float* v, int R, int D, int M, int segs, int span,
                        WT* __restrict__ out, int64_t ldo, int beta)
 {
     static_assert(VEC == 8 || MODE == 2, "single elements are checked one by one");
@@ -85,22 +88,35 @@ expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
 #pragma unroll
     for (int i = 0; i < CH; ++i)
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) vr[i][e] = ld_chained(v + VEC * (q + LPS * i) + e);
+        for (int e = 0; e < VEC; ++e) vr[i][e] = v[VEC * (q + LPS * i) + e];
 
-    // One warp per output row at a time.  The row's scalars are fetched for up to PB blocks of 32 sub-tokens
+    // One warp per output row (or span of it) at a time.  The row's scalars are fetched for up to PB blocks of 32 sub-tokens
     // before the first store, so a row costs one load latency per PB blocks instead of one per block (a row of
     // 172 sub-tokens went through six dependent round trips to memory before).
     constexpr int PB = 4;
     const int warps = gridDim.x * (kStreamThreads / 32);
-    for (int r = blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5); r < R; r += warps)
-    for (int mb0 = 0; mb0 < mblocks; mb0 += PB) {
+    const int items = R * segs;                  // spans of `span` sub-tokens, a multiple of SPW (segs == 1: whole rows)
+    for (int item = blockIdx.x * (kStreamThreads / 32) + (threadIdx.x >> 5); item < items; item += warps) {
+    const int r = segs == 1 ? item : item / segs;
+    const ST* row_s = S + static_cast<int64_t>(r) * lds;
+    WT* row_out = out + static_cast<int64_t>(r) * ldo;
+    int end = M, M_left = M, D_left = D;         // sub-tokens to do, sub-tokens and columns from where the span starts
+    if (segs > 1) {
+        const int m_begin = (item - r * segs) * span;
+        row_s += m_begin;
+        row_out += m_begin * (L * VEC);
+        M_left -= m_begin;
+        D_left -= m_begin * (L * VEC);
+        end = M_left < span ? M_left : span;
+    }
+    for (int mb0 = 0; mb0 < end; mb0 += 32 * PB) {
         float pb[PB];
 #pragma unroll
         for (int b = 0; b < PB; ++b) {
-            const int m = (mb0 + b) * 32 + lane;
+            const int m = mb0 + b * 32 + lane;
             float p = 0.f;
-            if (mb0 + b < mblocks && (MODE == 0 || m < M)) {
-                const ST* sp = S + static_cast<int64_t>(r) * lds + m;
+            if (m < end) {
+                const ST* sp = row_s + m;
 #pragma unroll 4
                 for (int s = 0; s < splits; ++s) p += load_scalar<ST>(sp + s * split_stride);   // fixed order
             }
@@ -108,20 +124,46 @@ expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
         }
 #pragma unroll
         for (int b = 0; b < PB; ++b) {
-            const int m0 = (mb0 + b) * 32;
-            if (mb0 + b >= mblocks) break;
+            const int m0 = mb0 + b * 32;
+            if (m0 >= end) break;
+            const int steps = (end - m0 + SPW - 1) / SPW < LPS ? (end - m0 + SPW - 1) / SPW : LPS;
             const float p = pb[b];
             // Element pointer of this lane's first chunk; each step moves on by SPW sub-tokens.
-            WT* ptr = out + static_cast<int64_t>(r) * ldo + (static_cast<int64_t>(m0 + sub) * L + q) * VEC;
+            WT* ptr = row_out + (static_cast<int64_t>(m0 + sub) * L + q) * VEC;
+            if (VEC == 1 && beta && segs > 1) {
+                // Few rows: eight elements of a lane at a time, what is there read first.  (With a warp per row this form takes
+                // 382 us on 8192 x 11005 fp32 with Dsub 16, the one below 210.)
+                constexpr int G = CH < 8 ? 8 / CH : 1;
+                for (int it = 0; it < steps; it += G, ptr += G * SPW * L) {
+                    float y[G][CH];
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const int ms = (it + g) * SPW + sub;
+                        const float pm = __shfl_sync(kFull, p, ms & 31);
+#pragma unroll
+                        for (int i = 0; i < CH; ++i) {
+                            y[g][i] = pm * vr[i][0];
+                            if (it + g < steps && (m0 + ms) * L + q + LPS * i < D_left) y[g][i] += Elem<WT>::load(ptr + g * SPW * L + i * LPS);
+                        }
+                    }
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+#pragma unroll
+                        for (int i = 0; i < CH; ++i)
+                            if (it + g < steps && (m0 + (it + g) * SPW + sub) * L + q + LPS * i < D_left)
+                                Elem<WT>::store(ptr + g * SPW * L + i * LPS, y[g][i]);
+                }
+                continue;
+            }
 #pragma unroll 8
-            for (int it = 0; it < LPS; ++it, ptr += SPW * L * VEC) {
+            for (int it = 0; it < steps; ++it, ptr += SPW * L * VEC) {
                 const int ms = it * SPW + sub;
                 const float pm = __shfl_sync(kFull, p, ms);
-                if (MODE != 0 && m0 + ms >= M) continue;
+                if (MODE != 0 && m0 + ms >= M_left) continue;
 #pragma unroll
                 for (int i = 0; i < CH; ++i) {
                     if constexpr (VEC == 1) {
-                        if ((m0 + ms) * L + q + LPS * i < D) {
+                        if ((m0 + ms) * L + q + LPS * i < D_left) {
                             WT* pe = ptr + i * LPS;
                             float f = pm * vr[i][0];
                             if (beta) f += Elem<WT>::load(pe);
@@ -136,12 +178,12 @@ expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
                         Out8<WT>::store(ptr + i * LPS * 8, y, beta);
                     } else {
                         const int col = ((m0 + ms) * L + q + LPS * i) * 8;
-                        if (col + 8 <= D) {
+                        if (col + 8 <= D_left) {
                             Out8<WT>::store(ptr + i * LPS * 8, y, beta);
                         } else {
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
-                                if (col + e < D) {
+                                if (col + e < D_left) {
                                     WT* pe = ptr + i * LPS * 8 + e;
                                     float f = y[e];
                                     if (beta) f += Elem<WT>::load(pe);
@@ -153,11 +195,12 @@ expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
             }
         }
     }
+    }
 }
 
 template <int VEC, int LPS, int CH, typename ST, typename WT>
 int launch_mode(int mode, int grid, const void* S, int splits, int64_t split_stride, int lds, const float* v,
-                int R, int D, int M, int mblocks, void* out, int64_t ldo, int beta, cudaStream_t stream)
+                int R, int D, int M, int segs, int span, void* out, int64_t ldo, int beta, cudaStream_t stream)
 {
     const ST* s = static_cast<const ST*>(S);
     WT* o = static_cast<WT*>(out);
@@ -170,11 +213,11 @@ int launch_mode(int mode, int grid, const void* S, int splits, int64_t split_str
     cfg.numAttrs = 1;
     cudaError_t e;
     if (mode == 0 && VEC == 8)
-        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, VEC == 8 ? 0 : 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, mblocks, o, ldo, beta);
+        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, VEC == 8 ? 0 : 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, segs, span, o, ldo, beta);
     else if (mode == 1 && VEC == 8)
-        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, VEC == 8 ? 1 : 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, mblocks, o, ldo, beta);
+        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, VEC == 8 ? 1 : 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, segs, span, o, ldo, beta);
     else
-        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, mblocks, o, ldo, beta);
+        e = cudaLaunchKernelEx(&cfg, expand_rows_vec_kernel<VEC, LPS, CH, 2, ST, WT>, s, splits, split_stride, lds, v, R, D, M, segs, span, o, ldo, beta);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return VELORA_ERR_CUDA;
@@ -184,11 +227,11 @@ int launch_mode(int mode, int grid, const void* S, int splits, int64_t split_str
 
 template <typename ST, typename WT>
 int launch_shape(int vec, int lps, int ch, int mode, int grid, const void* S, int splits, int64_t split_stride, int lds,
-                 const float* v, int R, int D, int M, int mblocks, void* out, int64_t ldo, int beta, cudaStream_t stream)
+                 const float* v, int R, int D, int M, int segs, int span, void* out, int64_t ldo, int beta, cudaStream_t stream)
 {
 #define VELORA_EXPAND_CASE(VECV, LPSV, CHV)                                                                    \
     if (vec == VECV && lps == LPSV && ch == CHV)                                                               \
-        return launch_mode<VECV, LPSV, CHV, ST, WT>(mode, grid, S, splits, split_stride, lds, v, R, D, M, mblocks, out, ldo, beta, stream)
+        return launch_mode<VECV, LPSV, CHV, ST, WT>(mode, grid, S, splits, split_stride, lds, v, R, D, M, segs, span, out, ldo, beta, stream)
     VELORA_EXPAND_CASE(8, 1, 1);
     VELORA_EXPAND_CASE(8, 2, 1);
     VELORA_EXPAND_CASE(8, 4, 1);
@@ -222,23 +265,27 @@ int launch_expand_rows_vec(const void* S, int s_dtype, int splits, int64_t split
     if ((s_dtype == VELORA_BF16 || s_dtype == VELORA_FP8_E4M3) && out_dtype != VELORA_BF16) return VELORA_ERR_UNSUPPORTED;
     const int lps = L < 32 ? L : 32, ch = L / lps;
     const int M = static_cast<int>(ceil_div64(D, Dsub));
-    const int mblocks = (M + 31) / 32;
     const int mode = (D % Dsub) ? 2 : ((M % 32) ? 1 : 0);
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc != VELORA_OK) return rc;
-    int64_t ctas = ceil_div64(R, kStreamThreads / 32);
-    const int64_t cap = static_cast<int64_t>(di.sm_count) * kStreamCtasPerSm;
-    if (ctas > cap) ctas = cap;
-    const int grid = static_cast<int>(ctas < 1 ? 1 : ctas);
+    const int64_t cap = static_cast<int64_t>(di.sm_count) * kStreamCtasPerSm, warps = cap * (kStreamThreads / 32);
+    // Rows are cut while there are fewer of them than warps, into spans of eight store instructions or more (four of 16 bytes).
+    const int spw = 32 / lps, least = spw * ceil_div64(vec == 1 ? 8 : 4, ch);
+    int64_t n_segs = R < warps ? ceil_div64(warps, R) : 1;
+    if (n_segs > ceil_div64(M, least)) n_segs = ceil_div64(M, least);
+    const int span = static_cast<int>(ceil_div64(ceil_div64(M, n_segs), spw) * spw);
+    const int segs = static_cast<int>(ceil_div64(M, span));
+    const int64_t ctas = ceil_div64(R * segs, kStreamThreads / 32);
+    const int grid = static_cast<int>(ctas < cap ? ctas : cap);
     const int r = static_cast<int>(R), d = static_cast<int>(D), ld = static_cast<int>(lds);
     if (s_dtype == VELORA_BF16)
-        return launch_shape<__nv_bfloat16, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, mblocks, out, ldo, beta, stream);
+        return launch_shape<__nv_bfloat16, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, segs, span, out, ldo, beta, stream);
     if (s_dtype == VELORA_FP8_E4M3)
-        return launch_shape<e4m3_t, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, mblocks, out, ldo, beta, stream);
+        return launch_shape<e4m3_t, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, segs, span, out, ldo, beta, stream);
     if (out_dtype == VELORA_BF16)
-        return launch_shape<float, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, mblocks, out, ldo, beta, stream);
-    return launch_shape<float, float>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, mblocks, out, ldo, beta, stream);
+        return launch_shape<float, __nv_bfloat16>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, segs, span, out, ldo, beta, stream);
+    return launch_shape<float, float>(vec, lps, ch, mode, grid, S, splits, split_stride, ld, v, r, d, M, segs, span, out, ldo, beta, stream);
 }
 
 }  // namespace velora

@@ -67,7 +67,7 @@ template <int CH> struct VSlice {
         for (int i = 0; i < CH; ++i) {
             const int pos = (32 * i + lane) & (L - 1);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[i][e] = ld_chained(vg + 8 * pos + e);
+            for (int e = 0; e < 8; ++e) v[i][e] = vg[8 * pos + e];
         }
     }
 };

@@ -47,7 +47,7 @@ struct Tile {
                 const int64_t fast_left = row_fast ? rows - (row0 + row) : k_end - (k0 + kk);
                 const bool slow_in = row_fast ? k0 + kk < k_end : row0 + row < rows;
                 if (sizeof(T) == 4 && slow_in && fast_left >= 4) {
-                    const float4 x = ld_chained(reinterpret_cast<const float4*>(q));
+                    const float4 x = *reinterpret_cast<const float4*>(q);
                     r[4 * i] = x.x; r[4 * i + 1] = x.y; r[4 * i + 2] = x.z; r[4 * i + 3] = x.w;
                 } else {
 #pragma unroll

@@ -33,7 +33,7 @@ struct PackArgs {
 // The aligned 16 bytes at `a`; bytes outside the matrix are not touched and read as zero.
 __device__ __forceinline__ uint4 load_aligned(const char* a, const char* lo_limit, const char* hi_limit)
 {
-    if (a >= lo_limit && a + 16 <= hi_limit) return ld_chained<true>(reinterpret_cast<const uint4*>(a));
+    if (a >= lo_limit && a + 16 <= hi_limit) return ld_stream_if(a, true);
     uint32_t o[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int e = 0; e < 8; ++e)

@@ -20,6 +20,9 @@
 // the lane at position 0 stores Z[row, m].  init_v: the lane adds what it loads into VEC * CH running sums; the
 // CTA then adds the sums of the lanes that share a position in a fixed order and writes one row of partials.
 //
+// Fewer rows than warps: a row is cut into runs of whole rounds, one warp each.  16 rows of 11005 unpadded bf16 elements with Dsub 64:
+// compress 2 us, 17 with a warp per row; the sub-token sum 7 us, 14.
+//
 // Columns at or beyond D count as zeros: chunks past the row's end are not loaded and a last chunk that
 // straddles D is masked, which is the zero extension of a ragged last sub-token.
 #include "common.cuh"
@@ -46,10 +49,12 @@ template <> struct Chunk<__nv_bfloat16, 8> {
     static __device__ __forceinline__ Raw load(const __nv_bfloat16* row, int c, int full, int tail)
     {
         const uint4* q = reinterpret_cast<const uint4*>(row) + c;
-        if (c < full) return ld_chained<!KEEP>(q);
+        // A last partial chunk lies inside the row's pitch (a multiple of 8 elements).
+        const bool take = c < full || (c == full && tail);
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (!KEEP) x = ld_stream_if(q, take);
+        else if (take) x = *q;
         if (c == full && tail) {
-            x = ld_chained<true>(q);                       // inside the row's pitch (a multiple of 8 elements)
             uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -74,8 +79,13 @@ template <> struct Chunk<float, 4> {
     static __device__ __forceinline__ Raw load(const float* row, int c, int full, int tail)
     {
         const float4* q = reinterpret_cast<const float4*>(row) + c;
-        if (c < full) return ld_chained<!KEEP>(q);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (KEEP) {
+            if (c < full) x = *q;
+        } else {
+            const uint4 w = ld_stream_if(q, c < full);
+            x = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+        }
         if (c == full && tail) {                 // the row may end inside the chunk and so may the buffer
             x.x = row[4 * c];
             if (tail > 1) x.y = row[4 * c + 1];
@@ -90,14 +100,14 @@ template <typename XT> struct Chunk<XT, 1> {
     template <bool KEEP>
     static __device__ __forceinline__ Raw load(const XT* row, int c, int full, int)
     {
-        return c < full ? ld_chained(row + c) : static_cast<XT>(0.f);
+        return c < full ? row[c] : static_cast<XT>(0.f);
     }
     static __device__ __forceinline__ void unpack(const Raw& d, float (&x)[1]) { x[0] = static_cast<float>(d); }
 };
 
 template <typename XT, int VEC, int LPS, int CH, bool INIT, typename ZT>
 __global__ void __launch_bounds__(RW_THREADS)
-stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M,
+stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M, int segs, int seg_rounds,
                    const float* v, ZT* __restrict__ Z, int64_t ldz, float* __restrict__ partials)
 {
     constexpr int U = CH > RW_U ? CH : RW_U;
@@ -116,19 +126,30 @@ stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M,
 #pragma unroll
     for (int i = 0; i < CH; ++i)
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) vr[i][e] = INIT ? 0.f : ld_chained(v + VEC * (q + LPS * i) + e);
+        for (int e = 0; e < VEC; ++e) vr[i][e] = INIT ? 0.f : v[VEC * (q + LPS * i) + e];
 
     // compress goes through the rows from the last to the first: whatever read or wrote X before it went the other way, so the
     // last rows are the ones still in L2 (a 180 MB X right behind its sub-token sum: 32 -> 23 us).
     const int warps = gridDim.x * RW_WARPS;
-    for (int at = blockIdx.x * RW_WARPS + (threadIdx.x >> 5); at < N; at += warps) {
-        const int row = INIT ? at : N - 1 - at;
+    const int items = N * segs;                   // runs of seg_rounds rounds (segs == 1: whole rows)
+    for (int at = blockIdx.x * RW_WARPS + (threadIdx.x >> 5); at < items; at += warps) {
+        const int item = INIT ? at : items - 1 - at;
+        const int row = segs == 1 ? item : item / segs;
         const XT* rp = X + static_cast<int64_t>(row) * ldx;
         ZT* zrow = INIT ? nullptr : Z + static_cast<int64_t>(row) * ldz;
-        for (int c0 = 0; c0 < cpr; c0 += 32 * U) {
+        int left = full, end = cpr, M_left = M;   // whole chunks, chunks to walk and sub-tokens from where the run starts
+        if (segs > 1) {
+            const int c_begin = (item - row * segs) * seg_rounds * (32 * U), m_begin = c_begin / (LPS * CH);
+            rp += c_begin * VEC;
+            if (!INIT) zrow += m_begin;
+            left -= c_begin;
+            M_left -= m_begin;
+            end = cpr - c_begin < seg_rounds * (32 * U) ? cpr - c_begin : seg_rounds * (32 * U);
+        }
+        for (int c0 = 0; c0 < end; c0 += 32 * U) {
             typename C::Raw d[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) d[u] = C::template load<INIT>(rp, c0 + 32 * u + lane, full, tail);
+            for (int u = 0; u < U; ++u) d[u] = C::template load<INIT>(rp, c0 + 32 * u + lane, left, tail);
             float part = 0.f;                     // CH > 1: sum over the parts of one sub-token so far
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -153,7 +174,7 @@ stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M,
                         for (int off = LPS / 2; off >= 1; off >>= 1) k += __shfl_xor_sync(0xffffffffu, k, off);
                         // first chunk of the sub-token: c0 + 32 * (u - i); its index m = that / (LPS * CH) (+ lane / LPS)
                         const int m = (c0 + 32 * (u - i)) / (LPS * CH) + (CH == 1 ? lane / LPS : 0);
-                        if (q == 0 && m < M) put_z<ZT>(zrow + m, k);
+                        if (q == 0 && m < M_left) put_z<ZT>(zrow + m, k);
                     }
                 }
             }
@@ -181,10 +202,10 @@ stream_rows_kernel(const XT* X, int N, int D, int64_t ldx, int M,
 
 struct RowsPlan {
     bool ok;
-    int vec, lps, ch, M, grid;
+    int vec, lps, ch, M, segs, seg_rounds, grid;
 };
 
-RowsPlan plan_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx, int Dsub, int sm_count, int max_grid)
+RowsPlan plan_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx, int Dsub, int sm_count, int max_grid, bool sum)
 {
     RowsPlan p{};
     if (Dsub < 8 || Dsub > 1024 || (Dsub & (Dsub - 1))) return p;
@@ -195,11 +216,18 @@ RowsPlan plan_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx
     p.lps = L < 32 ? L : 32;
     p.ch = L / p.lps;
     p.M = static_cast<int>(ceil_div64(D, Dsub));
-    int64_t grid = ceil_div64(N, RW_WARPS);
-    const int64_t cap = static_cast<int64_t>(sm_count) * kStreamCtasPerSm;
-    if (grid > cap) grid = cap;
-    if (max_grid > 0 && grid > max_grid) grid = max_grid;
-    p.grid = static_cast<int>(grid);
+    int64_t cap = static_cast<int64_t>(sm_count) * kStreamCtasPerSm;
+    if (max_grid > 0 && cap > max_grid) cap = max_grid;
+    // Rows are cut while there are fewer of them than warps; for the sub-token sum than four warps per SM, because each CTA adds
+    // a row to what the finalize kernel's one CTA adds up (512 x 2045 fp32, Dsub 256: 16 us with as many runs as compress).
+    const int64_t rounds = ceil_div64(ceil_div64(D, p.vec), 32 * (p.ch > RW_U ? p.ch : RW_U));
+    const int64_t wanted = sum ? 4 * static_cast<int64_t>(sm_count) : cap * RW_WARPS;
+    int64_t segs = N < wanted ? ceil_div64(wanted, N) : 1;
+    if (segs > rounds) segs = rounds;
+    p.seg_rounds = static_cast<int>(ceil_div64(rounds, segs));
+    p.segs = static_cast<int>(ceil_div64(rounds, p.seg_rounds));
+    const int64_t grid = ceil_div64(N * p.segs, RW_WARPS);
+    p.grid = static_cast<int>(grid < cap ? grid : cap);
     p.ok = true;
     return p;
 }
@@ -216,7 +244,7 @@ int launch_rows(const RowsPlan& p, const void* X, int64_t N, int64_t D, int64_t 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, stream_rows_kernel<XT, VEC, LPS, CH, INIT, ZT>, static_cast<const XT*>(X), static_cast<int>(N),
-                           static_cast<int>(D), ldx, p.M, v, Z, ldz, partials) != cudaSuccess) {
+                           static_cast<int>(D), ldx, p.M, p.segs, p.seg_rounds, v, Z, ldz, partials) != cudaSuccess) {
         cudaGetLastError();
         return VELORA_ERR_CUDA;
     }
@@ -267,7 +295,7 @@ int launch_compress_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64
     DeviceInfo di;
     const int rc = device_info(&di);
     if (rc != VELORA_OK) return rc;
-    const RowsPlan p = plan_rows(X, x_dtype, N, D, ldx, Dsub, di.sm_count, 0);
+    const RowsPlan p = plan_rows(X, x_dtype, N, D, ldx, Dsub, di.sm_count, 0, false);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
     if (z_dtype == VELORA_F32)
         return dispatch_rows<false, float>(p, X, x_dtype, N, D, ldx, v, static_cast<float*>(Z), ldz, nullptr, stream);
@@ -286,7 +314,7 @@ int launch_init_v_partials_rows(const void* X, int x_dtype, int64_t N, int64_t D
     // that each walk a few rows; a larger grid would only add partial rows for the finalize kernel to add up.
     int cap = di.sm_count * 4;
     if (max_partials > 0 && cap > max_partials) cap = max_partials;
-    const RowsPlan p = plan_rows(X, x_dtype, N, D, ldx, Dsub, di.sm_count, cap);
+    const RowsPlan p = plan_rows(X, x_dtype, N, D, ldx, Dsub, di.sm_count, cap, true);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
     *num_partials = p.grid;
     return dispatch_rows<true, float>(p, X, x_dtype, N, D, ldx, nullptr, static_cast<float*>(nullptr), 0, partials, stream);
