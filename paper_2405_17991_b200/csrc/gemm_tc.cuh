@@ -38,7 +38,7 @@ int launch_linear_forward_skinny(const void* X, int64_t ldx, const void* W, int6
 bool gemm_pair_preferred(int64_t Mdim, int64_t Ndim);
 
 // Tensor map of a row-major bf16 matrix: `inner` contiguous elements per row, `outer` rows, row pitch
-// ld_elems; 128-byte swizzle (or none), zero fill outside the matrix.  (gemm_tc.cu)
+// ld_elems; 128-byte swizzle (or none), zero fill outside the matrix.  (tensor_maps.cu)
 int make_tmap_bf16_2d(CUtensorMap* map, const void* base, int64_t inner, int64_t outer, int64_t ld_elems,
                       int box_inner, int box_outer, bool swizzle128 = true);
 bool tc_operand_ok(const void* p, int64_t ld_elems);
