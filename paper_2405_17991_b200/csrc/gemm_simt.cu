@@ -274,6 +274,8 @@ int launch_tiles(const void* A, int64_t a_sm, int64_t a_sk, int a_mode, const vo
                            static_cast<const BT*>(B), b_sn, b_sk, b_mode, static_cast<CT*>(C), ldc, beta, c_vec, Mdim, Ndim, Kdim,
                            k_per_split) != cudaSuccess) {
         cudaGetLastError();
+        if (splits > 1)                                         // a refused cluster: the same tiles, one CTA each
+            return launch_tiles<GM, GN, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, 1, stream);
         return VELORA_ERR_CUDA;
     }
     return after_launch();

@@ -378,8 +378,8 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, kern, ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, kb_per_split, c_vec,
                            status, fz) != cudaSuccess) {
-        cudaGetLastError();
-        return VELORA_ERR_CUDA;
+        cudaGetLastError();                                           // a refused cluster: the same tiles, one CTA each
+        return launch_kernel<A_MN, B_MN, CT, FUSE, BN>(ta, tb, C, ldc, beta, Mdim, Ndim, Kdim, 1, status, stream, fz);
     }
     return after_launch();
 }

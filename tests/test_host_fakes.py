@@ -44,3 +44,29 @@ int main()
 }
 """)
     assert r.stdout.split() == ["0"] * 4, r.stdout + r.stderr
+
+
+def test_a_refused_cluster_launch_falls_back_to_single_ctas(tmp_path):
+    r = _run(tmp_path, "gemm_simt.cu", r"""
+namespace velora {
+int device_info(DeviceInfo* d) { *d = DeviceInfo{148, 227 * 1024}; return VELORA_OK; }
+int after_launch() { return VELORA_OK; }
+}
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void** args)
+{
+    unsigned cluster = 1;
+    for (unsigned i = 0; i < c->numAttrs; ++i)
+        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.z;
+    std::printf("cluster %u grid %u %u %u slice %lld\n", cluster, c->gridDim.x, c->gridDim.y, c->gridDim.z, (long long)*static_cast<int64_t*>(args[15]));
+    return cluster > 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+int main()
+{
+    float x[4];
+    const int rc = velora::launch_gemm_simt(x, VELORA_F32, 1280, 1, x, VELORA_F32, 1280, 1, x, VELORA_F32, 288, 0, 171, 288, 1280, nullptr);
+    std::printf("status %d\n", rc);
+}
+""")
+    lines = r.stdout.splitlines()
+    assert lines[-1] == "status 0", r.stdout + r.stderr
+    assert lines[0].startswith("cluster 8 grid 5 3 8") and lines[1] == "cluster 1 grid 5 3 1 slice 1280", r.stdout
