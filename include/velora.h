@@ -46,9 +46,9 @@
  *     leading dimensions are multiples of 16 bytes and Dsub is a multiple of 8
  *     (fastest for 8 * 2^k) or one of 1, 2, 4; otherwise kernels that take one element at a time
  *     run (same results, lower speed).  The
- *     tensor-core GEMMs read 16-byte aligned bf16 rows; operands whose rows are not are copied
- *     into the workspace first, where it has the room that velora_workspace_bytes reports
- *     for widths that are no multiple of 8.  Without it, and for fp32, the CUDA-core GEMM runs.
+ *     tensor-core GEMMs read 16-byte aligned bf16 rows; a layer's operands whose rows are not are copied
+ *     into the workspace first, where it has the room (VELORA_OP_ANY_ROWS).  Without it, for fp32 and in
+ *     velora_dense_product, the CUDA-core GEMM runs.
  *     The factored weight gradient of such bf16 rows runs on the CUDA cores in either case, with Z
  *     as stored; on aligned rows of more than 64 columns it rounds an fp32 Z to bf16 for the tensor cores.
  */
@@ -90,7 +90,9 @@ typedef enum {
     VELORA_OP_LINEAR_BACKWARD_FACTORED = 4,
     VELORA_OP_LINEAR_BACKWARD_EXPLICIT = 5,
     VELORA_OP_UPDATE_V = 6,
-    VELORA_OP_Z8_CALIBRATE = 7
+    VELORA_OP_Z8_CALIBRATE = 7,
+    /* added to one of the layer's or the explicit gradient's: with room for copies of operands on odd rows */
+    VELORA_OP_ANY_ROWS = 256
 } velora_op;
 
 #define VELORA_MAX_DSUB 1024
@@ -106,9 +108,11 @@ const char* velora_status_string(int status);
 
 /*
  * Bytes of device workspace the given entry point needs for these sizes
- * (0 if it needs none).  Independent of pointer values; deterministic.  Where D or O is no multiple of 8 the
- * figure includes room for aligned copies of the bf16 operands of that width; a workspace
- * smaller by that much is accepted and costs speed on rows that are not 16-byte aligned.
+ * (0 if it needs none).  Independent of pointer values; deterministic.  Calls that may be in flight at the same
+ * time (on two streams) must not share a workspace.
+ * With op | VELORA_OP_ANY_ROWS the figure includes, where D or O is no multiple of 8, room for aligned copies of the
+ * bf16 operands of that width (X and W of the forward, dY and W of the backward): worth it for rows that are not
+ * 16-byte aligned, which run on the CUDA cores without it, and for nothing else (padded rows and fp32 never use it).
  */
 size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub);
 

@@ -23,6 +23,7 @@ WG_FACTORED, WG_EXPLICIT = 0, 1
 PRODUCT_A_BT, PRODUCT_A_B, PRODUCT_AT_B = 0, 1, 2
 (OP_INIT_V, OP_WEIGHT_GRAD_FACTORED, OP_WEIGHT_GRAD_EXPLICIT, OP_LINEAR_FORWARD,
  OP_LINEAR_BACKWARD_FACTORED, OP_LINEAR_BACKWARD_EXPLICIT, OP_UPDATE_V, OP_Z8_CALIBRATE) = range(8)
+OP_ANY_ROWS = 256                                    # see velora_workspace_bytes
 
 _p, _i64, _int, _sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_size_t
 
@@ -179,8 +180,14 @@ def velora_status_string(status: int) -> str:
     return lib().velora_status_string(status).decode()
 
 
-def velora_workspace_bytes(op: int, N: int, D: int, O: int, Dsub: int) -> int:
-    return int(lib().velora_workspace_bytes(op, N, D, O, Dsub))
+def velora_workspace_bytes(op: int, N: int, D: int, O: int, Dsub: int, any_rows: bool = True) -> int:
+    """Bytes that ``op`` needs.  ``any_rows``: with room for aligned copies of bf16 operands where D or O is no multiple of 8 and
+    the rows may lie as torch.empty leaves them, without padding; False where they are padded to 16 bytes, or fp32."""
+    return int(lib().velora_workspace_bytes(op | OP_ANY_ROWS if any_rows else op, N, D, O, Dsub))
+
+
+def _odd_rows(t: torch.Tensor, ptr: int, ld: int) -> bool:
+    return t.dtype == torch.bfloat16 and (ptr % 16 != 0 or ld % 8 != 0)
 
 
 def velora_init_v(X: torch.Tensor, Dsub: int, v: Optional[torch.Tensor] = None,
@@ -248,7 +255,7 @@ def velora_weight_grad(dY: torch.Tensor, Z: torch.Tensor, v: torch.Tensor, D: in
     wp, lddw = _mat(dW, "dW")
     op = OP_WEIGHT_GRAD_FACTORED if mode == WG_FACTORED else OP_WEIGHT_GRAD_EXPLICIT
     if ws is None:
-        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
+        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub, _odd_rows(dY, yp, lddy)), dY.device)
     rc = lib().velora_weight_grad(yp, _dt(dY), N, O, lddy, zp, _dt(Z), ldz, _vec(v), D, Dsub,
                                   wp, _dt(dW), lddw, beta, mode, ws.data_ptr(), ws.numel(),
                                   _stream(stream))
@@ -273,7 +280,8 @@ def velora_linear_forward(X: torch.Tensor, W: torch.Tensor, v: torch.Tensor,
     yp, ldy = _mat(Y, "Y")
     zp, ldz = _mat(Z, "Z")
     if ws is None:
-        ws = velora_workspace_alloc(velora_workspace_bytes(OP_LINEAR_FORWARD, N, D, O, Dsub), X.device)
+        odd = _odd_rows(X, xp, ldx) or _odd_rows(W, wp, ldw)
+        ws = velora_workspace_alloc(velora_workspace_bytes(OP_LINEAR_FORWARD, N, D, O, Dsub, odd), X.device)
     rc = lib().velora_linear_forward(xp, ldx, wp, ldw, _vec(v), yp, ldy, zp, _dt(Z), ldz,
                                      _dt(X), N, D, O, Dsub, ws.data_ptr(), ws.numel(),
                                      _stream(stream))
@@ -299,7 +307,8 @@ def velora_linear_backward(dY: torch.Tensor, W: torch.Tensor, Z: torch.Tensor, v
     gp, lddw = _mat(dW, "dW") if need_dW else (None, D)
     op = OP_LINEAR_BACKWARD_FACTORED if mode == WG_FACTORED else OP_LINEAR_BACKWARD_EXPLICIT
     if ws is None:
-        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub), dY.device)
+        odd = _odd_rows(dY, yp, lddy) or (need_dX and _odd_rows(W, wp, ldw))
+        ws = velora_workspace_alloc(velora_workspace_bytes(op, N, D, O, Dsub, odd), dY.device)
     rc = lib().velora_linear_backward(yp, lddy, wp, ldw, zp, _dt(Z), ldz, _vec(v), xp, lddx,
                                       gp, _dt(dW) if need_dW else _dt(dY), lddw, beta, mode,
                                       _dt(dY), N, D, O, Dsub, ws.data_ptr(), ws.numel(),

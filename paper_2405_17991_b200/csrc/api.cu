@@ -72,14 +72,14 @@ size_t factored_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
 // ---- operands that TMA cannot address ----
 // A bf16 operand whose rows do not all start on 16-byte boundaries is copied to the end of the workspace with a padded
 // pitch (pack_rows.cu) and the tensor-core kernels run on the copy.  velora_workspace_bytes reports the room for the
-// operands whose width is no multiple of 8; a workspace without that room is as good as it ever was (the call then
-// runs on the CUDA cores), and other misaligned operands (an offset view) are copied where the room happens to be
-// there.  Measured on a 4096 x 2048 -> 5461 layer with dense rows: 3360 us a product on the CUDA cores.
+// operands whose width is no multiple of 8 when asked with VELORA_OP_ANY_ROWS (a forward of 4096 x 5461 -> 2048: 68 MB instead
+// of 256 bytes, which padded rows and fp32 have no use for); without that room the call runs on the CUDA cores, and other
+// misaligned operands (an offset view) are copied where the room happens to be there.  Measured on a 4096 x 2048 -> 5461 layer with dense rows: 3360 us a product on the CUDA cores.
 bool packable(int64_t rows, int64_t cols) { return rows >= 1 && rows < (1 << 30) && cols >= 1 && cols < (1 << 30); }
 
-size_t pack_bytes_if_ragged(int64_t rows, int64_t cols)
+size_t pack_bytes_if_ragged(int64_t rows, int64_t cols, bool any_rows)
 {
-    return cols % 8 && packable(rows, cols) ? pack_rows_bytes(rows, cols) : 0;
+    return any_rows && cols % 8 && packable(rows, cols) ? pack_rows_bytes(rows, cols) : 0;
 }
 
 struct Operand {
@@ -251,14 +251,15 @@ const char* velora_status_string(int status)
 size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub)
 {
     if (N < 0 || D < 1 || Dsub < 1 || Dsub > D || Dsub > VELORA_MAX_DSUB) return 0;
-    switch (op) {
+    const bool any_rows = (op & VELORA_OP_ANY_ROWS) != 0;
+    switch (op & ~VELORA_OP_ANY_ROWS) {
         case VELORA_OP_INIT_V: return init_v_workspace_bytes(Dsub);
         case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub);
         case VELORA_OP_LINEAR_BACKWARD_FACTORED:
-            return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O) + pack_bytes_if_ragged(O, D);
-        case VELORA_OP_WEIGHT_GRAD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O);
-        case VELORA_OP_LINEAR_BACKWARD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O) + pack_bytes_if_ragged(O, D);
-        case VELORA_OP_LINEAR_FORWARD: return kStatusBytes + pack_bytes_if_ragged(N, D) + pack_bytes_if_ragged(O, D);
+            return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
+        case VELORA_OP_WEIGHT_GRAD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O, any_rows);
+        case VELORA_OP_LINEAR_BACKWARD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
+        case VELORA_OP_LINEAR_FORWARD: return kStatusBytes + pack_bytes_if_ragged(N, D, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
         case VELORA_OP_UPDATE_V: return update_v_workspace_bytes(Dsub);
         case VELORA_OP_Z8_CALIBRATE: return z8_calibrate_workspace_bytes(N, D, Dsub);
         default: return 0;

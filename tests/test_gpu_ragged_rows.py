@@ -172,3 +172,19 @@ def test_explicit_fp32_gradient_on_odd_rows_is_a_rounded_sum(vl, guard, dy_pad, 
     dW = vl.velora_weight_grad(dY, Z, v, D, dW=guard.mat(O, D, torch.float32, ld=D + dw_pad), mode=vl.WG_EXPLICIT)
     ref = dY.double().T @ vl.velora_reconstruct(Z, v, D, x_dtype=torch.bfloat16).double()
     assert float((dW.double() - ref).norm() / ref.norm()) < 3.6e-6
+
+
+# A call without a workspace allocates room for copies only where it makes them.
+@pytest.mark.parametrize("dtype,pad,copies", [(torch.bfloat16, 0, True), (torch.bfloat16, 3, False), (torch.float32, 0, False)])
+def test_own_workspace_of_a_call(vl, monkeypatch, dtype, pad, copies):
+    from paper_2405_17991_b200 import binding
+    N, D, O, Dsub = 64, 1021, 509, 16
+    asked = []
+    alloc = binding.velora_workspace_alloc
+    monkeypatch.setattr(binding, "velora_workspace_alloc", lambda n, device: asked.append(n) or alloc(n, device))
+    X, W, dY = (torch.randn((r, c + pad), device=DEV).to(dtype)[:, :c] for r, c in ((N, D), (O, D), (N, O)))
+    v = torch.full((Dsub,), 0.25, device=DEV)
+    _, Z = vl.velora_linear_forward(X, W, v)
+    vl.velora_linear_backward(dY, W, Z, v)
+    need = [vl.velora_workspace_bytes(op, N, D, O, Dsub, any_rows=copies) for op in (vl.OP_LINEAR_FORWARD, vl.OP_LINEAR_BACKWARD_FACTORED)]
+    assert asked == need

@@ -141,6 +141,17 @@ def test_memory_model_matches_table_5b_structure():
         assert abs(full / saved_activation_bytes(1 << 20, D, 64, z_bytes=zb) / ratio - 1) < 1e-3
 
 
+# Copies of operands on odd rows are asked for, not part of what padded rows and fp32 need.
+def test_workspace_without_room_for_copies(lib):
+    from paper_2405_17991_b200 import binding as b
+    for op in (b.OP_LINEAR_FORWARD, b.OP_LINEAR_BACKWARD_FACTORED, b.OP_LINEAR_BACKWARD_EXPLICIT):
+        odd, even = (4096, 5461, 2041, 128), (4096, 5461 // 8 * 8, 2040, 128)
+        assert lib.velora_workspace_bytes(op, *odd) == b.velora_workspace_bytes(op, *odd, any_rows=False)
+        assert b.velora_workspace_bytes(op, *odd) >= lib.velora_workspace_bytes(op, *odd) + 4096 * 2041 * 2
+        assert b.velora_workspace_bytes(op, *even) == lib.velora_workspace_bytes(op, *even)
+    assert lib.velora_workspace_bytes(b.OP_LINEAR_FORWARD, 4096, 5461, 2048, 128) == 256
+
+
 # A kernel that waits for the one before it while that one runs may not read through the read-only path: ld.global.nc is for data
 # that nothing writes while the reader lives, and the compiler makes it of const __restrict__ inputs too.  Exempt: the conversion of
 # Z, which is launched when everything before it has completed, and the kernel behind it, which reads nothing else early.
