@@ -230,7 +230,7 @@ int velora_weight_grad(const void* dY, int dy_dtype, int64_t N, int64_t O, int64
  * be kept by the caller afterwards: (Z, W, v) is all the backward needs.
  * With bf16 data, 16-byte aligned rows and Dsub a power of two in 8 .. 1024, X is read
  * from HBM once for both results: inside the tensor-core product for wide layers
- * (O > 768), in a single streaming pass for adapter-shaped ones (O <= 64, Section 4:
+ * (O > 1792; O > 2816 where ldx is no multiple of 64), in a single streaming pass for adapter-shaped ones (O <= 64, Section 4:
  * down projections of adapters); other shapes run the product and then velora_compress.
  * ws: velora_workspace_bytes(VELORA_OP_LINEAR_FORWARD, ...) bytes.
  */

@@ -81,9 +81,8 @@ template <int CH> struct VSlice {
 // load takes microseconds: one batch at a time kept 16 KB per SM in flight and moved 3.4 GB/s per SM).
 // L = Dsub / 8 chunks form a sub-token: lps = min(L, 32) adjacent lanes hold (a part of) it, for L > 32 the CH = L / 32
 // consecutive instructions complete it.  fp32 products and sums, xor-shuffle reduction, one lane stores Z[row, m].
-// Columns at or beyond D count as zeros (ragged last sub-token), rows at or beyond N are skipped.  No shared memory and
-// no barrier (v sits in registers): the warps that do this never touch the GEMM's pipeline, and in particular not
-// the shared-memory bandwidth the tensor cores live on.
+// Columns at or beyond D count as zeros (ragged last sub-token), rows at or beyond N are skipped.  No shared-memory tile and
+// no barrier (v sits in registers): what these warps take from the tensor cores is the shared-memory pipe under their shuffles.
 template <int ZK, int CH> struct CompressWalk {
     const FuseArgs& fz;
     const VSlice<CH>& vs;

@@ -34,8 +34,6 @@ int launch_linear_forward_tc_pair(const void* X, int64_t ldx, const void* W, int
 int launch_linear_forward_skinny(const void* X, int64_t ldx, const void* W, int64_t ldw, const float* v,
                                  void* Y, int64_t ldy, void* Z, int z_dtype, int64_t ldz,
                                  int64_t N, int64_t D, int64_t O, int Dsub, int* status, cudaStream_t stream);
-// True when a product with this output shape fills the device with 256 x 256 pair tiles.
-bool gemm_pair_preferred(int64_t Mdim, int64_t Ndim);
 
 // Tensor map of a row-major bf16 matrix: `inner` contiguous elements per row, `outer` rows, row pitch
 // ld_elems; 128-byte swizzle (or none), zero fill outside the matrix.  (tensor_maps.cu)

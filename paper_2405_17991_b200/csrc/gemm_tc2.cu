@@ -20,8 +20,8 @@
 // FUSE = 1 / 2 / 3 (forward only, both operands K-major): four more warps per CTA compute Z = compress(X, v)
 // (fp32 / bf16 / E4M3 storage) for the row block the CTA is multiplying, from lines of X that are in L2 for
 // the GEMM anyway, so X crosses HBM once for both results.  The CTA pair working on n-tile j handles the
-// sub-token groups g with g % tiles_n == j.  These warps read X with plain 16-byte loads and share nothing
-// with the GEMM's pipeline: no stage, no barrier, no producer work (a second copy of the X tile fetched by the
+// sub-token groups g with g % tiles_n == j.  These warps read X with plain 16-byte loads and share no
+// stage, no barrier and no producer work with the GEMM's pipeline (a second copy of the X tile fetched by the
 // TMA producer into a buffer of their own cost 4-9 % of the product's time).
 #include <cooperative_groups.h>
 

@@ -70,7 +70,7 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, int tiles_m, int tiles
 // that are on their way through L2 for the GEMM anyway, so X crosses HBM once for both results.  The CTA
 // working on n-tile j handles the sub-token groups g with g % tiles_n == j, so the work is spread over the
 // CTAs that share a row block.  The compress warps read X with plain 16-byte loads and keep v in registers:
-// they share no stage, no barrier and no shared-memory bandwidth with the GEMM's pipeline (gemm_fuse.cuh),
+// they share no stage and no barrier with the GEMM's pipeline, only the pipe of their shuffles (gemm_fuse.cuh),
 // and they sit on warps 6, 7, 10, 11 so that none of them shares a warp scheduler (warp % 4) with the TMA
 // producer (warp 0) or the MMA issuer (warp 1).
 template <bool A_MN, bool B_MN, typename CT, int FUSE, int BN>
