@@ -27,9 +27,9 @@ def guard():
     g.check()
 
 
-# One element; tile edges; a K that leaves the last of eight splits empty (9 slices of 32); one that splits evenly; the
+# One element; tile edges; two shares of unequal length (9 slices of 32); eight of five slices, the last one empty; eight even ones; the
 # 128-wide tile (at least 148 of them) with ragged edges in all three directions; 304 of those, which run as half tiles.
-SIZES = [(1, 1, 1), (64, 64, 32), (65, 63, 33), (130, 70, 288), (171, 288, 1280), (40, 1000, 257), (1700, 1500, 77), (1664, 1536, 64), (2370, 2000, 50)]
+SIZES = [(1, 1, 1), (64, 64, 32), (65, 63, 33), (130, 70, 288), (130, 70, 1056), (171, 288, 1280), (40, 1000, 257), (1700, 1500, 77), (1664, 1536, 64), (2370, 2000, 50)]
 
 
 @pytest.mark.parametrize("Mdim,Ndim,Kdim", SIZES)

@@ -159,7 +159,7 @@ def test_init_v_compress_reconstruct_full_size(vl, outs, c, li, Dsub):
     assert abs(float(Z.double().sum()) - norm) < 1e-3 * norm + 1e-2 * np.sqrt(Z.numel())
 
 
-def test_unpadded_odd_rows_take_the_elementwise_kernels(vl, guard):
+def test_unpadded_odd_rows_give_the_results_of_padded_ones(vl, guard):
     cfg = vi.CONFIGS[4]
     li = 6                                            # down projection: D = 5461, odd row pitch
     Xa = vi.make_X(cfg, li, N=512)
@@ -236,33 +236,48 @@ def test_edge_shapes_all_entry_points(vl, outs, N, D, O, Dsub, dtype):
 
 
 FUSED_EDGE = [
-    # N, D, O, Dsub: outputs wide enough (>= 4 column tiles) for the forward to compute Z inside the GEMM
-    (300, 320, 1100, 16),    # four sub-tokens per 64-column block
-    (200, 264, 1024, 8),     # eight per block; D not a multiple of 64
-    (257, 1376, 1040, 64),   # ragged last sub-token (32 of 64 columns)
-    (130, 320, 1025, 256),   # sub-token spans four blocks, the last one has only one block of columns
-    (513, 640, 1536, 128),   # sub-token spans two blocks
-    (129, 2048, 1030, 1024), # longest sub-token
-    (260, 1536, 1100, 512),  # sub-token of 64 chunks: two loads per lane complete it
-    (140, 1000, 1026, 32),   # D a multiple of 8 only: the last 64-column block and the last sub-token are ragged
+    # N, D, O, Dsub: outputs of at least 12 column tiles of 256, for which the forward computes Z inside the product in every
+    # pitch; ragged in rows, columns and contraction.  Single CTAs of 128 columns where nothing else is said.
+    (300, 320, 2900, 16),    # four sub-tokens per 64-column block
+    (200, 264, 2824, 8),     # eight per block; D not a multiple of 64
+    (257, 1376, 2832, 64),   # ragged last sub-token (32 of 64 columns)
+    (130, 320, 2825, 256),   # sub-token spans four blocks, the last one has only one block of columns
+    (513, 640, 3072, 128),   # sub-token spans two blocks
+    (129, 2048, 2830, 1024), # longest sub-token; two CTAs share a tile's contraction
+    (260, 1536, 2900, 512),  # sub-token of 64 chunks: two loads per lane complete it
+    (140, 1000, 2826, 32),   # D a multiple of 8 only: the last 64-column block and the last sub-token are ragged
+    (60, 4096, 3072, 8),     # five CTAs share a tile's contraction
+    (120, 8192, 3072, 16),   # the same
+    (1300, 512, 3000, 64),   # single CTAs of 256 columns
+    (2300, 1376, 3600, 16),  # CTA pairs
+    (1900, 2040, 3072, 128), # the same, ragged last sub-token
 ]
 
 
 @pytest.mark.parametrize("N,D,O,Dsub", FUSED_EDGE)
-@pytest.mark.parametrize("z_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("z_dtype", [torch.float32, torch.bfloat16, torch.uint8])
 def test_forward_with_compress_inside_the_gemm(vl, outs, N, D, O, Dsub, z_dtype):
     case = vi.small_case(9000 + D + Dsub, N, D, O, dtype="bf16", mean_offset=0.25)
     Xa, Wa = case["X"], case["W"]
-    X, W = Xa.torch(DEV), Wa.torch(DEV)
+    X, W = Xa.torch(DEV), Wa.torch(DEV, ld=-(-D // 8) * 8)
     v = vl.velora_init_v(X, Dsub)
     v64 = to_f64(v)
     ws = outs.ws(vl.OP_LINEAR_FORWARD, N, D, O, Dsub)
+    before = vl.velora_launch_count()
     Y, Z = outs.forward(X, W, v, z_dtype=z_dtype, ws=ws)
+    assert vl.velora_launch_count() == before + 1              # one kernel for both results
     assert vl.velora_workspace_status(ws) == 0
     assert_matches(Y, oracle.linear_forward(Xa.f64(), Wa.f64()), TOL_GEMM, "Y")
-    assert_matches(Z, oracle.compress(Xa.f64(), v64), TOL_Z, "Z")
-    # the stand-alone kernel and the fused path agree to fp32 rounding
-    assert rel_err(to_f64(Z), to_f64(vl.velora_compress(X, v, z_dtype=z_dtype))) < (4e-3 if z_dtype == torch.bfloat16 else 1e-5)
+    alone = vl.velora_compress(X, v, z_dtype=torch.float32)
+    if z_dtype == torch.uint8:
+        # the code of the fp32 value, or its neighbour where that sits on the border of two
+        assert float((Z != alone.to(torch.float8_e4m3fn).view(torch.uint8)).double().mean()) < 1e-3
+        got, ref = Z.view(torch.float8_e4m3fn).double(), alone.double()
+        assert bool(((got - ref).abs() <= torch.clamp(ref.abs() / 16, min=2.0 ** -10) * 1.001).all())
+    else:
+        assert_matches(Z, oracle.compress(Xa.f64(), v64), TOL_Z, "Z")
+        # the stand-alone kernel and the fused path agree to fp32 rounding
+        assert rel_err(to_f64(Z), to_f64(alone)) < (4e-3 if z_dtype == torch.bfloat16 else 1e-5)
     assert vl.velora_device_error() == 0
 
 

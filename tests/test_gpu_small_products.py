@@ -1,4 +1,4 @@
-"""Tensor-core products of few tiles: every tile width, every number of CTAs that may share a contraction, ragged in all three
+"""Tensor-core products of few tiles: every tile width, 2, 3, 4, 5 and 8 CTAs that share a contraction, ragged in all three
 directions, with accumulation, unaligned outputs, and the compress that rides on a split forward."""
 import pytest
 import torch
@@ -26,10 +26,11 @@ def guard():
     g.check()
 
 
-# One k-block; 2 .. 8 CTAs per tile, with a short last share (71 and 33 k-blocks); tiles of 64, 128, 192 and 256 columns;
-# more tiles than SMs; rows and columns that end inside a tile.
+# One k-block; 2 .. 8 CTAs per tile (3: rows of the exchange that do not divide evenly), with a short last share (71 and 33
+# k-blocks); tiles of 64, 128, 192 and 256 columns, each alone and shared; more tiles than SMs; rows and columns that end inside a tile.
 SIZES = [(100, 40, 8), (128, 64, 128), (386, 320, 9032), (615, 296, 4536), (130, 1000, 2104), (1000, 264, 1000), (300, 2000, 520),
-         (2114, 576, 4096), (700, 1300, 3000), (3100, 768, 1024)]
+         (2114, 576, 4096), (700, 1300, 3000), (3100, 768, 1024),
+         (300, 768, 2048), (640, 1000, 3000), (640, 1000, 4096), (1500, 1000, 6000), (700, 1000, 4096), (4700, 1024, 512)]
 
 
 @pytest.mark.parametrize("Mdim,Ndim,Kdim", SIZES)
@@ -58,7 +59,7 @@ def test_products(vl, guard, Mdim, Ndim, Kdim, kind, c_dtype):
     assert torch.equal(C1, vl.velora_dense_product(kind, A, B, c_dtype=c_dtype))
 
 
-@pytest.mark.parametrize("N,D,O,Dsub", [(200, 4096, 3072, 64), (130, 1000, 2304, 8), (60, 2048, 2560, 512), (500, 1376, 4096, 1024)])
+@pytest.mark.parametrize("N,D,O,Dsub", [(200, 4096, 3072, 64), (130, 1000, 2880, 8), (60, 2048, 2560, 512), (500, 1376, 4096, 1024)])
 @pytest.mark.parametrize("z_dtype", [torch.float32, torch.bfloat16])
 def test_forward_of_few_tiles(vl, guard, N, D, O, Dsub, z_dtype):
     case = vi.small_case(N + D, N, D, O, dtype="bf16", mean_offset=0.1)
