@@ -33,7 +33,7 @@ constexpr int SK_DIRECT_PARTS = 8;    // slices that the expansion kernel adds u
 // Thread (warp w, lane l) owns outputs o = OI w + i (i < OI; one or two broadcast loads bring them), m = l + 32 j (j < MJ)
 // of the 8 OI columns of block blockIdx.y.
 template <typename YT, typename ZT, int OI, int MJ>
-__global__ void __launch_bounds__(SK_THREADS)
+__global__ void __launch_bounds__(SK_THREADS, MJ == 8 ? 2 : 1)
 wg_skinny_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
                          int N, int O, int M, int tokens_per_cta, float* __restrict__ partials)
 {
@@ -67,14 +67,18 @@ wg_skinny_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
     };
     pdl_wait();
     pdl_trigger();
-    fetch(n_begin);
+    // Each chunk is on its way while the one before is multiplied; for 129 sub-tokens and more that would leave an SM one CTA
+    // (164 registers), which costs more (gradient of 10161 x 60 with 152 sub-tokens: 32 us instead of 28).
+    constexpr bool AHEAD = MJ < 8;
+    if (AHEAD) fetch(n_begin);
     for (int n0 = n_begin; n0 < n_end; n0 += SK_CHUNK) {
+        if (!AHEAD) fetch(n0);
 #pragma unroll
         for (int u = 0; u < NY; ++u) (&sdy[0][0])[threadIdx.x + u * SK_THREADS] = ly[u];
 #pragma unroll
         for (int u = 0; u < NZ; ++u) (&sz[0][0])[threadIdx.x + u * SK_THREADS] = lz[u];
         __syncthreads();
-        if (n0 + SK_CHUNK < n_end) fetch(n0 + SK_CHUNK);      // on its way while this chunk is multiplied
+        if (AHEAD && n0 + SK_CHUNK < n_end) fetch(n0 + SK_CHUNK);
 #pragma unroll 4
         for (int r = 0; r < SK_CHUNK; ++r) {
             float y[OI], z[MJ];
@@ -594,6 +598,9 @@ int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O
     if (O > SK_MAX_O && dy_dtype == VELORA_BF16 && tc_operand_ok(dY, lddy)) return VELORA_ERR_UNSUPPORTED;
     const SkinnyPlan p = skinny_plan(N, D, O, Dsub, 148);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
+    // One slice of a wide layer's factor is one small product; the general kernel makes it without a reduction behind it
+    // (11 tokens, 1954 x 38: 4.7 us, 6.1 here).
+    if (O > SK_MAX_O && P_out && p.parts == 1) return VELORA_ERR_UNSUPPORTED;
     if (ws_bytes < p.partial_bytes + p.p_bytes) return VELORA_ERR_WORKSPACE;
     float* partials = static_cast<float*>(ws);
     float* P = reinterpret_cast<float*>(static_cast<char*>(ws) + p.partial_bytes);
