@@ -528,7 +528,6 @@ SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
     p.mj = static_cast<int>((M + 31) / 32);
     p.mj = p.mj <= 1 ? 1 : (p.mj <= 2 ? 2 : (p.mj <= 4 ? 4 : 8));
     p.o_blocks = static_cast<int>(ceil_div64(O, 8 * p.oi));
-    p.tile = O > SK_MAX_O && M <= SK_TILE_M;
     // One 32-token chunk per CTA where that gives at most 512 partials: the partial kernel is a single round
     // trip to memory plus a little arithmetic, so more, shorter CTAs finish sooner.
     int64_t max_parts = 512;
@@ -537,10 +536,13 @@ SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
         // workspace holds (that size is what velora_workspace_bytes has always reported for them).
         const int64_t bytes = static_cast<int64_t>(weight_grad_tc_workspace_bytes(N, D, O, Dsub)) - 512;   // two roundings to 256
         const int64_t room = bytes / static_cast<int64_t>(sizeof(float) * O * M) - 1;                       // and P itself
-        // Four CTAs per SM; the tile kernel's three (up to 16 sub-tokens) or two without a second wave.
-        max_parts = M <= SK_TILE_M ? (M <= 16 ? 3 : 2) * static_cast<int64_t>(sm_count) / p.o_blocks
-                                   : ceil_div64(4 * static_cast<int64_t>(sm_count), p.o_blocks);
-        if (max_parts < 1) max_parts = 1;
+        // Four CTAs per SM.  The tile kernel has three (up to 16 sub-tokens) or two, without a second wave, and takes slices of
+        // 256 tokens and more: adding up its eight warps costs several microseconds (45 tokens, 936 x 21: 12.4 us instead of 4.4).
+        max_parts = ceil_div64(4 * static_cast<int64_t>(sm_count), p.o_blocks);
+        int64_t tile_parts = (M <= 16 ? 3 : 2) * static_cast<int64_t>(sm_count) / p.o_blocks;
+        if (tile_parts < 1) tile_parts = 1;
+        p.tile = M <= SK_TILE_M && N >= 256 * tile_parts;
+        if (p.tile) max_parts = tile_parts;
         if (max_parts > room) max_parts = room;
         if (max_parts < 1 || p.o_blocks > 65535) return p;
     }
