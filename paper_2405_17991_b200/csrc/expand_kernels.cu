@@ -270,9 +270,9 @@ int launch_expand_rows_vec(const void* S, int s_dtype, int splits, int64_t split
     int rc = device_info(&di);
     if (rc != VELORA_OK) return rc;
     const int64_t cap = static_cast<int64_t>(di.sm_count) * kStreamCtasPerSm, warps = cap * (kStreamThreads / 32);
-    // Rows are cut while there are fewer of them than warps, into spans of eight store instructions or more (four of 16 bytes).
+    // Rows are cut while there are two warps and more for each, into spans of eight store instructions or more (four of 16 bytes).
     const int spw = 32 / lps, least = spw * ceil_div64(vec == 1 ? 8 : 4, ch);
-    int64_t n_segs = R < warps ? ceil_div64(warps, R) : 1;
+    int64_t n_segs = R < warps ? warps / R : 1;
     if (n_segs > ceil_div64(M, least)) n_segs = ceil_div64(M, least);
     const int span = static_cast<int>(ceil_div64(ceil_div64(M, n_segs), spw) * spw);
     const int segs = static_cast<int>(ceil_div64(M, span));

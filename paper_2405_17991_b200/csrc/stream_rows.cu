@@ -218,11 +218,11 @@ RowsPlan plan_rows(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx
     p.M = static_cast<int>(ceil_div64(D, Dsub));
     int64_t cap = static_cast<int64_t>(sm_count) * kStreamCtasPerSm;
     if (max_grid > 0 && cap > max_grid) cap = max_grid;
-    // Rows are cut while there are fewer of them than warps; for the sub-token sum than four warps per SM, because each CTA adds
+    // Rows are cut while there are two warps and more for each; for the sub-token sum of four warps per SM, because each CTA adds
     // a row to what the finalize kernel's one CTA adds up (512 x 2045 fp32, Dsub 256: 16 us with as many runs as compress).
     const int64_t rounds = ceil_div64(ceil_div64(D, p.vec), 32 * (p.ch > RW_U ? p.ch : RW_U));
     const int64_t wanted = sum ? 4 * static_cast<int64_t>(sm_count) : cap * RW_WARPS;
-    int64_t segs = N < wanted ? ceil_div64(wanted, N) : 1;
+    int64_t segs = N < wanted ? wanted / N : 1;
     if (segs > rounds) segs = rounds;
     p.seg_rounds = static_cast<int>(ceil_div64(rounds, segs));
     p.segs = static_cast<int>(ceil_div64(rounds, p.seg_rounds));
