@@ -47,8 +47,9 @@
  *     (fastest for 8 * 2^k) or one of 1, 2, 4; otherwise kernels that take one element at a time
  *     run (same results, lower speed).  The
  *     tensor-core GEMMs read 16-byte aligned bf16 rows; a layer's operands whose rows are not are copied
- *     into the workspace first, where it has the room (VELORA_OP_ANY_ROWS).  Without it, for fp32 and in
- *     velora_dense_product, the CUDA-core GEMM runs.
+ *     into the workspace first, where it has the room (VELORA_OP_ANY_ROWS).  Without it and in
+ *     velora_dense_product, the CUDA-core GEMM runs.  fp32 products run on the tensor cores as bf16 parts, with an
+ *     error no larger than that of fp32 multiply-adds in sequence, or where they are small on the CUDA cores.
  *     The factored weight gradient of such bf16 rows runs on the CUDA cores in either case, with Z
  *     as stored; on aligned rows of more than 64 columns it rounds an fp32 Z to bf16 for the tensor cores.
  */
@@ -226,7 +227,7 @@ int velora_weight_grad(const void* dY, int dy_dtype, int64_t N, int64_t O, int64
  * Forward of the VeLoRA linear (Algorithm 1, forward):
  *     Y[N, O] = X W^T      and      Z = compress(X, v)
  * `dtype` is the storage type of X, W and Y (bf16: tensor cores with fp32
- * accumulation; f32: CUDA cores).  Z as in velora_compress.  X itself need not
+ * accumulation; f32: tensor cores to fp32 accuracy, or CUDA cores).  Z as in velora_compress.  X itself need not
  * be kept by the caller afterwards: (Z, W, v) is all the backward needs.
  * With bf16 data, 16-byte aligned rows and Dsub a power of two in 8 .. 1024, X is read
  * from HBM once for both results: inside the tensor-core product for wide layers
@@ -290,8 +291,8 @@ int velora_z8_calibrate(const void* X, int x_dtype, int64_t N, int64_t D, int64_
  *   VELORA_PRODUCT_A_BT:  A[Mdim, Kdim], B[Ndim, Kdim]    (C = A B^T)
  *   VELORA_PRODUCT_A_B:   A[Mdim, Kdim], B[Kdim, Ndim]    (C = A B)
  *   VELORA_PRODUCT_AT_B:  A[Kdim, Mdim], B[Kdim, Ndim]    (C = A^T B)
- * `dtype`: storage type of A and B (bf16: tensor cores when their rows are 16-byte aligned; otherwise and for
- * f32 the CUDA-core product).  C: c_dtype, bf16 or f32.  ws: at least 256 bytes, initialised (status header).
+ * `dtype`: storage type of A and B (bf16: tensor cores when their rows are 16-byte aligned, otherwise the CUDA-core product;
+ * f32: either, see above).  C: c_dtype, bf16 or f32.  ws: at least 256 bytes, initialised (status header).
  */
 typedef enum { VELORA_PRODUCT_A_BT = 0, VELORA_PRODUCT_A_B = 1, VELORA_PRODUCT_AT_B = 2 } velora_product;
 int velora_dense_product(int kind, const void* A, int64_t lda, const void* B, int64_t ldb,

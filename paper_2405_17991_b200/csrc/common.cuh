@@ -137,11 +137,13 @@ int launch_reconstruct(const void* Z, int z_dtype, int64_t ldz, int64_t N, int64
 
 // ---- GEMMs ----
 // C[m, n] = sum_k A(m, k) * B(n, k) with element strides; fp32 accumulation on CUDA cores.
-// Serves the all-fp32 case and shapes the tensor-core path does not take.
+// Serves the shapes that the tensor-core paths do not take.
 int launch_gemm_simt(const void* A, int a_dtype, int64_t a_sm, int64_t a_sk,
                      const void* B, int b_dtype, int64_t b_sn, int64_t b_sk,
                      void* C, int c_dtype, int64_t ldc, int beta,
                      int64_t Mdim, int64_t Ndim, int64_t Kdim, cudaStream_t stream);
+// Estimate of its time for fp32 operands, in microseconds.
+double gemm_simt_f32_us(int64_t Mdim, int64_t Ndim, int64_t Kdim, int sm_count);
 
 // dW[o, m*Dsub + j] = beta*dW + (sum over `splits` partial P[s][o][m], fp32) * v[j].
 int launch_expand_p(const float* P, int splits, int64_t split_stride, int64_t ldp, const float* v,

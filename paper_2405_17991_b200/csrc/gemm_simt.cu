@@ -1,7 +1,7 @@
 // CUDA-core GEMM with arbitrary element strides and fp32 accumulation.
 //   C[m, n] = beta * C[m, n] + sum_k A(m, k) * B(n, k)
-// It computes the dense products of Algorithm 1 (arxiv 2405.17991) for the all-fp32 case, where tensor cores would
-// drop mantissa bits, and for bf16 operands that neither TMA nor the packed copies can serve.
+// It computes the dense products of Algorithm 1 (arxiv 2405.17991) for small all-fp32 ones (gemm_f32_tc.cu has the others)
+// and for bf16 operands that neither TMA nor the packed copies can serve.
 //
 // Bound by the fp32 pipes (74 TFLOP/s at 1965 MHz).  Three shapes of the same kernel, 256 threads each:
 //   128 x 128 tile, 16-deep slices, 8 x 8 outputs a thread: 64 multiply-adds for four 16-byte shared-memory loads, and
@@ -281,6 +281,28 @@ int launch_tiles(const void* A, int64_t a_sm, int64_t a_sk, int a_mode, const vo
     return after_launch();
 }
 
+struct SimtShape {
+    int rows, cols, splits;                                     // of a tile; CTAs that share its contraction
+};
+
+SimtShape simt_shape(int64_t Mdim, int64_t Ndim, int64_t Kdim, int sm_count)
+{
+    // The large tile once it gives every SM one; two of them fit on an SM.  Half of it in rows where that saves more of the
+    // last wave than its extra loads cost: 12608 x 768 is 594 large tiles on 296 places, two of which ran alone for a third
+    // of the time, and 1182 half tiles (layer of two such products: 887 -> 813 us).
+    const int64_t large = ceil_div64(Mdim, 128) * ceil_div64(Ndim, 128), half = ceil_div64(Mdim, 64) * ceil_div64(Ndim, 128);
+    if (large >= sm_count) {
+        const int64_t places = 2 * static_cast<int64_t>(sm_count);
+        if (11 * ceil_div64(half, places) < 20 * ceil_div64(large, places)) return SimtShape{64, 128, 1};
+        return SimtShape{128, 128, 1};
+    }
+    // Few small tiles: share the contraction while that leaves every CTA four slices and no more than two CTAs per SM.
+    const int64_t tiles = ceil_div64(Mdim, 64) * ceil_div64(Ndim, 64);
+    int splits = 1;
+    while (splits < SG_MAX_SPLITS && tiles * splits * 2 <= 2 * sm_count && ceil_div64(Kdim, 32) >= 8 * splits) splits *= 2;
+    return SimtShape{64, 64, splits};
+}
+
 template <typename AT, typename BT, typename CT>
 int dispatch_tiles(const void* A, int a_dtype, int64_t a_sm, int64_t a_sk, const void* B, int b_dtype, int64_t b_sn, int64_t b_sk,
                    void* C, int c_dtype, int64_t ldc, int beta, int64_t Mdim, int64_t Ndim, int64_t Kdim, cudaStream_t stream)
@@ -290,24 +312,24 @@ int dispatch_tiles(const void* A, int a_dtype, int64_t a_sm, int64_t a_sk, const
     if (rc != VELORA_OK) return rc;
     const int a_mode = load_mode(A, a_dtype, a_sm, a_sk), b_mode = load_mode(B, b_dtype, b_sn, b_sk);
     const int c_vec = c_dtype == VELORA_F32 && aligned16(C) && ldc % 4 == 0;
-    // The large tile once it gives every SM one; two of them fit on an SM.  Half of it in rows where that saves more of the
-    // last wave than its extra loads cost: 12608 x 768 is 594 large tiles on 296 places, two of which ran alone for a third
-    // of the time, and 1182 half tiles (layer of two such products: 887 -> 813 us).
-    const int64_t large = ceil_div64(Mdim, 128) * ceil_div64(Ndim, 128), half = ceil_div64(Mdim, 64) * ceil_div64(Ndim, 128);
-    if (large >= di.sm_count) {
-        const int64_t places = 2 * static_cast<int64_t>(di.sm_count);
-        if (11 * ceil_div64(half, places) < 20 * ceil_div64(large, places))
-            return launch_tiles<1, 2, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, 1, stream);
+    const SimtShape shape = simt_shape(Mdim, Ndim, Kdim, di.sm_count);
+    if (shape.rows == 128)
         return launch_tiles<2, 2, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, 1, stream);
-    }
-    // Few small tiles: share the contraction while that leaves every CTA four slices and no more than two CTAs per SM.
-    const int64_t tiles = ceil_div64(Mdim, 64) * ceil_div64(Ndim, 64);
-    int splits = 1;
-    while (splits < SG_MAX_SPLITS && tiles * splits * 2 <= 2 * di.sm_count && ceil_div64(Kdim, 32) >= 8 * splits) splits *= 2;
-    return launch_tiles<1, 1, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, splits, stream);
+    if (shape.cols == 128)
+        return launch_tiles<1, 2, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, 1, stream);
+    return launch_tiles<1, 1, AT, BT, CT>(A, a_sm, a_sk, a_mode, B, b_sn, b_sk, b_mode, C, ldc, beta, c_vec, Mdim, Ndim, Kdim, shape.splits, stream);
 }
 
 }  // namespace
+
+// Waves of CTAs, each its share of K at what a step of its tile takes on a full chip; a cluster costs its launch and the exchange.
+double gemm_simt_f32_us(int64_t Mdim, int64_t Ndim, int64_t Kdim, int sm_count)
+{
+    const SimtShape t = simt_shape(Mdim, Ndim, Kdim, sm_count);
+    const int64_t ctas = ceil_div64(Mdim, t.rows) * ceil_div64(Ndim, t.cols) * t.splits;
+    const double step = t.rows == 128 ? 0.22 : (t.cols == 128 ? 0.121 : 0.061);
+    return (t.splits > 1 ? 9.0 : 5.0) + ceil_div64(ctas, 2 * static_cast<int64_t>(sm_count)) * step * ceil_div64(Kdim, t.splits);
+}
 
 int launch_gemm_simt(const void* A, int a_dtype, int64_t a_sm, int64_t a_sk,
                      const void* B, int b_dtype, int64_t b_sn, int64_t b_sk,

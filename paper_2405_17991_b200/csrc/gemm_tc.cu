@@ -45,6 +45,8 @@ int launch_gemm_tc(int kind, const void* A, int64_t lda, const void* B, int64_t 
                    void* C, int c_dtype, int64_t ldc, int beta,
                    int64_t Mdim, int64_t Ndim, int64_t Kdim, int in_dtype, int* status, cudaStream_t stream)
 {
+    if (in_dtype == VELORA_F32 && c_dtype == VELORA_F32)
+        return launch_gemm_f32_tc(kind, A, lda, B, ldb, C, ldc, beta, Mdim, Ndim, Kdim, status, stream);
     if (in_dtype != VELORA_BF16) return VELORA_ERR_UNSUPPORTED;
     if (Mdim < 1 || Ndim < 1 || Kdim < 1) return VELORA_ERR_UNSUPPORTED;
     if (Mdim > (1 << 30) || Ndim > (1 << 30) || Kdim > (1 << 30)) return VELORA_ERR_UNSUPPORTED;

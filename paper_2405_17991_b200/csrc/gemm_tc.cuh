@@ -22,6 +22,11 @@ int launch_gemm_tc(int kind, const void* A, int64_t lda, const void* B, int64_t 
                    void* C, int c_dtype, int64_t ldc, int beta,
                    int64_t Mdim, int64_t Ndim, int64_t Kdim, int in_dtype, int* status, cudaStream_t stream);
 
+// The same products for fp32 operands and an fp32 result, to fp32 accuracy, any row pitch and alignment.  VELORA_ERR_UNSUPPORTED
+// (nothing launched) where the CUDA cores are faster.  (gemm_f32_tc.cu)
+int launch_gemm_f32_tc(int kind, const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, int beta,
+                       int64_t Mdim, int64_t Ndim, int64_t Kdim, int* status, cudaStream_t stream);
+
 // The same product with CTA pairs (tcgen05 cta_group::2, 256 x 256 tile per pair).  (gemm_tc2.cu)
 int launch_gemm_tc_pair(int kind, const void* A, int64_t lda, const void* B, int64_t ldb,
                         void* C, int c_dtype, int64_t ldc, int beta,

@@ -28,7 +28,7 @@
 #include "gemm_fuse.cuh"
 #include "gemm_store.cuh"
 #include "gemm_tc.cuh"
-#include "tc_common.cuh"
+#include "tc_pair.cuh"
 
 namespace velora {
 
@@ -50,70 +50,6 @@ constexpr int P_FUSE_THREADS = P_THREADS + 192;      // + four compress warps (6
 constexpr int P_STAGE_OFF = 256;                     // behind the ring: barriers, then the staging of unaligned output rows
 constexpr size_t P_SMEM = 1024 + static_cast<size_t>(P_STAGES) * P_STAGE_BYTES + P_STAGE_OFF + 4 * kStageFloats * sizeof(float);
 constexpr size_t P_FUSE_SMEM = P_SMEM;
-
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank)
-{
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
-    return remote;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// Tile load of a CTA pair: data to this CTA's shared memory, completion bytes to a barrier given by its
-// cluster address (the leader's).
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* m, uint32_t bar_cluster, int c0, int c1)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(c0), "r"(c1)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem, uint32_t cols)
-{
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish_pair()
-{
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols)
-{
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate ? 1u : 0u)
-        : "memory");
-}
-// Arrives on the barrier at this shared-memory offset in BOTH CTAs of the pair once the MMAs issued so
-// far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(bar), "h"(static_cast<uint16_t>(3)) : "memory");
-}
-
-struct PairTile {
-    int m0, n0;
-};
-// Pair tiles (256 x 256) walked in bands of 4 m-tiles so that pairs running together share B in L2.
-__device__ __forceinline__ PairTile pair_tile(int tile, int tiles_m, int tiles_n)
-{
-    constexpr int BAND = 4;
-    const int per_band = BAND * tiles_n;
-    const int band = tile / per_band;
-    const int in_band = tile - band * per_band;
-    const int band_rows = (tiles_m - band * BAND < BAND) ? tiles_m - band * BAND : BAND;
-    const int tn = in_band / band_rows;
-    const int tm = band * BAND + (in_band - tn * band_rows);
-    return {tm * 2 * P_BM, tn * P_BN};
-}
 
 template <bool A_MN, bool B_MN, typename CT, int FUSE>
 __global__ void __launch_bounds__(FUSE ? P_FUSE_THREADS : P_THREADS, 1)
@@ -177,7 +113,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int started = 0;
             for (int tile = pair; tile < num_tiles && !failed; tile += num_pairs) {
                 if (FUSE) *tiles_started = ++started;          // the compress warps may take this tile's row block now
-                const PairTile t0 = pair_tile(tile, tiles_m, tiles_n);
+                const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * P_BM, P_BN);
                 const int m0 = t0.m0 + static_cast<int>(rank) * P_BM;
                 const int n0 = t0.n0 + static_cast<int>(rank) * (P_BN / 2);
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
@@ -268,7 +204,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int ti = 0;
             for (int tile = pair; tile < num_tiles; tile += num_pairs, ++ti) {
                 if (!wait_for_tile(tiles_started, ti, abort_flag)) { failed = true; break; }
-                const PairTile t0 = pair_tile(tile, tiles_m, tiles_n);
+                const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * P_BM, P_BN);
                 const int r0 = t0.m0 + static_cast<int>(rank) * P_BM + cwi * 32;
                 CompressWalk<FUSE, vs.kParts>(fz, vs, r0, Mdim, Kdim, lane).run(t0.n0 / P_BN, tiles_n, n_groups);
             }
@@ -282,7 +218,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint32_t lead_tempty0 = map_to_cta(tempty, 0);
         uint32_t t = 0;
         for (int tile = pair; tile < num_tiles && !failed; tile += num_pairs, ++t) {
-            const PairTile t0 = pair_tile(tile, tiles_m, tiles_n);
+            const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * P_BM, P_BN);
             const uint32_t acc = t & 1u, aph = (t >> 1) & 1u;
             if (!mbar_wait_warp(tfull + 8 * acc, aph, abort_flag, 256)) { failed = true; break; }
             tc_fence_after_sync();
