@@ -3,6 +3,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace velora {
 
@@ -147,6 +148,37 @@ __device__ __forceinline__ void store_rows_staged(CT* block, int64_t ldc, int ro
         }
     }
     __syncwarp();
+}
+
+// How outputs are written: rows on odd boundaries by store_rows_staged, others by Store32 or as tiles by store_block.
+enum CRows { C_ELEMENTS = 0, C_VECTORS = 1, C_TILES = 2 };
+
+// bf16 outputs on 16-byte boundaries leave as tiles, 32 rows x 64 columns a warp: a lane that stores its own row writes 32 sectors of
+// 32 lines per instruction, and a product with little else to do waits for those (8192 x 4096 with K = 16: 19.5 us, 14.0 as
+// tiles, 67 MB at 4.8 TB/s; 8192 x 1024, K = 256: 9.6 and 8.1; 4096 x 4096 products of long contractions the same).  A tile
+// store clips whole 16-byte chunks: where the width is no multiple of 8 the last columns' block is left to Store32.
+constexpr int kStoreBytes = 32 * 128;
+
+// A warp's 32 x 64 outputs, r[h] the columns 32 h .. of this lane's row, through its block of shared memory (128-byte swizzle) to
+// C at (row0, col0).
+__device__ __forceinline__ void store_block(const CUtensorMap* tmC, uint32_t block, const uint32_t (&r)[2][32], int col0, int row0, int lane)
+{
+    if (lane == 0) tc::bulk_wait_read();                            // the block's last content is on its way
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int k = 8 * (c % 4) + 2 * e;
+            w[e] = pack_bf16x2(__uint_as_float(r[c / 4][k]), __uint_as_float(r[c / 4][k + 1]));
+        }
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(block + lane * 128 + ((c ^ (lane & 7)) << 4)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+    }
+    tc::fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) tc::tma_store_2d(tmC, block, col0, row0);
 }
 
 }  // namespace velora

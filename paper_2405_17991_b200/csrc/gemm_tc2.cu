@@ -47,14 +47,16 @@ constexpr int P_SLAB = 64 * P_BK * 2;               // 8 KB, one 64-wide MN-majo
 constexpr int P_THREADS = 192;
 constexpr int P_TMEM_COLS = 512;
 constexpr int P_FUSE_THREADS = P_THREADS + 192;      // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
-constexpr int P_STAGE_OFF = 256;                     // behind the ring: barriers, then the staging of unaligned output rows
-constexpr size_t P_SMEM = 1024 + static_cast<size_t>(P_STAGES) * P_STAGE_BYTES + P_STAGE_OFF + 4 * kStageFloats * sizeof(float);
+constexpr int P_BARRIER_BYTES = 256;
+constexpr int P_STAGING_BYTES = 17 * 1024;           // behind the ring: output blocks of the four epilogue warps on their way to memory
+static_assert(P_STAGING_BYTES >= 4 * kStageFloats * 4 && P_STAGING_BYTES >= 4 * kStoreBytes, "staging");
+constexpr size_t P_SMEM = 1024 + static_cast<size_t>(P_STAGES) * P_STAGE_BYTES + P_STAGING_BYTES + P_BARRIER_BYTES;
 constexpr size_t P_FUSE_SMEM = P_SMEM;
 
 template <bool A_MN, bool B_MN, typename CT, int FUSE>
 __global__ void __launch_bounds__(FUSE ? P_FUSE_THREADS : P_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
+                 const __grid_constant__ CUtensorMap tmC, CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
                  int tiles_m, int tiles_n, int c_vec, int* __restrict__ status, const FuseArgs fz)
 {
     static_assert(FUSE == 0 || (!A_MN && !B_MN), "compress rides on the K-major forward GEMM only");
@@ -68,8 +70,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
-    uint8_t* tail = smem + P_STAGES * P_STAGE_BYTES;
-    const uint32_t bars = base + P_STAGES * P_STAGE_BYTES;
+    uint8_t* staging = smem + P_STAGES * P_STAGE_BYTES;
+    uint8_t* tail = staging + P_STAGING_BYTES;
+    const uint32_t bars = base + P_STAGES * P_STAGE_BYTES + P_STAGING_BYTES;
     const uint32_t full = bars, empty = bars + 8 * P_STAGES;
     const uint32_t tfull = bars + 16 * P_STAGES, tempty = tfull + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 16 * P_STAGES + 48);
@@ -94,6 +97,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         fence_mbar_init();
         prefetch_tensormap(&tmA);
         prefetch_tensormap(&tmB);
+        if (c_vec == C_TILES) prefetch_tensormap(&tmC);
     }
     if (warp == 1) {
         tmem_alloc_pair(smem_u32(tmem_slot), P_TMEM_COLS);
@@ -216,6 +220,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // ------------------------------------------------ epilogue: this CTA's 128 rows of the pair tile
         const int quarter = warp & 3;
         const uint32_t lead_tempty0 = map_to_cta(tempty, 0);
+        const uint32_t block = smem_u32(staging) + quarter * kStoreBytes;
         uint32_t t = 0;
         for (int tile = pair; tile < num_tiles && !failed; tile += num_pairs, ++t) {
             const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * P_BM, P_BN);
@@ -237,7 +242,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8 * acc);
                 }
                 const int valid = Ndim - (t0.n0 + c * 32);
-                if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
+                if (sizeof(CT) == 2 && c_vec == C_TILES && (valid >= 64 || Ndim % 8 == 0)) {
+                    if (row - lane < Mdim && valid > 0) store_block(&tmC, block, r, t0.n0 + c * 32, row - lane, lane);
+                } else if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
                         if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);
@@ -246,10 +253,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int h = 0; h < 2; ++h)
                         if (valid > 32 * h)
                             store_rows_staged<CT>(crow - static_cast<int64_t>(lane) * ldc + (c + h) * 32, ldc, Mdim - (row - lane), valid - 32 * h,
-                                                  r[h], beta, reinterpret_cast<float*>(tail + P_STAGE_OFF) + quarter * kStageFloats, lane);
+                                                  r[h], beta, reinterpret_cast<float*>(staging) + quarter * kStageFloats, lane);
                 }
             }
         }
+        if (sizeof(CT) == 2 && c_vec == C_TILES && lane == 0) bulk_wait_all();
         if (failed) *abort_flag = 1;
     }
     if (failed && status) atomicExch(status, VELORA_ERR_TIMEOUT);
@@ -295,8 +303,10 @@ int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t l
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n,
-                           c_rows_vec(C, ldc, sizeof(CT)), status, fz) !=
+    int c_vec = c_rows_vec(C, ldc, sizeof(CT)) ? C_VECTORS : C_ELEMENTS;
+    CUtensorMap tc = ta;
+    if (sizeof(CT) == 2 && c_vec && !beta && tc_operand_ok(C, ldc) && make_tmap_bf16_2d(&tc, C, Ndim, Mdim, ldc, 64, 32) == VELORA_OK) c_vec = C_TILES;
+    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, c_vec, status, fz) !=
         cudaSuccess) {
         cudaGetLastError();
         return VELORA_ERR_CUDA;

@@ -34,7 +34,7 @@ constexpr int GEMM_THREADS = 192;                   // producer, issuer, four ep
 constexpr int GEMM_THREADS_SHORT = 320;             // eight epilogue warps, for contractions of up to SHORT_KBLOCKS k-blocks
 constexpr int SHORT_KBLOCKS = 8;
 constexpr int FUSE_THREADS = 384;    // + four compress warps (6, 7, 10, 11) and two idle ones (8, 9)
-constexpr int STAGE_OFF = 256;                    // behind the ring: barriers, then the staging of unaligned output rows
+constexpr int BARRIER_BYTES = 256;
 
 // What depends on the tile's width: as many stages as fit 200 KB, at most eight.
 template <int BN> struct TileShape {
@@ -42,7 +42,12 @@ template <int BN> struct TileShape {
     static constexpr int kFit = 200 * 1024 / (A_BYTES + kBBytes);
     static constexpr int kStages = kFit < 8 ? kFit : 8;
     static constexpr int kTmemCols = BN > 128 ? 512 : (BN > 64 ? 256 : 128);       // two accumulators, a power of two
-    static constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * (A_BYTES + kBBytes) + STAGE_OFF + 4 * kStageFloats * sizeof(float);
+    // Behind the ring: output blocks on their way to memory, of eight warps (four at BN = 192, whose ring has the room of the
+    // others) or, unaligned rows, of four.
+    static constexpr int kStoreWarps = BN == 192 ? 4 : 8;
+    static constexpr int kStagingBytes = kStoreWarps == 8 ? 8 * kStoreBytes : 17 * 1024;
+    static_assert(kStagingBytes >= 4 * kStageFloats * 4 && kStagingBytes >= kStoreWarps * kStoreBytes && kStagingBytes % 1024 == 0, "staging");
+    static constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * (A_BYTES + kBBytes) + kStagingBytes + BARRIER_BYTES;
     static constexpr int kPartialPitch = BN + 4;                                    // floats per row of a parked partial tile
     static_assert(static_cast<size_t>(BM) * kPartialPitch * 4 <= static_cast<size_t>(kStages) * (A_BYTES + kBBytes), "fits the ring");
 };
@@ -76,7 +81,7 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, int tiles_m, int tiles
 template <bool A_MN, bool B_MN, typename CT, int FUSE, int BN>
 __global__ void __launch_bounds__(FUSE ? FUSE_THREADS : GEMM_THREADS_SHORT, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
+               const __grid_constant__ CUtensorMap tmC, CT* __restrict__ C, int64_t ldc, int beta, int Mdim, int Ndim, int Kdim,
                int tiles_m, int tiles_n, int kb_per_split, int c_vec, int* __restrict__ status, const FuseArgs fz)
 {
     typedef TileShape<BN> S;
@@ -88,8 +93,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint8_t* smem = smem_raw + (base - raw);
     const uint32_t sA = base;
     const uint32_t sB = base + STAGES * A_BYTES;
-    uint8_t* tail = smem + STAGES * (A_BYTES + B_BYTES);
-    const uint32_t bars = base + STAGES * (A_BYTES + B_BYTES);
+    uint8_t* staging = smem + STAGES * (A_BYTES + B_BYTES);
+    uint8_t* tail = staging + S::kStagingBytes;
+    const uint32_t bars = base + STAGES * (A_BYTES + B_BYTES) + S::kStagingBytes;
     const uint32_t full = bars, empty = bars + 8 * STAGES;
     const uint32_t tfull = bars + 16 * STAGES, tempty = tfull + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 16 * STAGES + 48);
@@ -118,6 +124,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         fence_mbar_init();
         prefetch_tensormap(&tmA);
         prefetch_tensormap(&tmB);
+        if (c_vec == C_TILES) prefetch_tensormap(&tmC);
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
@@ -231,6 +238,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int quarter = warp & 3;
         const int set = FUSE ? 0 : (warp - 2) >> 2;
         const int sets = FUSE || blockDim.x == GEMM_THREADS || (sizeof(CT) == 2 && !c_vec && splits == 1) ? 1 : 2;     // staging room for four warps
+        const uint32_t block = smem_u32(staging) + (warp - 2) * kStoreBytes;
         uint32_t t = 0;
         for (int tile = blockIdx.x; tile < num_tiles && !failed; tile += gridDim.x, ++t) {
             const TileCoord tc0 = tile_coord<BN>(tile, tiles_m, tiles_n);
@@ -271,7 +279,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (lane == 0) mbar_arrive(tempty + 8 * acc);
                 }
                 const int valid = Ndim - (tc0.n0 + c * 32);
-                if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
+                if (sizeof(CT) == 2 && c_vec == C_TILES && (valid >= 64 || Ndim % 8 == 0)) {
+                    if (row - lane < Mdim && valid > 0) store_block(&tmC, block, r, tc0.n0 + c * 32, row - lane, lane);
+                } else if (sizeof(CT) == 4 || c_vec) {            // fp32 rows always are (host)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
                         if (row < Mdim && valid > 32 * h) Store32<CT>::run(crow + (c + h) * 32, r[h], valid - 32 * h, beta);
@@ -280,10 +290,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     for (int h = 0; h < 2; ++h)
                         if (valid > 32 * h)
                             store_rows_staged<CT>(crow - static_cast<int64_t>(lane) * ldc + (c + h) * 32, ldc, Mdim - (row - lane), valid - 32 * h,
-                                                  r[h], beta, reinterpret_cast<float*>(tail + STAGE_OFF) + quarter * kStageFloats, lane);
+                                                  r[h], beta, reinterpret_cast<float*>(staging) + quarter * kStageFloats, lane);
                 }
             }
         }
+        if (sizeof(CT) == 2 && c_vec == C_TILES && lane == 0) bulk_wait_all();
         if (failed) *abort_flag = 1;
     }
     if (failed && status) atomicExch(status, VELORA_ERR_TIMEOUT);
@@ -356,11 +367,16 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     const int64_t tiles = static_cast<int64_t>(tiles_m) * tiles_n;
     const int kblocks = (Kdim + BK - 1) / BK;
     const int threads = FUSE ? FUSE_THREADS : (kblocks <= SHORT_KBLOCKS * splits ? GEMM_THREADS_SHORT : GEMM_THREADS);
-    const int c_vec = c_rows_vec(C, ldc, sizeof(CT));
+    int c_vec = c_rows_vec(C, ldc, sizeof(CT)) ? C_VECTORS : C_ELEMENTS;
+    // bf16 rows on 16-byte boundaries leave as tiles.
+    CUtensorMap tc = ta;
+    if (sizeof(CT) == 2 && c_vec && !beta && splits <= 1 && ((threads - 64) / 32 <= S::kStoreWarps || FUSE) && tc_operand_ok(C, ldc) &&
+        make_tmap_bf16_2d(&tc, C, Ndim, Mdim, ldc, 64, 32) == VELORA_OK)
+        c_vec = C_TILES;
     if (splits <= 1) {
         const int grid = static_cast<int>(tiles < di.sm_count ? tiles : di.sm_count);
         return launch_chained(kern, dim3(static_cast<unsigned>(grid)), threads, S::kSmem, stream,
-                              ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, kblocks, c_vec, status, fz);
+                              ta, tb, tc, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, kblocks, c_vec, status, fz);
     }
     const int kb_per_split = (kblocks + splits - 1) / splits;
     splits = (kblocks + kb_per_split - 1) / kb_per_split;             // no split without k-blocks
@@ -376,7 +392,7 @@ int launch_kernel(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, kb_per_split, c_vec,
+    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, static_cast<CT*>(C), ldc, beta, Mdim, Ndim, Kdim, tiles_m, tiles_n, kb_per_split, c_vec,
                            status, fz) != cudaSuccess) {
         cudaGetLastError();                                           // a refused cluster: the same tiles, one CTA each
         return launch_kernel<A_MN, B_MN, CT, FUSE, BN>(ta, tb, C, ldc, beta, Mdim, Ndim, Kdim, 1, status, stream, fz);
