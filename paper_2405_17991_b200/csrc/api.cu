@@ -143,7 +143,7 @@ int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t
         // Adapter-shaped layers (O <= 64; too few output tiles for the tensor-core kernel to spread), fp32 and bf16 rows
         // on odd boundaries first.
         int rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
-                                           beta, body, ws_bytes - kStatusBytes, stream, nullptr, 0);
+                                           beta, body, ws_bytes - kStatusBytes, status, stream, nullptr, 0);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;
         rc = launch_weight_grad_tc(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub,
                                        dW, dw_dtype, lddw, beta, body, ws_bytes - kStatusBytes, status, stream);
@@ -578,7 +578,7 @@ int velora_weight_grad_p(const void* dY, int dy_dtype, int64_t N, int64_t O, int
     char* body = static_cast<char*>(ws) + kStatusBytes;
     if (N > 0) {
         rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D,
-                                       beta, body, ws_bytes - kStatusBytes, st, P, ldp);
+                                       beta, body, ws_bytes - kStatusBytes, status, st, P, ldp);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;
     }
     rc = launch_weight_grad_tc(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D, beta,

@@ -39,6 +39,7 @@
 
 #include "gemm_store.cuh"
 #include "gemm_tc.cuh"
+#include "split_bf16.cuh"
 #include "tc_pair.cuh"
 
 namespace velora {
@@ -67,17 +68,6 @@ struct F32Operand {
     int64_t ld;                                    // pitch of the contiguous rows in memory
     int vec;                                       // whether they start on 16-byte boundaries
 };
-
-// x less the two bf16 numbers nearest to it: exact, the remainder has 16 significant bits the first time and 8 the second.
-__device__ __forceinline__ float2 minus_parts(float2 x, uint32_t parts)
-{
-    float2 r;
-    asm("{\n\t.reg .b64 x, h, n;\n\t"
-        "mov.b64 x, {%2, %3};\n\tmov.b64 h, {%4, %5};\n\tmov.b64 n, {%6, %6};\n\t"
-        "fma.rn.f32x2 x, h, n, x;\n\tmov.b64 {%0, %1}, x;\n\t}"
-        : "=f"(r.x), "=f"(r.y) : "f"(x.x), "f"(x.y), "f"(bf16_lo(parts)), "f"(bf16_hi(parts)), "f"(-1.f));
-    return r;
-}
 
 // Four elements of a row, of which `left` exist; zeros for the others.
 __device__ __forceinline__ float4 load4(const float* q, int left, int vec)
@@ -154,23 +144,6 @@ struct F32Shape {
     static constexpr size_t kSmem = 1024 + static_cast<size_t>(F_STAGES) * kStageBytes + F_BARRIER_BYTES +
                                     F_SUM_WARPS * 32 * F_STAGE_PITCH * sizeof(float);
 };
-
-// 32 lanes x 8 consecutive fp32 columns: few registers beside the sums.
-__device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-
-// True for an output that the split may have got wrong (see the head of this file); zero is right either way, since the products
-// that vanish then are below the smallest fp32 number.
-__device__ __forceinline__ bool suspect(float x)
-{
-    const float a = fabsf(x);
-    return !(a <= 3.402823466e+38f) || (a < 5.421010862e-20f && a != 0.f);
-}
 
 // Computes again those of a warp's 32 x 16 outputs that `bad` marks (bit c of a lane: its row, column n0 + c).
 template <bool A_MN, bool B_MN>
@@ -374,12 +347,12 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
                 if (m0 >= Mdim || valid <= 0) continue;      // the same for the whole warp
                 bool odd = false;
 #pragma unroll
-                for (int e = 0; e < 16; ++e) odd |= suspect(sum[c + e]);
+                for (int e = 0; e < 16; ++e) odd |= split_suspect(sum[c + e]);
                 uint32_t bad = 0;
                 if (odd && m0 + lane < Mdim) {
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
-                        if (e < valid && suspect(sum[c + e])) bad |= 1u << e;
+                        if (e < valid && split_suspect(sum[c + e])) bad |= 1u << e;
                 }
                 const bool again = __any_sync(0xffffffffu, bad != 0);
                 if (again || !c_vec) {

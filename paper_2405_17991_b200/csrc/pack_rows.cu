@@ -12,6 +12,7 @@
 // its chunk begins, takes the rest from its neighbour (whose chunk begins there) and shifts; only the last lane of the
 // last step loads a second time.
 #include "gemm_tc.cuh"
+#include "row_chunks.cuh"
 
 namespace velora {
 namespace {
@@ -29,35 +30,6 @@ struct PackArgs {
     int chunks[2], segs[2];
     int64_t items[2];                                      // rows x segments
 };
-
-// The aligned 16 bytes at `a`; bytes outside the matrix are not touched and read as zero.
-__device__ __forceinline__ uint4 load_aligned(const char* a, const char* lo_limit, const char* hi_limit)
-{
-    if (a >= lo_limit && a + 16 <= hi_limit) return ld_stream_if(a, true);
-    uint32_t o[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-        if (a + 2 * e >= lo_limit && a + 2 * e < hi_limit)
-            o[e >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(a + 2 * e)) << (16 * (e & 1));
-    return make_uint4(o[0], o[1], o[2], o[3]);
-}
-
-// Sixteen bytes from byte s (even) of the 32 in x, y.
-__device__ __forceinline__ uint4 shift_pair(const uint4& x, const uint4& y, uint32_t s)
-{
-    uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-    if (s & 8u) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
-    }
-    if (s & 4u) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
-    }
-    const uint32_t bits = (s & 2u) * 8u;
-    return make_uint4(__funnelshift_r(w[0], w[1], bits), __funnelshift_r(w[1], w[2], bits),
-                      __funnelshift_r(w[2], w[3], bits), __funnelshift_r(w[3], w[4], bits));
-}
 
 __global__ void __launch_bounds__(PK_THREADS)
 pack_rows_kernel(const PackArgs a)
@@ -78,9 +50,9 @@ pack_rows_kernel(const PackArgs a)
         uint4 d[PK_U], over = make_uint4(0u, 0u, 0u, 0u);     // chunks at or beyond the row's end are loaded, not used
 #pragma unroll
         for (int u = 0; u < PK_U; ++u)
-            d[u] = c0 - lane + 32 * u <= a.chunks[k] ? load_aligned(ap + 16 * static_cast<int64_t>(c0 + 32 * u), a.src[k], a.src_end[k])
+            d[u] = c0 - lane + 32 * u <= a.chunks[k] ? load_aligned_chunk(ap + 16 * static_cast<int64_t>(c0 + 32 * u), a.src[k], a.src_end[k])
                                                      : make_uint4(0u, 0u, 0u, 0u);
-        if (lane == 31) over = load_aligned(ap + 16 * static_cast<int64_t>(c0 + 32 * PK_U - 31), a.src[k], a.src_end[k]);
+        if (lane == 31) over = load_aligned_chunk(ap + 16 * static_cast<int64_t>(c0 + 32 * PK_U - 31), a.src[k], a.src_end[k]);
         over.x = __shfl_sync(0xffffffffu, over.x, 31); over.y = __shfl_sync(0xffffffffu, over.y, 31);
         over.z = __shfl_sync(0xffffffffu, over.z, 31); over.w = __shfl_sync(0xffffffffu, over.w, 31);
         uint4* op = a.dst[k] + static_cast<int64_t>(row) * a.dst_pitch[k];
@@ -93,7 +65,7 @@ pack_rows_kernel(const PackArgs a)
             uint4 y;
             y.x = __shfl_sync(0xffffffffu, give.x, from); y.y = __shfl_sync(0xffffffffu, give.y, from);
             y.z = __shfl_sync(0xffffffffu, give.z, from); y.w = __shfl_sync(0xffffffffu, give.w, from);
-            if (c0 + 32 * u < a.chunks[k]) op[c0 + 32 * u] = shift_pair(d[u], y, shift);
+            if (c0 + 32 * u < a.chunks[k]) op[c0 + 32 * u] = shift_chunks(d[u], y, shift);
         }
     }
 }

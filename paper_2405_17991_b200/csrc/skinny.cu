@@ -10,7 +10,7 @@
 // kernel writes dW.  All sums are fp32, products are formed from the stored values (Z is not rounded to bf16).
 // The same kernel, with the output columns in blocks of 64, serves fp32 layers of any width (12608 tokens, 768 columns, 24
 // sub-tokens: 904 us as a general fp32 product whose 12 output tiles left most SMs idle) and bf16 gradients whose
-// rows are not 16-byte aligned, with Z as stored.
+// rows are not 16-byte aligned, with Z as stored, where weight_grad_parts.cu does not form the partial sums of these.
 //
 //  2. the forward, Y = X W^T and Z = compress(X, v) in one pass over X (further down).
 #include "common.cuh"
@@ -109,100 +109,6 @@ wg_skinny_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
             const int o = o0 + warp * OI + i, m = lane + 32 * j;
             if (o < O && m < M) out[o * M + m] = acc[i][j];
         }
-}
-
-// The partial P of wide layers with up to 32 sub-tokens: 64 columns of dY (block blockIdx.y) by 4 MT sub-tokens.  Every warp
-// computes the whole tile for every eighth token, 8 x MT outputs a thread, and the warps' sums are added up in order at
-// the end: 2 + MT / 4 shared-memory loads feed 8 MT multiply-adds, where the mapping above spends three on eight.
-// Layer of 4096 x 2048 -> 5461 on odd rows, 16 sub-tokens: 240 us, 271 with the mapping above (P alone: 46 us); fp32 gradient of
-// 12608 x 768, 24 sub-tokens: 50 -> 36 us.  What holds it is the 2-byte loads: one chunk of them is in flight per CTA, and deeper
-// chunks or a third CTA per SM gained nothing.
-constexpr int SK_TILE_O = 64, SK_TILE_M = 32;
-
-template <typename YT, typename ZT, int MT>
-__global__ void __launch_bounds__(SK_THREADS, MT == 4 ? 3 : 2)
-wg_tile_partial_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz,
-                       int N, int O, int M, int tokens_per_cta, float* __restrict__ partials)
-{
-    constexpr int TM = 4 * MT;
-    __shared__ __align__(16) float sdy[2][SK_CHUNK][SK_TILE_O];
-    __shared__ __align__(16) float sz[2][SK_CHUNK][TM];
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int og = lane & 7, mg = lane >> 3;               // outputs o = 4 og + {0 .. 3}, + 32; m = 4 mg + {0 .. 3} (, + 16)
-    const int o0 = blockIdx.y * SK_TILE_O;
-    const int n_begin = blockIdx.x * tokens_per_cta;
-    const int n_end = (n_begin + tokens_per_cta < N) ? n_begin + tokens_per_cta : N;
-    float acc[8][MT];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < MT; ++j) acc[i][j] = 0.f;
-
-    constexpr int NY = SK_CHUNK * SK_TILE_O / SK_THREADS, NZ = SK_CHUNK * TM / SK_THREADS;
-    float ly[NY], lz[NZ];
-    // Element u of this thread: token t / 64 + 4 u, column t % 64 of dY; token t / TM + u 256 / TM, sub-token t % TM of Z.
-    const int yo = o0 + t % SK_TILE_O, zm = t % TM;
-    const YT* yp = dY + static_cast<int64_t>(n_begin + t / SK_TILE_O) * lddy + yo;
-    const ZT* zp = Z + static_cast<int64_t>(n_begin + t / TM) * ldz + zm;
-    auto fetch = [&](int left) {                              // of the slice's tokens, from where yp and zp stand
-#pragma unroll
-        for (int u = 0; u < NY; ++u, yp += SK_THREADS / SK_TILE_O * lddy)
-            ly[u] = (t / SK_TILE_O + u * (SK_THREADS / SK_TILE_O) < left && yo < O) ? Elem<YT>::load(yp) : 0.f;
-#pragma unroll
-        for (int u = 0; u < NZ; ++u, zp += SK_THREADS / TM * ldz)
-            lz[u] = (t / TM + u * (SK_THREADS / TM) < left && zm < M) ? Elem<ZT>::load(zp) : 0.f;
-    };
-    pdl_wait();
-    pdl_trigger();
-    fetch(n_end - n_begin);
-    int buf = 0;
-    for (int n0 = n_begin; n0 < n_end; n0 += SK_CHUNK, buf ^= 1) {
-#pragma unroll
-        for (int u = 0; u < NY; ++u) (&sdy[buf][0][0])[t + u * SK_THREADS] = ly[u];
-#pragma unroll
-        for (int u = 0; u < NZ; ++u) (&sz[buf][0][0])[t + u * SK_THREADS] = lz[u];
-        __syncthreads();
-        if (n0 + SK_CHUNK < n_end) fetch(n_end - n0 - SK_CHUNK);      // on its way while this chunk is multiplied
-#pragma unroll 2
-        for (int r = warp; r < SK_CHUNK; r += SK_THREADS / 32) {
-            float y[8], z[MT];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float4 q = *reinterpret_cast<const float4*>(&sdy[buf][r][32 * h + 4 * og]);
-                y[4 * h] = q.x; y[4 * h + 1] = q.y; y[4 * h + 2] = q.z; y[4 * h + 3] = q.w;
-            }
-#pragma unroll
-            for (int h = 0; h < MT / 4; ++h) {
-                const float4 q = *reinterpret_cast<const float4*>(&sz[buf][r][16 * h + 4 * mg]);
-                z[4 * h] = q.x; z[4 * h + 1] = q.y; z[4 * h + 2] = q.z; z[4 * h + 3] = q.w;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < MT; ++j) acc[i][j] = fmaf(y[i], z[j], acc[i][j]);
-        }
-    }
-    __syncthreads();
-    // The tile lies over sdy as [o][m]: 64 x TM floats.
-    float* red = &sdy[0][0][0];
-    static_assert(TM <= SK_CHUNK, "the tile fits in sdy");
-    for (int w = 0; w < SK_THREADS / 32; ++w) {
-        if (warp == w) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < MT; ++j) {
-                    float* p = red + (32 * (i / 4) + 4 * og + i % 4) * TM + 16 * (j / 4) + 4 * mg + j % 4;
-                    *p = w == 0 ? acc[i][j] : *p + acc[i][j];
-                }
-        }
-        __syncthreads();
-    }
-    float* out = partials + static_cast<int64_t>(blockIdx.x) * O * M;
-    for (int idx = t; idx < SK_TILE_O * TM; idx += SK_THREADS) {
-        const int o = o0 + idx / TM, m = idx % TM;
-        if (o < O && m < M) out[o * M + m] = red[idx];
-    }
 }
 
 // P[o*ldp + m] = beta * P + sum over the partials.  A block takes 32 consecutive elements; its eight warps
@@ -512,12 +418,12 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 }
 
 struct SkinnyPlan {
-    bool ok, tile;
+    bool ok, tensor;              // `tensor`: launch_wg_parts
     int M, oi, mj, o_blocks, tokens_per_cta, parts;
     size_t partial_bytes, p_bytes;
 };
 
-SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
+SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count, int dy_dtype)
 {
     SkinnyPlan p{};
     const int64_t M = ceil_div64(D, Dsub);
@@ -536,18 +442,20 @@ SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
         // workspace holds (that size is what velora_workspace_bytes has always reported for them).
         const int64_t bytes = static_cast<int64_t>(weight_grad_tc_workspace_bytes(N, D, O, Dsub)) - 512;   // two roundings to 256
         const int64_t room = bytes / static_cast<int64_t>(sizeof(float) * O * M) - 1;                       // and P itself
-        // Four CTAs per SM.  The tile kernel has three (up to 16 sub-tokens) or two, without a second wave, and takes slices of
-        // 256 tokens and more: adding up its eight warps costs several microseconds (45 tokens, 936 x 21: 12.4 us instead of 4.4).
+        // Four CTAs per SM.  Up to 32 sub-tokens go to the tensor cores (weight_grad_parts.cu), in one wave of slices of 192 tokens or more
+        // (three stages: filling and emptying such a CTA costs several microseconds), where that gives every other SM one.
         max_parts = ceil_div64(4 * static_cast<int64_t>(sm_count), p.o_blocks);
-        int64_t tile_parts = (M <= 16 ? 3 : 2) * static_cast<int64_t>(sm_count) / p.o_blocks;
-        if (tile_parts < 1) tile_parts = 1;
-        p.tile = M <= SK_TILE_M && N >= 256 * tile_parts;
-        if (p.tile) max_parts = tile_parts;
+        int64_t tc_parts = wg_parts_slices(dy_dtype, O, sm_count);
+        if (tc_parts > N / 192) tc_parts = N / 192;
+        if (tc_parts > room) tc_parts = room;
+        p.tensor = M <= 32 && tc_parts >= 1 && 2 * tc_parts * ceil_div64(O, 128) >= sm_count;
+        if (p.tensor) max_parts = tc_parts;
         if (max_parts > room) max_parts = room;
         if (max_parts < 1 || p.o_blocks > 65535) return p;
     }
     int64_t tpc = ceil_div64(N, max_parts);
-    tpc = ceil_div64(tpc, SK_CHUNK) * SK_CHUNK;
+    const int64_t chunk = p.tensor ? 64 : SK_CHUNK;
+    tpc = ceil_div64(tpc, chunk) * chunk;
     p.tokens_per_cta = static_cast<int>(tpc);
     p.parts = static_cast<int>(ceil_div64(N, tpc));
     p.partial_bytes = ((static_cast<size_t>(p.parts) * O * M * sizeof(float) + 255) / 256) * 256;
@@ -560,13 +468,6 @@ template <typename YT, typename ZT>
 int launch_partial(const SkinnyPlan& p, const void* dY, int64_t lddy, const void* Z, int64_t ldz, int N, int O,
                    float* partials, cudaStream_t stream)
 {
-    if (p.tile) {
-        const dim3 grid(p.parts, p.o_blocks);
-        return p.M <= 16 ? launch_chained(wg_tile_partial_kernel<YT, ZT, 4>, grid, SK_THREADS, 0, stream, static_cast<const YT*>(dY), lddy,
-                                          static_cast<const ZT*>(Z), ldz, N, O, p.M, p.tokens_per_cta, partials)
-                         : launch_chained(wg_tile_partial_kernel<YT, ZT, 8>, grid, SK_THREADS, 0, stream, static_cast<const YT*>(dY), lddy,
-                                          static_cast<const ZT*>(Z), ldz, N, O, p.M, p.tokens_per_cta, partials);
-    }
 #define VELORA_SK_CASE(OIV, MJV)                                                                                  \
     if (p.oi == OIV && p.mj == MJV) {                                                                             \
         return launch_chained(wg_skinny_partial_kernel<YT, ZT, OIV, MJV>, dim3(p.parts, p.o_blocks), SK_THREADS, 0, stream, \
@@ -584,7 +485,7 @@ int launch_partial(const SkinnyPlan& p, const void* dY, int64_t lddy, const void
 size_t weight_grad_skinny_workspace_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
 {
     if (O > SK_MAX_O) return 0;                          // planned into the tensor-core form's room
-    const SkinnyPlan p = skinny_plan(N > 0 ? N : 1, D, O, Dsub, 148);
+    const SkinnyPlan p = skinny_plan(N > 0 ? N : 1, D, O, Dsub, 148, VELORA_BF16);
     // The token range is always cut into at most 512 slices, whatever the device, so the size is fixed.
     return p.ok ? p.partial_bytes + p.p_bytes : 0;
 }
@@ -595,10 +496,10 @@ size_t weight_grad_skinny_workspace_bytes(int64_t N, int64_t D, int64_t O, int D
 int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
                               const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
                               void* dW, int dw_dtype, int64_t lddw, int beta,
-                              void* ws, size_t ws_bytes, cudaStream_t stream, float* P_out, int64_t ldp_out)
+                              void* ws, size_t ws_bytes, int* status, cudaStream_t stream, float* P_out, int64_t ldp_out)
 {
     if (O > SK_MAX_O && dy_dtype == VELORA_BF16 && tc_operand_ok(dY, lddy)) return VELORA_ERR_UNSUPPORTED;
-    const SkinnyPlan p = skinny_plan(N, D, O, Dsub, 148);
+    const SkinnyPlan p = skinny_plan(N, D, O, Dsub, 148, dy_dtype);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
     // One slice of a wide layer's factor is one small product; the general kernel makes it without a reduction behind it
     // (11 tokens, 1954 x 38: 4.7 us, 6.1 here).
@@ -608,7 +509,9 @@ int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O
     float* P = reinterpret_cast<float*>(static_cast<char*>(ws) + p.partial_bytes);
     const int n = static_cast<int>(N), o = static_cast<int>(O);
     int rc;
-    if (z_dtype == VELORA_FP8_E4M3)
+    if (p.tensor)
+        rc = launch_wg_parts(dY, dy_dtype, lddy, Z, z_dtype, ldz, n, o, p.M, p.tokens_per_cta, p.parts, partials, status, stream);
+    else if (z_dtype == VELORA_FP8_E4M3)
         rc = dy_dtype == VELORA_BF16 ? launch_partial<__nv_bfloat16, e4m3_t>(p, dY, lddy, Z, ldz, n, o, partials, stream)
                                      : launch_partial<float, e4m3_t>(p, dY, lddy, Z, ldz, n, o, partials, stream);
     else if (dy_dtype == VELORA_BF16)

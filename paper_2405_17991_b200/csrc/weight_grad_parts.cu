@@ -1,0 +1,371 @@
+// Partial factors P[o, m] = sum_n dY[n, o] * Z[n, m] of token slices on the tensor cores, to fp32 accuracy, for the gradients that
+// weight_grad_tc.cu does not take: fp32 rows, and bf16 rows on odd boundaries with Z as stored.
+//
+// An fp32 Z is split into three bf16 parts (exact, as in gemm_f32_tc.cu) that lie side by side as columns of one operand: 64
+// tokens of a bf16 dY are four tcgen05.mma of M = 128 columns of dY by N = 3 x round16(sub-tokens).  An fp32 dY has three parts as well, and
+// three times the products.  After every 64 tokens the accumulator is read out and added to fp32 sums, rounded to nearest (the
+// tensor cores' own sums truncate).
+//
+// A CTA takes 128 columns of dY and one slice of the tokens.  Roles (416 threads): warps 0..3 sums (a lane has a column of dY);
+// warps 4..11 operands (plain loads of any alignment, split, swizzled MN-major tiles: tokens are the contraction, rows of both
+// matrices are rows of the tiles); warp 12 issues.  Two stages and two accumulators, a barrier pair each:
+//   full[s] (eight operand warps), done[s] (commit: the stage may be written, the accumulator read), drained[s] (four warps).
+// Two CTAs share an SM (bf16); bound by the loads and stores of the operand warps.  Rows that start on odd boundaries are
+// read as the aligned 16 bytes that a chunk begins in and shifted against the neighbouring lane's.
+//
+// An infinity or NaN, a Z too large for bf16, or numbers so small that their parts vanish: outputs that come out not finite or below
+// 2^-64 are computed again by fp32 multiply-adds.
+#include "gemm_tc.cuh"
+#include "row_chunks.cuh"
+#include "split_bf16.cuh"
+#include "tc_common.cuh"
+
+namespace velora {
+
+using namespace tc;
+
+namespace {
+
+constexpr int WP_O = 128, WP_K = 64;
+constexpr int WP_SUM_WARPS = 4, WP_OPERAND_WARPS = 8;
+constexpr int WP_OPERAND_THREADS = 32 * WP_OPERAND_WARPS;
+constexpr int WP_THREADS = 32 * (WP_SUM_WARPS + WP_OPERAND_WARPS + 1);
+constexpr int WP_SLAB = WP_K * 128;                     // 64 columns of 64 tokens
+constexpr int WP_A_PART = 2 * WP_SLAB;
+
+template <typename YT, typename ZT, int MP>
+struct PartsShape {
+    static constexpr int kParts = sizeof(YT) == 2 ? 1 : 3;                      // of dY
+    static constexpr int kZParts = sizeof(ZT) == 4 ? 3 : 1;                     // a stored bf16 or E4M3 value is a bf16 number
+    static constexpr int kN = kZParts * MP;
+    static constexpr int kSlabsB = (kN + 63) / 64;
+    static constexpr int kStageBytes = kParts * WP_A_PART + kSlabsB * WP_SLAB;
+    static constexpr int kAccCols = kN <= 32 ? 32 : (kN <= 64 ? 64 : 128);
+    static constexpr size_t kSmem = 1024 + 2 * static_cast<size_t>(kStageBytes) + 128;
+    static constexpr int kCtasPerSm = kParts == 1 ? 2 : 1;
+    // Accumulators that share a stage's 64 tokens, as many as the 512 columns of an SM have room for: less truncation.
+    static constexpr int kSets = kAccCols * 8 * kCtasPerSm <= 512 ? 4 : (kAccCols * 4 * kCtasPerSm <= 512 ? 2 : 1);
+    static constexpr int kTmemCols = 2 * kSets * kAccCols;
+};
+
+// dY of a stage: 64 tokens x 128 columns, four passes of sixteen tokens; a thread has eight columns of every sixteenth token.
+template <typename YT> struct RowsOfY;
+
+template <> struct RowsOfY<__nv_bfloat16> {
+    uint4 x[4], over[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16* dY, int64_t ld, int n, int n_end, int o0, const char* end, int t)
+    {
+        const int l = t & 15;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = n + (t >> 4) + 16 * i;
+            const char* rp = reinterpret_cast<const char*>(dY + static_cast<int64_t>(row) * ld + o0);
+            const char* ap = rp - (reinterpret_cast<uintptr_t>(rp) & 15u) + 16 * l;
+            x[i] = over[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (row < n_end) {
+                x[i] = load_aligned_chunk(ap, reinterpret_cast<const char*>(dY), end);
+                if (l == 15) over[i] = load_aligned_chunk(ap + 16, reinterpret_cast<const char*>(dY), end);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t a0, const __nv_bfloat16* dY, int64_t ld, int n, int o0, int t)
+    {
+        const int r = t >> 4, l = t & 15;
+        const uint32_t at = a0 + (l >> 3) * WP_SLAB + r * 128 + (((l & 7) ^ (r & 7)) << 4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(dY + static_cast<int64_t>(n + r + 16 * i) * ld + o0) & 15u);
+            uint4 y;
+            y.x = __shfl_down_sync(0xffffffffu, x[i].x, 1, 16); y.y = __shfl_down_sync(0xffffffffu, x[i].y, 1, 16);
+            y.z = __shfl_down_sync(0xffffffffu, x[i].z, 1, 16); y.w = __shfl_down_sync(0xffffffffu, x[i].w, 1, 16);
+            const uint4 w = shift_chunks(x[i], l == 15 ? over[i] : y, shift);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + i * 16 * 128), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w) : "memory");
+        }
+    }
+};
+
+template <> struct RowsOfY<float> {
+    float4 x[8];                                       // eight tokens a pass: four columns of every eighth token
+    __device__ __forceinline__ void load(const float* dY, int64_t ld, int n, int n_end, int o0, const char* end, int t)
+    {
+        const int c = (t & 31) * 4;
+        const bool vec = (reinterpret_cast<uintptr_t>(dY) & 15u) == 0 && ld % 4 == 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = n + (t >> 5) + 8 * i;
+            const float* q = dY + static_cast<int64_t>(row) * ld + o0 + c;
+            const int64_t left = (end - reinterpret_cast<const char*>(q)) / 4;            // what follows in memory: columns beyond O feed nothing
+            x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row >= n_end) continue;
+            if (vec && left >= 4) {
+                x[i] = *reinterpret_cast<const float4*>(q);
+            } else {
+                if (left > 0) x[i].x = q[0];
+                if (left > 1) x[i].y = q[1];
+                if (left > 2) x[i].z = q[2];
+                if (left > 3) x[i].w = q[3];
+            }
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t a0, const float*, int64_t, int, int, int t)
+    {
+        const int r = t >> 5, c = (t & 31) * 4;
+        const uint32_t at = a0 + (c >> 6) * WP_SLAB + r * 128 + ((((c >> 3) & 7) ^ r) << 4) + (c & 4) * 2;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float2 a = make_float2(x[i].x, x[i].y), b = make_float2(x[i].z, x[i].w);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                const uint32_t u = pack_bf16x2(a.x, a.y), w = pack_bf16x2(b.x, b.y);
+                asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + i * 8 * 128 + p * WP_A_PART), "r"(u), "r"(w) : "memory");
+                if (p < 2) {
+                    a = minus_parts(a, u);
+                    b = minus_parts(b, w);
+                }
+            }
+        }
+    }
+};
+
+// Z of a stage: 64 tokens x MP sub-tokens (zeros beyond M and n_end), a thread has pairs of neighbours.
+template <typename ZT, int MP>
+struct RowsOfZ {
+    static constexpr int kPairs = WP_K * MP / 2 / WP_OPERAND_THREADS;
+    float2 x[kPairs];
+    __device__ __forceinline__ void load(const ZT* Z, int64_t ld, int n, int n_end, int M, int t)
+    {
+#pragma unroll
+        for (int i = 0; i < kPairs; ++i) {
+            const int idx = t + WP_OPERAND_THREADS * i, row = n + idx / (MP / 2), m = idx % (MP / 2) * 2;
+            const ZT* q = Z + static_cast<int64_t>(row) * ld + m;
+            x[i].x = row < n_end && m < M ? Elem<ZT>::load(q) : 0.f;
+            x[i].y = row < n_end && m + 1 < M ? Elem<ZT>::load(q + 1) : 0.f;
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t b0, int t)
+    {
+#pragma unroll
+        for (int i = 0; i < kPairs; ++i) {
+            const int idx = t + WP_OPERAND_THREADS * i, r = idx / (MP / 2), m = idx % (MP / 2) * 2;
+            float2 a = x[i];
+#pragma unroll
+            for (int p = 0; p < (sizeof(ZT) == 4 ? 3 : 1); ++p) {
+                const int c = p * MP + m;
+                const uint32_t u = pack_bf16x2(a.x, a.y);
+                asm volatile("st.shared.b32 [%0], %1;"
+                             ::"r"(b0 + (c >> 6) * WP_SLAB + r * 128 + ((((c >> 3) & 7) ^ (r & 7)) << 4) + (c & 7) * 2), "r"(u) : "memory");
+                if (p < 2 && sizeof(ZT) == 4) a = minus_parts(a, u);
+            }
+        }
+    }
+};
+
+template <typename YT, typename ZT, int MP>
+__global__ void __launch_bounds__(WP_THREADS, PartsShape<YT, ZT, MP>::kCtasPerSm)
+wg_parts_kernel(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz, int N, int O, int M, int tokens_per_cta,
+                float* __restrict__ partials, int* __restrict__ status)
+{
+    using S = PartsShape<YT, ZT, MP>;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* tail = smem_raw + (base - raw) + 2 * S::kStageBytes;
+    const uint32_t full = base + 2 * S::kStageBytes, done = full + 16, drained = full + 32;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 48);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 56);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int o0 = blockIdx.y * WP_O;
+    const int n_begin = blockIdx.x * tokens_per_cta;
+    const int n_end = n_begin + tokens_per_cta < N ? n_begin + tokens_per_cta : N;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(full + 8 * s, WP_OPERAND_WARPS);
+            mbar_init(done + 8 * s, 1);
+            mbar_init(drained + 8 * s, WP_SUM_WARPS);
+        }
+        *abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == WP_SUM_WARPS + WP_OPERAND_WARPS) {
+        tmem_alloc(smem_u32(tmem_slot), S::kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
+
+    bool failed = false;
+    if (warp == WP_SUM_WARPS + WP_OPERAND_WARPS) {
+        // ------------------------------------------------ products
+        if (lane == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16(WP_O, S::kN, true, true);
+            uint32_t it = 0;
+            for (int n = n_begin; n < n_end; n += WP_K, ++it) {
+                const uint32_t s = it & 1u, ph = (it >> 1) & 1u;
+                if (!mbar_wait(drained + 8 * s, ph ^ 1u, abort_flag) || !mbar_wait(full + 8 * s, ph, abort_flag)) { failed = true; break; }
+                tc_fence_after_sync();
+                const uint32_t a0 = base + s * S::kStageBytes, b0 = a0 + S::kParts * WP_A_PART;
+#pragma unroll
+                for (int p = S::kParts - 1; p >= 0; --p)              // the small parts first
+#pragma unroll
+                    for (int j = 0; j < WP_K / 16; ++j)
+                        umma_bf16(tmem_base + (s * S::kSets + j * S::kSets / 4) * S::kAccCols, umma_smem_desc(a0 + p * WP_A_PART + j * 2048, WP_SLAB, 1024),
+                                  umma_smem_desc(b0 + j * 2048, WP_SLAB, 1024), idesc, p != S::kParts - 1 || j % (4 / S::kSets) != 0);
+                umma_commit(done + 8 * s);
+            }
+            if (failed) *abort_flag = 1;
+        }
+    } else if (warp >= WP_SUM_WARPS) {
+        // ------------------------------------------------ operands
+        const int t = threadIdx.x - 32 * WP_SUM_WARPS;
+        const char* end = reinterpret_cast<const char*>(dY + static_cast<int64_t>(N - 1) * lddy + O);
+        RowsOfY<YT> y;
+        RowsOfZ<ZT, MP> z;
+        y.load(dY, lddy, n_begin, n_end, o0, end, t);
+        z.load(Z, ldz, n_begin, n_end, M, t);
+        uint32_t it = 0;
+        for (int n = n_begin; n < n_end; n += WP_K, ++it) {
+            const uint32_t s = it & 1u, ph = (it >> 1) & 1u;
+            if (!mbar_wait_warp(done + 8 * s, ph ^ 1u, abort_flag)) { failed = true; break; }
+            const uint32_t a0 = base + s * S::kStageBytes;
+            y.store(a0, dY, lddy, n, o0, t);
+            z.store(a0 + S::kParts * WP_A_PART, t);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full + 8 * s);
+            if (n + WP_K < n_end) {
+                y.load(dY, lddy, n + WP_K, n_end, o0, end, t);
+                z.load(Z, ldz, n + WP_K, n_end, M, t);
+            }
+        }
+        if (failed) *abort_flag = 1;
+    } else {
+        // ------------------------------------------------ sums: lane = column o of dY
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+        float sum[MP];
+#pragma unroll
+        for (int m = 0; m < MP; ++m) sum[m] = 0.f;
+        uint32_t it = 0;
+        for (int n = n_begin; n < n_end; n += WP_K, ++it) {
+            const uint32_t s = it & 1u, ph = (it >> 1) & 1u;
+            if (!mbar_wait_warp(done + 8 * s, ph, abort_flag, 32)) { failed = true; break; }
+            tc_fence_after_sync();
+#pragma unroll
+            for (int m = 0; m < MP; m += 8) {                        // a stage's accumulators and parts first, then one rounding of the sum
+                float stage_sum[8];
+#pragma unroll
+                for (int i = 0; i < S::kSets; ++i) {
+                    const uint32_t at = taddr + (s * S::kSets + i) * S::kAccCols + m;
+                    uint32_t h[8], mid[8] = {}, l[8] = {};
+                    tmem_ld_32x8(at, h);
+                    if (S::kZParts == 3) {
+                        tmem_ld_32x8(at + MP, mid);
+                        tmem_ld_32x8(at + 2 * MP, l);
+                    }
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        float f = __uint_as_float(h[e]);
+                        if (S::kZParts == 3) f += __uint_as_float(mid[e]) + __uint_as_float(l[e]);
+                        stage_sum[e] = i == 0 ? f : stage_sum[e] + f;
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) sum[m + e] += stage_sum[e];
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(drained + 8 * s);
+        }
+        const int o = o0 + warp * 32 + lane;
+        float* out = partials + (static_cast<int64_t>(blockIdx.x) * O + o) * M;
+        uint32_t bad = 0;
+#pragma unroll
+        for (int m = 0; m < MP; ++m) {
+            if (o < O && m < M) {
+                out[m] = sum[m];
+                if (split_suspect(sum[m])) bad |= 1u << m;
+            }
+        }
+        if (!failed)
+            for (uint32_t cols = __ballot_sync(0xffffffffu, bad != 0); cols; cols &= cols - 1) {
+                const int c = __ffs(cols) - 1;                       // the column of dY: this warp's lane c
+                const YT* yc = dY + o0 + warp * 32 + c;
+                int nan = 0;                                         // with a NaN in it all its outputs are NaN
+                for (int n = n_begin + lane; n < n_end; n += 32) {
+                    const float f = Elem<YT>::load(yc + static_cast<int64_t>(n) * lddy);
+                    nan |= f != f;
+                }
+                if (__any_sync(0xffffffffu, nan)) continue;
+                for (uint32_t ms = __shfl_sync(0xffffffffu, bad, c); ms; ms &= ms - 1) {
+                    const int m = __ffs(ms) - 1;
+                    float f = 0.f;
+                    for (int n = n_begin + lane; n < n_end; n += 32)
+                        f = fmaf(Elem<YT>::load(yc + static_cast<int64_t>(n) * lddy), Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m), f);
+                    for (int off = 16; off >= 1; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
+                    if (lane == c) out[m] = f;
+                }
+            }
+        if (failed) *abort_flag = 1;
+    }
+    if (failed && status) atomicExch(status, VELORA_ERR_TIMEOUT);
+
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (warp == WP_SUM_WARPS + WP_OPERAND_WARPS) {
+        __syncwarp();
+        tmem_dealloc(tmem_base, S::kTmemCols);
+    }
+}
+
+template <typename YT, typename ZT, int MP>
+int launch_shape(const void* dY, int64_t lddy, const void* Z, int64_t ldz, int N, int O, int M, int tokens_per_cta, int parts,
+                 float* partials, int* status, cudaStream_t stream)
+{
+    using S = PartsShape<YT, ZT, MP>;
+    static DeviceOnce configured;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return VELORA_ERR_CUDA;
+    auto kern = wg_parts_kernel<YT, ZT, MP>;
+    if (!configured.get(dev)) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::kSmem)) != cudaSuccess) return VELORA_ERR_CUDA;
+        configured.set(dev);
+    }
+    const dim3 grid(static_cast<unsigned>(parts), static_cast<unsigned>(ceil_div64(O, WP_O)));
+    kern<<<grid, WP_THREADS, S::kSmem, stream>>>(static_cast<const YT*>(dY), lddy, static_cast<const ZT*>(Z), ldz, N, O, M, tokens_per_cta,
+                                                 partials, status);
+    return after_launch();
+}
+
+template <typename YT, typename ZT>
+int launch_types(const void* dY, int64_t lddy, const void* Z, int64_t ldz, int N, int O, int M, int tokens_per_cta, int parts,
+                 float* partials, int* status, cudaStream_t stream)
+{
+    return M <= 16 ? launch_shape<YT, ZT, 16>(dY, lddy, Z, ldz, N, O, M, tokens_per_cta, parts, partials, status, stream)
+                   : launch_shape<YT, ZT, 32>(dY, lddy, Z, ldz, N, O, M, tokens_per_cta, parts, partials, status, stream);
+}
+
+}  // namespace
+
+int wg_parts_slices(int dy_dtype, int64_t O, int sm_count)
+{
+    const int64_t slices = static_cast<int64_t>(sm_count) * (dy_dtype == VELORA_BF16 ? 2 : 1) / ceil_div64(O, WP_O);
+    return slices < 1 ? 1 : static_cast<int>(slices);
+}
+
+int launch_wg_parts(const void* dY, int dy_dtype, int64_t lddy, const void* Z, int z_dtype, int64_t ldz, int N, int O, int M,
+                    int tokens_per_cta, int parts, float* partials, int* status, cudaStream_t stream)
+{
+#define VELORA_WP_CASE(YT)                                                                                                              \
+    if (z_dtype == VELORA_FP8_E4M3) return launch_types<YT, e4m3_t>(dY, lddy, Z, ldz, N, O, M, tokens_per_cta, parts, partials, status, stream); \
+    if (z_dtype == VELORA_BF16) return launch_types<YT, __nv_bfloat16>(dY, lddy, Z, ldz, N, O, M, tokens_per_cta, parts, partials, status, stream); \
+    return launch_types<YT, float>(dY, lddy, Z, ldz, N, O, M, tokens_per_cta, parts, partials, status, stream)
+    if (dy_dtype == VELORA_BF16) { VELORA_WP_CASE(__nv_bfloat16); }
+    VELORA_WP_CASE(float);
+#undef VELORA_WP_CASE
+}
+
+}  // namespace velora

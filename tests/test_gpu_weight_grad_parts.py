@@ -1,0 +1,68 @@
+"""The factor P = dY^T Z on the tensor cores to fp32 accuracy (fp32 dY, bf16 dY on odd rows): edges of slices, stages and tiles,
+every storage of Z, and values that the bf16 parts cannot carry.  Bound: fp32 sums of N terms as in ``test_gpu_fp32_products``."""
+import pytest
+import torch
+
+from _util import Guard, assert_matches
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def vl():
+    import paper_2405_17991_b200 as pkg
+    pkg.lib()
+    return pkg
+
+
+@pytest.fixture
+def guard():
+    g = Guard(DEV)
+    yield g
+    g.check()
+
+
+def _inputs(N, O, M, dtype, z, pad, offset, seed):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(seed)
+    dY = torch.full((offset + N * (O + pad),), float("nan"), device=DEV, dtype=dtype).as_strided((N, O), (O + pad, 1), offset)
+    dY.copy_(torch.randn((N, O), generator=gen, device=DEV))
+    return dY, torch.randn((N, M), generator=gen, device=DEV).to(z)
+
+
+# 16 sub-tokens and one column over a tile, the last slice one token; 17 and 32 sub-tokens; one token less than whole stages.
+@pytest.mark.parametrize("N,O,M", [(3009, 4993, 16), (3841, 1153, 17), (8191, 383, 32), (1600, 11001, 3)])
+@pytest.mark.parametrize("dtype,pad,offset", [(torch.bfloat16, 0, 0), (torch.bfloat16, 2, 3), (torch.float32, 0, 0), (torch.float32, 3, 0), (torch.float32, 7, 1)])
+@pytest.mark.parametrize("z", [torch.float32, torch.bfloat16, torch.float8_e4m3fn])
+def test_factor(vl, guard, N, O, M, dtype, pad, offset, z):
+    dY, Z = _inputs(N, O, M, dtype, z, pad, offset, N + M)
+    ws = guard.workspace(vl, vl.velora_workspace_bytes(vl.OP_WEIGHT_GRAD_FACTORED, N, 16 * M, O, 16))
+    ref = dY.double().T @ Z.double()
+    P0 = torch.randn((O, M), device=DEV)
+    for beta in (0, 1):
+        P = guard.mat(O, M, torch.float32, ld=M + 1, init=P0)
+        vl.velora_weight_grad_p(dY, Z, 16 * M, 16, P=P, beta=beta, ws=ws)
+        assert_matches(P, (ref + beta * P0.double()).cpu().numpy(), 1e-6, "P", c=3.84 * N * 2.0 ** -24)
+    assert vl.velora_workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_values_that_the_parts_cannot_carry(vl, guard, dtype):
+    N, O, M = 4000, 1301, 9
+    dY, Z = _inputs(N, O, M, dtype, torch.float32, 0, 0, 7)
+    dY[5, 3], dY[6, 700], dY[6, 1300], dY[7, 1300] = float("inf"), float("nan"), float("inf"), float("-inf")
+    dY[:, 10] = 0.0
+    dY[:, 11] *= 2.0 ** -118
+    Z[100, 2], Z[3999, 8] = float("-inf"), float("nan")
+    P = guard.mat(O, M, torch.float32)
+    vl.velora_weight_grad_p(dY, Z, 16 * M, 16, P=P)
+    y, z = dY.double(), Z.double()
+    ref = y.T @ z
+    assert torch.equal(P.isnan(), ref.isnan())
+    assert torch.equal(torch.where(P.isinf(), P, 0.0), torch.where(ref.isinf(), ref, 0.0).float())
+    fin = ref.isfinite()
+    scale = y.abs().nan_to_num(0, 0, 0).T @ z.abs().nan_to_num(0, 0, 0)
+    # N roundings of 2^-24 at most, and numbers below the smallest normal fp32 one to its last place
+    assert bool(((P.double() - ref).abs()[fin] <= (N * 2.0 ** -24 * scale + 2.0 ** -140)[fin]).all())
