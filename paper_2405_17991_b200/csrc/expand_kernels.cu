@@ -117,7 +117,7 @@ expand_rows_vec_kernel(const ST* S, int splits, int64_t split_stride, int lds,
             float p = 0.f;
             if (m < end) {
                 const ST* sp = row_s + m;
-#pragma unroll 4
+#pragma unroll 8
                 for (int s = 0; s < splits; ++s) p += load_scalar<ST>(sp + s * split_stride);   // fixed order
             }
             pb[b] = p;
