@@ -124,7 +124,8 @@ int pack_operands(Operand** ops, int count, void* ws, size_t ws_bytes, size_t us
 bool weight_grad_packs(int mode, int dw_dtype) { return mode == VELORA_WG_EXPLICIT && dw_dtype == VELORA_BF16; }
 
 // ---- weight gradient routing ----
-int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
+// `packed` (may be NULL): a packed copy of a bf16 dY that the call has made for another product.
+int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy, const void* packed, int64_t ld_packed,
                      const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
                      void* dW, int dw_dtype, int64_t lddw, int beta, int mode,
                      void* ws, size_t ws_bytes, cudaStream_t stream)
@@ -142,7 +143,7 @@ int weight_grad_impl(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t
         if (ws_bytes < factored_bytes(N, D, O, Dsub)) return VELORA_ERR_WORKSPACE;
         // Adapter-shaped layers (O <= 64; too few output tiles for the tensor-core kernel to spread), fp32 and bf16 rows
         // on odd boundaries first.
-        int rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
+        int rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, packed, ld_packed, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
                                            beta, body, ws_bytes - kStatusBytes, status, stream, nullptr, 0);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;
         rc = launch_weight_grad_tc(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, v, D, Dsub,
@@ -326,7 +327,7 @@ int velora_weight_grad(const void* dY, int dy_dtype, int64_t N, int64_t O, int64
         rc = pack_operands(ops, 1, ws, ws_bytes, need, static_cast<cudaStream_t>(stream));
         if (rc != VELORA_OK) return rc;
     }
-    return weight_grad_impl(y.p, dy_dtype, N, O, y.ld, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
+    return weight_grad_impl(y.p, dy_dtype, N, O, y.ld, nullptr, 0, Z, z_dtype, ldz, v, D, Dsub, dW, dw_dtype, lddw,
                             beta, mode, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }
 
@@ -408,7 +409,7 @@ int velora_linear_backward(const void* dY, int64_t lddy, const void* W, int64_t 
         if (rc != VELORA_OK) return rc;
     }
     if (dW)
-        return weight_grad_impl(pack_for_dw ? y.p : dY, dtype, N, O, pack_for_dw ? y.ld : lddy, Z, z_dtype, ldz, v, D, Dsub,
+        return weight_grad_impl(pack_for_dw ? y.p : dY, dtype, N, O, pack_for_dw ? y.ld : lddy, y.p != dY ? y.p : nullptr, y.ld, Z, z_dtype, ldz, v, D, Dsub,
                                 dW, dw_dtype, lddw, beta, mode, ws, ws_bytes, s);
     return VELORA_OK;
 }
@@ -577,7 +578,7 @@ int velora_weight_grad_p(const void* dY, int dy_dtype, int64_t N, int64_t O, int
     int* status = static_cast<int*>(ws);
     char* body = static_cast<char*>(ws) + kStatusBytes;
     if (N > 0) {
-        rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D,
+        rc = launch_weight_grad_skinny(dY, dy_dtype, N, O, lddy, nullptr, 0, Z, z_dtype, ldz, nullptr, D, Dsub, nullptr, VELORA_F32, D,
                                        beta, body, ws_bytes - kStatusBytes, status, st, P, ldp);
         if (rc != VELORA_ERR_UNSUPPORTED) return rc;
     }

@@ -116,14 +116,15 @@ int launch_init_v(const void* X, int x_dtype, int64_t N, int64_t D, int64_t ldx,
 int launch_normalize_v(const float* s, int Dsub, float* v, void* ws, size_t ws_bytes, cudaStream_t stream);
 // ---- adapter-shaped layers (skinny.cu) ----
 size_t weight_grad_skinny_workspace_bytes(int64_t N, int64_t D, int64_t O, int Dsub);
-int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
+int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy, const void* packed, int64_t ld_packed,
                               const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
                               void* dW, int dw_dtype, int64_t lddw, int beta,
                               void* ws, size_t ws_bytes, int* status, cudaStream_t stream, float* P_out, int64_t ldp_out);
-// Partial factors of `parts` token slices, partials[slice][O][M], M <= 32, any rows.  (weight_grad_parts.cu)
+// Partial factors of `parts` token slices, partials[slice][O][M], M <= 32, any rows.  `packed` (may be NULL): a copy of a bf16 dY
+// with rows that a tensor map can describe.  (weight_grad_parts.cu)
 int wg_parts_slices(int dy_dtype, int64_t O, int sm_count);          // slices that fill the chip once
-int launch_wg_parts(const void* dY, int dy_dtype, int64_t lddy, const void* Z, int z_dtype, int64_t ldz, int N, int O, int M,
-                    int tokens_per_cta, int parts, float* partials, int* status, cudaStream_t stream);
+int launch_wg_parts(const void* dY, int dy_dtype, int64_t lddy, const void* packed, int64_t ld_packed, const void* Z, int z_dtype, int64_t ldz,
+                    int N, int O, int M, int tokens_per_cta, int parts, float* partials, int* status, cudaStream_t stream);
 size_t init_v_workspace_bytes(int Dsub);
 // Scale of the 8-bit Z store from a batch: zscale = headroom * max|compress(X, v)| / 448 (1 if that maximum is
 // zero or not finite), v_store = v / zscale, v_load = v * zscale.  Asynchronous.

@@ -493,7 +493,7 @@ size_t weight_grad_skinny_workspace_bytes(int64_t N, int64_t D, int64_t O, int D
 // Returns VELORA_ERR_UNSUPPORTED (nothing launched) for more than 256 sub-tokens, and for bf16 gradients of more than 64
 // columns on 16-byte aligned rows (those have the tensor cores).
 // P_out != NULL: only the factor, P_out = beta * P_out + dY^T Z (dW, v unused).
-int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
+int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy, const void* packed, int64_t ld_packed,
                               const void* Z, int z_dtype, int64_t ldz, const float* v, int64_t D, int Dsub,
                               void* dW, int dw_dtype, int64_t lddw, int beta,
                               void* ws, size_t ws_bytes, int* status, cudaStream_t stream, float* P_out, int64_t ldp_out)
@@ -510,7 +510,7 @@ int launch_weight_grad_skinny(const void* dY, int dy_dtype, int64_t N, int64_t O
     const int n = static_cast<int>(N), o = static_cast<int>(O);
     int rc;
     if (p.tensor)
-        rc = launch_wg_parts(dY, dy_dtype, lddy, Z, z_dtype, ldz, n, o, p.M, p.tokens_per_cta, p.parts, partials, status, stream);
+        rc = launch_wg_parts(dY, dy_dtype, lddy, packed, ld_packed, Z, z_dtype, ldz, n, o, p.M, p.tokens_per_cta, p.parts, partials, status, stream);
     else if (z_dtype == VELORA_FP8_E4M3)
         rc = dy_dtype == VELORA_BF16 ? launch_partial<__nv_bfloat16, e4m3_t>(p, dY, lddy, Z, ldz, n, o, partials, stream)
                                      : launch_partial<float, e4m3_t>(p, dY, lddy, Z, ldz, n, o, partials, stream);
