@@ -15,6 +15,7 @@
 //  2. the forward, Y = X W^T and Z = compress(X, v) in one pass over X (further down).
 #include "common.cuh"
 #include "gemm_fuse.cuh"
+#include "gemm_store.cuh"
 #include "gemm_tc.cuh"
 #include "tc_common.cuh"
 
@@ -148,27 +149,26 @@ wg_skinny_reduce_kernel(const float* partials, int parts, int O, int M, float* _
 
 // ------------------------------------------------------------------ forward of an adapter-shaped layer
 // Y[N, O] = X W^T and Z = compress(X, v) for O <= 64 in ONE pass over X (Algorithm 1, forward).  The work is
-// one HBM read of X; the product runs on tcgen05 with the roles of the operands swapped so that tokens are
-// the N dimension of the MMA and 64-token tiles give every SM a CTA:
-//     D[o, t] (TMEM, 128 lanes x 64 columns) += W_tile[o, k] * X_tile[t, k]      (M = 128, N = 64, K = 16)
-// Only the first O lanes of the accumulator mean anything: the A descriptor spans 128 rows of shared memory
-// but only round_up(O, 8) rows are loaded; whatever lies behind them feeds lanes that are never read.
-// A stage holds 256 columns of the 64 tokens as four 8 KB tiles (64 rows x 128 bytes, 128-byte swizzle) plus
+// one HBM read of X; the product runs on tcgen05 with tiles of up to 64 tokens, so that every SM has one:
+//     D[t, o] (64 rows of TMEM) += X_tile[t, k] * W_tile[o, k]      (M = 64, N = round_up(O, 8), K = 16)
+// (with the operands' roles swapped, M = 128 rows of W of which O mean anything, the products held the stream up: 8192 x 4096,
+// rank 16, 23.2 us, now 20.6; 12608 x 768 16.6 and 12.1).
+// A stage holds 256 columns of the tokens as four tiles (of 64 rows x 128 bytes at most, 128-byte swizzle) plus
 // the four W tiles.  Where D is a multiple of 64 ONE three-dimensional TMA box (64 elements x 64 rows x 4
 // column chunks) brings the X tiles in, 512 contiguous bytes per token row: with one box per 128-byte-wide
-// tile the same pass ran at 2.5 TB/s however deep the ring was.  Warp 0 produces, warp 1 issues the MMAs, the
-// other sixteen warps compress: four sets of four warps take the stages in turn (a sub-token that spans
+// tile the same pass ran at 2.5 TB/s however deep the ring was.  Warp 0 produces, warp 1 issues the MMAs, the last warp
+// announces stages, the other sixteen compress: four sets of four warps take the stages in turn (a sub-token that spans
 // several stages stays with one set; spreading the four tiles of a stage over the sets instead was slower,
 // every set then waking for every stage).  Within a set a warp takes 16 of the 64 token rows; eight lanes per row
 // read the row's eight 16-byte chunks of a tile in one instruction, multiply with their slice of v and add up
 // over the lanes of a sub-token with shuffles.  They read the tiles in place and release the stage together
 // with the MMA's commit (the kernel waits on HBM, so a stage held a little longer costs nothing here).  Warps 4
-// and 5 finally read lanes 0..63 of the accumulator and store Y.
+// to 7 finally read the accumulator and store Y.
 constexpr int SF_TOKENS = 64, SF_BK = 64, SF_SB = 4, SF_MAX_STAGES = 6;
-constexpr int SF_X_BYTES = SF_TOKENS * SF_BK * 2;      // 8 KB: one tile
+constexpr int SF_ROW_BYTES = SF_BK * 2;
 constexpr int SF_RING_BYTES = 200 * 1024;
 constexpr int SF_SETS = 4;                             // compress warp sets (four warps each)
-constexpr int SF_THREADS = 64 + SF_SETS * 128;
+constexpr int SF_THREADS = 64 + SF_SETS * 128 + 32;     // producer, issuer, compress sets, herald
 constexpr int SF_BAR_BYTES = 1024;                     // barriers, TMEM slot, abort flag
 constexpr size_t SF_SMEM = 1024 + SF_RING_BYTES + 16384 /* A descriptor overhang */ + SF_BAR_BYTES + VELORA_MAX_DSUB * 4;
 
@@ -184,7 +184,7 @@ template <bool Z_BF16>
 __global__ void __launch_bounds__(SF_THREADS, 1)
 skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmX3,
                       const __grid_constant__ CUtensorMap tmW, int use3d,
-                      __nv_bfloat16* __restrict__ Y, int64_t ldy, int N, int O, int D, int w_rows, int stages,
+                      __nv_bfloat16* __restrict__ Y, int64_t ldy, int N, int O, int D, int tokens, int w_rows, int stages, int y_vec,
                       int* __restrict__ status, const FuseArgs fz)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -193,11 +193,12 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     uint8_t* smem = smem_raw + (base - raw);
     constexpr int TAIL_OFF = SF_RING_BYTES + 16384;
     const int w_tile = (w_rows * 128 + 1023) & ~1023;
-    const int stage_bytes = SF_SB * (SF_X_BYTES + w_tile);      // four X tiles, then four W tiles
+    const int x_bytes = tokens * SF_ROW_BYTES;                  // one tile: `tokens` rows, a multiple of 8 (the swizzle's period)
+    const int stage_bytes = SF_SB * (x_bytes + w_tile);         // four X tiles, then four W tiles
     uint8_t* tail = smem + TAIL_OFF;
     const uint32_t bars = base + TAIL_OFF;
     const uint32_t full = bars, empty = bars + 8 * SF_MAX_STAGES, tfull = bars + 16 * SF_MAX_STAGES;
-    // ready[set][s]: stage s holds landed tiles for compress set `set`.  Signalled by the MMA thread, which
+    // ready[set][s]: stage s holds landed tiles for compress set `set`.  Signalled by the herald warp, which
     // sees every phase of full[s] in order; a set that only looked at full[s] for its own stages would skip
     // phases and could not tell them apart by parity.
     const uint32_t ready = tfull + 8;
@@ -207,12 +208,13 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     float* sv = reinterpret_cast<float*>(tail + SF_BAR_BYTES);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = blockIdx.x * SF_TOKENS;
+    const int t0 = blockIdx.x * tokens;
+    const int t_end = t0 + tokens < N ? t0 + tokens : N;
     const int kblocks = (D + SF_BK - 1) / SF_BK;
     const int nsb = (kblocks + SF_SB - 1) / SF_SB;              // stages' worth of columns
     const int cw = fz.Dsub >= SF_BK ? fz.Dsub / SF_BK : 1;      // k-blocks per sub-token (a power of two)
     const int cwshift = 31 - __clz(cw);
-    const uint32_t stage_tx = static_cast<uint32_t>(SF_SB * (SF_X_BYTES + w_rows * 128));
+    const uint32_t stage_tx = static_cast<uint32_t>(SF_SB * (x_bytes + w_rows * 128));
     // The set that compresses stage-load sb: sub-tokens longer than a stage stay with one set.
     auto set_of = [&](int sb) { return (cw > SF_SB ? (sb * SF_SB) >> cwshift : sb) & (SF_SETS - 1); };
 
@@ -256,11 +258,11 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                 } else {
 #pragma unroll
                     for (int j = 0; j < SF_SB; ++j)
-                        tma_load_2d(dst + j * SF_X_BYTES, &tmX, full + 8 * s, (sb * SF_SB + j) * SF_BK, t0);
+                        tma_load_2d(dst + j * x_bytes, &tmX, full + 8 * s, (sb * SF_SB + j) * SF_BK, t0);
                 }
 #pragma unroll
                 for (int j = 0; j < SF_SB; ++j)
-                    tma_load_2d(dst + SF_SB * SF_X_BYTES + j * w_tile, &tmW, full + 8 * s, (sb * SF_SB + j) * SF_BK, 0);
+                    tma_load_2d(dst + SF_SB * x_bytes + j * w_tile, &tmW, full + 8 * s, (sb * SF_SB + j) * SF_BK, 0);
                 if (++s == static_cast<uint32_t>(stages)) { s = 0; ph ^= 1u; }
             }
             if (failed) {
@@ -276,29 +278,39 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, SF_TOKENS, false, false);
+            const uint32_t idesc = umma_idesc_bf16(SF_TOKENS, w_rows, false, false);
             uint32_t s = 0, ph = 0;
             for (int sb = 0; sb < nsb; ++sb) {
                 if (!mbar_wait(full + 8 * s, ph, abort_flag)) { failed = true; break; }
-                // Relaxed: a release in this thread would wait for the MMAs in flight.  The compress warps
-                // take their acquire from full[s] itself.
-                asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];"
-                             ::"r"(ready + 8 * (set_of(sb) * SF_MAX_STAGES + s)) : "memory");
                 tc_fence_after_sync();
-                const uint32_t x0 = base + s * stage_bytes, w0 = x0 + SF_SB * SF_X_BYTES;
+                const uint32_t x0 = base + s * stage_bytes, w0 = x0 + SF_SB * x_bytes;
 #pragma unroll
                 for (int j = 0; j < SF_SB; ++j) {
                     if (sb * SF_SB + j >= kblocks) break;            // nothing but zero fill beyond D
 #pragma unroll
                     for (int k = 0; k < SF_BK / 16; ++k)
-                        umma_bf16(tmem_base, umma_smem_desc(w0 + j * w_tile + k * 32, 16, 1024),
-                                  umma_smem_desc(x0 + j * SF_X_BYTES + k * 32, 16, 1024), idesc, (sb | j | k) != 0);
+                        umma_bf16(tmem_base, umma_smem_desc(x0 + j * x_bytes + k * 32, 16, 1024),
+                                  umma_smem_desc(w0 + j * w_tile + k * 32, 16, 1024), idesc, (sb | j | k) != 0);
                 }
                 umma_commit(empty + 8 * s);
                 if (++s == static_cast<uint32_t>(stages)) { s = 0; ph ^= 1u; }
             }
             if (!failed) umma_commit(tfull);
             else *abort_flag = 1;
+        }
+    } else if (warp == SF_THREADS / 32 - 1) {
+        // ---- herald: tells a stage's set that its tiles have landed.  The issuer did this once, and the sets waited for its products
+        // (the sets cannot watch full[s] themselves: they meet a stage in some of its phases only).
+        if (lane == 0) {
+            uint32_t s = 0, ph = 0;
+            for (int sb = 0; sb < nsb; ++sb) {
+                if (!mbar_wait(full + 8 * s, ph, abort_flag)) { failed = true; break; }
+                // Relaxed: the compress warps take their acquire from full[s] itself.
+                asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];"
+                             ::"r"(ready + 8 * (set_of(sb) * SF_MAX_STAGES + s)) : "memory");
+                if (++s == static_cast<uint32_t>(stages)) { s = 0; ph ^= 1u; }
+            }
+            if (failed) *abort_flag = 1;
         }
     } else {
         // ---- compress: warp cwp of a set takes tile rows 16 cwp .. 16 cwp + 15, four at a time, eight lanes per row
@@ -332,7 +344,7 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     const int r = 16 * cwp + 4 * i + sub;
                     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(d[i].x), "=r"(d[i].y), "=r"(d[i].z), "=r"(d[i].w)
-                                 : "r"(x0 + j * SF_X_BYTES + r * 128 + (static_cast<uint32_t>(c ^ (r & 7)) << 4)));
+                                 : "r"(x0 + j * x_bytes + r * 128 + (static_cast<uint32_t>(c ^ (r & 7)) << 4)));
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -371,7 +383,7 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const int row = t0 + 16 * cwp + 4 * i + sub;
-                        if (row < N) {
+                        if (row < t_end) {
                             if (Z_BF16) static_cast<__nv_bfloat16*>(fz.Z)[static_cast<int64_t>(row) * fz.ldz + m] = __float2bfloat16_rn(zval[j][i]);
                             else static_cast<float*>(fz.Z)[static_cast<int64_t>(row) * fz.ldz + m] = zval[j][i];
                         }
@@ -381,25 +393,28 @@ skinny_forward_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             if (++s == static_cast<uint32_t>(stages)) { s = 0; ph ^= 1u; }
         }
         if (failed) *abort_flag = 1;
-        // ---- epilogue: warps 4 and 5 own TMEM lanes 0..31 and 32..63 (= output columns o)
-        if (!failed && warp >= 4 && warp <= 5 && (warp - 4) * 32 < O) {
+        // ---- epilogue: row r of a product of 64 rows is in TMEM lane 32 (r / 16) + r % 16; warps 4 .. 7 have a quarter each
+        if (!failed && warp >= 4 && warp <= 7) {
             if (!mbar_wait_warp(tfull, 0u, abort_flag, 64)) {
                 failed = true;
                 *abort_flag = 1;
             } else {
                 tc_fence_after_sync();
-                const int o = (warp - 4) * 32 + lane;
-                const uint32_t taddr = tmem_base + (static_cast<uint32_t>((warp - 4) * 32) << 16);
+                const int quarter = warp & 3, t = t0 + quarter * 16 + lane;
+                const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+                __nv_bfloat16* row = Y + static_cast<int64_t>(t) * ldy;
 #pragma unroll 1
-                for (int cc = 0; cc < SF_TOKENS / 32; ++cc) {
+                for (int o = 0; o < O; o += 32) {
                     uint32_t r[32];
-                    tmem_ld_32x32(taddr + cc * 32, r);
+                    tmem_ld_32x32(taddr + o, r);
                     tmem_ld_wait();
-                    if (o < O) {
+                    if (lane < 16 && t < t_end) {
+                        if (y_vec) {
+                            Store32<__nv_bfloat16>::run(row + o, r, O - o, 0);
+                        } else {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const int t = t0 + cc * 32 + i;
-                            if (t < N) Y[static_cast<int64_t>(t) * ldy + o] = __float2bfloat16_rn(__uint_as_float(r[i]));
+                            for (int i = 0; i < 32; ++i)
+                                if (o + i < O) row[o + i] = __float2bfloat16_rn(__uint_as_float(r[i]));
                         }
                     }
                 }
@@ -550,15 +565,27 @@ int launch_linear_forward_skinny(const void* X, int64_t ldx, const void* W, int6
     if (static_cast<size_t>(di.smem_optin) < SF_SMEM) return VELORA_ERR_UNSUPPORTED;
     const int w_rows = static_cast<int>((O + 7) / 8 * 8);
     const int w_tile = (w_rows * 128 + 1023) & ~1023;
-    int stages = SF_RING_BYTES / (SF_SB * (SF_X_BYTES + w_tile));
+    // Tokens per CTA: as many as leave the fewest rows to stream one after the other, since one CTA fits an SM and a row costs the
+    // same in any of them (8192 tokens: 147 CTAs of 56 instead of 128 of 64; 1024: 64 of 16 instead of 16 of 64); eight rows stand
+    // for what a CTA costs besides.
+    int tokens = SF_TOKENS;
+    int64_t least = INT64_MAX;
+    for (int t = SF_TOKENS; t >= 16; t -= 8) {
+        const int64_t cost = ceil_div64(ceil_div64(N, t), di.sm_count) * (t + 8);
+        if (cost < least) {
+            least = cost;
+            tokens = t;
+        }
+    }
+    int stages = SF_RING_BYTES / (SF_SB * (tokens * SF_ROW_BYTES + w_tile));
     if (stages > SF_MAX_STAGES) stages = SF_MAX_STAGES;
     CUtensorMap tx, tx3, tw;
-    rc = make_tmap_bf16_2d(&tx, X, D, N, ldx, SF_BK, SF_TOKENS);
+    rc = make_tmap_bf16_2d(&tx, X, D, N, ldx, SF_BK, tokens);
     if (rc != VELORA_OK) return rc;
     rc = make_tmap_bf16_2d(&tw, W, D, O, ldw, SF_BK, w_rows);
     if (rc != VELORA_OK) return rc;
     // One box for four 64-column tiles needs whole 64-column chunks; otherwise four two-dimensional boxes.
-    int use3d = (D % SF_BK == 0 && make_tmap_bf16_chunks3d(&tx3, X, D, N, ldx, SF_TOKENS, SF_SB) == VELORA_OK) ? 1 : 0;
+    int use3d = (D % SF_BK == 0 && make_tmap_bf16_chunks3d(&tx3, X, D, N, ldx, tokens, SF_SB) == VELORA_OK) ? 1 : 0;
     if (!use3d) tx3 = tx;
     static DeviceOnce configured;
     int dev = 0;
@@ -570,14 +597,15 @@ int launch_linear_forward_skinny(const void* X, int64_t ldx, const void* W, int6
         configured.set(dev);
     }
     FuseArgs fz{v, Z, ldz, Dsub, static_cast<int>(ceil_div64(D, Dsub))};
-    const int grid = static_cast<int>(ceil_div64(N, SF_TOKENS));
+    const int y_vec = c_rows_vec(Y, ldy, sizeof(__nv_bfloat16)) ? 1 : 0;
+    const int grid = static_cast<int>(ceil_div64(N, tokens));
     if (z_dtype == VELORA_BF16)
         return launch_chained(skinny_forward_kernel<true>, dim3(grid), SF_THREADS, SF_SMEM, stream,
-            tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D),
-            w_rows, stages, status, fz);
+            tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D), tokens,
+            w_rows, stages, y_vec, status, fz);
     return launch_chained(skinny_forward_kernel<false>, dim3(grid), SF_THREADS, SF_SMEM, stream,
-            tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D),
-            w_rows, stages, status, fz);
+            tx, tx3, tw, use3d, static_cast<__nv_bfloat16*>(Y), ldy, static_cast<int>(N), static_cast<int>(O), static_cast<int>(D), tokens,
+            w_rows, stages, y_vec, status, fz);
 }
 
 }  // namespace velora
