@@ -118,9 +118,10 @@ int pack_operands(Operand** ops, int count, void* ws, size_t ws_bytes, size_t us
     return VELORA_OK;
 }
 
-// Whether the weight gradient runs on a packed copy of dY: the dense product with a bf16 result only.  The factored form
-// keeps such rows on the CUDA cores: its tensor-core kernel rounds an fp32 Z to bf16 (error of P at 4096 tokens: 2e-3
-// instead of 2e-7) and adds up with truncation, as the tensor cores do (P from a bf16 Z of 12608 tokens: 3.4e-6 instead of 2e-7).
+// Whether the weight gradient runs on a packed copy of dY instead of dY: the dense product with a bf16 result only.  The factored form
+// keeps Z as stored and its fp32 sums for such rows (it takes a packed copy that is there anyway as another source of the same
+// numbers): the kernel for aligned rows rounds an fp32 Z to bf16 (error of P at 4096 tokens: 2e-3 instead of 1e-7) and adds
+// up with truncation, as the tensor cores do (P from a bf16 Z of 12608 tokens: 3.4e-6 instead of 1e-7).
 bool weight_grad_packs(int mode, int dw_dtype) { return mode == VELORA_WG_EXPLICIT && dw_dtype == VELORA_BF16; }
 
 // ---- weight gradient routing ----
