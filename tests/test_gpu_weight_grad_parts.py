@@ -66,3 +66,17 @@ def test_values_that_the_parts_cannot_carry(vl, guard, dtype):
     scale = y.abs().nan_to_num(0, 0, 0).T @ z.abs().nan_to_num(0, 0, 0)
     # N roundings of 2^-24 at most, and numbers below the smallest normal fp32 one to its last place
     assert bool(((P.double() - ref).abs()[fin] <= (N * 2.0 ** -24 * scale + 2.0 ** -140)[fin]).all())
+
+
+# One sub-token block of 16 columns of Z and one of 32; the last slice ragged.
+@pytest.mark.parametrize("N,D,O,Dsub", [(4001, 1024, 3003, 64), (2200, 2048, 9001, 64)])
+def test_packed_copy_gives_the_same_bits(vl, N, D, O, Dsub):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(N)
+    dY, Z = _inputs(N, O, D // Dsub, torch.bfloat16, torch.float32, 0, 0, N)
+    W = torch.randn((O, D), generator=gen, device=DEV).bfloat16()
+    v = torch.randn(Dsub, generator=gen, device=DEV)
+    _, dW = vl.velora_linear_backward(dY, W, Z, v)                      # packs dY for dX
+    alone = vl.velora_weight_grad(dY, Z, v, D, ws=vl.velora_workspace_alloc(
+        vl.velora_workspace_bytes(vl.OP_WEIGHT_GRAD_FACTORED, N, D, O, Dsub), DEV))
+    assert torch.equal(dW, alone)
