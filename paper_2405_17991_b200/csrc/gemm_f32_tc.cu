@@ -31,8 +31,10 @@
 //
 // Numbers that the split cannot carry.  An infinity, a NaN or a number that rounds to infinity in bf16 has no finite h or m, so
 // every output it enters comes out not finite; below 2^-110 the last bits of l are lost (at most 2^-134 of absolute value), which
-// shows only where an output is tiny altogether.  Outputs that are not finite or below 2^-64 are therefore computed again
-// by fp32 multiply-adds (a warp per output) before they are written.
+// shows only where an output is tiny altogether.  A warp whose 32 x BN / 3 outputs hold one that is not finite or below 2^-64 leaves
+// them unwritten and marks them.  Marked outputs are computed by fp32 multiply-adds behind the last tile, when no role waits for another any
+// more (computed in between they kept the pair's other roles waiting, for longer than those do when a contraction is long), at the
+// rate of the CUDA-core product.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -141,31 +143,102 @@ struct F32Shape {
     using TileB = SplitTile<B_MN, BN / 2>;
     static constexpr int kStageBytes = 3 * (TileA::kPartBytes + TileB::kPartBytes);
     static constexpr int kAccCols = BN > 128 ? 256 : 128;             // TMEM columns from one accumulator to the next
+    static constexpr int kMaxTiles = BN > 128 ? 2048 : 1024;          // of a pair in one launch, one word of marks each
     static constexpr size_t kSmem = 1024 + static_cast<size_t>(F_STAGES) * kStageBytes + F_BARRIER_BYTES +
-                                    F_SUM_WARPS * 32 * F_STAGE_PITCH * sizeof(float);
+                                    F_SUM_WARPS * 32 * F_STAGE_PITCH * sizeof(float) + kMaxTiles * sizeof(uint32_t);
 };
 
-// Computes again those of a warp's 32 x 16 outputs that `bad` marks (bit c of a lane: its row, column n0 + c).
-template <bool A_MN, bool B_MN>
-__device__ __noinline__ void recompute(const F32Operand A, const F32Operand B, int m0, int n0, int Kdim, uint32_t bad, float* stage, int lane)
+__device__ __forceinline__ void sum_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * F_SUM_WARPS) : "memory"); }
+// The same; true in all of them if `p` is in one.
+__device__ __forceinline__ bool sum_warps_any(bool p)
 {
-    const int64_t a_sm = A_MN ? 1 : A.ld, a_sk = A_MN ? A.ld : 1, b_sn = B_MN ? 1 : B.ld, b_sk = B_MN ? B.ld : 1;
-    for (uint32_t rows = __ballot_sync(0xffffffffu, bad != 0); rows; rows &= rows - 1) {
-        const int r = __ffs(rows) - 1;
-        const float* a = A.p + static_cast<int64_t>(m0 + r) * a_sm;
-        int nan = 0;                                        // a row with a NaN in it has nothing but NaN outputs
-        for (int k = lane; k < Kdim; k += 32) nan |= a[k * a_sk] != a[k * a_sk];
-        if (__any_sync(0xffffffffu, nan)) continue;
-        for (uint32_t cols = __shfl_sync(0xffffffffu, bad, r); cols; cols &= cols - 1) {
-            const int c = __ffs(cols) - 1;
-            const float* b = B.p + static_cast<int64_t>(n0 + c) * b_sn;
-            float s = 0.f;
-            for (int k = lane; k < Kdim; k += 32) s = fmaf(a[k * a_sk], b[k * b_sk], s);
-            for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (lane == 0) stage[r * F_STAGE_PITCH + c] = s;
-        }
+    uint32_t any;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(any) : "r"(static_cast<uint32_t>(p)), "n"(32 * F_SUM_WARPS) : "memory");
+    return any != 0;
+}
+
+// Four bytes to shared memory, zero where `take` is false.
+__device__ __forceinline__ void copy4_async(uint32_t dst, const float* src, bool take)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(take ? 4 : 0) : "memory");
+}
+
+// The marked outputs of a CTA's 128 x BN (bit w: those of sum warp w) by fp32 multiply-adds, all sum warps: blocks of 96 columns, 8 x 4
+// outputs a thread, slices of 32 through the ring's memory, the next one on its way while one is multiplied.
+constexpr int F_REDO_COLS = 96, F_REDO_K = 32, F_REDO_PITCH_A = F_BM + 4, F_REDO_PITCH_B = F_REDO_COLS + 4;
+constexpr int F_REDO_SLICE = F_REDO_K * (F_REDO_PITCH_A + F_REDO_PITCH_B);          // floats
+
+template <bool A_MN, bool B_MN>
+__device__ __forceinline__ void redo_load(const F32Operand& A, const F32Operand& B, int m0, int n0, int k0, int Mdim, int Ndim, int Kdim,
+                                          uint32_t slice, int t)
+{
+#pragma unroll 4
+    for (int i = t; i < F_BM * F_REDO_K; i += 32 * F_SUM_WARPS) {
+        const int r = A_MN ? i % F_BM : i / F_REDO_K, k = A_MN ? i / F_BM : i % F_REDO_K, m = m0 + r;
+        const bool in = m < Mdim && k0 + k < Kdim;
+        const float* q = A.p + (A_MN ? static_cast<int64_t>(k0 + k) * A.ld + m : static_cast<int64_t>(m) * A.ld + (k0 + k));
+        copy4_async(slice + (k * F_REDO_PITCH_A + r) * 4, in ? q : A.p, in);
     }
-    __syncwarp();
+#pragma unroll 4
+    for (int i = t; i < F_REDO_COLS * F_REDO_K; i += 32 * F_SUM_WARPS) {
+        const int c = B_MN ? i % F_REDO_COLS : i / F_REDO_K, k = B_MN ? i / F_REDO_COLS : i % F_REDO_K, n = n0 + c;
+        const bool in = n < Ndim && k0 + k < Kdim;
+        const float* q = B.p + (B_MN ? static_cast<int64_t>(k0 + k) * B.ld + n : static_cast<int64_t>(n) * B.ld + (k0 + k));
+        copy4_async(slice + (F_REDO_K * F_REDO_PITCH_A + k * F_REDO_PITCH_B + c) * 4, in ? q : B.p, in);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <bool A_MN, bool B_MN, int BN>
+__device__ __noinline__ void redo_tile(const F32Operand A, const F32Operand B, float* C, int64_t ldc, int beta, int m0, int n0,
+                                       int Mdim, int Ndim, int Kdim, uint32_t marked, float* ring)
+{
+    static_assert(F_SUM_WARPS * 32 == F_BM / 8 * (F_REDO_COLS / 4) && BN % F_REDO_COLS == 0, "one block at a time");
+    const int t = threadIdx.x, tr = t / (F_REDO_COLS / 4) * 8, tc = t % (F_REDO_COLS / 4) * 4;
+    for (int u0 = 0; u0 < BN && n0 + u0 < Ndim; u0 += F_REDO_COLS) {
+        // Eight rows of a thread are within a warp's 32, four columns within its third.
+        const bool mine = (marked >> ((u0 + tc) / (BN / 3) * 4 + tr / 32)) & 1u, work = __any_sync(0xffffffffu, mine);
+        float acc[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        sum_warps_sync();                                   // the last block's slices have been read
+        redo_load<A_MN, B_MN>(A, B, m0, n0 + u0, 0, Mdim, Ndim, Kdim, smem_u32(ring), t);
+        int odd = 0;
+        for (int k0 = 0; k0 < Kdim; k0 += F_REDO_K, odd ^= 1) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            sum_warps_sync();                               // this slice is there, the one before it has been read
+            if (k0 + F_REDO_K < Kdim)
+                redo_load<A_MN, B_MN>(A, B, m0, n0 + u0, k0 + F_REDO_K, Mdim, Ndim, Kdim, smem_u32(ring + (odd ^ 1) * F_REDO_SLICE), t);
+            if (!work) continue;
+            const float* sA = ring + odd * F_REDO_SLICE + tr;
+            const float* sB = ring + odd * F_REDO_SLICE + F_REDO_K * F_REDO_PITCH_A + tc;
+#pragma unroll 4
+            for (int k = 0; k < F_REDO_K; ++k) {
+                const float4 a0 = *reinterpret_cast<const float4*>(sA + k * F_REDO_PITCH_A), a1 = *reinterpret_cast<const float4*>(sA + k * F_REDO_PITCH_A + 4);
+                const float4 b = *reinterpret_cast<const float4*>(sB + k * F_REDO_PITCH_B);
+                const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    acc[i][0] = fmaf(a[i], b.x, acc[i][0]);
+                    acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
+                    acc[i][2] = fmaf(a[i], b.z, acc[i][2]);
+                    acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (mine && m0 + tr + i < Mdim && n0 + u0 + tc + j < Ndim) {
+                    float* p = C + static_cast<int64_t>(m0 + tr + i) * ldc + (n0 + u0 + tc + j);
+                    *p = beta ? acc[i][j] + *p : acc[i][j];
+                }
+        __syncwarp();
+    }
 }
 
 // One k-block: six products of four steps each, the small ones first (l h', h l', m m', m h', h m', h h').
@@ -212,6 +285,7 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
     const uint32_t full = base + F_STAGES * S::kStageBytes, done = full + 16, drained = full + 32;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 48);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 56);
+    uint32_t* marks = reinterpret_cast<uint32_t*>(tail + F_BARRIER_BYTES + F_SUM_WARPS * 32 * F_STAGE_PITCH * sizeof(float));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int num_tiles = tiles_m * tiles_n;
@@ -226,6 +300,7 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
         *abort_flag = 0;
         fence_mbar_init();
     }
+    for (int i = threadIdx.x; pair + i * num_pairs < num_tiles; i += F_THREADS) marks[i] = 0;
     if (warp == F_SUM_WARPS + F_OPERAND_WARPS) {
         tmem_alloc_pair(smem_u32(tmem_slot), 2 * S::kAccCols);
         tmem_relinquish_pair();
@@ -317,7 +392,8 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
         float* stage = reinterpret_cast<float*>(tail + F_BARRIER_BYTES) + warp * 32 * F_STAGE_PITCH;
         const uint32_t taddr = tmem_base + third * COLS + (static_cast<uint32_t>(quarter * 32) << 16);
         uint32_t it = 0;
-        for (int tile = pair; tile < num_tiles && !failed; tile += num_pairs) {
+        uint32_t* mark = marks;
+        for (int tile = pair; tile < num_tiles && !failed; tile += num_pairs, ++mark) {
             float sum[COLS];
 #pragma unroll
             for (int c = 0; c < COLS; ++c) sum[c] = 0.f;
@@ -340,26 +416,30 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
             if (failed) break;
             const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * F_BM, BN);
             const int m0 = t0.m0 + rank * F_BM + quarter * 32, n0 = t0.n0 + third * COLS;
+            SplitCheck check;
+#pragma unroll
+            for (int c = 0; c < COLS; ++c) check.add(sum[c]);
+            bool odd = check.suspect() && m0 + lane < Mdim;
+            if (odd && n0 + COLS > Ndim) {                   // columns beyond the matrix do not count
+                check = SplitCheck();
+#pragma unroll
+                for (int c = 0; c < COLS; ++c)
+                    if (n0 + c < Ndim) check.add(sum[c]);
+                odd = check.suspect();
+            }
+            if (__any_sync(0xffffffffu, odd)) {
+                if (lane == 0) atomicOr(mark, 1u << warp);
+                continue;
+            }
             float* crow = C + static_cast<int64_t>(m0 + lane) * ldc + n0;
 #pragma unroll
             for (int c = 0; c < COLS; c += 16) {
                 const int valid = Ndim - (n0 + c);
                 if (m0 >= Mdim || valid <= 0) continue;      // the same for the whole warp
-                bool odd = false;
-#pragma unroll
-                for (int e = 0; e < 16; ++e) odd |= split_suspect(sum[c + e]);
-                uint32_t bad = 0;
-                if (odd && m0 + lane < Mdim) {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (e < valid && split_suspect(sum[c + e])) bad |= 1u << e;
-                }
-                const bool again = __any_sync(0xffffffffu, bad != 0);
-                if (again || !c_vec) {
+                if (!c_vec) {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) stage[lane * F_STAGE_PITCH + e] = sum[c + e];
                     __syncwarp();
-                    if (again) recompute<A_MN, B_MN>(A, B, m0, n0 + c, Kdim, bad, stage, lane);
                     // A row at a time, half a warp each: consecutive lanes to consecutive columns.
                     const int e = lane & 15;
                     if (e < valid) {
@@ -394,6 +474,17 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
             }
         }
         if (failed) *abort_flag = 1;
+        // Marked outputs: every product is done, the ring is free, and nobody waits but for the end.  All sum warps get here.
+        __syncwarp();
+        if (!sum_warps_any(failed)) {
+            mark = marks;
+            for (int tile = pair; tile < num_tiles; tile += num_pairs, ++mark) {
+                if (!*mark) continue;
+                const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * F_BM, BN);
+                redo_tile<A_MN, B_MN, BN>(A, B, C, ldc, beta, t0.m0 + rank * F_BM, t0.n0, Mdim, Ndim, Kdim, *mark,
+                                          reinterpret_cast<float*>(smem_raw + (base - raw)));
+            }
+        }
     }
     if (failed && status) atomicExch(status, VELORA_ERR_TIMEOUT);
 
@@ -424,6 +515,13 @@ int launch_shape(const F32Operand& A, const F32Operand& B, float* C, int64_t ldc
     const int tiles_m = static_cast<int>(ceil_div64(Mdim, 2 * F_BM)), tiles_n = static_cast<int>(ceil_div64(Ndim, BN));
     const int64_t tiles = static_cast<int64_t>(tiles_m) * tiles_n;
     const int pairs = tiles < di.sm_count / 2 ? static_cast<int>(tiles) : di.sm_count / 2;
+    if (ceil_div64(tiles, pairs) > F32Shape<A_MN, B_MN, BN>::kMaxTiles) {             // 7 GB of outputs and more: half of the rows at a time
+        if (tiles_m < 2) return VELORA_ERR_UNSUPPORTED;
+        const int rows = tiles_m / 2 * 2 * F_BM;
+        const F32Operand A2{A.p + static_cast<int64_t>(rows) * (A_MN ? 1 : A.ld), A.ld, A.vec};
+        const int rc = launch_shape<A_MN, B_MN, BN>(A, B, C, ldc, beta, rows, Ndim, Kdim, status, di, stream);
+        return rc != VELORA_OK ? rc : launch_shape<A_MN, B_MN, BN>(A2, B, C + rows * ldc, ldc, beta, Mdim - rows, Ndim, Kdim, status, di, stream);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs), 1, 1);
     cfg.blockDim = dim3(F_THREADS, 1, 1);

@@ -25,4 +25,16 @@ __device__ __forceinline__ bool split_suspect(float x)
     return !(a <= 3.402823466e+38f) || (a < 5.421010862e-20f && a != 0.f);
 }
 
+// The same for many outputs at once, two instructions each.
+struct SplitCheck {
+    float finite = 0.f;                  // NaN once an output is not finite
+    uint32_t least = 0xffffffffu;        // twice the bits of the smallest magnitude less one: zero, which is right, counts as the largest
+    __device__ __forceinline__ void add(float x)
+    {
+        finite = fmaf(x, 0.f, finite);
+        least = min(least, 2u * __float_as_uint(x) - 1u);
+    }
+    __device__ __forceinline__ bool suspect() const { return finite != 0.f || least < 2u * 0x1f800000u - 1u; }      // 2^-64
+};
+
 }  // namespace velora

@@ -87,3 +87,30 @@ def test_values_that_the_parts_cannot_carry(vl, guard, kind, pad):
     # 200 roundings of 2^-24 at most, and numbers below the smallest normal fp32 one to its last place
     assert bool((err <= torch.where(fin, 200 * 2.0 ** -24 * scale + 2.0 ** -140, float("inf"))).all())
     assert bool((C[201][fin[201]] == 0).all())
+
+
+@pytest.mark.parametrize("what", ["infinite token", "NaN token", "2^-118"])
+def test_every_output_of_a_long_contraction_is_computed_again(vl, guard, what):
+    """A token that is not finite, or an operand of very small numbers, takes all outputs off the tensor cores; several tiles per CTA
+    pair.  None may be left out, and no wait of the kernel may run out meanwhile."""
+    Kdim, Mdim, Ndim = 40000, 2300, 2310
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(11)
+    A = torch.randn((Kdim, Mdim), generator=gen, device=DEV)
+    B = torch.randn((Kdim, Ndim), generator=gen, device=DEV)
+    if what == "2^-118":
+        A *= 2.0 ** -118
+    else:
+        B[31234] = float("inf") if what == "infinite token" else float("nan")
+    ws = guard.workspace(vl, 256)
+    C0 = torch.randn((Mdim, Ndim), generator=gen, device=DEV) * (2.0 ** -112 if what == "2^-118" else 1.0)
+    C = guard.mat(Mdim, Ndim, torch.float32, init=C0)
+    vl.velora_dense_product(vl.PRODUCT_AT_B, A, B, C=C, beta=1, ws=ws)
+    assert vl.velora_workspace_status(ws) == 0
+    if what == "2^-118":
+        ref = A.double().T @ B.double() + C0.double()
+        assert_matches(C * 2.0 ** 118, (ref * 2.0 ** 118).cpu().numpy(), 1e-5, "C", c=3.84 * Kdim * 2.0 ** -24)
+    elif what == "infinite token":
+        assert torch.equal(C, torch.where(A[31234] > 0, float("inf"), float("-inf"))[:, None].expand(Mdim, Ndim))
+    else:
+        assert bool(C.isnan().all())
