@@ -29,12 +29,11 @@
 // An arrival on the other CTA's barrier holds its warp up for 700 to 1000 cycles, which the operand and sum warps do not have.
 // Every wait is bounded; both CTAs always reach the closing cluster barrier.  No copies are in flight when they do.
 //
-// Numbers that the split cannot carry.  An infinity, a NaN or a number that rounds to infinity in bf16 has no finite h or m, so
-// every output it enters comes out not finite; below 2^-110 the last bits of l are lost (at most 2^-134 of absolute value), which
-// shows only where an output is tiny altogether.  A warp whose 32 x BN / 3 outputs hold one that is not finite or below 2^-64 leaves
-// them unwritten and marks them.  Marked outputs are computed by fp32 multiply-adds behind the last tile, when no role waits for another any
-// more (computed in between they kept the pair's other roles waiting, for longer than those do when a contraction is long), at the
-// rate of the CUDA-core product.
+// Numbers that the split cannot carry (split_bf16.cuh).  The operand warps look at what they split and leave a tile's flags in its word of
+// marks, in both CTAs, before its last full[s]; a warp whose 32 x BN / 3 outputs may be wrong by them or by what came out leaves the outputs
+// unwritten and sets its bit there.  Marked outputs are computed by fp32 multiply-adds behind the last tile, when no role waits for
+// another any more (computed in between they kept the pair's other roles waiting, for longer than those do when a contraction is long), at
+// about the rate of the CUDA-core product: 12608 x 768 x 768 with every output marked 640 us, with one row 229.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -62,6 +61,7 @@ constexpr int F_SLAB = 64 * F_BK * 2;              // 64 columns of an MN-major 
 constexpr int F_STAGES = 2;                        // stage = accumulator = k-block mod 2
 constexpr int F_STAGE_PITCH = 17;                  // 16 columns of 32 unaligned output rows, no bank conflicts either way
 constexpr int F_BARRIER_BYTES = 128;
+constexpr int F_FLAG_SHIFT = 16;                   // of the operands' flags in a tile's word of marks
 
 template <int N> using Int = std::integral_constant<int, N>;
 
@@ -119,14 +119,20 @@ struct SplitTile {
         return load4(q + pass * (kRowsPerPass * op.ld), pass * kRowsPerPass < rows ? cols : 0, op.vec);
     }
     // The three parts, kPartBytes apart.
-    static __device__ __forceinline__ void store(uint32_t part0, int pass, int t, const float4& x)
+    static __device__ __forceinline__ void store(uint32_t part0, int pass, int t, const float4& x, SplitOperandCheck& seen)
     {
         const int r = t / kLanes, c = t % kLanes * 4;
         if (c >= kCols || (kRows % kRowsPerPass && r + pass * kRowsPerPass >= kRows)) return;
         const uint32_t at = part0 + (c >> 6) * F_SLAB + r * 128 + ((((c >> 3) & 7) ^ (r & 7)) << 4) + (c & 4) * 2 + pass * (kRowsPerPass * 128);
         float2 a = make_float2(x.x, x.y), b = make_float2(x.z, x.w);
+        seen.add(a);
+        seen.add(b);
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
+            if (p == 2) {
+                seen.add_rest(a);
+                seen.add_rest(b);
+            }
             const uint32_t u = pack_bf16x2(a.x, a.y), w = pack_bf16x2(b.x, b.y);
             asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + p * kPartBytes), "r"(u), "r"(w) : "memory");
             if (p < 2) {
@@ -156,6 +162,15 @@ __device__ __forceinline__ bool sum_warps_any(bool p)
     asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
                  : "=r"(any) : "r"(static_cast<uint32_t>(p)), "n"(32 * F_SUM_WARPS) : "memory");
     return any != 0;
+}
+
+// Sets bits of a word of shared memory in both CTAs of the pair, before any arrival that this thread makes afterwards.
+__device__ __noinline__ void flag_tile(uint32_t* word, uint32_t bits)
+{
+    const uint32_t local = smem_u32(word);
+    for (uint32_t rank = 0; rank < 2; ++rank)
+        asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(map_to_cta(local, rank)), "r"(bits) : "memory");
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
 }
 
 // Four bytes to shared memory, zero where `take` is false.
@@ -352,6 +367,7 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
         };
         // A waits in registers while the stage is being read; B is fetched while A is split, into the registers that frees.
         float4 x[4];
+        SplitOperandCheck seen;
         int tile = pair, kb = 0;
         if (tile < num_tiles) {
             start(tile);
@@ -364,11 +380,17 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
             const uint32_t a0 = base + s * S::kStageBytes;
 #pragma unroll
             for (int i = 0; i < TileA::kPasses; ++i) {
-                TileA::store(a0, i, t, x[i]);
+                TileA::store(a0, i, t, x[i], seen);
                 if (i < TileB::kPasses) x[i] = tb.load(B, i);
             }
 #pragma unroll
-            for (int i = 0; i < TileB::kPasses; ++i) TileB::store(a0 + 3 * TileA::kPartBytes, i, t, x[i]);
+            for (int i = 0; i < TileB::kPasses; ++i) TileB::store(a0 + 3 * TileA::kPartBytes, i, t, x[i], seen);
+            if (kb + 1 == kblocks) {
+                const uint32_t flags = (__any_sync(0xffffffffu, seen.flags() & SPLIT_TINY) ? SPLIT_TINY : 0u) |
+                                       (__any_sync(0xffffffffu, seen.flags() & SPLIT_BIG) ? SPLIT_BIG : 0u);
+                if (flags && lane == 0) flag_tile(marks + (tile - pair) / num_pairs, flags << F_FLAG_SHIFT);
+                seen = SplitOperandCheck();
+            }
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(full + 8 * s);
@@ -416,18 +438,12 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
             if (failed) break;
             const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * F_BM, BN);
             const int m0 = t0.m0 + rank * F_BM + quarter * 32, n0 = t0.n0 + third * COLS;
-            SplitCheck check;
+            const uint32_t operands = *const_cast<volatile uint32_t*>(mark) >> F_FLAG_SHIFT;
+            SplitOutputCheck check;
 #pragma unroll
             for (int c = 0; c < COLS; ++c) check.add(sum[c]);
-            bool odd = check.suspect() && m0 + lane < Mdim;
-            if (odd && n0 + COLS > Ndim) {                   // columns beyond the matrix do not count
-                check = SplitCheck();
-#pragma unroll
-                for (int c = 0; c < COLS; ++c)
-                    if (n0 + c < Ndim) check.add(sum[c]);
-                odd = check.suspect();
-            }
-            if (__any_sync(0xffffffffu, odd)) {
+            // Columns beyond the matrix are not finite where their row has others that are not, or zeros: looked at again for nothing at worst.
+            if (__any_sync(0xffffffffu, m0 + lane < Mdim && n0 < Ndim && check.suspect(operands, Kdim))) {
                 if (lane == 0) atomicOr(mark, 1u << warp);
                 continue;
             }
@@ -479,7 +495,7 @@ gemm_f32_pair_kernel(const F32Operand A, const F32Operand B, float* __restrict__
         if (!sum_warps_any(failed)) {
             mark = marks;
             for (int tile = pair; tile < num_tiles; tile += num_pairs, ++mark) {
-                if (!*mark) continue;
+                if (!(*mark & ((1u << F_SUM_WARPS) - 1u))) continue;
                 const PairTile t0 = pair_tile(tile, tiles_m, tiles_n, 2 * F_BM, BN);
                 redo_tile<A_MN, B_MN, BN>(A, B, C, ldc, beta, t0.m0 + rank * F_BM, t0.n0, Mdim, Ndim, Kdim, *mark,
                                           reinterpret_cast<float*>(smem_raw + (base - raw)));

@@ -25,16 +25,37 @@ __device__ __forceinline__ bool split_suspect(float x)
     return !(a <= 3.402823466e+38f) || (a < 5.421010862e-20f && a != 0.f);
 }
 
-// The same for many outputs at once, two instructions each.
-struct SplitCheck {
+// What a product of split operands has to be checked for.
+//   Operands: a number other than zero below 2^-110 loses up to 2^-134 ("tiny").  Where no operand is 2^30 or more ("big") that is at most
+//   2^-104 a product: outputs of K * 2^-79 and more have lost 2^-25 of themselves at most.
+//   Outputs: one that is not finite (operands that round to infinity in bf16, infinities, NaN), or is below 2^-120 without being zero
+//   (products of last parts fall below the smallest number).
+constexpr uint32_t SPLIT_TINY = 1u, SPLIT_BIG = 2u;
+
+// Half an instruction an operand each.
+struct SplitOperandCheck {
+    uint32_t rests = 0;                  // what is left for the last part has its low 16 bits clear where a bf16 number holds it
+    float most = 0.f;                    // NaN does not show here, but in the outputs
+    __device__ __forceinline__ void add_rest(float2 x) { rests |= __float_as_uint(x.x) | __float_as_uint(x.y); }
+    __device__ __forceinline__ void add(float2 x) { asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(x.x), "f"(x.y)); }
+    __device__ __forceinline__ uint32_t flags() const { return (rests & 0xffffu ? SPLIT_TINY : 0u) | (most >= 1073741824.f ? SPLIT_BIG : 0u); }
+};
+
+struct SplitOutputCheck {
     float finite = 0.f;                  // NaN once an output is not finite
-    uint32_t least = 0xffffffffu;        // twice the bits of the smallest magnitude less one: zero, which is right, counts as the largest
+    uint32_t least = 0xffffffffu;        // as above
+    float least_or_zero = 3.402823466e+38f;
     __device__ __forceinline__ void add(float x)
     {
         finite = fmaf(x, 0.f, finite);
         least = min(least, 2u * __float_as_uint(x) - 1u);
+        least_or_zero = fminf(least_or_zero, fabsf(x));
     }
-    __device__ __forceinline__ bool suspect() const { return finite != 0.f || least < 2u * 0x1f800000u - 1u; }      // 2^-64
+    __device__ __forceinline__ bool suspect(uint32_t operands, int Kdim) const
+    {
+        if (finite != 0.f || least < 2u * 0x03800000u - 1u) return true;
+        return (operands & SPLIT_TINY) && ((operands & SPLIT_BIG) || least_or_zero < Kdim * 1.6543612251060553e-24f);       // K * 2^-79
+    }
 };
 
 }  // namespace velora

@@ -114,3 +114,39 @@ def test_every_output_of_a_long_contraction_is_computed_again(vl, guard, what):
         assert torch.equal(C, torch.where(A[31234] > 0, float("inf"), float("-inf"))[:, None].expand(Mdim, Ndim))
     else:
         assert bool(C.isnan().all())
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("ea,eb", [(-140, 0), (-140, 30), (-128, 70), (-120, 60), (60, -120), (-100, -30), (-70, -70)])
+@pytest.mark.parametrize("where", ["operand", "row", "element"])
+def test_very_small_operands(vl, guard, kind, ea, eb, where):
+    """Numbers whose last bits no bf16 part holds, against partners so large (or small) that those bits show in the outputs: a whole
+    operand of them, a row (or column) and single elements among ordinary ones, of either operand."""
+    Mdim, Ndim, Kdim = 1500, 1000, 200
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(3)
+    a = torch.randn((Mdim, Kdim), generator=gen, device=DEV)
+    b = torch.randn((Ndim, Kdim), generator=gen, device=DEV)
+    small, large, e, f = (a, b, ea, eb) if ea <= eb else (b, a, eb, ea)
+    large *= 2.0 ** f
+    if where == "operand":
+        small *= 2.0 ** e
+    elif where == "row":
+        small[77] *= 2.0 ** e
+    else:
+        small[::5, ::7] *= 2.0 ** e
+        small[77] = 0.0
+        small[77, 11] = 2.0 ** e * 1.23456789
+    A = a.T.contiguous() if kind == vl.PRODUCT_AT_B else a
+    B = b if kind == vl.PRODUCT_A_BT else b.T.contiguous()
+    C = guard.mat(Mdim, Ndim, torch.float32)
+    vl.velora_dense_product(kind, A, B, C=C)
+    ref = a.double() @ b.double().T
+    # 200 roundings of 2^-24 at most, and of numbers below the smallest normal fp32 one to the last place
+    bound = 200 * 2.0 ** -24 * (a.double().abs() @ b.double().abs().T) + 200 * 2.0 ** -149
+    assert bool(((C.double() - ref).abs() <= bound).all())
+    # in norm too, as fp32 sums of 200 terms have it (2.1e-7 for ordinary numbers), where the outputs are normal numbers
+    if ea + eb > -100:
+        for rows in (slice(None), 77):
+            r, c = (ref[rows], C[rows]) if small is a else (ref[:, rows], C[:, rows])
+            assert float((c.double() - r).norm() / r.norm()) <= 4e-7
