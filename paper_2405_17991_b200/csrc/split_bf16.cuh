@@ -17,14 +17,6 @@ __device__ __forceinline__ float2 minus_parts(float2 x, uint32_t parts)
     return r;
 }
 
-// True for an output that the split may have got wrong (not finite, or so small altogether that vanished last parts could show); zero is right either way, since the products
-// that vanish then are below the smallest fp32 number.
-__device__ __forceinline__ bool split_suspect(float x)
-{
-    const float a = fabsf(x);
-    return !(a <= 3.402823466e+38f) || (a < 5.421010862e-20f && a != 0.f);
-}
-
 // What a product of split operands has to be checked for.
 //   Operands: a number other than zero below 2^-110 loses up to 2^-134 ("tiny").  Where no operand is 2^30 or more ("big") that is at most
 //   2^-104 a product: outputs of K * 2^-79 and more have lost 2^-25 of themselves at most.
@@ -43,7 +35,7 @@ struct SplitOperandCheck {
 
 struct SplitOutputCheck {
     float finite = 0.f;                  // NaN once an output is not finite
-    uint32_t least = 0xffffffffu;        // as above
+    uint32_t least = 0xffffffffu;        // twice the bits of the smallest magnitude less one: zero counts as the largest
     float least_or_zero = 3.402823466e+38f;
     __device__ __forceinline__ void add(float x)
     {

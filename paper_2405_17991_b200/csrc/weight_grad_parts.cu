@@ -15,8 +15,9 @@
 // copy of dY for the input gradient already (TILED), a thirteenth warp fetches tiles of that instead, four stages deep, and the
 // operand warps have Z only (layer of 4096 x 2048 -> 5461 with dense rows: 217 -> 203 us).
 //
-// An infinity or NaN, a Z too large for bf16, or numbers so small that their parts vanish: outputs that come out not finite or below
-// 2^-64 are computed again by fp32 multiply-adds.
+// Numbers that the parts cannot carry (split_bf16.cuh): the 32 columns of dY of a sum warp whose outputs may be wrong by what the operand
+// warps have seen (in fp32 operands; how large a bf16 dY is they do not look at) or by what came out are computed by fp32 multiply-adds at
+// the end.  12608 x 768 fp32, 24 sub-tokens: 21 us, 68 with every output computed again (32 on the CUDA cores).
 #include "gemm_tc.cuh"
 #include "row_chunks.cuh"
 #include "split_bf16.cuh"
@@ -32,6 +33,7 @@ constexpr int WP_O = 128, WP_K = 64;
 constexpr int WP_SUM_WARPS = 4, WP_OPERAND_WARPS = 8;
 constexpr int WP_OPERAND_THREADS = 32 * WP_OPERAND_WARPS;
 constexpr int WP_THREADS = 32 * (WP_SUM_WARPS + WP_OPERAND_WARPS + 1);
+constexpr int WP_FLAG_SHIFT = 16;                       // of the operands' flags in the word that says what to compute again
 constexpr int WP_SLAB = WP_K * 128;                     // 64 columns of 64 tokens
 constexpr int WP_A_PART = 2 * WP_SLAB;
 
@@ -57,7 +59,7 @@ template <typename YT> struct RowsOfY;
 
 template <> struct RowsOfY<__nv_bfloat16> {
     uint4 x[4], over[4];
-    __device__ __forceinline__ void load(const __nv_bfloat16* dY, int64_t ld, int n, int n_end, int o0, const char* end, int t)
+    __device__ __forceinline__ void load(const __nv_bfloat16* dY, int64_t ld, int n, int n_end, int o0, int, const char* end, int t)
     {
         const int l = t & 15;
 #pragma unroll
@@ -72,7 +74,7 @@ template <> struct RowsOfY<__nv_bfloat16> {
             }
         }
     }
-    __device__ __forceinline__ void store(uint32_t a0, const __nv_bfloat16* dY, int64_t ld, int n, int o0, int t)
+    __device__ __forceinline__ void store(uint32_t a0, const __nv_bfloat16* dY, int64_t ld, int n, int o0, int t, SplitOperandCheck&)
     {
         const int r = t >> 4, l = t & 15;
         const uint32_t at = a0 + (l >> 3) * WP_SLAB + r * 128 + (((l & 7) ^ (r & 7)) << 4);
@@ -90,15 +92,14 @@ template <> struct RowsOfY<__nv_bfloat16> {
 
 template <> struct RowsOfY<float> {
     float4 x[8];                                       // eight tokens a pass: four columns of every eighth token
-    __device__ __forceinline__ void load(const float* dY, int64_t ld, int n, int n_end, int o0, const char* end, int t)
+    __device__ __forceinline__ void load(const float* dY, int64_t ld, int n, int n_end, int o0, int O, const char*, int t)
     {
-        const int c = (t & 31) * 4;
+        const int c = (t & 31) * 4, left = O - (o0 + c);
         const bool vec = (reinterpret_cast<uintptr_t>(dY) & 15u) == 0 && ld % 4 == 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int row = n + (t >> 5) + 8 * i;
             const float* q = dY + static_cast<int64_t>(row) * ld + o0 + c;
-            const int64_t left = (end - reinterpret_cast<const char*>(q)) / 4;            // what follows in memory: columns beyond O feed nothing
             x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (row >= n_end) continue;
             if (vec && left >= 4) {
@@ -111,15 +112,21 @@ template <> struct RowsOfY<float> {
             }
         }
     }
-    __device__ __forceinline__ void store(uint32_t a0, const float*, int64_t, int, int, int t)
+    __device__ __forceinline__ void store(uint32_t a0, const float*, int64_t, int, int, int t, SplitOperandCheck& seen)
     {
         const int r = t >> 5, c = (t & 31) * 4;
         const uint32_t at = a0 + (c >> 6) * WP_SLAB + r * 128 + ((((c >> 3) & 7) ^ r) << 4) + (c & 4) * 2;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             float2 a = make_float2(x[i].x, x[i].y), b = make_float2(x[i].z, x[i].w);
+            seen.add(a);
+            seen.add(b);
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
+                if (p == 2) {
+                    seen.add_rest(a);
+                    seen.add_rest(b);
+                }
                 const uint32_t u = pack_bf16x2(a.x, a.y), w = pack_bf16x2(b.x, b.y);
                 asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + i * 8 * 128 + p * WP_A_PART), "r"(u), "r"(w) : "memory");
                 if (p < 2) {
@@ -132,7 +139,7 @@ template <> struct RowsOfY<float> {
 };
 
 // Z of a stage: 64 tokens x MP sub-tokens (zeros beyond M and n_end), a thread has pairs of neighbours.
-template <typename ZT, int MP>
+template <typename YT, typename ZT, int MP>
 struct RowsOfZ {
     static constexpr int kPairs = WP_K * MP / 2 / WP_OPERAND_THREADS;
     float2 x[kPairs];
@@ -146,14 +153,16 @@ struct RowsOfZ {
             x[i].y = row < n_end && m + 1 < M ? Elem<ZT>::load(q + 1) : 0.f;
         }
     }
-    __device__ __forceinline__ void store(uint32_t b0, int t)
+    __device__ __forceinline__ void store(uint32_t b0, int t, SplitOperandCheck& seen)
     {
 #pragma unroll
         for (int i = 0; i < kPairs; ++i) {
             const int idx = t + WP_OPERAND_THREADS * i, r = idx / (MP / 2), m = idx % (MP / 2) * 2;
             float2 a = x[i];
+            if (sizeof(YT) == 4) seen.add(a);
 #pragma unroll
             for (int p = 0; p < (sizeof(ZT) == 4 ? 3 : 1); ++p) {
+                if (p == 2) seen.add_rest(a);                        // columns beyond M and rows beyond n_end are zeros
                 const int c = p * MP + m;
                 const uint32_t u = pack_bf16x2(a.x, a.y);
                 asm volatile("st.shared.b32 [%0], %1;"
@@ -163,6 +172,51 @@ struct RowsOfZ {
         }
     }
 };
+
+// The marked outputs (bit w: those of sum warp w) by fp32 multiply-adds, whole CTA: warps 0 .. 11 have 32 columns of dY by 8 sub-tokens
+// each, 64 tokens of Z at a time in shared memory (`zs`, 64 x 24) and added to the sum.
+template <typename YT, typename ZT>
+__device__ __noinline__ void redo_outputs(const YT* dY, int64_t lddy, const ZT* Z, int64_t ldz, int n_begin, int n_end, int o0, int O, int M,
+                                          uint32_t marked, float* zs, float* out)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, block = warp & 3, third = warp >> 2;
+    const int o = o0 + block * 32 + lane;
+    const YT* y = dY + (o < O ? o : O - 1);
+    for (int m_first = 0; m_first < M; m_first += 24) {
+        const int m0 = m_first + 8 * third;
+        const bool mine = third < 3 && m0 < M && ((marked >> block) & 1u);
+        float sum[8] = {};
+        for (int n0 = n_begin; n0 < n_end; n0 += WP_K) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < WP_K * 24; i += blockDim.x) {
+                const int n = n0 + i / 24, m = m_first + i % 24;
+                zs[i] = n < n_end && m < M ? Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m) : 0.f;
+            }
+            __syncthreads();
+            if (!mine) continue;
+            float part[8] = {};
+#pragma unroll 1
+            for (int h = 0; h < WP_K; h += 16) {
+                float f[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) f[i] = n0 + h + i < n_end ? Elem<YT>::load(y + static_cast<int64_t>(n0 + h + i) * lddy) : 0.f;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float4 u = *reinterpret_cast<const float4*>(zs + (h + i) * 24 + 8 * third), w = *reinterpret_cast<const float4*>(zs + (h + i) * 24 + 8 * third + 4);
+                    part[0] = fmaf(f[i], u.x, part[0]); part[1] = fmaf(f[i], u.y, part[1]);
+                    part[2] = fmaf(f[i], u.z, part[2]); part[3] = fmaf(f[i], u.w, part[3]);
+                    part[4] = fmaf(f[i], w.x, part[4]); part[5] = fmaf(f[i], w.y, part[5]);
+                    part[6] = fmaf(f[i], w.z, part[6]); part[7] = fmaf(f[i], w.w, part[7]);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) sum[e] += part[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (mine && o < O && m0 + e < M) out[static_cast<int64_t>(o) * M + m0 + e] = sum[e];
+    }
+}
 
 template <typename YT, typename ZT, int MP, bool TILED>
 __global__ void __launch_bounds__(PartsShape<YT, ZT, MP, TILED>::kThreads, PartsShape<YT, ZT, MP, TILED>::kCtasPerSm)
@@ -178,6 +232,7 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
     const uint32_t full = base + ST * S::kStageBytes, done = full + 32, drained = full + 64;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 80);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 88);
+    uint32_t* redo = reinterpret_cast<uint32_t*>(tail + 92);              // bit w: the columns of sum warp w
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int o0 = blockIdx.y * WP_O;
     const int n_begin = blockIdx.x * tokens_per_cta;
@@ -191,6 +246,7 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
         for (int a = 0; a < 2; ++a) mbar_init(drained + 8 * a, WP_SUM_WARPS);
         if (TILED) prefetch_tensormap(&tmY);
         *abort_flag = 0;
+        *redo = 0;
         fence_mbar_init();
     }
     if (warp == WP_SUM_WARPS + WP_OPERAND_WARPS) {
@@ -246,21 +302,23 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
         const int t = threadIdx.x - 32 * WP_SUM_WARPS;
         const char* end = reinterpret_cast<const char*>(dY + static_cast<int64_t>(N - 1) * lddy + O);
         RowsOfY<YT> y;
-        RowsOfZ<ZT, MP> z;
-        if (!TILED) y.load(dY, lddy, n_begin, n_end, o0, end, t);
+        RowsOfZ<YT, ZT, MP> z;
+        SplitOperandCheck seen;
+        if (!TILED) y.load(dY, lddy, n_begin, n_end, o0, O, end, t);
         z.load(Z, ldz, n_begin, n_end, M, t);
         uint32_t it = 0;
         for (int n = n_begin; n < n_end; n += WP_K, ++it) {
             const uint32_t s = it % ST, ph = (it / ST) & 1u;
             if (!mbar_wait_warp(done + 8 * s, ph ^ 1u, abort_flag)) { failed = true; break; }
             const uint32_t a0 = base + s * S::kStageBytes;
-            if (!TILED) y.store(a0, dY, lddy, n, o0, t);
-            z.store(a0 + S::kParts * WP_A_PART, t);
+            if (!TILED) y.store(a0, dY, lddy, n, o0, t, seen);
+            z.store(a0 + S::kParts * WP_A_PART, t, seen);
+            if (n + WP_K >= n_end && seen.flags()) atomicOr(redo, (sizeof(YT) == 2 ? SPLIT_TINY | SPLIT_BIG : seen.flags()) << WP_FLAG_SHIFT);
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(full + 8 * s);
             if (n + WP_K < n_end) {
-                if (!TILED) y.load(dY, lddy, n + WP_K, n_end, o0, end, t);
+                if (!TILED) y.load(dY, lddy, n + WP_K, n_end, o0, O, end, t);
                 z.load(Z, ldz, n + WP_K, n_end, M, t);
             }
         }
@@ -305,33 +363,16 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
         }
         const int o = o0 + warp * 32 + lane;
         float* out = partials + (static_cast<int64_t>(blockIdx.x) * O + o) * M;
-        uint32_t bad = 0;
+        SplitOutputCheck check;
 #pragma unroll
         for (int m = 0; m < MP; ++m) {
             if (o < O && m < M) {
                 out[m] = sum[m];
-                if (split_suspect(sum[m])) bad |= 1u << m;
+                check.add(sum[m]);
             }
         }
-        if (!failed)
-            for (uint32_t cols = __ballot_sync(0xffffffffu, bad != 0); cols; cols &= cols - 1) {
-                const int c = __ffs(cols) - 1;                       // the column of dY: this warp's lane c
-                const YT* yc = dY + o0 + warp * 32 + c;
-                int nan = 0;                                         // with a NaN in it all its outputs are NaN
-                for (int n = n_begin + lane; n < n_end; n += 32) {
-                    const float f = Elem<YT>::load(yc + static_cast<int64_t>(n) * lddy);
-                    nan |= f != f;
-                }
-                if (__any_sync(0xffffffffu, nan)) continue;
-                for (uint32_t ms = __shfl_sync(0xffffffffu, bad, c); ms; ms &= ms - 1) {
-                    const int m = __ffs(ms) - 1;
-                    float f = 0.f;
-                    for (int n = n_begin + lane; n < n_end; n += 32)
-                        f = fmaf(Elem<YT>::load(yc + static_cast<int64_t>(n) * lddy), Elem<ZT>::load(Z + static_cast<int64_t>(n) * ldz + m), f);
-                    for (int off = 16; off >= 1; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
-                    if (lane == c) out[m] = f;
-                }
-            }
+        const uint32_t operands = *const_cast<volatile uint32_t*>(redo) >> WP_FLAG_SHIFT;
+        if (check.suspect(operands, n_end - n_begin)) atomicOr(redo, 1u << warp);
         if (failed) *abort_flag = 1;
     }
     if (failed && status) atomicExch(status, VELORA_ERR_TIMEOUT);
@@ -343,6 +384,9 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
         __syncwarp();
         tmem_dealloc(tmem_base, S::kTmemCols);
     }
+    if ((*redo & 0xfu) && !*abort_flag)
+        redo_outputs<YT, ZT>(dY, lddy, Z, ldz, n_begin, n_end, o0, O, M, *redo, reinterpret_cast<float*>(smem_raw + (base - raw)),
+                             partials + static_cast<int64_t>(blockIdx.x) * O * M);
 }
 
 struct PartsArgs {

@@ -80,3 +80,32 @@ def test_packed_copy_gives_the_same_bits(vl, N, D, O, Dsub):
     alone = vl.velora_weight_grad(dY, Z, v, D, ws=vl.velora_workspace_alloc(
         vl.velora_workspace_bytes(vl.OP_WEIGHT_GRAD_FACTORED, N, D, O, Dsub), DEV))
     assert torch.equal(dW, alone)
+
+
+@pytest.mark.parametrize("dtype,pad", [(torch.bfloat16, 2), (torch.bfloat16, 0), (torch.float32, 0), (torch.float32, 3)])
+@pytest.mark.parametrize("ey,ez", [(0, -140), (30, -140), (70, -128), (60, -120), (-120, 60), (-70, -70)])
+@pytest.mark.parametrize("where", ["operand", "token", "element"])
+def test_very_small_operands(vl, guard, dtype, pad, ey, ez, where):
+    """Numbers whose last bits no bf16 part holds against partners that make them show: a whole operand of them, whole tokens, single
+    elements among ordinary ones."""
+    N, O, M = 4000, 1301, 9
+    dY, Z = _inputs(N, O, M, dtype, torch.float32, pad, 0, 9)
+    small, large, e, f = (Z, dY, ez, ey) if ez <= ey else (dY, Z, ey, ez)
+    large *= 2.0 ** f
+    if where == "operand":
+        small *= 2.0 ** e
+    elif where == "token":
+        small[5::3] *= 2.0 ** e
+    else:
+        small[::5, ::7] *= 2.0 ** e
+        small[:, 8] = 0.0
+        small[77, 8] = 2.0 ** e * 1.23456789
+    P = guard.mat(O, M, torch.float32)
+    vl.velora_weight_grad_p(dY, Z, 16 * M, 16, P=P)
+    y, z = dY.double(), Z.double()
+    ref = y.T @ z
+    # N roundings of 2^-24 at most, and of numbers below the smallest normal fp32 one to the last place; in norm as fp32 sums have it
+    assert bool(((P.double() - ref).abs() <= N * 2.0 ** -24 * (y.abs().T @ z.abs()) + N * 2.0 ** -149).all())
+    if ey + ez > -100:
+        for part in (slice(None), (slice(None), 8) if small is Z else 8):
+            assert float((P[part].double() - ref[part]).norm() / ref[part].norm()) <= 1e-6
