@@ -42,6 +42,9 @@ constexpr int WG_A_BYTES = WG_BM * WG_BK * 2;         // 16 KB: two 64-wide slab
 constexpr int WG_SLAB = 64 * WG_BK * 2;               // 8 KB
 constexpr int WG_THREADS = 192;
 constexpr int WG_MAX_SPLITS = 8;                      // also the portable cluster size limit
+// Layers whose token range may be cut into twice as many: 16 splits of 9 row blocks fill 148 SMs once, one slab of Z.
+constexpr int64_t WG_NARROW_O = 148 / 16 * 128;
+constexpr int WG_NARROW_PAD = 64;
 constexpr int WG_MAX_M = 256;
 
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -421,8 +424,9 @@ WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
     int best = 1;
     double best_eff = 0.0;
     // Where even eight splits would keep half of the SMs idle, up to sixteen through the workspace, of four k-blocks or more
-    // (8192 x 512 -> 512: the partial products take 6 us instead of 9).
-    const int most = !p.fat && 2 * WG_MAX_SPLITS * static_cast<int64_t>(p.tiles_o) <= sm_count && p.kblocks >= 8 * WG_MAX_SPLITS ? 2 * WG_MAX_SPLITS : WG_MAX_SPLITS;
+    // (8192 x 512 -> 512: the partial products take 6 us instead of 9).  By a fixed count of SMs, as the room is asked for without a device.
+    const bool narrow = p.npad <= WG_NARROW_PAD && O <= WG_NARROW_O && p.kblocks >= 8 * WG_MAX_SPLITS;
+    const int most = narrow ? 2 * WG_MAX_SPLITS : WG_MAX_SPLITS;
     for (int s = 1; s <= most && s <= p.kblocks; ++s) {
         const int64_t ctas = static_cast<int64_t>(p.tiles_o) * s;
         const int64_t waves = ceil_div64(ctas, slots);
@@ -432,7 +436,13 @@ WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
     p.kb_per_split = static_cast<int>(ceil_div64(p.kblocks, best));
     p.splits = static_cast<int>(ceil_div64(p.kblocks, p.kb_per_split));
     p.zb_bytes = static_cast<size_t>(round_up(static_cast<int64_t>(N) * p.pitch * 2, 256));
-    p.part_bytes = static_cast<size_t>(most) * static_cast<size_t>(O) * p.npad * sizeof(float);
+    // Room for the partial products: never less for a wider layer or more tokens, so that a workspace sized for the largest layer serves all.
+    size_t part_values = static_cast<size_t>(WG_MAX_SPLITS) * static_cast<size_t>(O) * p.npad;
+    if (p.kblocks >= 8 * WG_MAX_SPLITS) {
+        const size_t narrow_values = 2 * WG_MAX_SPLITS * static_cast<size_t>(O < WG_NARROW_O ? O : WG_NARROW_O) * (p.npad < WG_NARROW_PAD ? p.npad : WG_NARROW_PAD);
+        if (narrow_values > part_values) part_values = narrow_values;
+    }
+    p.part_bytes = part_values * sizeof(float);
     p.ok = true;
     return p;
 }
@@ -567,7 +577,7 @@ int launch_weight_grad_tc(const void* dY, int dy_dtype, int64_t N, int64_t O, in
     // 2a. one launch: cluster of the tile's splits, reduction through distributed shared memory
     const int L = (Dsub % 8 == 0) ? Dsub / 8 : 0;
     const bool filled = p.fat || static_cast<int64_t>(p.tiles_o) * p.splits > di.sm_count;
-    const bool vec = filled && L >= 1 && L <= 128 && (L & (L - 1)) == 0 && aligned16(dW) &&
+    const bool vec = filled && p.splits <= WG_MAX_SPLITS && L >= 1 && L <= 128 && (L & (L - 1)) == 0 && aligned16(dW) &&
                      (lddw * static_cast<int64_t>(dtype_size(dw_dtype))) % 16 == 0 &&
                      static_cast<size_t>(WG_BM) * (p.npad + 4) * 4 <= static_cast<size_t>(p.tail_off);
     if (vec) {

@@ -187,3 +187,19 @@ def test_kernels_trigger_the_next_one_after_they_have_allocated():
                 allocated = body.index("__syncthreads()", body.index("tmem_alloc("))
                 assert body.index("pdl_wait()") < body.index("pdl_trigger()") and allocated < body.index("pdl_trigger()"), name
     assert seen >= 2
+
+
+# A workspace sized for a model's widest layer (or its longest batch, or its widest input) serves the narrower ones.
+def test_workspace_of_a_larger_layer_serves_a_smaller_one(lib):
+    from paper_2405_17991_b200 import binding as b
+    widths = [65, 128, 129, 512, 1024, 1152, 1153, 1280, 2304, 2305, 4096, 11008]
+    tokens = [1, 64, 500, 2048, 4032, 4033, 8192, 12608]
+    subtokens = [1, 16, 17, 64, 65, 80, 172, 256]
+    for op in (b.OP_WEIGHT_GRAD_FACTORED, b.OP_LINEAR_BACKWARD_FACTORED):
+        for Dsub in (16, 64):
+            size = {(n, m, o): lib.velora_workspace_bytes(op, n, m * Dsub, o, Dsub) for n in tokens for m in subtokens for o in widths}
+            for (n, m, o), s in size.items():
+                for axis, i in ((tokens, tokens.index(n)), (subtokens, subtokens.index(m)), (widths, widths.index(o))):
+                    if i + 1 < len(axis):
+                        larger = (axis[i + 1] if axis is tokens else n, axis[i + 1] if axis is subtokens else m, axis[i + 1] if axis is widths else o)
+                        assert s <= size[larger], (op, Dsub, (n, m, o), larger)
