@@ -1,15 +1,19 @@
 // Partial factors P[o, m] = sum_n dY[n, o] * Z[n, m] of token slices on the tensor cores, to fp32 accuracy, for the gradients that
 // weight_grad_tc.cu does not take: fp32 rows, and bf16 rows on odd boundaries with Z as stored.
 //
-// An fp32 Z is split into three bf16 parts (exact, as in gemm_f32_tc.cu) that lie side by side as columns of one operand: 64
-// tokens of a bf16 dY are four tcgen05.mma of M = 128 columns of dY by N = 3 x round16(sub-tokens).  An fp32 dY has three parts as well, and
-// three times the products.  After every 64 tokens the accumulator is read out and added to fp32 sums, rounded to nearest (the
-// tensor cores' own sums truncate).
+// An fp32 Z is split into three bf16 parts (exact, as in gemm_f32_tc.cu), the second and third side by side as columns of one operand: 64
+// tokens of a bf16 dY are four tcgen05.mma of M = 128 columns of dY by N = round16(sub-tokens) and four by twice that.  An fp32 dY has three
+// parts as well, and three times the products.  The tensor cores' sums truncate, so the products of the first parts, the only ones that
+// reach the result's size, are added up there for 16 tokens and no further: 16 products of 16 significant bits hardly reach 24.
+// The others share an accumulator for the 64 tokens of a stage, below 2^-7 of the result; after each stage all are read out
+// and added to fp32 sums, rounded to nearest.
+// Error in norm against 64 bits, 12608 x 768, 24 sub-tokens in fp32, this form / the 64 tokens in one accumulator / fp32
+// multiply-adds on the CUDA cores, times 1e-8: |N(0, 1)| with a bf16 dY 4.7 / 8.9 / 4.8, fp32 4.1 / 7.1 / 4.8; N(0, 1) 9.9 / 11 / 17, 8.2 / 11 / 17.
 //
 // A CTA takes 128 columns of dY and one slice of the tokens.  Roles (416 threads): warps 0..3 sums (a lane has a column of dY);
 // warps 4..11 operands (plain loads of any alignment, split, swizzled MN-major tiles: tokens are the contraction, rows of both
 // matrices are rows of the tiles); warp 12 issues.  Two stages and two accumulators, a barrier pair each:
-//   full[s] (eight operand warps), done[s] (commit: the stage may be written, the accumulator read), drained[s] (four warps).
+//   full[s] (eight operand warps), done[s] (commit: the stage may be written, the accumulator read), drained[a] (four warps).
 // Two CTAs share an SM (bf16); bound by the loads and stores of the operand warps.  Rows that start on odd boundaries are
 // read as the aligned 16 bytes that a chunk begins in and shifted against the neighbouring lane's.  Where the call has made a packed
 // copy of dY for the input gradient already (TILED), a thirteenth warp fetches tiles of that instead, four stages deep, and the
@@ -41,17 +45,24 @@ template <typename YT, typename ZT, int MP, bool TILED>
 struct PartsShape {
     static constexpr int kParts = sizeof(YT) == 2 ? 1 : 3;                      // of dY
     static constexpr int kZParts = sizeof(ZT) == 4 ? 3 : 1;                     // a stored bf16 or E4M3 value is a bf16 number
-    static constexpr int kN = kZParts * MP;
-    static constexpr int kSlabsB = (kN + 63) / 64;
+    static constexpr int kSlabsB = kZParts == 3 ? 2 : 1;                        // second and third parts of Z, then the first
+    static constexpr int kHeadSlab = kSlabsB - 1;
     static constexpr int kStageBytes = kParts * WP_A_PART + kSlabsB * WP_SLAB;
-    static constexpr int kAccCols = kN <= 32 ? 32 : (kN <= 64 ? 64 : 128);
-    static constexpr int kStages = TILED ? (MP == 16 ? 4 : 3) : 2;
+    static constexpr int kStages = TILED ? (kStageBytes * 4 <= 100 * 1024 && MP == 16 ? 4 : 3) : 2;
     static constexpr int kThreads = WP_THREADS + (TILED ? 32 : 0);
-    static constexpr size_t kSmem = 1024 + kStages * static_cast<size_t>(kStageBytes) + 128;
+    // What the roundings of the sums leave is kept beside them, in registers or, where those do not suffice, in shared memory.  An fp32 Z with
+    // a bf16 dY does without: fp32 sums of its products on the CUDA cores were further off than this form is already.
+    static constexpr bool kRests = kParts == 3 || kZParts == 1, kRestsInSmem = kParts == 1 && kRests && MP == 32;
+    static constexpr size_t kSmem = 1024 + kStages * static_cast<size_t>(kStageBytes) + 128 + (kRestsInSmem ? WP_O * MP * 4 : 0);
     static constexpr int kCtasPerSm = kParts == 1 ? 2 : 1;
-    // Accumulators that share a stage's 64 tokens, as many as the 512 columns of an SM have room for: less truncation.
-    static constexpr int kSets = kAccCols * 8 * kCtasPerSm <= 512 ? 4 : (kAccCols * 4 * kCtasPerSm <= 512 ? 2 : 1);
-    static constexpr int kTmemCols = 2 * kSets * kAccCols;
+    // TMEM columns of a stage: first parts by first parts, four times 16 tokens; dY by the other parts of Z; the other parts of dY by the
+    // first of Z.  Two such sets where the 512 columns of an SM have the room (not for a bf16 dY by an fp32 Z of more than 16 sub-tokens: 4096 x
+    // 5461, 32 of them, 45 us instead of 42).
+    static constexpr int kTailCol = (WP_K / 16) * MP, kSideCol = kTailCol + (kZParts == 3 ? 2 * MP : 0);
+    static constexpr int kAccCols = kSideCol + (kParts == 3 ? MP : 0);
+    static constexpr int kBuffers = 2 * kAccCols * kCtasPerSm <= 512 ? 2 : 1;
+    static constexpr int kTmemCols = kBuffers * kAccCols <= 128 ? 128 : (kBuffers * kAccCols <= 256 ? 256 : 512);
+    static_assert(kBuffers * kAccCols <= kTmemCols && kTmemCols * kCtasPerSm <= 512 && 2 * MP <= 64, "TMEM columns");
 };
 
 // dY of a stage: 64 tokens x 128 columns, four passes of sixteen tokens; a thread has eight columns of every sixteenth token.
@@ -163,10 +174,10 @@ struct RowsOfZ {
 #pragma unroll
             for (int p = 0; p < (sizeof(ZT) == 4 ? 3 : 1); ++p) {
                 if (p == 2) seen.add_rest(a);                        // columns beyond M and rows beyond n_end are zeros
-                const int c = p * MP + m;
+                const int c = p == 0 ? m : (p - 1) * MP + m;
                 const uint32_t u = pack_bf16x2(a.x, a.y);
                 asm volatile("st.shared.b32 [%0], %1;"
-                             ::"r"(b0 + (c >> 6) * WP_SLAB + r * 128 + ((((c >> 3) & 7) ^ (r & 7)) << 4) + (c & 7) * 2), "r"(u) : "memory");
+                             ::"r"(b0 + (p == 0 && sizeof(ZT) == 4 ? WP_SLAB : 0) + r * 128 + (((c >> 3) ^ (r & 7)) << 4) + (c & 7) * 2), "r"(u) : "memory");
                 if (p < 2 && sizeof(ZT) == 4) a = minus_parts(a, u);
             }
         }
@@ -280,19 +291,23 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
     } else if (warp == WP_SUM_WARPS + WP_OPERAND_WARPS) {
         // ------------------------------------------------ products
         if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(WP_O, S::kN, true, true);
+            constexpr uint32_t idesc_head = umma_idesc_bf16(WP_O, MP, true, true), idesc_tail = umma_idesc_bf16(WP_O, 2 * MP, true, true);
             uint32_t it = 0;
             for (int n = n_begin; n < n_end; n += WP_K, ++it) {
-                const uint32_t s = it % ST, ph = (it / ST) & 1u, acc = it & 1u;
-                if (!mbar_wait(drained + 8 * acc, ((it >> 1) & 1u) ^ 1u, abort_flag) || !mbar_wait(full + 8 * s, ph, abort_flag)) { failed = true; break; }
+                const uint32_t s = it % ST, ph = (it / ST) & 1u, acc = it % S::kBuffers;
+                if (!mbar_wait(drained + 8 * acc, ((it / S::kBuffers) & 1u) ^ 1u, abort_flag) || !mbar_wait(full + 8 * s, ph, abort_flag)) { failed = true; break; }
                 tc_fence_after_sync();
-                const uint32_t a0 = base + s * S::kStageBytes, b0 = a0 + S::kParts * WP_A_PART;
+                const uint32_t a0 = base + s * S::kStageBytes, b0 = a0 + S::kParts * WP_A_PART, d = tmem_base + acc * S::kAccCols;
 #pragma unroll
-                for (int p = S::kParts - 1; p >= 0; --p)              // the small parts first
+                for (int p = S::kParts - 1; p >= 0; --p)
 #pragma unroll
-                    for (int j = 0; j < WP_K / 16; ++j)
-                        umma_bf16(tmem_base + (acc * S::kSets + j * S::kSets / 4) * S::kAccCols, umma_smem_desc(a0 + p * WP_A_PART + j * 2048, WP_SLAB, 1024),
-                                  umma_smem_desc(b0 + j * 2048, WP_SLAB, 1024), idesc, p != S::kParts - 1 || j % (4 / S::kSets) != 0);
+                    for (int j = 0; j < WP_K / 16; ++j) {
+                        const bool more = p != S::kParts - 1 || j != 0;
+                        const uint64_t a = umma_smem_desc(a0 + p * WP_A_PART + j * 2048, WP_SLAB, 1024);
+                        if (S::kZParts == 3) umma_bf16(d + S::kTailCol, a, umma_smem_desc(b0 + j * 2048, WP_SLAB, 1024), idesc_tail, more);
+                        umma_bf16(d + (p == 0 ? j * MP : S::kSideCol), a, umma_smem_desc(b0 + S::kHeadSlab * WP_SLAB + j * 2048, WP_SLAB, 1024), idesc_head,
+                                  p != 0 && more);
+                    }
                 umma_commit(done + 8 * s);
             }
             if (failed) *abort_flag = 1;
@@ -326,36 +341,59 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
     } else {
         // ------------------------------------------------ sums: lane = column o of dY
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
-        float sum[MP];
+        float sum[MP], rest[MP];
+        float* shared_rest = reinterpret_cast<float*>(tail + 128) + threadIdx.x;
 #pragma unroll
-        for (int m = 0; m < MP; ++m) sum[m] = 0.f;
+        for (int m = 0; m < MP; ++m) {
+            sum[m] = rest[m] = 0.f;
+            if (S::kRestsInSmem) shared_rest[m * WP_O] = 0.f;
+        }
         uint32_t it = 0;
         for (int n = n_begin; n < n_end; n += WP_K, ++it) {
-            const uint32_t s = it % ST, ph = (it / ST) & 1u, acc = it & 1u;
+            const uint32_t s = it % ST, ph = (it / ST) & 1u, acc = it % S::kBuffers;
             if (!mbar_wait_warp(done + 8 * s, ph, abort_flag, 32)) { failed = true; break; }
             tc_fence_after_sync();
 #pragma unroll
-            for (int m = 0; m < MP; m += 8) {                        // a stage's accumulators and parts first, then one rounding of the sum
-                float stage_sum[8];
+            for (int m = 0; m < MP; m += 8) {                        // what a stage brings first, then one rounding of the sum
+                const uint32_t at = taddr + acc * S::kAccCols + m;
+                float head[8];
 #pragma unroll
-                for (int i = 0; i < S::kSets; ++i) {
-                    const uint32_t at = taddr + (acc * S::kSets + i) * S::kAccCols + m;
-                    uint32_t h[8], mid[8] = {}, l[8] = {};
-                    tmem_ld_32x8(at, h);
-                    if (S::kZParts == 3) {
-                        tmem_ld_32x8(at + MP, mid);
-                        tmem_ld_32x8(at + 2 * MP, l);
-                    }
+                for (int j = 0; j < WP_K / 16; j += 2) {
+                    uint32_t x[8], y[8];
+                    tmem_ld_32x8(at + j * MP, x);
+                    tmem_ld_32x8(at + (j + 1) * MP, y);
                     tmem_ld_wait();
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        float f = __uint_as_float(h[e]);
-                        if (S::kZParts == 3) f += __uint_as_float(mid[e]) + __uint_as_float(l[e]);
-                        stage_sum[e] = i == 0 ? f : stage_sum[e] + f;
+                        const float f = __uint_as_float(x[e]) + __uint_as_float(y[e]);
+                        head[e] = j == 0 ? f : head[e] + f;
+                    }
+                }
+                if (S::kAccCols > S::kTailCol) {
+                    uint32_t mid[8] = {}, l[8] = {}, side[8] = {};
+                    if (S::kZParts == 3) {
+                        tmem_ld_32x8(at + S::kTailCol, mid);
+                        tmem_ld_32x8(at + S::kTailCol + MP, l);
+                    }
+                    if (S::kParts == 3) tmem_ld_32x8(at + S::kSideCol, side);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        float f = S::kZParts == 3 ? __uint_as_float(mid[e]) + __uint_as_float(l[e]) : 0.f;
+                        if (S::kParts == 3) f += __uint_as_float(side[e]);
+                        head[e] += f;
                     }
                 }
 #pragma unroll
-                for (int e = 0; e < 8; ++e) sum[m + e] += stage_sum[e];
+                for (int e = 0; e < 8; ++e) {
+                    if (S::kRests) {
+                        const float next = sum[m + e] + head[e];
+                        (S::kRestsInSmem ? shared_rest[(m + e) * WP_O] : rest[m + e]) += head[e] - (next - sum[m + e]);
+                        sum[m + e] = next;
+                    } else {
+                        sum[m + e] += head[e];
+                    }
+                }
             }
             tc_fence_before_sync();
             __syncwarp();
@@ -366,6 +404,7 @@ wg_parts_kernel(const __grid_constant__ CUtensorMap tmY, const YT* dY, int64_t l
         SplitOutputCheck check;
 #pragma unroll
         for (int m = 0; m < MP; ++m) {
+            if (S::kRests) sum[m] += S::kRestsInSmem ? shared_rest[m * WP_O] : rest[m];
             if (o < O && m < M) {
                 out[m] = sum[m];
                 check.add(sum[m]);

@@ -109,3 +109,18 @@ def test_very_small_operands(vl, guard, dtype, pad, ey, ez, where):
     if ey + ez > -100:
         for part in (slice(None), (slice(None), 8) if small is Z else 8):
             assert float((P[part].double() - ref[part]).norm() / ref[part].norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("dtype,pad", [(torch.bfloat16, 1), (torch.float32, 0)])
+@pytest.mark.parametrize("z_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("M", [12, 24])
+@pytest.mark.parametrize("what", ["magnitudes", "offset"])
+def test_products_of_one_sign_add_up_as_fp32_sums_do(vl, guard, dtype, pad, z_dtype, M, what):
+    """Sums that truncate show on products of one sign, where sums that round to nearest err by little more than their last rounding: 2^-24
+    in norm (4.6e-8 to 5.3e-8 for fp32 multiply-adds in slices, any of these inputs)."""
+    dY, Z = _inputs(12608, 768, M, dtype, z_dtype, pad, 0, 4)
+    for t in (dY, Z):
+        t.copy_(t.abs() if what == "magnitudes" else t + 1.0)
+    P = vl.velora_weight_grad_p(dY, Z, 32 * M, 32)
+    ref = dY.double().T @ Z.double()
+    assert float((P.double() - ref).norm() / ref.norm()) <= 2.0 ** -24
