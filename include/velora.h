@@ -50,8 +50,8 @@
  *     into the workspace first, where it has the room (VELORA_OP_ANY_ROWS).  Without it and in
  *     velora_dense_product, the CUDA-core GEMM runs.  fp32 products run on the tensor cores as bf16 parts, with an
  *     error no larger than that of fp32 multiply-adds in sequence, or where they are small on the CUDA cores.
- *     The factored weight gradient of such bf16 rows takes Z as stored and adds up in fp32, on tensor or CUDA
- *     cores; on aligned rows of more than 64 columns it rounds an fp32 Z to bf16 for the tensor cores.
+ *     The factored weight gradient of such bf16 rows and of fp32 rows takes Z as stored and adds up in fp32 or, on the
+ *     tensor cores, with no larger an error; on aligned bf16 rows of more than 64 columns it rounds an fp32 Z to bf16 for the tensor cores.
  */
 #ifndef VELORA_H
 #define VELORA_H

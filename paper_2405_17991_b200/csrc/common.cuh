@@ -53,10 +53,11 @@ inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 //   griddepcontrol.wait  waits for the kernel before, all of whose CTAs are resident or done when this one starts (each has
 //                        triggered): nothing that this kernel occupies can keep it from ending.
 //   tcgen05.alloc        never finds TMEM short.  Every kernel that allocates TMEM takes more than half of an SM's 228 KB of shared
-//                        memory and so has an SM to itself among them (products 210 KB or more, adapter forward 222 KB; the fp32 product 162 KB or more),
+//                        memory and so has an SM to itself among them (products 210 KB or more, adapter forward 222 KB; the fp32 product 162 KB or more, and every register),
 //                        but for wg_kernel, of which two CTAs fit (96 KB or more each) with at most 256 of the 512 columns each.
-//                        wg_parts_kernel (41 KB or more, as many columns as its CTAs on an SM can share) is launched the ordinary way
-//                        and lets nothing in before its end; CTAs of other streams wait for columns of kernels that end by themselves.
+//                        wg_parts_kernel (49 KB or more) has as many CTAs on an SM as its registers allow, two for a bf16 dY with at
+//                        most 256 columns each, one for fp32.  It is launched the ordinary way and lets nothing in before its end;
+//                        CTAs of other streams wait for columns of kernels that end by themselves.
 //   cluster barriers     all CTAs of a cluster are placed together, and each reaches both barriers whatever happened before.
 // What such a kernel reads is still being written while it is resident, so none of it may go through the read-only path:
 // neither __ldg nor ld.global.nc, and no `const __restrict__` on its inputs, of which the compiler makes the same loads (a line

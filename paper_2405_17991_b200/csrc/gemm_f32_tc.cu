@@ -7,12 +7,13 @@
 // their sum is not left to grow: after every k-block the accumulator is read out and added, rounded to nearest, to sums in
 // registers.  Error in norm against 64 bits, 2048 x 2048 outputs, this form / fp32 multiply-adds in sequence:
 //   K = 64: 0.8e-7 / 1.4e-7,  K = 768: 1.0e-7 / 5.0e-7,  K = 3072: 1.5e-7 / 9.9e-7
-// (accumulators read out every 128 instead of every 64: 5.9e-7 at any K).
+// (accumulators read out every 128 instead of every 64: 5.9e-7 at any K), and on |N(0, 1)|, whose products are all of one sign,
+//   K = 64: 0.9e-7 / 1.2e-7,  K = 768: 1.0e-7 / 3.7e-7,  K = 3072: 1.3e-7 / 7.4e-7.
 //
 // CTA pairs (cta_group::2), 256 x BN outputs a pair, BN = 192 (or 96).  12608 x 768, K = 768: 97 us, 153 TFLOP/s of fp32 arithmetic
-// (372 us on the CUDA cores).  Bound by the shared-memory pipe: a k-block's 24 products read 172 KB of operands, the split
-// writes 86 KB and its loads pass 114 KB through, 2900 cycles of 128 bytes where the tensor cores need 2310; the block takes
-// 3400.  Registers decide the split of roles: 12 warps of sums with 64 columns each, so few registers for the operand warps that
+// (372 us on the CUDA cores).  Nearest to a limit by count is shared memory: a k-block's 24 products read 172 KB of operands, the
+// split writes 86 KB and its loads pass 114 KB through, 2900 cycles of 128 bytes where the tensor cores need 2310; the block takes
+// 3400 (over the whole launch the tensor pipe is busy for 51 % of the cycles, the schedulers issue in 52 %).  Registers decide the split of roles: 12 warps of sums with 64 columns each, so few registers for the operand warps that
 // only A of the next k-block waits in them (both operands, and spills: 115 us; eight operand warps: 101).
 //
 // Roles per CTA (1024 threads):
