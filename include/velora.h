@@ -110,7 +110,8 @@ const char* velora_status_string(int status);
 /*
  * Bytes of device workspace the given entry point needs for these sizes
  * (0 if it needs none).  Independent of pointer values; deterministic.  Calls that may be in flight at the same
- * time (on two streams) must not share a workspace.
+ * time (on two streams) must not share a workspace.  A workspace for the widest layer and the longest batch serves the others.  The
+ * factored gradient of up to 1152 outputs also runs in less, with fewer splits of its tokens.
  * With op | VELORA_OP_ANY_ROWS the figure includes, where D or O is no multiple of 8, room for aligned copies of the
  * bf16 operands of that width (X and W of the forward, dY and W of the backward): worth it for rows that are not
  * 16-byte aligned, which run on the CUDA cores without it, and for nothing else (padded rows and fp32 never use it).

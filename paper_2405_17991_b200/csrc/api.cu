@@ -60,10 +60,11 @@ size_t xhat_bytes(int64_t N, int64_t D)
     return kStatusBytes + align256(static_cast<size_t>(N) * round_up8(D) * 4);
 }
 
-size_t factored_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
+// What a call needs, or (`ask`) what velora_workspace_bytes reports: room for the form that is fastest.
+size_t factored_bytes(int64_t N, int64_t D, int64_t O, int Dsub, bool ask = false)
 {
     const size_t simt = align256(static_cast<size_t>(O) * num_subtokens(D, Dsub) * sizeof(float));
-    const size_t tc = weight_grad_tc_workspace_bytes(N, D, O, Dsub);
+    const size_t tc = weight_grad_tc_workspace_bytes(N, D, O, Dsub, ask);
     const size_t skinny = weight_grad_skinny_workspace_bytes(N, D, O, Dsub);
     const size_t most = simt > tc ? simt : tc;
     return kStatusBytes + (most > skinny ? most : skinny);
@@ -256,9 +257,9 @@ size_t velora_workspace_bytes(int op, int64_t N, int64_t D, int64_t O, int Dsub)
     const bool any_rows = (op & VELORA_OP_ANY_ROWS) != 0;
     switch (op & ~VELORA_OP_ANY_ROWS) {
         case VELORA_OP_INIT_V: return init_v_workspace_bytes(Dsub);
-        case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub);
+        case VELORA_OP_WEIGHT_GRAD_FACTORED: return O < 1 ? 0 : factored_bytes(N, D, O, Dsub, true);
         case VELORA_OP_LINEAR_BACKWARD_FACTORED:
-            return O < 1 ? 0 : factored_bytes(N, D, O, Dsub) + pack_bytes_if_ragged(N, O, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
+            return O < 1 ? 0 : factored_bytes(N, D, O, Dsub, true) + pack_bytes_if_ragged(N, O, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
         case VELORA_OP_WEIGHT_GRAD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O, any_rows);
         case VELORA_OP_LINEAR_BACKWARD_EXPLICIT: return xhat_bytes(N, D) + pack_bytes_if_ragged(N, O, any_rows) + pack_bytes_if_ragged(O, D, any_rows);
         case VELORA_OP_LINEAR_FORWARD: return kStatusBytes + pack_bytes_if_ragged(N, D, any_rows) + pack_bytes_if_ragged(O, D, any_rows);

@@ -453,8 +453,8 @@ SkinnyPlan skinny_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count, 
     int64_t max_parts = 512;
     if (O > SK_MAX_O) {
         // Wide layers: as many slices as fill the chip over all column blocks and as the tensor-core form's
-        // workspace holds (the size that velora_workspace_bytes reports for them).
-        const int64_t bytes = static_cast<int64_t>(weight_grad_tc_workspace_bytes(N, D, O, Dsub)) - 512;   // two roundings to 256
+        // workspace holds at the least.
+        const int64_t bytes = static_cast<int64_t>(weight_grad_tc_workspace_bytes(N, D, O, Dsub, false)) - 512;   // two roundings to 256
         const int64_t room = bytes / static_cast<int64_t>(sizeof(float) * O * M) - 1;                       // and P itself
         // Four CTAs per SM.  Up to 32 sub-tokens go to the tensor cores (weight_grad_parts.cu), in one wave of slices of 192 tokens or more
         // (three stages: filling and emptying such a CTA costs several microseconds), where that gives every other SM one.

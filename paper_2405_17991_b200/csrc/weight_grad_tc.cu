@@ -383,10 +383,11 @@ struct WgPlan {
     int M, npad, pitch, n_slabs, tmem_cols, kblocks, splits, kb_per_split, tiles_o, stages, tail_off;
     bool after_conversion;    // the launch follows z_to_bf16_kernel in the stream
     bool fat;                 // one CTA of twelve warps per SM instead of two CTAs of six
-    size_t zb_bytes, part_bytes, smem;
+    bool narrow;              // may be cut into sixteen splits
+    size_t zb_bytes, part_bytes, narrow_bytes, ask_bytes, smem;
 };
 
-WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
+WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count, bool narrow_room)
 {
     WgPlan p{};
     const int64_t M = ceil_div64(D, Dsub);
@@ -424,9 +425,11 @@ WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
     int best = 1;
     double best_eff = 0.0;
     // Where even eight splits would keep half of the SMs idle, up to sixteen through the workspace, of four k-blocks or more
-    // (8192 x 512 -> 512: the partial products take 6 us instead of 9).  By a fixed count of SMs, as the room is asked for without a device.
-    const bool narrow = p.npad <= WG_NARROW_PAD && O <= WG_NARROW_O && p.kblocks >= 8 * WG_MAX_SPLITS;
-    const int most = narrow ? 2 * WG_MAX_SPLITS : WG_MAX_SPLITS;
+    // (8192 x 512 -> 512: the partial products take 6 us instead of 9), if it has the room.  By a fixed count of SMs, as room is asked for
+    // without a device.
+    const bool long_range = p.kblocks >= 8 * WG_MAX_SPLITS;
+    p.narrow = p.npad <= WG_NARROW_PAD && O <= WG_NARROW_O && long_range;
+    const int most = p.narrow && narrow_room ? 2 * WG_MAX_SPLITS : WG_MAX_SPLITS;
     for (int s = 1; s <= most && s <= p.kblocks; ++s) {
         const int64_t ctas = static_cast<int64_t>(p.tiles_o) * s;
         const int64_t waves = ceil_div64(ctas, slots);
@@ -436,13 +439,11 @@ WgPlan make_plan(int64_t N, int64_t D, int64_t O, int Dsub, int sm_count)
     p.kb_per_split = static_cast<int>(ceil_div64(p.kblocks, best));
     p.splits = static_cast<int>(ceil_div64(p.kblocks, p.kb_per_split));
     p.zb_bytes = static_cast<size_t>(round_up(static_cast<int64_t>(N) * p.pitch * 2, 256));
-    // Room for the partial products: never less for a wider layer or more tokens, so that a workspace sized for the largest layer serves all.
-    size_t part_values = static_cast<size_t>(WG_MAX_SPLITS) * static_cast<size_t>(O) * p.npad;
-    if (p.kblocks >= 8 * WG_MAX_SPLITS) {
-        const size_t narrow_values = 2 * WG_MAX_SPLITS * static_cast<size_t>(O < WG_NARROW_O ? O : WG_NARROW_O) * (p.npad < WG_NARROW_PAD ? p.npad : WG_NARROW_PAD);
-        if (narrow_values > part_values) part_values = narrow_values;
-    }
-    p.part_bytes = part_values * sizeof(float);
+    const auto partials = [](int splits, int64_t rows, int pad) { return static_cast<size_t>(splits) * static_cast<size_t>(rows) * pad * sizeof(float); };
+    p.part_bytes = partials(WG_MAX_SPLITS, O, p.npad);
+    p.narrow_bytes = partials(2 * WG_MAX_SPLITS, O < WG_NARROW_O ? O : WG_NARROW_O, p.npad < WG_NARROW_PAD ? p.npad : WG_NARROW_PAD);
+    // Asked for: never less for a wider layer or more tokens, so that a workspace sized for the largest layer serves all.
+    p.ask_bytes = long_range && p.narrow_bytes > p.part_bytes ? p.narrow_bytes : p.part_bytes;
     p.ok = true;
     return p;
 }
@@ -486,11 +487,11 @@ int launch_wg(const CUtensorMap& tmY, const CUtensorMap& tmZ, const WgArgs& a, c
 
 }  // namespace
 
-size_t weight_grad_tc_workspace_bytes(int64_t N, int64_t D, int64_t O, int Dsub)
+size_t weight_grad_tc_workspace_bytes(int64_t N, int64_t D, int64_t O, int Dsub, bool ask)
 {
-    const WgPlan p = make_plan(N > 0 ? N : 1, D, O, Dsub, 148);
+    const WgPlan p = make_plan(N > 0 ? N : 1, D, O, Dsub, 148, false);
     if (!p.ok) return 0;
-    return p.zb_bytes + static_cast<size_t>(round_up(static_cast<int64_t>(p.part_bytes), 256));
+    return p.zb_bytes + static_cast<size_t>(round_up(static_cast<int64_t>(ask ? p.ask_bytes : p.part_bytes), 256));
 }
 
 int launch_weight_grad_tc(const void* dY, int dy_dtype, int64_t N, int64_t O, int64_t lddy,
@@ -504,9 +505,12 @@ int launch_weight_grad_tc(const void* dY, int dy_dtype, int64_t N, int64_t O, in
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc != VELORA_OK) return rc;
-    const WgPlan p = make_plan(N, D, O, Dsub, di.sm_count);
+    WgPlan p = make_plan(N, D, O, Dsub, di.sm_count, false);
     if (!p.ok) return VELORA_ERR_UNSUPPORTED;
-    if (ws_bytes < weight_grad_tc_workspace_bytes(N, D, O, Dsub) || !aligned16(ws)) return VELORA_ERR_WORKSPACE;
+    if (ws_bytes < weight_grad_tc_workspace_bytes(N, D, O, Dsub, false) || !aligned16(ws)) return VELORA_ERR_WORKSPACE;
+    // The room behind the least may hold copies that the call has made of its products' operands: those have been read, since nothing
+    // here starts before the products have ended.
+    if (p.narrow && ws_bytes >= p.zb_bytes + p.narrow_bytes) p = make_plan(N, D, O, Dsub, di.sm_count, true);
     if (p.smem > static_cast<size_t>(di.smem_optin)) return VELORA_ERR_UNSUPPORTED;
 
     uint4* Zb = static_cast<uint4*>(ws);

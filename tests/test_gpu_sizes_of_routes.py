@@ -109,6 +109,28 @@ def test_narrow_layers_gradient_of_many_splits(vl, guard, N, D, O, Dsub, z_dtype
     assert_matches(P, P64.cpu().numpy(), TOL_GEMM, "P", c=c)
 
 
+@pytest.mark.parametrize("N,D,O,Dsub", [(4159, 512, 512, 64), (8192, 515, 1152, 64)])
+def test_narrow_layers_gradient_in_the_room_of_eight_splits(vl, guard, N, D, O, Dsub):
+    """Half of the partial products' room is enough, with copies of the other product's operands behind it or without."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(N)
+    M = vl.num_subtokens(D, Dsub)
+    dY = torch.randn((N, O), generator=gen, device=DEV).bfloat16()
+    W = torch.randn((O, D), generator=gen, device=DEV).bfloat16()
+    Z = torch.randn((N, M), generator=gen, device=DEV).bfloat16()
+    v = torch.randn(Dsub, generator=gen, device=DEV)
+    ref = ((dY.double().T @ Z.double())[:, :, None] * v.double()).reshape(O, M * Dsub)[:, :D]
+    dX_ref = dY.double() @ W.double()
+    full = vl.velora_workspace_bytes(vl.OP_LINEAR_BACKWARD_FACTORED, N, D, O, Dsub)
+    for need in (full, full - 8 * O * 16 * 4):
+        ws = guard.workspace(vl, need)
+        for _ in range(2):
+            dX, dW = vl.velora_linear_backward(dY, W, Z, v, dX=guard.mat(N, D), dW=guard.mat(O, D), ws=ws)
+            assert_matches(dX, dX_ref.cpu().numpy(), TOL_GEMM, "dX")
+            assert_matches(dW, ref.cpu().numpy(), TOL_GEMM, "dW")
+        assert vl.velora_workspace_status(ws) == 0
+
+
 def test_kernels_with_tensor_memory_on_two_streams(vl):
     """fp32 products beside partial factors and bf16 products, none of which waits for another: what each computes alone, bit for bit."""
     gen = torch.Generator(device=DEV)
