@@ -10,7 +10,8 @@ from cache between steps.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints one JSON line (rank 0).  ``--impl reference`` times the fp64 CPU oracle on a bounded sample.
+Prints one JSON line (rank 0) on stdout, a few KB at most, and the tables behind it (every kernel and shape, timed three ways) as
+JSON lines on stderr.  ``--impl reference`` times the fp64 CPU oracle on a bounded sample.
 """
 from __future__ import annotations
 
@@ -203,6 +204,35 @@ def run_reference(args):
     print(json.dumps(line))
 
 
+def rounded(x):
+    """The same with six significant digits."""
+    if isinstance(x, float):
+        return float("%.6g" % x)
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+LINE_TABLES = ("timing_floor_us", "compress", "reconstruct", "weight_grad_factored")     # of the roofline object: one column each on stdout
+
+
+def emit(line):
+    """The line on stdout and its tables on stderr: with them in it (19 KB) it no longer fits what keeps the end of a program's output."""
+    line = rounded(line)
+    for row in line.pop("kernels", []):
+        print(json.dumps({"table": "kernels", **row}), file=sys.stderr)
+    roofline = line["roofline"]
+    for name in LINE_TABLES:
+        table = roofline.pop(name, None)
+        if table is None:
+            continue
+        print(json.dumps({"table": name, "rows": table}), file=sys.stderr)
+        if isinstance(table, list):
+            roofline[name + "_us"] = {"%s/%s" % (r["shape"], r["Dsub"]): r.get("us_graph", r["us"]) for r in table}
+    sys.stderr.flush()
+    print(json.dumps(line), flush=True)
+
+
 def workload_config(cfg):
     if cfg.index == 5:
         layers = "7 projections (q,k,v,o 4096x4096; up,gate 4096x11008; down 11008x4096)"
@@ -370,8 +400,7 @@ def run_ours(args):
                 "fwd_ms_per_step": fwd_ms / args.steps, "bwd_ms_per_step": bwd_ms / args.steps}
     overhead = {"velora_ms_per_step": elapsed_ms / args.steps, "plain_ms_per_step": plain_ms,
                 "velora_over_plain": (elapsed_ms / args.steps) / plain_ms,
-                "plain": "the same layers without the method: Y = X W^T, dX = dY W, dW = dY^T X (dense), X kept",
-                "paper": "Table 7 reports VeLoRA 4-9 % slower than full fine-tuning (other hardware, whole model)"}
+                "plain": "the same layers without the method: dense dW = dY^T X, X kept"}
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": max(args.warmup, 3),
@@ -422,7 +451,7 @@ def run_ours(args):
                               "every buffer so that nothing is found in L2"}
         if rank == 0:
             line["roofline"]["traffic"] = None         # the capture behind the ratio was taken on configuration 5
-            print(json.dumps(line))
+            emit(line)
         if world > 1:
             dist.destroy_process_group()
         return
@@ -523,8 +552,8 @@ def run_ours(args):
             set_oracle_threads(threads)
             line["cpu_baseline"]["single_thread"] = {
                 "value": CPU_SINGLE_TOKENS / t_one, "unit": UNIT, "cores": 1,
-                "sample": cpu_sample_text(CPU_SINGLE_TOKENS) % N + "; one pass, %.1f s" % t_one}
-        print(json.dumps(line))
+                "sample": "the same, first %d tokens, one pass, %.1f s" % (CPU_SINGLE_TOKENS, t_one)}
+        emit(line)
     if world > 1:
         dist.destroy_process_group()
 
